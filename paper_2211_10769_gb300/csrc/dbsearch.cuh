@@ -16,21 +16,36 @@
 // lane holds more rows of a short query and the skew of a wavefront is 15
 // steps rather than 31.  The query profile (int8, S + open, all passes) sits in
 // shared memory; the two residues' score bytes are merged into one packed
-// register with a single prmt.  The cell update is the pairwise one in
-// __viaddmax_s16x2 / __viaddmax_s16x2_relu form.
+// register with a single prmt.
+//
+// Cell update.  The kernel is bound by the ALU pipe (DPX, prmt, min/max: 64
+// lanes a clock and SM); plain 32-bit adds can run on the otherwise idle FMA
+// pipe.  A plain add or subtract moves two 16-bit halves at once as long as
+// the low half neither carries nor borrows, so the values are kept in a form
+// in which the two subtractions of a cell never borrow:
+//   U = H (>= 0);  E and F stored as E + open and F + open;  X = max(H(i-1,j-1) + S, E, 0)
+//   E  <- vimax3(E - extend, U, open)        E floored at 0: X has that floor, so H is unchanged,
+//                                            and E + open >= open >= extend, so no borrow
+//   X  <- viaddmax(U(i-1,j-1), S + open, E)  stored as X + open, at least open
+//   X - open                                 a plain subtraction, no borrow
+//   H  <- viaddmax(F, -open, X),  F of the next row <- viaddmax(F, -extend, X)
+// Four ALU operations a cell pair instead of five (the zero floor as a relu on
+// X, and X - open as a packed add on the ALU pipe); with the profile's prmt
+// and half a vimax3 for the running maximum 5.5 instead of 6.5.
+// 500,000 subjects, m = 1,000: 36.7 -> 33.6 ms (4,930 -> 5,382 GCUPS); m = 144:
+// 5.78 -> 5.25 ms.  (The subtractions as explicit IMADs: 34.7 ms.)
 //
 // Exactness of 16-bit lanes: every H value is exact while all H values of
-// the subject stay <= T = 32767 - max(S) (the largest intermediate is
-// H + S, E and F never drop below -open - extend - 16384).  The first cell
-// whose H exceeds T is still exact and raises the running maximum above T,
-// so a subject whose maximum exceeds T is flagged and rescored in 32 bits;
-// all other scores are exact.
+// the subject stay <= T = 32767 - max(S) - open (the largest intermediate is
+// H + S + open).  The first cell whose H exceeds T is still exact and raises
+// the running maximum above T, so a subject whose maximum exceeds T is
+// flagged and rescored in 32 bits; all other scores are exact.  A saturated
+// subject cannot disturb the other half: E and X stay >= open in any case
+// (signed maxima with open and E), so the subtractions never borrow.
 #pragma once
 #include "sw_device.cuh"
 
 namespace swgb {
-
-constexpr int kNeg16 = -16384;
 
 struct DbJob {
     const uint8_t *q;          // query codes (device)
@@ -167,8 +182,8 @@ __device__ __forceinline__ void load_prof_words(const int8_t *p, uint32_t (&w)[d
 // mpad = passes * 32 * db_lane_slot(R) (lane slots of whole words).
 constexpr int kDbCH = 8;      // steps per chunk of the packed fill (steady chunks skip all range tests)
 
-// Per-lane state of the packed fill: U = H - open and E of the lane's R query
-// rows for both subjects (16-bit halves), the bottom row's (U, F) of the
+// Per-lane state of the packed fill: U = H and E + open of the lane's R query
+// rows for both subjects (16-bit halves), the bottom row's (H, F + open) of the
 // previous step, the diagonal, the running maximum, and the prefetched
 // residue pair / top cell of the next step.
 template <int R>
@@ -186,7 +201,7 @@ struct DbLane {
 template <int R, int G, bool CHECK>
 __device__ __forceinline__ void db_step(DbLane<R> &st, int s, int gl, int n, const uint16_t *pr, uint2 *bnd,
                                         bool tops, bool last, int K, int mpad,
-                                        unsigned nge2, unsigned ngo2, unsigned neg2)
+                                        unsigned nge2, unsigned ngo2, unsigned ge2, unsigned go2)
 {
     const int j = s - gl;
     unsigned uup = __shfl_up_sync(kFull, st.ub, 1, G);
@@ -195,7 +210,7 @@ __device__ __forceinline__ void db_step(DbLane<R> &st, int s, int gl, int n, con
     // inputs of the next step
     const int jn = j + 1;
     unsigned cpn;
-    uint2 topn = make_uint2(ngo2, neg2);
+    uint2 topn = make_uint2(0u, 0u);
     if (CHECK) {
         cpn = (jn >= 0 && jn <= n) ? pr[jn] : 0xffffu;
         if (tops && s + 1 < n) topn = bnd[s + 1];
@@ -214,14 +229,13 @@ __device__ __forceinline__ void db_step(DbLane<R> &st, int s, int gl, int n, con
         for (int r = 0; r < R; ++r) {
             const unsigned sp = merge_row(wa, wb, r);
             const unsigned uold = st.U[r];
-            const unsigned e = __viaddmax_s16x2(st.E[r], nge2, uold);
-            const unsigned x = __viaddmax_s16x2_relu(udiag, sp, e);
-            const unsigned xgo = __viaddmax_s16x2(x, ngo2, neg2);   // x - open
-            const unsigned u = __viaddmax_s16x2(f, ngo2, xgo);      // H - open
+            const unsigned e = __vimax3_s16x2(st.E[r] - ge2, uold, go2);        // E + open, at least open
+            const unsigned x = __viaddmax_s16x2(udiag, sp, e) - go2;            // X
+            const unsigned u = __viaddmax_s16x2(f, ngo2, x);                    // H = max(F, X)
             st.E[r] = e;
             udiag = uold;
             st.U[r] = u;
-            if (r + 1 < R) f = __viaddmax_s16x2(f, nge2, xgo);
+            if (r + 1 < R) f = __viaddmax_s16x2(f, nge2, x);                    // F + open of the next row
         }
         st.ub = st.U[R - 1];
         st.fb = f;
@@ -278,13 +292,13 @@ db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
 
         int maxs = 0;
         for (int k = 0; k < K * K; ++k) maxs = max(maxs, (int)SC.mat[k]);
-        const int tmax_u = 32767 - maxs - go;            // overflow threshold on H - open
+        const int tmax = 32767 - maxs - go;              // overflow threshold on H
         const int lane = threadIdx.x & 31;
         const int gl = lane & (G - 1), grp = lane / G;          // the lane's wavefront and its place there
         const int gwarp = slot * W + (threadIdx.x >> 5);
         uint2 *bnd = scratch + ((size_t)gwarp * NG + grp) * (size_t)(D.maxlen + 1);
         const unsigned go2 = pack2(go, go), ge2 = pack2(ge, ge);
-        const unsigned ngo2 = pack2(-go, -go), nge2 = pack2(-ge, -ge), neg2 = pack2(kNeg16, kNeg16);
+        const unsigned ngo2 = pack2(-go, -go), nge2 = pack2(-ge, -ge);
 
         for (;;) {
             // the warp takes NG consecutive pairs (similar lengths: the pairs are sorted), one per wavefront
@@ -314,29 +328,29 @@ db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
                 nmax = max(n, o);
                 nmin = min(n, o);
             }
-            unsigned cmax = ngo2;                                   // running max of H - open (H = 0)
+            unsigned cmax = 0;                                      // running max of H
             for (int pass = 0; pass < passes; ++pass) {
                 DbLane<R> st;
                 st.prow = prof + pass * PROWS + gl * LS;
     #pragma unroll
-                for (int r = 0; r < R; ++r) { st.U[r] = ngo2; st.E[r] = neg2; }
-                st.ub = ngo2; st.fb = neg2; st.udiag0 = ngo2;
+                for (int r = 0; r < R; ++r) { st.U[r] = 0; st.E[r] = go2; }    // H = 0; E = 0 never shows
+                st.ub = 0; st.fb = 0; st.udiag0 = 0;                           // F = -open: F(1) = max(-inf, H - open)
                 st.cmax = cmax;
                 const bool last = pass + 1 == passes;
                 const bool tops = pass > 0;
                 // prefetched inputs of this lane's first column and of lane 0's first top cell
                 st.cp = gl == 0 && n > 0 ? pr[0] : 0xffffu;
-                st.topv = (tops && n > 0) ? bnd[0] : make_uint2(ngo2, neg2);
+                st.topv = (tops && n > 0) ? bnd[0] : make_uint2(0u, 0u);
                 for (int s0 = 0; s0 < nmax + G - 1; s0 += kDbCH) {
                     if (s0 >= G - 1 && s0 + kDbCH <= nmin) {
                         // steady state: every lane's column is inside its pair, the prefetched
                         // column at most the padding column n
     #pragma unroll
                         for (int k = 0; k < kDbCH; ++k)
-                            db_step<R, G, false>(st, s0 + k, gl, n, pr, bnd, tops, last, K, mpad, nge2, ngo2, neg2);
+                            db_step<R, G, false>(st, s0 + k, gl, n, pr, bnd, tops, last, K, mpad, nge2, ngo2, ge2, go2);
                     } else {
                         for (int k = 0; k < kDbCH && s0 + k < nmax + G - 1; ++k)
-                            db_step<R, G, true>(st, s0 + k, gl, n, pr, bnd, tops, last, K, mpad, nge2, ngo2, neg2);
+                            db_step<R, G, true>(st, s0 + k, gl, n, pr, bnd, tops, last, K, mpad, nge2, ngo2, ge2, go2);
                     }
                 }
                 cmax = st.cmax;
@@ -355,12 +369,12 @@ db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
                 for (int h = 0; h < 2; ++h) {
                     const int s = outs[h];
                     if (s < 0) continue;
-                    if (mx[h] > tmax_u) {
+                    if (mx[h] > tmax) {
                         J.scores[s] = -1;
                         const int slot = atomicAdd(J.novf, 1);
                         J.ovf[slot] = s;
                     } else {
-                        J.scores[s] = max(0, mx[h] + go);
+                        J.scores[s] = mx[h];
                     }
                 }
             }

@@ -117,6 +117,27 @@ def test_saturating_subjects_are_rescored(ctx, oracle_mod):
     assert (want > 32767 - 11).sum() >= 10
 
 
+@pytest.mark.parametrize("go,ge", [(0, 0), (1, 1), (10, 1), (11, 11), (60, 2), (110, 110)])
+def test_half_beside_a_saturated_one(ctx, oracle_mod, go, ge):
+    """A saturating subject in either half of a packed pair leaves its
+    neighbour's score exact (the halves share plain 32-bit subtractions), and
+    so do scores just below and above the flagging threshold."""
+    S = W.blosum62()
+    Wc = W.PROTEIN_ALPHABET.index("W")
+    q = np.full(3100, Wc, np.uint8)
+    q[np.arange(0, 3100, 150)] = 0
+    subjects = [q.copy(), W.random_protein(3100, W.BASE_SEED + 781),           # low half saturates
+                W.random_protein(3090, W.BASE_SEED + 782), q[:3090].copy()]    # high half saturates
+    # runs of W around (32767 - 11 - go) / 11 residues: on both sides of the threshold
+    edge = (32767 - 11 - go) // 11
+    q2 = np.full(edge + 6, Wc, np.uint8)
+    runs = [np.full(edge + d, Wc, np.uint8) for d in (-2, -1, 0, 1, 2, 3)]
+    for query, subj in ((q, subjects), (q2, runs)):
+        want = oracle_mod.db_scores(query, subj, S, go, ge)
+        hits, scores = _db(ctx, subj).search(query, S, go, ge, k=4, all_scores=True)
+        assert scores.tolist() == want.tolist()
+
+
 def test_degenerate_databases(ctx, oracle_mod):
     sc = W.protein_scoring()
     q = W.random_protein(200, W.BASE_SEED + 760)
