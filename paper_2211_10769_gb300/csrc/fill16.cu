@@ -18,10 +18,10 @@ constexpr size_t kPairProfileMax = 110 * 1024;
 template <int R, int W, int MODE, int PK, bool LEFT>
 int launch16(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int max_blocks) {
     auto kern = wavefront16_kernel<R, W, MODE, PK, LEFT>;
-    const size_t smem = p16_profile_bytes(R, W, K, PK);
+    const size_t smem = p16_shared_bytes<R, W>() + p16_profile_bytes(R, W, K, PK);
     static int attr_set[64] = {0};
     if (c->device >= 64 || !attr_set[c->device]) {
-        const size_t cap = PK == kP16Pair ? kPairProfileMax : p16_profile_bytes(R, W, kMaxAlphabet, PK);
+        const size_t cap = p16_shared_bytes<R, W>() + (PK == kP16Pair ? kPairProfileMax : p16_profile_bytes(R, W, kMaxAlphabet, PK));
         CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
         if (c->device < 64) attr_set[c->device] = 1;
     }
@@ -68,7 +68,7 @@ bool swgb::p16_fits(const DevScoring &s, int R) {
     if (s.alg != kAlgLocal) return false;            // the packed fill keeps the zero floor
     int lo = 127, hi = -128;
     for (int k = 0; k < s.K * s.K; ++k) { lo = std::min(lo, (int)s.mat[k]); hi = std::max(hi, (int)s.mat[k]); }
-    return p16_spread(R, s.go, s.ge, hi, lo) < kP16Span;
+    return p16_spread(R, s.go, s.ge, hi, lo) <= kP16Span;
 }
 
 int swgb::launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K,

@@ -410,17 +410,16 @@ __device__ __forceinline__ void split_staircase_prologue(const FillTask &T, Lane
 
 // Input warp of a fill block: streams the strip's top boundary row (the
 // matrix border, the task's top row or the previous strip's bottom row, as
-// (H - open, F), multiplied by 2^SHIFT) into channel 0 of the boundary ring and the column residues
+// (H - open, F)) into channel 0 of the boundary ring and the column residues
 // into the residue ring, ahead of the first compute warp.  Room in channel 0
 // is bounded by what warp 0 consumed, room in the residue ring by what the
 // last active warp (whose lanes read furthest back, `lag` columns behind its
 // published count) has published.
-template <int QS, int QB, int IOB, int SHIFT = 0>
+template <int QS, int QB, int IOB>
 __device__ __forceinline__ void fill_input_warp(const FillTask &T, const FillLaunch &L, int strip, long long slot,
                                                 int n, int go, int K, int Wa, int lag, int2 *ring0,
                                                 uint8_t *bring, int *prod, const int *cons,
-                                                volatile int *s_abort, int lane, int alg = kAlgLocal, int ge = 0,
-                                                int *poff = nullptr, int pk1 = 0, int pstride = 0)
+                                                volatile int *s_abort, int lane, int alg = kAlgLocal, int ge = 0)
 {
     int in_next = 0;
     long long idle = 0;
@@ -439,15 +438,8 @@ __device__ __forceinline__ void fill_input_warp(const FillTask &T, const FillLau
                 // the matrix's top border: H(0, j) of the algorithm, F = -infinity
                 const int2 v = src ? __ldcg(src + col)
                                    : make_int2((int)top_border_h(alg, (long long)T.col0 + col + 1, go, ge), kNeg);
-                if constexpr (SHIFT == 0)
-                    ring0[col & (QS - 1)] = make_int2(v.x - go, v.y);
-                else     // scaled values; -infinity stays far below every real value, without overflow
-                    ring0[col & (QS - 1)] = make_int2((v.x - go) * (1 << SHIFT), max(v.y, kNeg >> SHIFT) * (1 << SHIFT));
-                const int c = min((int)T.b[col], K);
-                bring[col & (QB - 1)] = (uint8_t)c;
-                // pair profile (packed fill): the byte offset of the entry for (b[col], b[col - 1])
-                if (poff)   // (column -1 is real for a task entered from a checkpoint column)
-                    poff[col & (QB - 1)] = (c * pk1 + ((col > 0 || T.left) ? min((int)T.b[col - 1], K) : K)) * pstride;
+                ring0[col & (QS - 1)] = make_int2(v.x - go, v.y);
+                bring[col & (QB - 1)] = (uint8_t)min((int)T.b[col], K);
             }
             __syncwarp();
             if (lane == 0) sts_release(&prod[0], target);
@@ -468,11 +460,11 @@ __device__ __forceinline__ void fill_input_warp(const FillTask &T, const FillLau
     }
 }
 
-// Output warp of a fill block: drains the strip's bottom row (H - open, F),
-// multiplied by 2^SHIFT, from the last active warp's channel to global memory as (H, F) -- the next
+// Output warp of a fill block: drains the strip's bottom row (H - open, F)
+// from the last active warp's channel to global memory as (H, F) -- the next
 // strip's input and, every ckpt_every-th strip, a checkpoint row -- and
 // publishes the stored column count with a release store.
-template <int QS, int SHIFT = 0>
+template <int QS>
 __device__ __forceinline__ void fill_output_warp(const FillTask &T, const FillLaunch &L, int strip, long long slot,
                                                  int n, int go, int SH, int Wa, const int2 *ringW,
                                                  const int *prod, int *cons, volatile int *s_abort, int lane)
@@ -493,7 +485,7 @@ __device__ __forceinline__ void fill_output_warp(const FillTask &T, const FillLa
             if (store || ck) {
                 for (int col = out_next + lane; col < avail_out; col += 32) {
                     const int2 u = ringW[col & (QS - 1)];
-                    const int2 v = make_int2((u.x >> SHIFT) + go, u.y >> SHIFT);
+                    const int2 v = make_int2(u.x + go, u.y);
                     if (store) dst[col] = v;
                     if (ck) cdst[col] = v;
                 }

@@ -17,37 +17,62 @@
 //   * so one __viaddmax_s16x2 advances two cells, and the vertical
 //     dependency chain of a step is R/2 packed operations long.
 //
-// Values are kept multiplied by 8 (scores and penalties scaled by 8: the
-// recurrence is linear, so every H, E and F is scaled by 8 too), which frees
-// the low 3 bits of every value for a row tag when the end cell is tracked.
+// What bounds it.  A pair's strips form one chain of warps, at 200 kbp one
+// compute warp per SM sub-partition, so a step runs at the pace of a single
+// warp: its dependent chain (the shuffle, then the F chain through R/2 rows)
+// and the instructions around it, which a lone warp issues at 0.73 a clock at
+// most (measured with all SMs busy, loops longer than about 100
+// instructions).  So the step is kept short; everything that can be done once
+// per chunk of 32 steps, or once per sweep, is:
 //
-// Exact 16-bit values.  H is Lipschitz along rows and columns:
-// H(i-1,j) - o <= H(i,j) <= H(i-1,j) + o + max(S, 0) (the same along j), and
-// E, F and H + S stay within o + e + |S| of a neighbouring H.  Every value a
-// lane touches during one chunk of kP16CH steps sits within D = R + kP16CH + 6 rows
-// plus columns of its top half's first row, so all of them lie within
-// 8 (D (o + max S) + o + e + |min S| + max S) of that reference, in scaled
-// units (p16_spread).  Each lane keeps a base B (a multiple of 8; absolute =
-// B + stored value) and, at every chunk boundary, sets B = max(0, ref -
-// kP16Center) rounded down to a multiple of 8, shifting its registers by the
-// change.  With the spread below kP16Span:
+//   * one base per warp and no scaling (below): a shuffled value needs no
+//     conversion;
+//   * the bottom half's (H - open, F) go to the next lane, and to the next
+//     warp's ring, as one packed word: one shuffle, one select, one store;
+//   * the end cell's row and column are not tracked; a chunk only keeps its
+//     largest value per half-lane (half a vimax3 a row), and the place is
+//     looked up once, at the end of the sweep (p16_locate);
+//   * the columns past the last one have profile offsets too (padding), so
+//     that every chunk runs the same unrolled loop.
+//
+// 45 instructions a step at 12 rows a lane (77 before), 91 clocks in the
+// loop.  200 kbp score fill 18.85 -> 15.2 ms, 1 Mbp (16 rows a lane) 332 ->
+// 276 ms (GB300, 2,070 MHz).  Tried on the same code: four ALU operations a
+// cell pair and two plain subtractions, as in the database search (no gain
+// with one warp a sub-partition); a third step of skew per lane to take the
+// shuffle off the chain (the longer fill eats the gain); unrolling 8 (16.4
+// ms) and 32 steps (18.4 ms) instead of 16.
+//
+// Exact 16-bit values.  A warp keeps one base B: absolute value = B + stored
+// value.  H cannot change faster than
+//   |H(p) - H(q)| <= D (max S + extend) + 2 open,   D = row + column distance
+// (a path through p or q bends to the other cell for one gap each way; a row
+// or column more earns max S at most and saves an extension).  U = H - open,
+// E, F, X and the sums the instructions form lie within 3 open + extend +
+// |S| + max S of a neighbouring H.  All cells a warp touches in one chunk lie
+// within 32R rows and kP16Pos + kP16CH columns of each other, so all its
+// values lie within p16_spread of lane 0's first row (the reference).  At each
+// chunk start the warp moves its base if the reference has left kP16Center
+// +- kP16Slack (never below 0).  With the spread at most kP16Span:
 //   * B = 0: values are absolute, the 0 floor of H is the hardware relu;
-//   * B > 0: every value of the lane lies in (0, 32767 - 8), so the relu
-//     never fires -- as in the true recurrence, where every such H is above
-//     B > 0.
-// A value shuffled in from lane t-1 is moved from its base to this lane's by
-// one packed add; lane 0 converts the absolute boundary row; lane 31 writes
-// absolute values.  The strips exchange absolute rows (scaled in shared
-// memory, plain int32 in global memory), so the result does not depend on
-// the bases.
+//   * B > 0: every value of the warp lies in (0, 32767), so the relu never
+//     fires -- as in the true recurrence, where every such H is above B > 0.
+// The strips exchange absolute rows (plain int32 in global memory); a warp's
+// ring entries are relative to its base of that chunk, which it stores beside
+// them.  The result does not depend on the bases.
 //
-// End cell without branches.  The key of packed row k is its value OR a
-// tag 7 - k in the low 3 bits: the maximum key of a column is the largest
-// value and, among equal ones, the earliest row.  Each half keeps its best
-// key and the column where that key first appeared (a strictly larger key
-// replaces it: a larger score, or the same score in an earlier row); the
-// best is kept absolute in int32 across chunk boundaries, so a base change
-// never loses it.
+// End cell: the first cell in row-major order that holds the largest H.  A
+// half-lane (R/2 rows of a lane) is a row range, ordered by 2 lane + half.  At a
+// chunk's end the warp compares the largest value of the chunk with its best:
+// larger, or equal in an earlier half-lane, makes this chunk the best's, and
+// the chunk's snapshot (the lane states at its start, written to shared memory
+// every chunk) is kept; equal in the same half-lane, the snapshot is kept
+// beside the first one, because that chunk may hold an earlier row.  At the
+// end of the sweep the kept chunks are run again with a test per cell
+// (p16_locate).  A third equal chunk makes the warp look the kept ones up at
+// once.  Cells outside the task never decide: a padding cell is below every
+// real one, or (gaps that cost nothing) equal to a real one in the same or an
+// earlier row of an earlier step, and p16_locate tests real cells only.
 //
 // Query profile: for small alphabets a pair profile, one packed word per
 // (residue of the top half, residue of the bottom half) and packed row; else
@@ -62,24 +87,28 @@
 namespace swgb {
 
 constexpr int kNeg16p = -16384;     // -infinity of a packed 16-bit lane
-constexpr int kP16Center = 16384;   // stored value of a lane's reference once B > 0
-constexpr int kP16Span = 16000;     // largest scaled value spread (p16_spread) the packed fill accepts
+constexpr int kP16Center = 16384;   // stored value of a warp's reference once B > 0
+constexpr int kP16Slack = 1024;     // drift of the reference from kP16Center before the base moves
+constexpr int kP16Span = 15000;     // largest value spread (p16_spread) the packed fill accepts
 constexpr int kP16QS = 512;         // boundary-ring columns per channel
 constexpr int kP16Pos = 64;         // wavefront positions per warp (two per lane)
-constexpr int kP16Shift = 3;        // values are multiplied by 2^3
 constexpr int kP16CH = 32;          // steps per chunk (hand-off, base change; 16 measured slower)
+constexpr int kP16Lag = kP16Pos - 1;   // lane 31's bottom half trails lane 0's top half
+constexpr int kP16Unroll = 16;      // steps per unrolled body (8 and 32 measured slower)
+// An I/O warp with nothing to move sleeps this long: polling takes issue slots from the compute warp
+// beside it (200 kbp: 48 ns 15.5 ms, 128 ns 15.25 ms, 256 ns 15.15 ms)
+constexpr int kP16IdleNs = 256;
 
 // Profile kinds of the packed fill.
 enum P16Prof { kP16Pair = 0, kP16Int16 = 1 };
 
-// Bound on the spread, in scaled units, of all values a lane touches during
-// one chunk (see the header); the packed fill is exact when it is below
-// kP16Span.
+// Bound on the spread of all values a warp touches during one chunk (see the header); the packed
+// fill is exact when it is at most kP16Span.
 inline long long p16_spread(int R, int go, int ge, int max_s, int min_s) {
-    const long long L = (long long)go + (max_s > 0 ? max_s : 0);
-    const long long D = (long long)R + kP16CH + 6;
+    const long long L = (long long)ge + (max_s > 0 ? max_s : 0);
+    const long long D = 32LL * R + kP16Pos + kP16CH + 4;
     const long long neg = -min_s > 128 ? -min_s : 128;          // padding residues score -128
-    return 8 * (D * L + go + ge + neg + (max_s > 0 ? max_s : 0));
+    return D * L + 3LL * go + ge + neg + (max_s > 0 ? max_s : 0);
 }
 
 // Bytes of the packed fill's query profile for K residue codes.
@@ -88,50 +117,71 @@ inline size_t p16_profile_bytes(int R, int W, int K, int pk) {
     return pk == kP16Pair ? (size_t)(K + 1) * (K + 1) * (HC / 2) * 4 : (size_t)(K + 1) * HC * 2;
 }
 
+// Words of a lane's state in a snapshot: U, E, fb, udiag0, rounded up to whole 16-byte stores.
+__host__ __device__ constexpr int p16_snap_words(int R) { return (R + 2 + 3) / 4 * 4; }
+
 __device__ __forceinline__ unsigned p16_pack(int lo, int hi) {
     return (unsigned)(lo & 0xffff) | ((unsigned)hi << 16);
 }
 __device__ __forceinline__ int p16_lo(unsigned v) { return (int)(short)(v & 0xffffu); }
 __device__ __forceinline__ int p16_hi(unsigned v) { return (int)v >> 16; }
 
-__device__ __forceinline__ unsigned prmt_r(unsigned a, unsigned b, unsigned sel) {
+template <unsigned sel>
+__device__ __forceinline__ unsigned prmt_c(unsigned a, unsigned b) {
     unsigned d;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "n"(sel));
     return d;
 }
 
 // low half = 16-bit half ha of a, high half = 16-bit half hb of b
 template <int ha, int hb>
 __device__ __forceinline__ unsigned p16_halves(uint32_t a, uint32_t b) {
-    constexpr uint32_t sel = (2 * ha) | ((2 * ha + 1) << 4) | ((4 + 2 * hb) << 8) | ((5 + 2 * hb) << 12);
-    uint32_t d;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "n"(sel));
-    return d;
+    return prmt_c<(2 * ha) | ((2 * ha + 1) << 4) | ((4 + 2 * hb) << 8) | ((5 + 2 * hb) << 12)>(a, b);
 }
 
-// Profile words of one step, R/2 per lane.  Pair profile: the lane's packed
-// words for (top residue, bottom residue).  int16 profile: the lane's R
-// scores at the top half's residue; the bottom half uses the previous step's.
-//
-// Pair profile layout: combination cc = c_top * (K + 1) + c_bottom, lane g of
-// NL, packed rows 2q, 2q+1 as one 8-byte chunk at word ((cc*(R/4) + q)*NL + g)*2
-// (conflict-free 8-byte loads).  int16 layout: row r of the strip at
-// prof16[c * HC + r].
+// pair profile: a lane's H words of one residue pair in chunks of 4, 2 and 1 words, each kind
+// [chunk][lane] so that a warp's load is conflict-free
+template <int H> struct P16Chunks {
+    static constexpr int N4 = H == 6 ? 0 : H / 4, N2 = H == 6 ? 3 : (H % 4) / 2, N1 = H % 2;
+};
+// word index of packed row k of lane g (of NL) within one residue pair's H * NL words
+template <int H>
+__device__ __forceinline__ int p16_pair_word(int k, int g, int NL) {
+    using C = P16Chunks<H>;
+    if (k < 4 * C::N4) return ((k >> 2) * NL + g) * 4 + (k & 3);
+    k -= 4 * C::N4;
+    if (k < 2 * C::N2) return 4 * C::N4 * NL + ((k >> 1) * NL + g) * 2 + (k & 1);
+    return (4 * C::N4 + 2 * C::N2) * NL + g;
+}
+
+// Profile words of one step (H per lane) for the column whose profile offset is off.
 template <int R, int PK, int NL>
-__device__ __forceinline__ void p16_load(const int8_t *p, uint32_t (&w)[R / 2]) {
+__device__ __forceinline__ void p16_load(const int8_t *prof, int g, int off, uint32_t (&w)[R / 2]) {
+    constexpr int H = R / 2;
     if constexpr (PK == kP16Pair) {
+        using C = P16Chunks<H>;
+        const int8_t *p = prof + off;
 #pragma unroll
-        for (int q = 0; q < R / 4; ++q) {
-            const uint2 v = *reinterpret_cast<const uint2 *>(p + (size_t)q * NL * 8);
-            w[2 * q] = v.x; w[2 * q + 1] = v.y;
+        for (int q = 0; q < C::N4; ++q) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(p + g * 16 + (size_t)q * NL * 16);
+            w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
         }
+#pragma unroll
+        for (int q = 0; q < C::N2; ++q) {
+            const uint2 v = *reinterpret_cast<const uint2 *>(p + g * 8 + (size_t)(C::N4 * 16 + q * 8) * NL);
+            w[4 * C::N4 + 2 * q] = v.x; w[4 * C::N4 + 2 * q + 1] = v.y;
+        }
+        if constexpr (C::N1 == 1)
+            w[H - 1] = *reinterpret_cast<const uint32_t *>(p + g * 4 + (size_t)(C::N4 * 16 + C::N2 * 8) * NL);
     } else if constexpr (R == 8 || R == 16) {
+        const int8_t *p = prof + off + 2 * g * R;
 #pragma unroll
         for (int q = 0; q < R / 8; ++q) {
             const uint4 v = *reinterpret_cast<const uint4 *>(p + 16 * q);
             w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
         }
     } else {
+        const int8_t *p = prof + off + 2 * g * R;
 #pragma unroll
         for (int q = 0; q < R / 4; ++q) {
             const uint2 v = *reinterpret_cast<const uint2 *>(p + 8 * q);
@@ -140,7 +190,7 @@ __device__ __forceinline__ void p16_load(const int8_t *p, uint32_t (&w)[R / 2]) 
     }
 }
 
-// Scaled score pair 8 (S + open) of packed row k.
+// Score pair S + open of packed row k.
 template <int R, int PK>
 __device__ __forceinline__ unsigned p16_score(const uint32_t (&cur)[R / 2], const uint32_t (&prev)[R / 2], int k) {
     if constexpr (PK == kP16Pair) {
@@ -157,93 +207,286 @@ __device__ __forceinline__ unsigned p16_score(const uint32_t (&cur)[R / 2], cons
     }
 }
 
-// Per-lane state.  U = 8 (H - open) and E (scaled) of the lane's R/2 packed
-// rows relative to the lane base B; ub the last packed row's U after the
-// previous step and fb the F of the row below it, max(F - extend, U) (the
-// first row's F of the half below, so the next step starts its F chain from
-// it); udiag0 the packed row above the two halves at their previous columns.  Tracking: the best key per half relative to B
-// (packed, valid inside a chunk) and absolute (int32, across chunks), and the
-// column where it first appeared.
+// Per-lane state: U = H - open and E of the lane's R/2 packed rows relative to the warp's base;
+// fb the F of the row below each half's last row; flast the F of that last row; udiag0 the packed
+// row above the two halves at their previous columns; w the bottom half's (U, F below) for the
+// next lane; cmx the largest U of the chunk per half.
 template <int R>
 struct P16Lane {
     unsigned U[R / 2], E[R / 2];
-    unsigned ub, fb, udiag0;
-    unsigned flast;                 // F of each half's last row (fb is the F of the row below)
-    unsigned kbest;
-    int B;                          // lane base
-    unsigned din2;                  // (lane t-1's base minus this one, 0); (0, 0) for lane 0
-    int best[2], bcol[2];
+    unsigned fb, flast, udiag0, w, cmx;
 };
 
-// One step of one lane: column j = s - 2 lane (top half) and j - 1 (bottom
-// half).  TAIL drops the keys of columns at or past n (the sweep's last steps
-// run on padding residues); the first steps need no mask because columns
-// left of the task hold the border state (H = 0), which is never a best.
-template <int R, int PK, int QS, bool TAIL>
+// -extend, -open and -infinity in both halves.
+struct P16Consts { unsigned nge2, ngo2, neg2; };
+
+// One step of one lane: column s - 2 lane (top half) and the one before (bottom half); top = lane 0's row
+// above for this step, (H - open, F of the first row).
+template <int R, int PK>
 __device__ __forceinline__ void p16_step(P16Lane<R> &st, const uint32_t (&pw)[R / 2], const uint32_t (&pwp)[R / 2],
-                                         uint2 top, int s, int lane, int n, unsigned nge2, unsigned ngo2,
-                                         unsigned neg2, int2 *rout)
+                                         unsigned top, bool lane0, const P16Consts &c)
 {
     constexpr int H = R / 2;
-    const int j = s - 2 * lane;
-    const unsigned su = __shfl_up_sync(kFull, st.ub, 1);
-    const unsigned sf = __shfl_up_sync(kFull, st.fb, 1);
-    // lane 0: the row above is the strip's boundary row, already in lane 0's base and in the
-    // high halves (p16_top_row)
-    const unsigned srcu = lane == 0 ? top.x : su;
-    const unsigned srcf = lane == 0 ? top.y : sf;
-    // low half: the row above the top half at j (the high half of the source, moved from
-    // lane t-1's base to this one); high half: this lane's top half's last row at j - 1.
-    // fb carries F of the row below a half's last row, so f is already the first row's F.
-    const unsigned uup = __viaddmax_s16x2(prmt_r(srcu, st.ub, 0x5432u), st.din2, neg2);
-    unsigned f = __viaddmax_s16x2(prmt_r(srcf, st.fb, 0x5432u), st.din2, neg2);
+    unsigned r = __shfl_up_sync(kFull, st.w, 1);
+    r = lane0 ? top : r;
+    // low half: the row above the top half (lane t-1's bottom half one step earlier); high half: this
+    // lane's own top half one step earlier
+    const unsigned uup = prmt_c<0x5410>(r, st.U[H - 1]);
+    unsigned f = prmt_c<0x5432>(r, st.fb);
     unsigned udiag = st.udiag0;
     st.udiag0 = uup;
 #pragma unroll
     for (int k = 0; k < H; ++k) {
-        const unsigned sp = p16_score<R, PK>(pw, pwp, k);           // 8 (S + open) of both cells
+        const unsigned sp = p16_score<R, PK>(pw, pwp, k);
         const unsigned uold = st.U[k];
-        const unsigned e = __viaddmax_s16x2(st.E[k], nge2, uold);
+        const unsigned e = __viaddmax_s16x2(st.E[k], c.nge2, uold);
         const unsigned x = __viaddmax_s16x2_relu(udiag, sp, e);    // max(H(i-1,j-1) + S, E, 0)
-        const unsigned xgo = __viaddmax_s16x2(x, ngo2, neg2);      // x - open
-        const unsigned u = __viaddmax_s16x2(f, ngo2, xgo);         // H - open
+        const unsigned xgo = __viaddmax_s16x2(x, c.ngo2, c.neg2);  // x - open
+        const unsigned u = __viaddmax_s16x2(f, c.ngo2, xgo);       // H - open
         st.E[k] = e;
         udiag = uold;
         st.U[k] = u;
-        if (k + 1 < H) f = __viaddmax_s16x2(f, nge2, xgo);         // F of the next row
-        else st.fb = __viaddmax_s16x2(f, nge2, xgo);                // F of the row below the half
+        if (k + 1 < H) f = __viaddmax_s16x2(f, c.nge2, xgo);       // F of the next row
+        else st.fb = __viaddmax_s16x2(f, c.nge2, xgo);             // F of the row below the half
     }
-    st.ub = st.U[H - 1];
     st.flast = f;
-    if (lane == 31)      // the warp's bottom row (H - open, F) at column s - 63, scaled absolute
-        rout[(j - 1) & (QS - 1)] = make_int2(p16_hi(st.ub) + st.B, p16_hi(f) + st.B);
-    // keys: value | (7 - k) in both halves; the column's largest key
-    // (the low 3 bits of a scaled value are 0, so adding the tag sets them without a carry: an
-    // integer add, which the FMA pipe takes, instead of an OR on the busier ALU pipe)
-    unsigned ck = __vimax3_s16x2(st.U[0] + 0x00070007u, st.U[1] + 0x00060006u, st.U[2] + 0x00050005u);
+    st.w = prmt_c<0x7632>(st.U[H - 1], st.fb);
 #pragma unroll
-    for (int k = 3; k < H; k += 2) {
-        const unsigned t0 = (unsigned)(7 - k) * 0x00010001u;
-        const int k1 = k + 1 < H ? k + 1 : k;
-        const unsigned t1 = (unsigned)(7 - k1) * 0x00010001u;
-        ck = __vimax3_s16x2(ck, st.U[k] + t0, st.U[k1] + t1);
+    for (int k = 0; k + 1 < H; k += 2) st.cmx = __vimax3_s16x2(st.cmx, st.U[k], st.U[k + 1]);
+    if constexpr (H % 2 == 1) st.cmx = __vmaxs2(st.cmx, st.U[H - 1]);
+}
+
+__device__ __forceinline__ int ld_relaxed(const int *p) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Input warp of a packed fill block, ahead of the first compute warp: every column's profile offset into the
+// offset ring (published in *res; it goes on past the last column with the padding residue) and the strip's top
+// boundary row (H - open, F; absolute) into channel 0 (published in prod[0]).
+template <int QS, int QB, int PK>
+__device__ __forceinline__ void p16_input_warp(const FillTask &T, const FillLaunch &L, int strip, long long slot,
+                                               int n, int n_ext, int go, int K, int Wa, int2 *ring0, int *poff,
+                                               int pstride, int *prod, int *res, const int *cons, volatile int *s_abort,
+                                               int lane)
+{
+    constexpr int kBatch = 64;                 // columns of either stream per turn
+    const uint8_t *const b = T.b;
+    const bool left = T.left != nullptr;
+    const int2 *const src = strip == 0 ? T.top : T.bnd + (size_t)((strip - 1) % T.nslot) * n;
+    const int *const pprev = L.prog + (slot - 1);
+    const long long spin_limit = L.spin_limit;
+    int next = 0, rnext = 0, avail = strip == 0 ? n : 0;
+    long long idle = 0;
+    bool warm = true;                          // the first turn runs the boundary code with nothing to move (instruction cache)
+    while (next < n || rnext < n_ext) {
+        bool moved = false;
+        if (next < n) {
+            const int room = lds_acquire(&cons[0]) + QS;
+            int target = min(n, min(next + kBatch, room));
+            if (target > next) {
+                if (avail < target) {
+                    const int seen = ld_relaxed(pprev);
+                    if (seen > avail) {
+                        asm volatile("fence.acq_rel.gpu;" ::: "memory");   // the row up to `seen` is visible now
+                        avail = seen;
+                    }
+                }
+                target = max(next, min(target, avail));
+            }
+            target = max(target, next);
+            if (target > next || warm) {
+                const int c0 = next + lane, c1 = c0 + 32;
+                int2 v0 = make_int2(0, kNeg), v1 = v0;
+                if (src && c0 < target) v0 = __ldcg(src + c0);
+                if (src && c1 < target) v1 = __ldcg(src + c1);
+                if (c0 < target) ring0[c0 & (QS - 1)] = make_int2(v0.x - go, v0.y);
+                if (c1 < target) ring0[c1 & (QS - 1)] = make_int2(v1.x - go, v1.y);
+                __syncwarp();
+                if (lane == 0) sts_release(&prod[0], target);
+                moved = target > next;
+                next = target;
+                warm = false;
+            }
+        }
+        // the offsets run ahead: in idle turns, and whenever they are less than two batches ahead
+        if (rnext < n_ext && (!moved || rnext < next + 2 * kBatch)) {
+            const int target = min(n_ext, min(rnext + kBatch, lds_acquire(&prod[Wa]) + QB - (kP16Pos + 2)));
+            if (target > rnext) {
+                for (int col = rnext + lane; col < target; col += 32) {
+                    const int c = col < n ? min((int)__ldg(b + col), K) : K;
+                    if constexpr (PK == kP16Pair) {
+                        const int cm = (col > 0 || left) && col <= n ? min((int)__ldg(b + col - 1), K) : K;
+                        poff[col & (QB - 1)] = (c * (K + 1) + cm) * pstride;
+                    } else {
+                        poff[col & (QB - 1)] = c * pstride;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) sts_release(res, target);
+                rnext = target;
+                moved = true;
+            }
+        }
+        if (moved) {
+            idle = 0;
+        } else {
+            if (*s_abort) break;
+            if (++idle > spin_limit) {
+                if (lane == 0) atomicCAS(L.err, 0, kErrTimeout);
+                *s_abort = 1;
+                break;
+            }
+            __nanosleep(kP16IdleNs);
+        }
     }
-    if (TAIL) ck = p16_pack(j < n ? p16_lo(ck) : -32768, j - 1 < n ? p16_hi(ck) : -32768);
-    bool ph, pl;
-    st.kbest = __vibmax_s16x2(st.kbest, ck, &ph, &pl);             // kept where best >= key
-    st.bcol[0] = pl ? st.bcol[0] : j;
-    st.bcol[1] = ph ? st.bcol[1] : j - 1;
+}
+
+// Output warp: the strip's bottom row from the last active warp's channel to global memory as
+// (H, F), absolute; publishes the stored column count with a release store.
+template <int QS>
+__device__ __forceinline__ void p16_output_warp(const FillTask &T, const FillLaunch &L, int strip, long long slot,
+                                                int n, int go, int SH, int Wa, const uint2 *ringW, const int *baseW,
+                                                const int *prod, int *cons, volatile int *s_abort, int lane)
+{
+    int out_next = 0;
+    long long idle = 0;
+    const bool ck = T.ckpt_every > 0 && ((strip + 1) % T.ckpt_every) == 0 &&
+                    (long long)(strip + 1) * SH <= (long long)T.rows;
+    int2 *const cdst = ck ? T.ckpt + (size_t)((strip + 1) / T.ckpt_every - 1) * n : nullptr;
+    const bool store = strip + 1 < T.nstrips;
+    int2 *const dst = store ? T.bnd + (size_t)(strip % T.nslot) * n : nullptr;
+    int *const prog = L.prog + slot;
+    const long long spin_limit = L.spin_limit;
+    bool warm = true;                          // the first turn runs with nothing to move (instruction cache)
+    while (out_next < n) {
+        const int avail_out = min(lds_acquire(&prod[Wa]), out_next + 64);
+        if (avail_out > out_next || warm) {
+            if (store || ck) {
+                const int c0 = out_next + lane, c1 = c0 + 32;
+                const bool p0 = c0 < avail_out, p1 = c1 < avail_out;
+                const int l0 = c0 + kP16Lag, l1 = c1 + kP16Lag;
+                const uint2 v0 = ringW[l0 & (QS - 1)], v1 = ringW[l1 & (QS - 1)];
+                const int B0 = baseW[(l0 / kP16CH) & (QS / kP16CH - 1)], B1 = baseW[(l1 / kP16CH) & (QS / kP16CH - 1)];
+                const int2 o0 = make_int2(p16_lo(v0.x) + B0 + go, p16_hi(v0.y) + B0);
+                const int2 o1 = make_int2(p16_lo(v1.x) + B1 + go, p16_hi(v1.y) + B1);
+                if (store && p0) __stcg(dst + c0, o0);
+                if (store && p1) __stcg(dst + c1, o1);
+                if (ck && p0) __stcg(cdst + c0, o0);
+                if (ck && p1) __stcg(cdst + c1, o1);
+            }
+            warm = false;
+            __syncwarp();
+            if (lane == 0) {
+                if (store) st_release(prog, avail_out);
+                sts_release(&cons[Wa], avail_out);
+            }
+            out_next = avail_out;
+            idle = 0;
+        } else {
+            if (*s_abort) break;
+            if (++idle > spin_limit) {
+                if (lane == 0) atomicCAS(L.err, 0, kErrTimeout);
+                *s_abort = 1;
+                break;
+            }
+            __nanosleep(kP16IdleNs);
+        }
+    }
+}
+
+// The warp waits until *a >= wa, *b >= wb and *c >= wc (bounded); false on timeout or when the block is aborting.
+__device__ __forceinline__ bool p16_wait3(const int *a, int wa, const int *b, int wb, const int *c, int wc,
+                                          const volatile int *abort_flag, long long limit, int *err) {
+    for (long long it = 0;; ++it) {
+        const int va = *(const volatile int *)a, vb = *(const volatile int *)b, vc = *(const volatile int *)c;
+        if (va >= wa && vb >= wb && vc >= wc) break;
+        if (*abort_flag) return false;
+        if (it > limit) { atomicCAS(err, 0, kErrTimeout); return false; }
+        if (it > 64) __nanosleep(20);
+    }
+    __threadfence_block();
+    return true;
+}
+
+// The first half-lane (2 lane + half) whose chunk maximum is v.
+__device__ __forceinline__ int p16_first_pos(unsigned cmx, int v) {
+    const unsigned b0 = __ballot_sync(kFull, p16_lo(cmx) == v), b1 = __ballot_sync(kFull, p16_hi(cmx) == v);
+    const int p0 = b0 ? 2 * (__ffs(b0) - 1) : 64, p1 = b1 ? 2 * (__ffs(b1) - 1) + 1 : 64;
+    return min(p0, p1);
+}
+
+// Snapshot of a warp's state at a chunk's start, for finding the end cell's row and column later.
+template <int R>
+struct P16Snap {
+    uint4 st[p16_snap_words(R) / 4][32];   // U, E, fb, udiag0 of every lane
+    unsigned top[kP16CH];                  // lane 0's rows above
+    int s0, B;
+};
+
+// The first cell in row-major order, among the valid cells of half-lane pos of the chunk in snapshot S,
+// whose H - open equals u: (row of the half, column), or (R, 0).
+template <int R, int PK, int NL>
+__device__ __noinline__ int2 p16_locate(const P16Snap<R> &S, const int8_t *prof, int g, int pstride, const FillTask &T,
+                                        int n, int K, int go, int ge, int pos, int u, int nrows)
+{
+    constexpr int H = R / 2;
+    const int lane = threadIdx.x & 31;
+    unsigned q[p16_snap_words(R)];
+#pragma unroll
+    for (int k = 0; k < p16_snap_words(R) / 4; ++k) {
+        const uint4 v = S.st[k][lane];
+        q[4 * k] = v.x; q[4 * k + 1] = v.y; q[4 * k + 2] = v.z; q[4 * k + 3] = v.w;
+    }
+    P16Lane<R> st;
+#pragma unroll
+    for (int k = 0; k < H; ++k) { st.U[k] = q[k]; st.E[k] = q[H + k]; }
+    st.fb = q[2 * H]; st.udiag0 = q[2 * H + 1];
+    st.flast = 0;
+    st.w = prmt_c<0x7632>(st.U[H - 1], st.fb);
+    st.cmx = 0x80008000u;
+    const P16Consts c{p16_pack(-ge, -ge), p16_pack(-go, -go), p16_pack(kNeg16p, kNeg16p)};
+    const int want = u - S.B;
+    const bool mine = lane == (pos >> 1);
+    const int h = pos & 1;
+    int row = R, col = 0;
+    auto code = [&](int j) { return ((j >= 0 || T.left) && j < n) ? min((int)T.b[j], K) : K; };
+#pragma unroll 1
+    for (int k = 0; k < kP16CH; ++k) {
+        const int j = S.s0 + k - 2 * lane;
+        uint32_t pw[H], pwp[H];
+        const int ct = code(j), cb = code(j - 1);
+        if constexpr (PK == kP16Pair) {
+            p16_load<R, PK, NL>(prof, g, (ct * (K + 1) + cb) * pstride, pw);
+#pragma unroll
+            for (int x = 0; x < H; ++x) pwp[x] = 0;
+        } else {
+            p16_load<R, PK, NL>(prof, g, ct * pstride, pw);
+            p16_load<R, PK, NL>(prof, g, cb * pstride, pwp);
+        }
+        p16_step<R, PK>(st, pw, pwp, S.top[k], lane == 0, c);
+        const int jj = j - h;
+        if (mine && jj >= 0 && jj < n) {
+#pragma unroll
+            for (int x = H - 1; x >= 0; --x)
+                if (x < row && x < nrows && (h ? p16_hi(st.U[x]) : p16_lo(st.U[x])) == want) { row = x; col = jj; }
+        }
+    }
+    row = __shfl_sync(kFull, row, pos >> 1);
+    col = __shfl_sync(kFull, col, pos >> 1);
+    return make_int2(row, col);
 }
 
 // A task that starts right of a checkpoint column written by this fill (the
 // two-positions staircase of the checkpoint mode, FillTask::left_split):
 // lane l's top half holds its rows at column -1 - 2l and its bottom half at
 // -2 - 2l (task columns), which is exactly the wavefront's state after step
-// -1.  The lane takes that state (scaled by 8, in a base of its own) and the
+// -1.  The lane takes that state (relative to a base taken from lane 0) and the
 // sweep goes on from step 0; its first steps recompute real columns left of
-// the task from real residues (the residue ring's slots left of column 0).
+// the task from real residues (the offset ring's slots left of column 0).
 template <int R>
-__device__ __forceinline__ void p16_enter_staircase(const FillTask &T, P16Lane<R> &st, int grow, int lane, int go,
+__device__ __forceinline__ void p16_enter_staircase(const FillTask &T, P16Lane<R> &st, int &B, int grow, int lane, int go,
                                                     int ge) {
     constexpr int H = R / 2;
     int vU[R], vE[R];
@@ -257,11 +500,8 @@ __device__ __forceinline__ void p16_enter_staircase(const FillTask &T, P16Lane<R
     const bool in = grow < T.rows;
     const int2 at = in ? __ldcg(T.left_aux + grow / H) : make_int2(-go, kNeg);       // top half
     const int2 ab = in ? __ldcg(T.left_aux + grow / H + 1) : make_int2(-go, kNeg);   // bottom half
-    // absolute values scaled by 8 (-infinity clamped first so that scaling cannot overflow), then
-    // relative to the lane's base, -infinity at kNeg16p
-    auto scaled = [](int v) { return max(v, -(1 << 20)) * 8; };
-    const int B = max(0, scaled(vU[0]) - kP16Center) & ~7;
-    auto rel = [&](int v) { return max(scaled(v) - B, kNeg16p); };
+    B = max(0, __shfl_sync(kFull, vU[0], 0) - kP16Center);
+    auto rel = [&](int v) { return max(min(v - B, 32767), kNeg16p); };
 #pragma unroll
     for (int k = 0; k < H; ++k) {
         st.U[k] = p16_pack(rel(vU[k]), rel(vU[H + k]));
@@ -269,29 +509,30 @@ __device__ __forceinline__ void p16_enter_staircase(const FillTask &T, P16Lane<R
     }
     st.udiag0 = p16_pack(rel(at.x), rel(ab.x));
     st.flast = p16_pack(rel(at.y), rel(ab.y));
-    st.ub = st.U[H - 1];
-    // F of the row below each half's last row: max(F - extend, H - open) of that row
-    st.fb = __viaddmax_s16x2(st.flast, p16_pack(-8 * ge, -8 * ge), st.U[H - 1]);
-    st.B = B;
-    const int bup = __shfl_up_sync(kFull, B, 1);
-    st.din2 = lane == 0 ? 0u : p16_pack(bup - B, 0);
-    // the best keys in the new base (H = 0 with the largest tag, never a best), kept above -32768
-    st.kbest = p16_pack(max(st.best[0] - B, -32768), max(st.best[1] - B, -32768));
+    st.fb = __viaddmax_s16x2(st.flast, p16_pack(-ge, -ge), st.U[H - 1]);
+    st.w = prmt_c<0x7632>(st.U[H - 1], st.fb);
 }
 
-// Lane 0's row above at one step, from the strip's boundary row v (scaled,
-// absolute: H - open and F): both taken to lane 0's base B0 and into the high
-// halves, the F as the first row's F, max(F - extend, H - open).
-__device__ __forceinline__ uint2 p16_top_row(int2 v, int B0, int ge8) {
-    const int tu = __viaddmax_s32(v.x, -B0, kNeg16p);
-    const int tf = __viaddmax_s32(__viaddmax_s32(v.y, -ge8, v.x), -B0, kNeg16p);
-    return make_uint2((unsigned)tu << 16, (unsigned)tf << 16);
-}
 
-// Steps per unrolled body of the steady loop, measured on GB300 (2, 4, 8, 16, 32 at 12 rows a lane): 8 for
-// the score fill; 16 with checkpoints above 8 rows a lane (its chunk-end code runs once per 16 steps); 32
-// is much slower (a body that large no longer stays in the instruction cache).
-constexpr int fill16_unroll(int R, int MODE) { return (R <= 8 || MODE == kModeScore) ? 8 : 16; }
+// Shared memory of a block ahead of its query profile.
+template <int R, int W>
+struct P16Shared {
+    P16Snap<R> snap[W][3];
+    int poff[kQB];                         // profile offset per column
+    int2 ring0[kP16QS];                    // (H - open, F), absolute: the strip's boundary row
+    uint2 ring[W][kP16QS];                 // channel w + 1: after step s of warp w, at slot s, (w, F of the bottom row)
+    int base[W][kP16QS / kP16CH];          // base of warp w per chunk
+    int4 cand[W];
+    long long tk;
+    int prod[W + 1];                       // columns available in channel k
+    int cons[W + 1];                       // columns consumed from channel k
+    int res;                               // columns with a profile offset
+    int task, strip;
+    int abort;
+};
+
+template <int R, int W>
+constexpr size_t p16_shared_bytes() { return (sizeof(P16Shared<R, W>) + 15) / 16 * 16; }
 
 // LEFT: the tasks may start right of a checkpoint column written by this fill
 // (p16_enter_staircase; the coarse-tile refills of a two-level reconstruction).
@@ -300,54 +541,56 @@ template <int R, int W, int MODE, int PK, bool LEFT = false>
 __global__ void __launch_bounds__((W + 2) * 32, 1)
 wavefront16_kernel(const FillLaunch L)
 {
-    static_assert(R % 4 == 0 && R >= 8 && R <= 16, "two halves of at most 8 rows (3-bit tags)");
+    static_assert(R % 2 == 0 && R >= 4, "two halves");
+    static_assert(PK == kP16Pair || R == 8 || R == 12 || R == 16, "int16 profile loads");
     static_assert(MODE == kModeScore || MODE == kModeScoreCk, "score modes only");
     constexpr int H = R / 2;
     constexpr int HC = W * 32 * R;
     constexpr int NL = W * 32;
-    constexpr int CH = kP16CH, QS = kP16QS, QB = kQB, IOB = kIOB;
-    constexpr int LAG = kP16Pos - 1;                 // lane 31's bottom half trails lane 0's top half
-    static_assert(QS >= 2 * IOB + 2 * CH + 2 * kP16Pos, "ring too small");
-    constexpr int UNR = fill16_unroll(R, MODE);
-    static_assert(CH % UNR == 0, "chunks are whole unrolled groups");
+    constexpr int CH = kP16CH, QS = kP16QS, QB = kQB, LAG = kP16Lag;
+    static_assert(QS >= 2 * 64 + 2 * CH + 2 * kP16Pos, "ring too small");
+    static_assert(QB >= W * (kP16Pos + CH) + kP16Pos + 2 + 128, "the last warp's offsets must not be overwritten");
+    constexpr int UNR = kP16Unroll;
+    static_assert(CH % UNR == 0 && UNR % 4 == 0, "chunks are whole unrolled groups of four steps");
+    static_assert(CH == 32, "one boundary entry a lane");
 
-    extern __shared__ __align__(16) int8_t prof[];   // p16_profile_bytes
-    __shared__ int2 ring[W + 1][QS];                 // (8 (H - open), 8 F), absolute
-    __shared__ uint8_t bring[QB];
-    __shared__ int s_poff[PK == kP16Pair ? QB : 1];   // pair profile: byte offset per column (fill_input_warp)
-    __shared__ int prod[W + 1];
-    __shared__ int cons[W + 1];
-    __shared__ long long s_tk;
-    __shared__ int s_task, s_strip;
-    __shared__ volatile int s_abort;
-    __shared__ int4 s_cand[W];
-    __shared__ uint2 s_top[W][CH];                   // lane 0's rows above for one chunk (p16_top_row)
-    static_assert(CH <= 32 && (CH & (CH - 1)) == 0, "one boundary entry a lane, a power of two");
+    extern __shared__ __align__(16) int8_t p16_smem[];   // P16Shared, then p16_profile_bytes
+    P16Shared<R, W> &S = *reinterpret_cast<P16Shared<R, W> *>(p16_smem);
+    int8_t *const prof = p16_smem + p16_shared_bytes<R, W>();
+    int2 *const ring0 = S.ring0;
+    uint2 (*const ring)[kP16QS] = S.ring;
+    int (*const s_base)[kP16QS / kP16CH] = S.base;
+    int *const s_poff = S.poff, *const prod = S.prod, *const cons = S.cons;
+    P16Snap<R> (*const s_snap)[3] = S.snap;
+    int4 *const s_cand = S.cand;
+    volatile int *const s_abort = &S.abort;
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    for (;;) {
+    for (bool first = true;; first = false) {
         if (threadIdx.x == 0) {
-            claim_strip(L, &s_tk, &s_task, &s_strip);
-            s_abort = 0;
+            claim_strip(L, &S.tk, &S.task, &S.strip);
+            *s_abort = 0;
         }
         if (threadIdx.x <= W) { prod[threadIdx.x] = 0; cons[threadIdx.x] = 0; }
+        if (threadIdx.x == 0) S.res = 0;
         __syncthreads();
-        const long long tk = s_tk;
+        const long long tk = S.tk;
         if (tk >= L.total) return;
-        const FillTask &T = L.tasks[s_task];
+        const FillTask &T = L.tasks[S.task];
         const DevScoring &SC = L.scorings[T.scoring];
         const int K = SC.K, go = SC.go, ge = SC.ge;
-        const int strip = s_strip;
+        const int strip = S.strip;
         const long long slot = T.ticket0 + strip;        // progress and candidate of (task, strip)
         const int SW = (T.strip_warps > 0 && T.strip_warps < W) ? T.strip_warps : W;
         const int SH = SW * 32 * R;
         const int rbase = strip * SH;
         const int n = T.ncols;
         const int Wa = min(SW, (T.rows - rbase + 32 * R - 1) / (32 * R));
+        const int n_ext = (n + LAG + CH - 1) / CH * CH + 2;
 
-        // ---- query profile of the strip's rows: 8 (S(a_r, c) + open), padding at 8 * -128
+        const int pstride = PK == kP16Pair ? H * NL * 4 : 2 * HC;   // bytes per profile entry
         if constexpr (PK == kP16Pair) {
             const int ncc = (K + 1) * (K + 1);
             uint32_t *pw32 = reinterpret_cast<uint32_t *>(prof);
@@ -357,236 +600,244 @@ wavefront16_kernel(const FillLaunch L)
                 const int rt = g * R + k, rb = g * R + H + k;
                 const bool okt = rt < SH && rbase + rt < T.rows && ct < K;
                 const bool okb = rb < SH && rbase + rb < T.rows && cb < K;
-                const int vt = okt ? 8 * (SC.mat[min((int)T.a[rbase + rt], K - 1) * K + ct] + go) : 8 * kPadScore;
-                const int vb = okb ? 8 * (SC.mat[min((int)T.a[rbase + rb], K - 1) * K + cb] + go) : 8 * kPadScore;
-                pw32[((cc * (R / 4) + (k >> 1)) * NL + g) * 2 + (k & 1)] = p16_pack(vt, vb);
+                const int vt = okt ? SC.mat[min((int)T.a[rbase + rt], K - 1) * K + ct] + go : kPadScore;
+                const int vb = okb ? SC.mat[min((int)T.a[rbase + rb], K - 1) * K + cb] + go : kPadScore;
+                pw32[cc * NL * H + p16_pair_word<H>(k, g, NL)] = p16_pack(vt, vb);
             }
         } else {
             int16_t *p16 = reinterpret_cast<int16_t *>(prof);
             for (int idx = threadIdx.x; idx < (K + 1) * HC; idx += blockDim.x) {
                 const int lr = idx % HC, c = idx / HC;
                 const bool ok = lr < SH && rbase + lr < T.rows && c < K;
-                p16[idx] = (int16_t)(ok ? 8 * (SC.mat[min((int)T.a[rbase + lr], K - 1) * K + c] + go) : 8 * kPadScore);
+                p16[idx] = (int16_t)(ok ? SC.mat[min((int)T.a[rbase + lr], K - 1) * K + c] + go : kPadScore);
             }
         }
-        // the residue ring's last kP16Pos slots hold the columns left of the task (down to -64),
-        // which lanes compute during their first two chunks: padding at the matrix border;
-        // the input warp reaches those slots only after the last warp has published a column,
-        // i.e. left those chunks
-        // bytes per profile entry: pair, per residue combination; int16, per residue
-        const int pstride = PK == kP16Pair ? (R / 4) * NL * 8 : 2 * HC;
-        // (a task entered from a checkpoint column: the real residues of those columns)
+        // the offset ring starts as padding (the warm-up chunk below reads columns down to -96); its last kP16Pos
+        // slots hold the columns left of the task: padding at the matrix border, real residues for a task entered from
+        // a checkpoint column.  The input warp reaches those slots only after the last warp has published a column,
+        // i.e. left them behind
+        if (first) {
+            for (int k = threadIdx.x; k < QB; k += blockDim.x) s_poff[k] = (PK == kP16Pair ? K * (K + 1) + K : K) * pstride;
+            __syncthreads();
+        }
         if (threadIdx.x < kP16Pos) {
             const int j = (int)threadIdx.x - kP16Pos;                       // column -64 .. -1
             const bool real = LEFT && T.left;
             const int cj = real ? min((int)T.b[j], K) : K;
-            bring[QB - kP16Pos + threadIdx.x] = (uint8_t)cj;
-            if constexpr (PK == kP16Pair) {
-                const int cjm = real ? min((int)T.b[j - 1], K) : K;
-                s_poff[QB - kP16Pos + threadIdx.x] = (cj * (K + 1) + cjm) * pstride;
-            }
+            const int cjm = real ? min((int)T.b[j - 1], K) : K;
+            s_poff[QB - kP16Pos + threadIdx.x] = PK == kP16Pair ? (cj * (K + 1) + cjm) * pstride : cj * pstride;
         }
         __syncthreads();
 
         if (warp == W) {
-            fill_input_warp<QS, QB, IOB, kP16Shift>(T, L, strip, slot, n, go, K, Wa, kP16Pos + 1, ring[0], bring,
-                                                    prod, cons, &s_abort, lane, kAlgLocal, 0,
-                                                    PK == kP16Pair ? s_poff : nullptr, K + 1, pstride);
+            p16_input_warp<QS, QB, PK>(T, L, strip, slot, n, n_ext, go, K, Wa, ring0, s_poff, pstride, prod, &S.res, cons,
+                                            s_abort, lane);
         } else if (warp == W + 1) {
-            fill_output_warp<QS, kP16Shift>(T, L, strip, slot, n, go, SH, Wa, ring[Wa], prod, cons, &s_abort, lane);
+            p16_output_warp<QS>(T, L, strip, slot, n, go, SH, Wa, ring[Wa - 1], s_base[Wa - 1], prod, cons, s_abort,
+                                lane);
         } else if (warp >= Wa) {
             if (lane == 0) s_cand[warp] = make_int4(0, 0x7fffffff, 0x7fffffff, 0);
         } else {
             // ================= compute warp =================
             const int g = warp * 32 + lane;
             const int grow = rbase + g * R;
-            // this lane's profile base (pair: its first chunk of combination 0; int16: its rows)
-            const int8_t *prow = PK == kP16Pair ? prof + g * 8 : prof + 2 * g * R;
-            const unsigned ngo2 = p16_pack(-8 * go, -8 * go), nge2 = p16_pack(-8 * ge, -8 * ge);
-            const unsigned neg2 = p16_pack(kNeg16p, kNeg16p);
+            const bool lane0 = lane == 0;
+            const P16Consts cst{p16_pack(-ge, -ge), p16_pack(-go, -go), p16_pack(kNeg16p, kNeg16p)};
             P16Lane<R> st;
+            int B = 0;
 #pragma unroll
-            for (int k = 0; k < H; ++k) { st.U[k] = ngo2; st.E[k] = neg2; }
-            st.ub = ngo2; st.fb = ngo2; st.flast = neg2; st.udiag0 = ngo2;   // matrix border: H = 0
-            st.B = 0; st.din2 = 0;
-            // H = 0 with the largest tag: never replaced by H = 0, always by H > 0
-            st.best[0] = st.best[1] = -8 * go + 7;
-            st.bcol[0] = st.bcol[1] = -1;
-            st.kbest = p16_pack(st.best[0], st.best[1]);
+            for (int k = 0; k < H; ++k) { st.U[k] = cst.ngo2; st.E[k] = cst.neg2; }
+            st.fb = cst.ngo2; st.flast = cst.neg2; st.udiag0 = cst.ngo2; st.w = cst.ngo2;   // matrix border: H = 0
             if constexpr (LEFT)
-                if (T.left) p16_enter_staircase<R>(T, st, grow, lane, go, ge);   // (a two-positions staircase)
+                if (T.left) p16_enter_staircase<R>(T, st, B, grow, lane, go, ge);
+            // the warp's best: H - open, half-lane (2 lane + half), and where: snapshot, or row and column once located
+            int bu = 1 - go, brow = R, bcol = 0, bcb = 0;
+            int pa = 0, pb = 0, npend = 0;      // snapshots that hold the best (the second: the same half-lane again)
+
+            unsigned bcm = 0x80008000u;
+            bool held = false;
+            int cur = 0;                        // snapshot buffer of the running chunk; the other holds the best's chunk
             int next_ck = (MODE == kModeScoreCk && T.colck && T.colck_every > 0) ? T.colck_every - 1 : 0x7fffffff;
-            int2 *rin = ring[warp];
-            int2 *rout = ring[warp + 1];
-            int seen_in = 0;
-            bool loaded = false;
-            uint32_t pw[R / 2], pwp[R / 2];
-            if constexpr (PK == kP16Pair || !LEFT) {
-#pragma unroll
-                for (int q = 0; q < R / 2; ++q) pwp[q] = p16_pack(8 * kPadScore, 8 * kPadScore);
-            } else {
-                // the int16 profile's bottom half takes the previous step's words: at step 0 those
-                // of column -1 - 2 lane (padding, or a real residue left of a checkpoint column)
-                p16_load<R, PK, NL>(prow + min((int)bring[(-1 - 2 * lane) & (QB - 1)], K) * pstride, pwp);
-            }
-            uint2 top;
-            for (int s0 = 0; s0 < n + LAG; s0 += CH) {
-                const int need_in = min(n, s0 + CH + 1);
-                if (need_in > seen_in) {
-                    if (!warp_wait_geq(&prod[warp], need_in, &s_abort, L.spin_limit, L.err)) { s_abort = 1; break; }
-                    seen_in = need_in;
+            uint2 *rout = ring[warp];
+            // rows and columns of the best in the pending snapshots: the smallest row, then the earlier chunk's column
+            auto resolve = [&](int pos) {
+                const int nr = T.rows - (rbase + (warp * 32 + (pos >> 1)) * R + (pos & 1) * H);
+                for (int q = 0; q < npend; ++q) {
+                    const int2 c = p16_locate<R, PK, NL>(s_snap[warp][q ? pb : pa], prof, g, pstride, T, n, K, go, ge, pos, bu, nr);
+                    if (c.x < brow) { brow = c.x; bcol = c.y; }
                 }
-                const int ring_hi = max(0, s0 + CH - LAG);
-                const int out_hi = min(n, ring_hi);
-                if (ring_hi > 0 && !warp_wait_geq(&cons[warp + 1], ring_hi - QS, &s_abort, L.spin_limit, L.err)) { s_abort = 1; break; }
-                if (!loaded) {
-                    const int c = min((int)bring[(s0 - 2 * lane) & (QB - 1)], K);
+            };
+            const long long spin_limit = L.spin_limit;
+            int *const err = L.err;
+            uint32_t pw[H], pwp[H];
+            int2 off;                           // profile offsets of the next two steps to load
+            bool ok = true;
+            // the block's first strip runs one chunk left of the task, which keeps the border state: it brings the
+            // loop into the instruction cache while the strip above has not produced its first columns yet
+            const int sbeg = first && !(LEFT && T.left) ? -CH : 0;
+            for (int s0 = sbeg; s0 < n + LAG; s0 += CH) {
+                // the chunk's rows above, the profile offsets one step ahead, and room in the ring below
+                const int ring_hi = s0 + CH - LAG, out_hi = min(n, ring_hi);
+                if (!p16_wait3(&prod[warp], min(n, s0 + CH), &S.res, s0 + CH + 2, &cons[warp + 1], ring_hi - QS, s_abort,
+                               spin_limit, err)) {
+                    *s_abort = 1;
+                    ok = false;
+                    break;
+                }
+                if (s0 == sbeg) {
                     if constexpr (PK == kP16Pair) {
-                        // the bottom halves' column is left of the task: padding, or (LEFT) a real residue
-                        if constexpr (LEFT) p16_load<R, PK, NL>(prow + s_poff[(s0 - 2 * lane) & (QB - 1)], pw);
-                        else p16_load<R, PK, NL>(prow + (c * (K + 1) + K) * pstride, pw);
-                    } else {
-                        p16_load<R, PK, NL>(prow + c * pstride, pw);
-                    }
-                    loaded = true;
-                }
-                {   // new lane base from the top half's first row at its last column; the best
-                    // keys go through their absolute copies
-                    const int oldB = st.B;
-                    if constexpr (LEFT) {   // (-32768: no key since the staircase entry put the best below the base)
-                        if (p16_lo(st.kbest) > -32768) st.best[0] = max(st.best[0], p16_lo(st.kbest) + oldB);
-                        if (p16_hi(st.kbest) > -32768) st.best[1] = max(st.best[1], p16_hi(st.kbest) + oldB);
-                    } else {
-                        st.best[0] = max(st.best[0], p16_lo(st.kbest) + oldB);
-                        st.best[1] = max(st.best[1], p16_hi(st.kbest) + oldB);
-                    }
-                    const int ref = p16_lo(st.U[0]) + oldB;
-                    const int Bn = max(0, ref - kP16Center) & ~7;
-                    const unsigned d2 = p16_pack(oldB - Bn, oldB - Bn);
 #pragma unroll
-                    for (int k = 0; k < H; ++k) {
-                        st.U[k] = __viaddmax_s16x2(st.U[k], d2, neg2);
-                        st.E[k] = __viaddmax_s16x2(st.E[k], d2, neg2);
+                        for (int q = 0; q < H; ++q) pwp[q] = 0;
+                    } else {
+                        p16_load<R, PK, NL>(prof, g, s_poff[(sbeg - 1 - 2 * lane) & (QB - 1)], pwp);
                     }
-                    st.ub = __viaddmax_s16x2(st.ub, d2, neg2);
-                    st.fb = __viaddmax_s16x2(st.fb, d2, neg2);
-                    st.flast = __viaddmax_s16x2(st.flast, d2, neg2);
-                    st.udiag0 = __viaddmax_s16x2(st.udiag0, d2, neg2);
-                    st.B = Bn;
-                    const int bup = __shfl_up_sync(kFull, Bn, 1);
-                    st.din2 = lane == 0 ? 0u : p16_pack(bup - Bn, 0);
-                    if constexpr (LEFT)
-                        st.kbest = p16_pack(max(min(st.best[0] - Bn, 32767), -32768), max(min(st.best[1] - Bn, 32767), -32768));
-                    else
-                        st.kbest = p16_pack(min(st.best[0] - Bn, 32767), min(st.best[1] - Bn, 32767));
+                    off = *reinterpret_cast<const int2 *>(&s_poff[(sbeg - 2 * lane) & (QB - 1)]);
+                    p16_load<R, PK, NL>(prof, g, off.x, pw);
                 }
-                {   // lane 0's rows above for the chunk's steps, taken to its new base once per
-                    // chunk (one entry a lane) rather than once per step; entries at or past n
-                    // read as -infinity.  The wait above made entries below s0 + CH + 1 ready.
-                    const int B0 = __shfl_sync(kFull, st.B, 0);
-                    __syncwarp();
-                    if (lane < CH) {
-                        const int sk = s0 + lane;
-                        const int2 v = sk < n ? rin[sk & (QS - 1)] : make_int2(kNeg, kNeg);
-                        s_top[warp][lane] = p16_top_row(v, B0, -p16_lo(nge2));
+                // lane 0's rows above for the chunk's steps (one entry a lane); -infinity at and past n
+                const int tcol = s0 + lane;
+                const bool treal = tcol >= 0 && tcol < n;
+                int2 tv = make_int2(0, 0);
+                int tB = 0;
+                if (treal) {
+                    if (warp == 0) {
+                        tv = ring0[tcol & (QS - 1)];
+                    } else {
+                        tv.x = (int)ring[warp - 1][(tcol + LAG) & (QS - 1)].x;
+                        tB = s_base[warp - 1][((tcol + LAG) / CH) & (QS / CH - 1)];
                     }
-                    __syncwarp();
-                    top = s_top[warp][0];
                 }
-                if (s0 + CH + 1 <= n) {
-                    // steady state: lane 0's prefetched column stays inside the task; columns
-                    // left of the task (first chunks) compute the border state on padding
-#pragma unroll UNR
-                    for (int k = 0; k < CH; ++k) {
-                        const int s = s0 + k;
-                        const uint2 topn = s_top[warp][(k + 1) & (CH - 1)];   // (unused after the last step)
-                        uint32_t pwn[R / 2];
-                        if constexpr (PK == kP16Pair) {
-                            p16_load<R, PK, NL>(prow + s_poff[(s + 1 - 2 * lane) & (QB - 1)], pwn);
-                        } else {
-                            const int cn = min((int)bring[(s + 1 - 2 * lane) & (QB - 1)], K);
-                            p16_load<R, PK, NL>(prow + cn * pstride, pwn);
+                {   // the warp's base follows lane 0's first row
+                    const int ref = p16_lo(__shfl_sync(kFull, st.U[0], 0));
+                    if (ref > kP16Center + kP16Slack || (B > 0 && ref < kP16Center - kP16Slack)) {
+                        const int Bn = max(0, ref + B - kP16Center);
+                        const unsigned d2 = p16_pack(B - Bn, B - Bn);
+#pragma unroll
+                        for (int k = 0; k < H; ++k) {
+                            st.U[k] = __viaddmax_s16x2(st.U[k], d2, cst.neg2);
+                            st.E[k] = __viaddmax_s16x2(st.E[k], d2, cst.neg2);
                         }
-                        p16_step<R, PK, QS, false>(st, pw, pwp, top, s, lane, n, nge2, ngo2, neg2, rout);
-#pragma unroll
-                        for (int q = 0; q < R / 2; ++q) { pwp[q] = pw[q]; pw[q] = pwn[q]; }
-                        top = topn;
+                        st.fb = __viaddmax_s16x2(st.fb, d2, cst.neg2);
+                        st.flast = __viaddmax_s16x2(st.flast, d2, cst.neg2);
+                        st.udiag0 = __viaddmax_s16x2(st.udiag0, d2, cst.neg2);
+                        st.w = prmt_c<0x7632>(st.U[H - 1], st.fb);
+                        B = Bn;
                     }
-                } else {
-                    // the sweep's last steps: columns past n read the padding residue and lane 0
-                    // an -inf row above; their keys are dropped.  Whole unrolled groups: up to
-                    // UNR - 1 steps past the last one (n + 62), whose ring writes past n the
-                    // wait on the consumer above covers.
-                    for (int gs = 0; gs < CH; gs += UNR) {
-                        if (s0 + gs >= n + LAG) break;
+                }
+                P16Snap<R> &snap = s_snap[warp][cur];
+                {
+                    unsigned q[p16_snap_words(R)];
 #pragma unroll
-                        for (int k = 0; k < UNR; ++k) {
-                            const int s = s0 + gs + k;
-                            const int jn = s + 1 - 2 * lane;
-                            const int cn = jn < n ? min((int)bring[jn & (QB - 1)], K) : K;
-                            const uint2 topn = s_top[warp][(gs + k + 1) & (CH - 1)];
-                            uint32_t pwn[R / 2];
-                            if constexpr (PK == kP16Pair) {   // the bottom half's residue: column jn - 1
-                                const int cb = jn - 1 < n ? min((int)bring[(jn - 1) & (QB - 1)], K) : K;
-                                p16_load<R, PK, NL>(prow + (cn * (K + 1) + cb) * pstride, pwn);
+                    for (int k = 0; k < H; ++k) { q[k] = st.U[k]; q[H + k] = st.E[k]; }
+                    q[2 * H] = st.fb; q[2 * H + 1] = st.udiag0;
+#pragma unroll
+                    for (int k = 2 * H + 2; k < p16_snap_words(R); ++k) q[k] = 0;
+#pragma unroll
+                    for (int k = 0; k < p16_snap_words(R) / 4; ++k)
+                        snap.st[k][lane] = make_uint4(q[4 * k], q[4 * k + 1], q[4 * k + 2], q[4 * k + 3]);
+                    if (lane0) {
+                        s_base[warp][(s0 / CH) & (QS / CH - 1)] = B;
+                        snap.s0 = s0; snap.B = B;
+                    }
+                    unsigned t = tcol < 0 ? cst.ngo2 : cst.neg2;
+                    if (treal) {
+                        if (warp == 0) t = p16_pack(max(tv.x - B, kNeg16p), max(max(tv.y - ge, tv.x) - B, kNeg16p));
+                        else t = __viaddmax_s16x2((unsigned)tv.x, p16_pack(tB - B, tB - B), cst.neg2);
+                    }
+                    snap.top[lane] = t;
+                    __syncwarp();
+                }
+                st.cmx = 0x80008000u;
+                uint2 *rc = rout + (s0 & (QS - 1));
+#pragma unroll 1
+                for (int gs = 0; gs < CH; gs += UNR) {                 // (a lane past the task's columns steps over padding)
+#pragma unroll
+                    for (int k4 = 0; k4 < UNR; k4 += 4) {
+                        const uint4 tops = *reinterpret_cast<const uint4 *>(&snap.top[gs + k4]);
+#pragma unroll
+                        for (int k2 = 0; k2 < 4; k2 += 2) {
+                            const int k = k4 + k2;
+                            // offsets of steps s + 2, s + 3 (slots an even distance apart from lane to lane)
+                            const int2 offn = *reinterpret_cast<const int2 *>(&s_poff[(s0 + gs + k + 2 - 2 * lane) & (QB - 1)]);
+                            uint32_t pwn[H];
+                            p16_load<R, PK, NL>(prof, g, off.y, pwn);
+                            p16_step<R, PK>(st, pw, pwp, k2 == 0 ? tops.x : tops.z, lane0, cst);
+                            if (lane == 31) rc[gs + k] = make_uint2(st.w, st.flast);
+                            p16_load<R, PK, NL>(prof, g, offn.x, PK == kP16Pair ? pw : pwp);
+                            if constexpr (PK == kP16Pair) {
+                                p16_step<R, PK>(st, pwn, pwp, k2 == 0 ? tops.y : tops.w, lane0, cst);
                             } else {
-                                p16_load<R, PK, NL>(prow + cn * pstride, pwn);
-                            }
-                            p16_step<R, PK, QS, true>(st, pw, pwp, top, s, lane, n, nge2, ngo2, neg2, rout);
+                                uint32_t t2[H];
 #pragma unroll
-                            for (int q = 0; q < R / 2; ++q) { pwp[q] = pw[q]; pw[q] = pwn[q]; }
-                            top = topn;
+                                for (int q = 0; q < H; ++q) t2[q] = pwp[q];      // words of step s + 2
+                                p16_step<R, PK>(st, pwn, pw, k2 == 0 ? tops.y : tops.w, lane0, cst);
+#pragma unroll
+                                for (int q = 0; q < H; ++q) { pwp[q] = pwn[q]; pw[q] = t2[q]; }
+                            }
+                            if (lane == 31) rc[gs + k + 1] = make_uint2(st.w, st.flast);
+                            off = offn;
                         }
                     }
                 }
                 if constexpr (MODE == kModeScoreCk) {
                     if (s0 + CH - 1 == next_ck && next_ck < n) {   // the same for every lane
-                        // staircase in the two-positions form: the top half's rows at column
-                        // next_ck - 2 lane, the bottom half's at next_ck - 2 lane - 1; unscaled
                         const long long kk = (next_ck + 1) / T.colck_every - 1;
                         int2 *cc = T.colck + kk * T.colck_ld + (T.row0 + grow);
-                        const int B = st.B;
 #pragma unroll
-                        for (int k = 0; k < H; k += 2) {
-                            *reinterpret_cast<int4 *>(cc + k) =
-                                make_int4((p16_lo(st.U[k]) + B) >> 3, (p16_lo(st.E[k]) + B) >> 3,
-                                          (p16_lo(st.U[k + 1]) + B) >> 3, (p16_lo(st.E[k + 1]) + B) >> 3);
-                            *reinterpret_cast<int4 *>(cc + H + k) =
-                                make_int4((p16_hi(st.U[k]) + B) >> 3, (p16_hi(st.E[k]) + B) >> 3,
-                                          (p16_hi(st.U[k + 1]) + B) >> 3, (p16_hi(st.E[k + 1]) + B) >> 3);
+                        for (int k = 0; k < H; ++k) {
+                            cc[k] = make_int2(p16_lo(st.U[k]) + B, p16_lo(st.E[k]) + B);
+                            cc[H + k] = make_int2(p16_hi(st.U[k]) + B, p16_hi(st.E[k]) + B);
                         }
                         int2 *ca = T.colck_aux + kk * (T.colck_ld / H) + (T.row0 + grow) / H;
-                        ca[0] = make_int2((p16_lo(st.udiag0) + B) >> 3, (p16_lo(st.flast) + B) >> 3);
-                        ca[1] = make_int2((p16_hi(st.udiag0) + B) >> 3, (p16_hi(st.flast) + B) >> 3);
+                        ca[0] = make_int2(p16_lo(st.udiag0) + B, p16_lo(st.flast) + B);
+                        ca[1] = make_int2(p16_hi(st.udiag0) + B, p16_hi(st.flast) + B);
                         next_ck += T.colck_every;
+                    }
+                }
+                {   // a best cell in this chunk?
+                    const int lo = p16_lo(st.cmx), hi = p16_hi(st.cmx);
+                    const int thr = min(bu - B, 32767);
+                    if (__any_sync(kFull, max(lo, hi) >= thr)) {
+                        const int wm = __reduce_max_sync(kFull, max(lo, hi)) + B;
+                        bool take = wm > bu || !held;          // a larger score
+                        if (!take) {
+                            // the same score again: the earlier half-lane holds the earlier rows; within one half-lane the
+                            // rows decide, which are found later
+                            const int bpos = p16_first_pos(bcm, bu - bcb), pos = p16_first_pos(st.cmx, bu - B);
+                            take = pos < bpos;
+                            if (pos == bpos && brow != 0) {
+                                if (npend == 2) {
+                                    resolve(bpos);
+                                    npend = 0;
+                                }
+                                if (brow != 0) {
+                                    if (npend++ == 0) pa = cur; else pb = cur;
+                                    cur = npend == 1 ? (pa + 1) % 3 : 3 - pa - pb;
+                                }
+                            }
+                        }
+                        if (take) {
+                            bu = wm; held = true; brow = R; bcm = st.cmx; bcb = B;
+                            pa = cur; npend = 1;
+                            cur = (cur + 1) % 3;
+                        }
                     }
                 }
                 __syncwarp();
                 if (lane == 0) {
-                    sts_release(&cons[warp], min(n, s0 + CH));
-                    if (out_hi > 0) sts_release(&prod[warp + 1], out_hi);
+                    __threadfence_block();
+                    *(volatile int *)&cons[warp] = s0 + CH;
+                    if (out_hi > 0) *(volatile int *)&prod[warp + 1] = out_hi;
                 }
             }
-            if (!LEFT || p16_lo(st.kbest) > -32768) st.best[0] = max(st.best[0], p16_lo(st.kbest) + st.B);
-            if (!LEFT || p16_hi(st.kbest) > -32768) st.best[1] = max(st.best[1], p16_hi(st.kbest) + st.B);
-
-            // the lane's candidate: the better of its halves (top rows come first)
             int cs = 0, cj = 0x7fffffff, ci = 0x7fffffff;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int key = st.best[h];
-                const int row = grow + h * H + (7 - (key & 7));      // tag 7 - k gives row k of the half
-                const int sc = (key >> 3) + go;                      // the value's multiple of 8, unscaled
-                if (sc > 0 && row < T.rows && cand_better(sc, st.bcol[h] + 1, T.row0 + row + 1, cs, cj, ci)) {
-                    cs = sc; cj = st.bcol[h] + 1; ci = T.row0 + row + 1;
+            if (ok && held) {
+                const int bpos = p16_first_pos(bcm, bu - bcb);
+                resolve(bpos);
+                if (brow < H) {
+                    cs = bu + go; cj = bcol + 1;
+                    ci = T.row0 + rbase + (warp * 32 + (bpos >> 1)) * R + (bpos & 1) * H + brow + 1;
                 }
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const int os = __shfl_xor_sync(kFull, cs, off);
-                const int oj = __shfl_xor_sync(kFull, cj, off);
-                const int oi = __shfl_xor_sync(kFull, ci, off);
-                if (cand_better(os, oj, oi, cs, cj, ci)) { cs = os; cj = oj; ci = oi; }
             }
             if (lane == 0) s_cand[warp] = make_int4(cs, ci, cj, 0);
         }

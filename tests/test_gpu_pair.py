@@ -451,3 +451,59 @@ def test_bounded_wait_timeout(oracle_mod, monkeypatch):
         assert (got.score, got.a_end, got.b_end) == want
     finally:
         c2.close()
+
+
+@pytest.fixture(scope="module", params=[8, 12, 16])
+def packed_ctx(request):
+    """A context on the packed fill with a fixed number of rows a lane."""
+    from paper_2211_10769_gb300 import binding
+    old = os.environ.get("SWGB_FWD")
+    os.environ["SWGB_FWD"] = "%d,4,0,2,1" % request.param
+    try:
+        c = binding.Context(0)
+    finally:
+        if old is None:
+            del os.environ["SWGB_FWD"]
+        else:
+            os.environ["SWGB_FWD"] = old
+    yield c
+    c.close()
+
+
+def test_packed_end_cell_among_ties(packed_ctx, oracle_mod):
+    """Many equal maxima: the packed fill keeps only chunk maxima during the
+    sweep and looks the first row and column up afterwards, from up to two kept
+    chunks, so ties within one half-lane over several chunks, between
+    half-lanes, warps and strips, and at the sweep's ends must all resolve to the
+    row-major first."""
+    g = np.random.default_rng(W.BASE_SEED + 8500)
+    for t in range(120):
+        K = int(g.integers(1, 5))
+        m = int(g.choice([3, 7, 40, 200, 600, 2100]))
+        n = int(g.choice([1, 31, 32, 33, 97, 160, 700, 1500]))
+        a, b = g.integers(0, K, size=m).astype(np.uint8), g.integers(0, K, size=n).astype(np.uint8)
+        if t % 3 == 0:                       # periodic: the same maximum in every chunk
+            b = np.resize(b[:int(g.integers(1, 40))], n)
+        if t % 6 == 1:
+            a = np.resize(a[:int(g.integers(1, 9))], m)
+        S = np.where(np.eye(4, dtype=bool), 1, -int(g.integers(1, 4))).astype(np.int8)
+        o = int(g.integers(0, 6))
+        _score_case(packed_ctx, oracle_mod, a, b, S, o, int(g.integers(0, o + 1)))
+
+
+def test_packed_base_moves(packed_ctx, oracle_mod):
+    """Scores far above 16 bits: the warps' bases follow the path up and the
+    decay beside it down, and penalties or scores at the edge of the packed
+    fill's exactness bound (some of them beyond it, which the int32 fill takes)."""
+    for S, o, e, K in ((100, 30, 2, 4), (20, 25, 25, 4), (24, 60, 1, 4), (11, 40, 1, 20), (127, 5, 5, 4)):
+        mat = np.full((K, K), -S // 2, np.int8)
+        np.fill_diagonal(mat, S)
+        g = np.random.default_rng(W.BASE_SEED + 8600 + S)
+        a = g.integers(0, K, size=5000).astype(np.uint8)
+        b = np.concatenate([g.integers(0, K, size=333).astype(np.uint8), W.mutate(a[200:4100], K, S),
+                            g.integers(0, K, size=1500).astype(np.uint8)])
+        _score_case(packed_ctx, oracle_mod, a, b, mat, o, e)
+        _score_case(packed_ctx, oracle_mod, b, a, mat, o, e)
+    S, o, e = W.protein_scoring().matrix, 10, 1
+    a = W.random_protein(4200, W.BASE_SEED + 8610)
+    _align_case(packed_ctx, oracle_mod, a, W.mutate(a, 20, W.BASE_SEED + 8611), S, o, e)
