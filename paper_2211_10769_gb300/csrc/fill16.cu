@@ -2,6 +2,7 @@
 // the test of whether a scoring scheme and tile shape keep it exact.
 #include "sw.h"
 #include "sw_ctx.h"
+#include "straighten.cuh"
 #include "wavefront16.cuh"
 
 #include <algorithm>
@@ -12,8 +13,13 @@ using namespace swgb;
 
 namespace {
 
+// steps by which a warp trails the one above, and clocks of a step (measured, R = 4 .. 26, one strip)
+constexpr double kP16ChainSteps = 105;
+constexpr double p16_step_clocks(int R) { return R <= 8 ? 70 + 3.3 * R : (R <= 16 ? 53 + 5.4 * R : 46 + 6.1 * R); }
+
 // largest pair profile (small alphabets); larger alphabets take the int16 profile
-constexpr size_t kPairProfileMax = 110 * 1024;
+constexpr size_t kPairProfileMax = 170 * 1024;
+constexpr size_t kSharedMax = 227 * 1024;          // shared memory a block can have
 
 template <int R, int W, int MODE, int PK, bool LEFT>
 int launch16(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int max_blocks) {
@@ -22,7 +28,7 @@ int launch16(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int max_b
     static int attr_set[64] = {0};
     if (c->device >= 64 || !attr_set[c->device]) {
         const size_t cap = p16_shared_bytes<R, W>() + (PK == kP16Pair ? kPairProfileMax : p16_profile_bytes(R, W, kMaxAlphabet, PK));
-        CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
+        CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(cap, kSharedMax)));
         if (c->device < 64) attr_set[c->device] = 1;
     }
     int occ = 0;
@@ -38,11 +44,18 @@ int launch16(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int max_b
     return SW_OK;
 }
 
+// Whether a block of W compute warps at R rows a lane takes the pair profile for K residue codes (it has to fit).
+template <int R, int W>
+bool pair_profile_fits(int K) {
+    const size_t p = p16_profile_bytes(R, W, K, kP16Pair);
+    return p <= kPairProfileMax && p16_shared_bytes<R, W>() + p <= kSharedMax;
+}
+
 template <int R, int MODE, bool LEFT = false, int W = 4>
 int launch16_pk(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int B) {
-    if (p16_profile_bytes(R, W, K, kP16Pair) <= kPairProfileMax)
-        return launch16<R, W, MODE, kP16Pair, LEFT>(c, L, K, tickets, B);
-    return launch16<R, W, MODE, kP16Int16, LEFT>(c, L, K, tickets, B);
+    if (pair_profile_fits<R, W>(K)) return launch16<R, W, MODE, kP16Pair, LEFT>(c, L, K, tickets, B);
+    if constexpr (R == 8 || R == 12 || R == 16) return launch16<R, W, MODE, kP16Int16, LEFT>(c, L, K, tickets, B);
+    else return SW_EINVAL;                          // (p16_fits keeps other shapes to small alphabets)
 }
 
 // left: the coarse-tile refills (checkpoint mode only), whose tasks enter the
@@ -51,7 +64,8 @@ int launch16_pk(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int B)
 // four warps runs its pair's width with one to four of them busy).
 template <int R>
 int launch16_mode(sw_ctx *c, int mode, bool left, int W, const FillLaunch &L, int K, long long tickets, int B) {
-    if (W == 2) return mode == kModeScore && !left ? launch16_pk<R, kModeScore, false, 2>(c, L, K, tickets, B) : SW_EINVAL;
+    if constexpr (R == 8 || R == 12 || R == 16)
+        if (W == 2) return mode == kModeScore && !left ? launch16_pk<R, kModeScore, false, 2>(c, L, K, tickets, B) : SW_EINVAL;
     if (W != 4) return SW_EINVAL;
     if (left) return mode == kModeScoreCk ? launch16_pk<R, kModeScoreCk, true>(c, L, K, tickets, B) : SW_EINVAL;
     switch (mode) {
@@ -61,10 +75,31 @@ int launch16_mode(sw_ctx *c, int mode, bool left, int W, const FillLaunch &L, in
     }
 }
 
+template <int R>
+int launch_straighten_r(sw_ctx *c, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc) {
+    const int wpt = (max_rows + 32 * R - 1) / (32 * R);
+    const long long threads = 32LL * wpt * ntasks;
+    straighten_kernel<R><<<(unsigned)((threads + kStraightThreads - 1) / kStraightThreads), kStraightThreads, 0,
+                           c->stream>>>(tasks, ntasks, wpt, sc);
+    CU(cudaGetLastError());
+    ++c->launches;
+    return SW_OK;
+}
+
+// shapes with a pair profile only, for pairs of small alphabets
+#define SWGB_P16_PAIR_SHAPES(X) X(10) X(14) X(20) X(26)
+#define SWGB_P16_SHAPES(X) X(8) X(12) X(16) SWGB_P16_PAIR_SHAPES(X)
+
 }  // namespace
 
 bool swgb::p16_fits(const DevScoring &s, int R) {
-    if (R != 8 && R != 12 && R != 16) return false;
+    switch (R) {
+        case 8: case 12: case 16: break;
+#define SWGB_P16_CASE(R) case R: if (!pair_profile_fits<R, 4>(s.K)) return false; break;
+        SWGB_P16_PAIR_SHAPES(SWGB_P16_CASE)
+#undef SWGB_P16_CASE
+        default: return false;
+    }
     if (s.alg != kAlgLocal) return false;            // the packed fill keeps the zero floor
     int lo = 127, hi = -128;
     for (int k = 0; k < s.K * s.K; ++k) { lo = std::min(lo, (int)s.mat[k]); hi = std::max(hi, (int)s.mat[k]); }
@@ -75,9 +110,50 @@ int swgb::launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, const FillLa
                         long long tickets) {
     if (tickets <= 0) return SW_OK;
     switch (cfg.R) {
-        case 8: return launch16_mode<8>(c, mode, cfg.left != 0, cfg.W, L, K, tickets, cfg.B);
-        case 12: return launch16_mode<12>(c, mode, cfg.left != 0, cfg.W, L, K, tickets, cfg.B);
-        case 16: return launch16_mode<16>(c, mode, cfg.left != 0, cfg.W, L, K, tickets, cfg.B);
+#define SWGB_P16_CASE(R) case R: return launch16_mode<R>(c, mode, cfg.left != 0, cfg.W, L, K, tickets, cfg.B);
+        SWGB_P16_SHAPES(SWGB_P16_CASE)
+#undef SWGB_P16_CASE
         default: return SW_EINVAL;
     }
+}
+
+int swgb::launch_straighten(sw_ctx *c, int R, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc) {
+    if (ntasks <= 0) return SW_OK;
+    switch (R) {
+#define SWGB_P16_CASE(R) case R: return launch_straighten_r<R>(c, tasks, ntasks, max_rows, sc);
+        SWGB_P16_SHAPES(SWGB_P16_CASE)
+#undef SWGB_P16_CASE
+        default: return SW_EINVAL;
+    }
+}
+
+// Rows a lane of the packed fill of one m x n pair, 0 where no shape is exact
+// for the scoring.  A pair's strips (128 R rows each) form one chain: each warp
+// trails the one above by kP16ChainSteps steps (64 positions and a chunk of
+// 32, and per strip of four warps the hand-off through global memory), and
+// strips beyond one per SM follow in waves.  So the fill takes about
+//   (columns x whole waves before the last strip + its place in the chain + columns) x step(R),
+// with step(R) the measured clocks of a step of one strip (GB300): few rows a
+// lane leave a long chain of short steps, many leave SMs idle.  Measured, score
+// fills: 8 kbp R = 4 / 6 / 8: 0.69 / 0.65 / 0.63 ms; 30 kbp R = 6 / 8 / 10:
+// 2.25 / 2.17 / 2.18; 200 kbp R = 12 / 14: 15.3 / 16.0; 1 Mbp R = 14 / 16 / 20:
+// 257 / 270 / 260 ms.
+int swgb::p16_rows_per_lane(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &s) {
+    static constexpr struct { int R; double clk; } kShapes[] = {
+#define SWGB_P16_ROW(R) {R, p16_step_clocks(R)},
+        SWGB_P16_SHAPES(SWGB_P16_ROW)
+#undef SWGB_P16_ROW
+    };
+    int best = 0;
+    double best_cost = 1e300;
+    for (const auto &q : kShapes) {
+        if (!p16_fits(s, q.R)) continue;
+        const int64_t last = (m + 128LL * q.R - 1) / (128LL * q.R) - 1;      // the last strip
+        const double wave = std::max((double)n, c->nsm * kP16ChainSteps * 4);
+        const double steps = (double)(last / c->nsm) * wave + (double)(last % c->nsm) * kP16ChainSteps * 4 + (double)n +
+                             kP16ChainSteps * std::min<double>(4.0, (double)m / (32.0 * q.R));
+        const double cost = steps * q.clk;
+        if (cost < best_cost) { best_cost = cost; best = q.R; }
+    }
+    return best;
 }

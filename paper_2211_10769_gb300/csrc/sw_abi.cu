@@ -252,11 +252,15 @@ FillConfig swgb::pair_fill_config(const sw_ctx *c, int64_t rows) {
     return FillConfig{16, 4, 0, 2};
 }
 
+constexpr int64_t kPackedMinSum = 2048;
+
 // Tile shape of a single-pair fill with scoring s: the packed 16-bit fill
-// (two cells per lane operation) where it is exact for the shape, with the
-// fewest rows per lane in {8, 12, 16} that give at most one strip per SM;
-// else the int32 fill of pair_fill_config.
-FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, const DevScoring &s) {
+// (two cells per lane operation) where it is exact, with the rows a lane that
+// p16_rows_per_lane picks; else the int32 fill of pair_fill_config.  Below
+// kPackedMinSum rows plus columns the int32 fill's shorter set-up wins (score:
+// 500 x 500 0.094 against 0.096 ms, 1,000 0.135 against 0.132, 2 kbp 0.221
+// against 0.199, 30 kbp 2.55 against 2.17).
+FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s) {
     if (s.alg != kAlgLocal) {
         FillConfig f = variant_fill_config(c, rows);
         if (!c->fwd_auto && (c->fwd.R == 8 || c->fwd.R == 12 || c->fwd.R == 16)) f.R = c->fwd.R;   // SWGB_FWD
@@ -267,18 +271,9 @@ FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, const DevSc
         f.P16 = f.P16 && p16_fits(s, f.R) && f.W == 4;
         return f;
     }
-    // Up to one 512-row strip per SM the int32 fill's 4-row lanes use twice the SMs of the packed
-    // fill's 8-row lanes, which outweighs the packed fill's cheaper cells (2 kbp: 0.170 against
-    // 0.190 ms); above that both take the same SM count and the packed fill wins (200 kbp: 19.8
-    // against 24.0 ms)
-    if (c->p16 && rows > (int64_t)c->nsm * 4 * 32 * 4) {
-        for (int R : {8, 12, 16}) {
-            const int64_t sh = 4LL * 32 * R;
-            if ((rows + sh - 1) / sh <= (int64_t)c->nsm || R == 16) {
-                if (p16_fits(s, R)) return FillConfig{R, 4, 0, 2, 1};
-                break;
-            }
-        }
+    if (c->p16 && rows + cols >= kPackedMinSum) {
+        const int R = p16_rows_per_lane(c, rows, cols, s);
+        if (R > 0) return FillConfig{R, 4, 0, 2, 1};
     }
     return pair_fill_config(c, rows);
 }
@@ -320,7 +315,7 @@ int swgb::launch_fill(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, con
 // Runs the fill over `tasks` (already in host memory, ticket0 assigned) on
 // stream st with buffers b, and leaves the per-strip candidates in b.cand.
 int swgb::run_fill_with(sw_ctx *c, const FillBufs &b, cudaStream_t st, const FillConfig &cfg, int mode, bool fold,
-                        const std::vector<FillTask> &tasks, long long tickets, int K) {
+                        const std::vector<FillTask> &tasks, long long tickets, int K, int straight_R) {
     const size_t tbytes = tasks.size() * sizeof(FillTask);
     RC(b.tasks->ensure(tbytes));
     RC(b.prog->ensure((size_t)tickets * sizeof(int)));
@@ -345,7 +340,13 @@ int swgb::run_fill_with(sw_ctx *c, const FillBufs &b, cudaStream_t st, const Fil
     // before they stage another fill on the same buffers (every ABI call ends with a sync)
     const cudaStream_t home = c->stream;
     c->stream = st;
-    const int rc = launch_fill(c, cfg, mode, fold, L, K, tickets);
+    int rc = SW_OK;
+    if (straight_R > 0) {
+        int max_rows = 0;
+        for (const FillTask &t : tasks) max_rows = std::max(max_rows, t.straight ? t.rows : 0);
+        if (max_rows > 0) rc = launch_straighten(c, straight_R, L.tasks, (int)tasks.size(), max_rows, L.scorings);
+    }
+    if (!rc) rc = launch_fill(c, cfg, mode, fold, L, K, tickets);
     c->stream = home;
     return rc;
 }
@@ -542,7 +543,7 @@ int sw_score(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b, int64_t n
     RC(validate_codes(c, db, n, ds.K));
     RC(upload_scorings(c, {ds}));
 
-    const FillConfig fwd = pair_fill_config_for(c, m, ds);
+    const FillConfig fwd = pair_fill_config_for(c, m, n, ds);
     const int sw = pair_strip_warps(c, fwd, m);
     const int SH = sw * 32 * fwd.R;
     FillTask t{};

@@ -182,7 +182,7 @@ int refill_coarse_tile(sw_ctx *c, const uint8_t *da, const uint8_t *db, int64_t 
     if (CJ > 0) {
         t.left = colck + (size_t)(CJ - 1) * colck_ld + R0c;
         t.left_aux = colaux + (size_t)(CJ - 1) * colaux_ld + R0c / aux_rows;
-        t.left_split = fwd.P16 ? 1 : 0;
+        t.left_split = fwd.P16 ? fwd.R : 0;
     }
     t.row0 = (int32_t)R0c;
     t.col0 = (int32_t)C0c;
@@ -213,6 +213,18 @@ int refill_coarse_tile(sw_ctx *c, const uint8_t *da, const uint8_t *db, int64_t 
 
 // Sides up to this many cells may take the one-round reconstruction below.
 constexpr int64_t kOneRoundSide = 8192;
+constexpr int64_t kOneRoundPackedSide = 4096;
+
+// Tile shape of the traceback fill after forward fill fwd: int32 (bits come from
+// the int32 fill); after the packed fill, whose checkpoint columns are
+// straightened, the context's shape (8 rows a lane); after an int32 fill the
+// tiles continue its staircase columns lane by lane, so they take its rows a lane.
+FillConfig traceback_config(const sw_ctx *c, const FillConfig &fwd) {
+    FillConfig t = (fwd.alg == kAlgLocal && (fwd.P16 || c->tbc.R == fwd.R)) ? c->tbc : FillConfig{fwd.R, 4};
+    t.P16 = 0;
+    t.alg = fwd.alg;
+    return t;
+}
 
 // Tile side of a small pair's reconstruction: a multiple of both fills' strip
 // heights and of the chunk, at least kWalkMinBT, the smallest whose tiles fit
@@ -220,17 +232,19 @@ constexpr int64_t kOneRoundSide = 8192;
 // none fits the chunk.
 long long small_pair_tile(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &ds, FillConfig *fwd_out,
                           FillConfig *tbc_out, int *sw_out, int *tsw_out) {
-    const FillConfig fwd = pair_fill_config_for(c, m, ds);
-    // strips of two compute warps (at R = 4: 256 rows) in both fills, so that a tile can be one
-    // two-warp strip of 256 rows: a small pair's forward chain has as many warps either way, and
-    // a tile recomputes in about half the steps of a 512-row one
-    const int sw = c->fwd_auto ? std::min(2, fwd.W) : pair_strip_warps(c, fwd, m);
+    // the packed fill at 8 rows a lane above kOneRoundPackedSide; below it the int32 fill, which needs no
+    // straightened columns (a launch and 63 dependent steps): 1,000 0.237 against 0.253 ms, 2,800 0.436 against
+    // 0.442, 8,000 1.185 against 1.134
+    FillConfig fwd = pair_fill_config_for(c, m, n, ds);
+    if (c->fwd_auto && fwd.P16)
+        fwd = std::max(m, n) > kOneRoundPackedSide && p16_fits(ds, 8) ? FillConfig{8, 4, 0, 2, 1} : pair_fill_config(c, m);
+    // strips of 256 rows where the fill allows it (one compute warp of the packed fill at 8 rows a lane, two of
+    // the int32 fill at 4): a small pair's forward chain has as many warps either way, and a 256-row tile
+    // recomputes in about half the steps of a 512-row one
+    const int sw = c->fwd_auto ? std::max(1, std::min(256 / (32 * fwd.R), fwd.W)) : pair_strip_warps(c, fwd, m);
     const int HC = sw * 32 * fwd.R;
-    // the traceback tiles continue the forward fill's staircase checkpoint columns lane by
-    // lane, so both fills must give each lane the same rows (R)
-    FillConfig tbc = (c->tbc.R == fwd.R && fwd.alg == kAlgLocal) ? c->tbc : FillConfig{fwd.R, 4};
-    tbc.P16 = 0;
-    tbc.alg = fwd.alg;
+    FillConfig tbc = traceback_config(c, fwd);
+    if (fwd.P16 && c->fwd_auto) tbc = FillConfig{4, 4, 0, 0, 0, fwd.alg};   // 256-row strips of two warps
     const int tsw = c->tb_strip_warps > 0 ? std::min(c->tb_strip_warps, tbc.W) : std::min(2, tbc.W);
     const long long BL = std::lcm((long long)HC, (long long)tsw * 32 * tbc.R);
     long long BT = BL * ((kWalkMinBT + BL - 1) / BL);
@@ -291,6 +305,7 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
 
     RC(c->tb.ensure((size_t)ntiles * tile_bytes));
     RC(c->tbbnd.ensure((size_t)ntiles * 2 * (size_t)BT * sizeof(int2)));
+    if (fwd.P16) RC(c->straight.ensure((size_t)ntiles * (size_t)BT * sizeof(int2)));
     std::vector<FillTask> tasks;                    // [0]: the forward fill; then every tile
     tasks.reserve((size_t)ntiles + 1);
     tasks.push_back(t);
@@ -311,9 +326,10 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
             if (c0 > 0) {
                 u.left = colck + (size_t)(c0 / BT - 1) * colck_ld + r0;
                 u.left_aux = colaux + (size_t)(c0 / BT - 1) * colaux_ld + r0 / aux_rows;
-                u.left_split = fwd.P16 ? 1 : 0;
+                u.left_split = fwd.P16 ? fwd.R : 0;
             }
             const size_t k = tasks.size() - 1;
+            if (u.left_split) u.straight = static_cast<int2 *>(c->straight.p) + k * (size_t)BT;
             u.nslot = std::min(u.nstrips, 2);
             u.bnd = static_cast<int2 *>(c->tbbnd.p) + k * 2 * (size_t)BT;
             u.row0 = (int32_t)r0;
@@ -369,6 +385,8 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
     Lt.cand = static_cast<int4 *>(c->cand.p) + t.nstrips;
     Lt.total = tickets;
     Lt.ntasks = ntiles;
+    if (fwd.P16 && nJ > 1)
+        RC(launch_straighten(c, fwd.R, dtasks + 1, ntiles, (int)std::min<int64_t>(BT, m), L.scorings));
     RC(launch_fill(c, tbc, kModeTb, fold, Lt, ds.K, tickets));
     walk_start_kernel<<<1, 32, 0, c->stream>>>(static_cast<const int4 *>(c->result.p), ds.alg == kAlgLocal ? 1 : 0,
                                                static_cast<WalkState *>(c->walk.p));
@@ -438,18 +456,16 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     // tiles are BT x BT; BT is a multiple of both fills' strip heights, so
     // checkpoint rows fall on forward-strip bottoms and tiles hold whole
     // traceback strips
-    const FillConfig fwd = pair_fill_config_for(c, m, ds);
+    const FillConfig fwd = pair_fill_config_for(c, m, n, ds);
     const int sw = pair_strip_warps(c, fwd, m);
     const int HC = sw * 32 * fwd.R;
-    // the traceback tiles continue the forward fill's staircase checkpoint columns lane by
-    // lane, so both fills must give each lane the same rows (R)
-    FillConfig tbc = (c->tbc.R == fwd.R && fwd.alg == kAlgLocal) ? c->tbc : FillConfig{fwd.R, 4};
-    tbc.P16 = 0;                                  // traceback bits come from the int32 fill
-    tbc.alg = fwd.alg;
+    const FillConfig tbc = traceback_config(c, fwd);
     // the packed forward fill stores its checkpoint columns with two positions per lane and
     // one auxiliary record per half-group of R/2 rows
     const int aux_rows = fwd.P16 ? fwd.R / 2 : fwd.R;
-    const int HT = fill_rows_per_strip(tbc);
+    // tiles hold whole traceback strips of an int32 forward fill's rows a lane; after the packed fill whole
+    // row groups are enough (the last strip of a tile may be partial)
+    const int HT = fwd.P16 ? 32 * tbc.R : fill_rows_per_strip(tbc);
     const int HC2 = 4 * 32 * fwd.R;                // strip height of a coarse tile's refill (int32, 4 warps)
     const long long BL = std::lcm((long long)HC, (long long)HT);
     const long long BL2 = std::lcm((long long)HC2, (long long)HT);
@@ -561,6 +577,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     const int maxtiles = 3 * band;
     RC(c->tb.ensure(tile_bytes * maxtiles));
     RC(c->tbbnd.ensure((size_t)maxtiles * 2 * (size_t)BT * sizeof(int2)));
+    if (fwd.P16) RC(c->straight.ensure((size_t)maxtiles * (size_t)BT * sizeof(int2)));
     RC(c->misc.ensure(table_cap * sizeof(void *)));
     // level 1: the forward fill's checkpoints (every BT1); level 2 (two levels only): those of
     // the current coarse tile's refill (every BT2 inside it), over rows [R0c, Wi0) and
@@ -586,6 +603,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
         bd.slot = slot;
         char *tbp = static_cast<char *>(slot ? c->tb_b.p : c->tb.p);
         int2 *bndp = static_cast<int2 *>(slot ? c->tbbnd_b.p : c->tbbnd.p);
+        int2 *strp = static_cast<int2 *>(slot ? c->straight_b.p : c->straight.p);
         const int I = (int)((wi - 1) / BT), J = (int)((wj - 1) / BT);
         const int It0 = (int)(R0c / BT), Jt0 = (int)(C0c / BT);       // the region's first tile row, column
         const int I0 = std::max(It0, I - band + 1);
@@ -631,13 +649,14 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
                 } else if (c0 % BT1 == 0) {
                     u.left = colck + (size_t)(c0 / BT1 - 1) * colck_ld + r0;
                     u.left_aux = colaux + (size_t)(c0 / BT1 - 1) * colaux_ld + r0 / aux_rows;
-                    u.left_split = fwd.P16 ? 1 : 0;
+                    u.left_split = fwd.P16 ? fwd.R : 0;
                 } else {
                     u.left = colck2 + (size_t)((c0 - C0c) / BT - 1) * ld2 + (r0 - R0c);
                     u.left_aux = colaux2 + (size_t)((c0 - C0c) / BT - 1) * (ld2 / aux_rows) + (r0 - R0c) / aux_rows;
-                    u.left_split = fwd.P16 ? 1 : 0;
+                    u.left_split = fwd.P16 ? fwd.R : 0;
                 }
                 const size_t k = bd.tasks.size();
+                if (u.left_split) u.straight = strp + k * (size_t)BT;
                 u.nslot = std::min(u.nstrips, 2);
                 u.bnd = bndp + k * 2 * (size_t)BT;
                 u.ckpt_every = 0; u.ckpt = nullptr; u.colck = nullptr; u.colck_every = 0;
@@ -659,6 +678,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     if (ahead) {
         RC(c->tb_b.ensure(tile_bytes * maxtiles));
         RC(c->tbbnd_b.ensure((size_t)maxtiles * 2 * (size_t)BT * sizeof(int2)));
+        if (fwd.P16) RC(c->straight_b.ensure((size_t)maxtiles * (size_t)BT * sizeof(int2)));
         RC(c->misc_b.ensure(table_cap * sizeof(void *)));
         if (!c->side) CU(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
         if (!c->side_go) CU(cudaEventCreateWithFlags(&c->side_go, cudaEventDisableTiming));
@@ -699,7 +719,8 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
         }
         if (!use_spec) {
             build_band(w.i, w.j, 0, cur);
-            RC(run_fill_with(c, main_bufs, c->stream, tbc, kModeTb, fold, cur.tasks, cur.tickets, ds.K));
+            RC(run_fill_with(c, main_bufs, c->stream, tbc, kModeTb, fold, cur.tasks, cur.tickets, ds.K,
+                             fwd.P16 ? fwd.R : 0));
         }
         const size_t tbytes = cur.table.size() * sizeof(void *);
         if (tbytes > c->stage2.cap) return SW_EINVAL;
@@ -717,7 +738,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
                 if (!spec.tasks.empty()) {
                     CU(cudaStreamWaitEvent(c->side, c->side_go, 0));
                     RC(run_fill_with(c, spec.slot ? side_bufs : main_bufs, c->side, tbc, kModeTb, fold, spec.tasks,
-                                     spec.tickets, ds.K));
+                                     spec.tickets, ds.K, fwd.P16 ? fwd.R : 0));
                     CU(cudaEventRecord(c->side_done, c->side));
                     have_spec = true;
                 }

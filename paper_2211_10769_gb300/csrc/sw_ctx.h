@@ -85,7 +85,7 @@ struct sw_ctx {
     size_t tb_budget = 0;             // bytes of traceback bits per row group
     swgb::DevBuf seq_a, seq_b, tasks, scorings, ticket, prog, cand, result, err, bnd, ckpt, colck, colaux, tb,
         ckpt2, colck2, colaux2,
-        tbbnd, runs, walk, misc, dbscratch, dbslots, dbovf, dbjob, dbscores, topk;
+        tbbnd, straight, straight_b, runs, walk, misc, dbscratch, dbslots, dbovf, dbjob, dbscores, topk;
     swgb::HostBuf stage, stage2, stage3;
     // sw_align's look-ahead band: a second set of traceback-fill buffers and a stream of their
     // own, so that the next band's tiles are recomputed while the walk goes through the current one
@@ -108,7 +108,10 @@ int map_kernel_error(int e);
 int fill_rows_per_strip(const FillConfig &cfg);
 int pair_strip_warps(const sw_ctx *c, const FillConfig &cfg, int64_t rows);
 FillConfig pair_fill_config(const sw_ctx *c, int64_t rows);
-FillConfig pair_fill_config_for(const sw_ctx *c, int64_t rows, const DevScoring &s);   // picks P16 where exact
+FillConfig pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s);   // picks P16 where exact
+int p16_rows_per_lane(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &s);
+// the packed checkpoint columns of tasks with FillTask::straight brought to one column (R: the writer's rows a lane)
+int launch_straighten(sw_ctx *c, int R, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc);
 bool p16_fits(const DevScoring &s, int R);
 int launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K, long long tickets);
 // the global, semi-global and overlap algorithms: 8 or 16 rows a lane, four compute warps
@@ -127,8 +130,9 @@ struct FillBufs {
     DevBuf *tasks, *prog, *cand, *ticket;
     HostBuf *stage;
 };
+// straight_R > 0: the tasks' packed checkpoint columns are straightened first (launch_straighten)
 int run_fill_with(sw_ctx *c, const FillBufs &b, cudaStream_t st, const FillConfig &cfg, int mode, bool fold,
-                  const std::vector<FillTask> &tasks, long long tickets, int K);
+                  const std::vector<FillTask> &tasks, long long tickets, int K, int straight_R = 0);
 int run_fill(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const std::vector<FillTask> &tasks,
              long long tickets, int K);
 int upload_scorings(sw_ctx *c, const std::vector<DevScoring> &s);

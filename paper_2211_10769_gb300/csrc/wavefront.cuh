@@ -81,10 +81,12 @@ struct FillTask {
     int64_t tb_ld;
     int32_t strip_warps;   // compute warps per strip (rows per strip = strip_warps * 32 * R);
                            // 0 = all W warps of the block
-    int32_t left_split;    // left / left_aux in the two-positions-per-lane form of the packed
-                           // fill (wavefront16.cuh): the first R/2 rows of lane l sit at column
-                           // c - 2l, the other R/2 at c - 2l - 1, and left_aux holds one record
+    int32_t left_split;    // rows a lane R of the packed fill (wavefront16.cuh) that wrote left / left_aux,
+                           // or 0: its two-positions-per-lane form, where the first R/2 rows of lane l sit at
+                           // column c - 2l, the other R/2 at c - 2l - 1, and left_aux holds one record
                            // per half-group of R/2 rows (first the top half's, then the bottom's)
+    int2 *straight;        // left brought to column c for every row, (H - open, E) (straighten_kernel):
+                           // traceback tiles of a packed fill's checkpoints enter from it
 };
 
 struct FillLaunch {
@@ -328,86 +330,6 @@ __device__ __forceinline__ void lane_step(LaneState<R> &st, const uint32_t (&pw)
     }
 }
 
-// Rows [r0, r1) of one lane advanced by one column (the Gotoh update of
-// column_update restricted to a range of the lane's rows), entered with the
-// row above's H - open and F at this column; udiag = H - open of the row
-// above at the previous column.  Returns the last row's F in *fout.
-template <int R, int PK, bool LOCAL>
-__device__ __forceinline__ void rows_update(LaneState<R> &st, const uint32_t (&pw)[ProfWords<R, PK>::N], int r0,
-                                            int r1, int uup, int fup, int udiag, int go, int ge, int *fout)
-{
-    int f = __viaddmax_s32(fup, -ge, uup);
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        if (r < r0 || r >= r1) continue;
-        int sp = score_at<PK>(pw, r);
-        if constexpr (PK == kProf8) sp += go;
-        const int uold = st.U[r];
-        const int e = __viaddmax_s32(st.E[r], -ge, uold);
-        const int x = LOCAL ? __viaddmax_s32_relu(udiag, sp, e) : __viaddmax_s32(udiag, sp, e);
-        const int xgo = x - go;
-        st.U[r] = __viaddmax_s32(f, -go, xgo);
-        st.E[r] = e;
-        udiag = uold;
-        if (r + 1 < r1) f = __viaddmax_s32(f, -ge, xgo);
-    }
-    *fout = f;
-}
-
-// A task entered from a checkpoint column written by the packed fill, whose
-// lanes hold two wavefront positions each: lane l's top half (rows
-// [0, R/2)) sits at column c - 2l, its bottom half at c - 2l - 1, where c is
-// the column left of the task.  Position v = 2l (top) or 2l + 1 (bottom)
-// advances v columns, in step with its neighbours -- the top half's k-th
-// column needs lane l-1's bottom half after its (k-1)-th, the bottom half's
-// needs this lane's top half after its (k-1)-th -- so that every row ends at
-// column c: a 63-step wavefront inside the warp.  Leaves st as the straight
-// boundary column the sweep starts from (U, E per row; ub / fb the last
-// row's H - open and F at c; udiag0 the row above at c for lane 0).
-template <int R, int W, int PK, bool LOCAL>
-__device__ __forceinline__ void split_staircase_prologue(const FillTask &T, LaneState<R> &st, const int8_t *prow,
-                                                         int grow, int lane, int K, int go, int ge)
-{
-    constexpr int H = R / 2;
-    constexpr int HC = W * 32 * R;
-    constexpr size_t PB = PK == kProf32 ? 4 : 1;
-    constexpr int NPW = ProfWords<R, PK>::N;
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (grow + r < T.rows) { const int2 v = __ldcg(T.left + grow + r); st.U[r] = v.x; st.E[r] = v.y; }
-    const bool in = grow < T.rows;
-    const int2 at = in ? __ldcg(T.left_aux + grow / H) : make_int2(-go, kNeg);       // top half
-    const int2 ab = in ? __ldcg(T.left_aux + grow / H + 1) : make_int2(-go, kNeg);   // bottom half
-    int udT = at.x, fT = at.y;        // row above the top half at its column; F of its last row
-    int udB = ab.x, fB = ab.y;        // the same for the bottom half
-    for (int k = 1; k < 64; ++k) {
-        // lane l-1's bottom half after its (k-1)-th column: the row above this lane's top half
-        const int uupT = __shfl_up_sync(kFull, st.U[R - 1], 1);
-        const int fupT = __shfl_up_sync(kFull, fB, 1);
-        // the bottom half moves first: its row above is the top half before this step
-        if (k <= 2 * lane + 1) {
-            const int cb = min((int)T.b[k - 2 * lane - 2], K);   // column c - 2l - 1 + k
-            uint32_t pwk[NPW];
-            load_profile<R, PK, W * 32>(prow + cb * HC * PB, pwk);
-            const int uup = st.U[H - 1];
-            rows_update<R, PK, LOCAL>(st, pwk, H, R, uup, fT, udB, go, ge, &fB);
-            udB = uup;
-        }
-        if (k <= 2 * lane) {
-            const int cb = min((int)T.b[k - 2 * lane - 1], K);   // column c - 2l + k
-            uint32_t pwk[NPW];
-            load_profile<R, PK, W * 32>(prow + cb * HC * PB, pwk);
-            rows_update<R, PK, LOCAL>(st, pwk, 0, H, uupT, fupT, udT, go, ge, &fT);
-            udT = uupT;
-        }
-    }
-    st.ub = st.U[R - 1];
-    st.fb = fB;
-    // the diagonal of the task's first column: the row above at column c
-    const int up = __shfl_up_sync(kFull, st.ub, 1);
-    st.udiag0 = lane > 0 ? up : udT;
-}
-
 // Input warp of a fill block: streams the strip's top boundary row (the
 // matrix border, the task's top row or the previous strip's bottom row, as
 // (H - open, F)) into channel 0 of the boundary ring and the column residues
@@ -610,8 +532,14 @@ wavefront_kernel(const FillLaunch L)
             }
             st.ub = st.U[R - 1];
             st.fb = kNeg;
-            if (T.left && T.left_split) {
-                split_staircase_prologue<R, W, PK, LOCAL>(T, st, prow, grow, lane, K, go, ge);
+            if (T.straight) {
+                // a straight left column: every lane starts at column c (c = the column left of the task)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (grow + r < T.rows) { const int2 v = __ldcg(T.straight + grow + r); st.U[r] = v.x; st.E[r] = v.y; }
+                // the row above at column c: the task's first row has it in the writer's first record
+                if (grow < T.rows) st.udiag0 = grow > 0 ? __ldcg(T.straight + grow - 1).x : __ldcg(T.left_aux).x;
+                st.ub = st.U[R - 1];
             } else if (T.left) {
                 // Staircase left boundary: lane l's rows hold column c - l (c = the column
                 // left of the task).  Lane l advances l columns, in step with its neighbours

@@ -90,11 +90,14 @@ constexpr int kNeg16p = -16384;     // -infinity of a packed 16-bit lane
 constexpr int kP16Center = 16384;   // stored value of a warp's reference once B > 0
 constexpr int kP16Slack = 1024;     // drift of the reference from kP16Center before the base moves
 constexpr int kP16Span = 15000;     // largest value spread (p16_spread) the packed fill accepts
-constexpr int kP16QS = 512;         // boundary-ring columns per channel
+constexpr int kP16QS = 512;         // columns of the strip's boundary ring (channel 0)
+constexpr int kP16RS = 256;         // steps of the rings between the warps
 constexpr int kP16Pos = 64;         // wavefront positions per warp (two per lane)
 constexpr int kP16CH = 32;          // steps per chunk (hand-off, base change; 16 measured slower)
 constexpr int kP16Lag = kP16Pos - 1;   // lane 31's bottom half trails lane 0's top half
-constexpr int kP16Unroll = 16;      // steps per unrolled body (8 and 32 measured slower)
+// steps per unrolled body (12 rows a lane at 200 kbp: 8, 16, 32 steps 16.4, 15.2, 18.4 ms; 26 rows: 8 and 16 steps
+// 212 and 205 clocks a step)
+constexpr int kP16Unroll = 16;
 // An I/O warp with nothing to move sleeps this long: polling takes issue slots from the compute warp
 // beside it (200 kbp: 48 ns 15.5 ms, 128 ns 15.25 ms, 256 ns 15.15 ms)
 constexpr int kP16IdleNs = 256;
@@ -345,7 +348,6 @@ __device__ __forceinline__ void p16_input_warp(const FillTask &T, const FillLaun
 
 // Output warp: the strip's bottom row from the last active warp's channel to global memory as
 // (H, F), absolute; publishes the stored column count with a release store.
-template <int QS>
 __device__ __forceinline__ void p16_output_warp(const FillTask &T, const FillLaunch &L, int strip, long long slot,
                                                 int n, int go, int SH, int Wa, const uint2 *ringW, const int *baseW,
                                                 const int *prod, int *cons, volatile int *s_abort, int lane)
@@ -367,8 +369,8 @@ __device__ __forceinline__ void p16_output_warp(const FillTask &T, const FillLau
                 const int c0 = out_next + lane, c1 = c0 + 32;
                 const bool p0 = c0 < avail_out, p1 = c1 < avail_out;
                 const int l0 = c0 + kP16Lag, l1 = c1 + kP16Lag;
-                const uint2 v0 = ringW[l0 & (QS - 1)], v1 = ringW[l1 & (QS - 1)];
-                const int B0 = baseW[(l0 / kP16CH) & (QS / kP16CH - 1)], B1 = baseW[(l1 / kP16CH) & (QS / kP16CH - 1)];
+                const uint2 v0 = ringW[l0 & (kP16RS - 1)], v1 = ringW[l1 & (kP16RS - 1)];
+                const int B0 = baseW[(l0 / kP16CH) & (kP16RS / kP16CH - 1)], B1 = baseW[(l1 / kP16CH) & (kP16RS / kP16CH - 1)];
                 const int2 o0 = make_int2(p16_lo(v0.x) + B0 + go, p16_hi(v0.y) + B0);
                 const int2 o1 = make_int2(p16_lo(v1.x) + B1 + go, p16_hi(v1.y) + B1);
                 if (store && p0) __stcg(dst + c0, o0);
@@ -451,26 +453,33 @@ __device__ __noinline__ int2 p16_locate(const P16Snap<R> &S, const int8_t *prof,
     const bool mine = lane == (pos >> 1);
     const int h = pos & 1;
     int row = R, col = 0;
-    auto code = [&](int j) { return ((j >= 0 || T.left) && j < n) ? min((int)T.b[j], K) : K; };
+    const uint8_t *const b = T.b;
+    const int first = T.left ? -(1 << 30) : 0;
+    auto code = [&](int j) { return (j >= first && j < n) ? min((int)__ldg(b + j), K) : K; };
 #pragma unroll 1
-    for (int k = 0; k < kP16CH; ++k) {
-        const int j = S.s0 + k - 2 * lane;
-        uint32_t pw[H], pwp[H];
-        const int ct = code(j), cb = code(j - 1);
-        if constexpr (PK == kP16Pair) {
-            p16_load<R, PK, NL>(prof, g, (ct * (K + 1) + cb) * pstride, pw);
+    for (int k0 = 0; k0 < kP16CH; k0 += 4) {
+        int cc[5];                                         // residues of columns j - 1 .. j + 3, loaded together
 #pragma unroll
-            for (int x = 0; x < H; ++x) pwp[x] = 0;
-        } else {
-            p16_load<R, PK, NL>(prof, g, ct * pstride, pw);
-            p16_load<R, PK, NL>(prof, g, cb * pstride, pwp);
-        }
-        p16_step<R, PK>(st, pw, pwp, S.top[k], lane == 0, c);
-        const int jj = j - h;
-        if (mine && jj >= 0 && jj < n) {
+        for (int x = 0; x < 5; ++x) cc[x] = code(S.s0 + k0 + x - 1 - 2 * lane);
 #pragma unroll
-            for (int x = H - 1; x >= 0; --x)
-                if (x < row && x < nrows && (h ? p16_hi(st.U[x]) : p16_lo(st.U[x])) == want) { row = x; col = jj; }
+        for (int x = 0; x < 4; ++x) {
+            const int j = S.s0 + k0 + x - 2 * lane;
+            uint32_t pw[H], pwp[H];
+            if constexpr (PK == kP16Pair) {
+                p16_load<R, PK, NL>(prof, g, (cc[x + 1] * (K + 1) + cc[x]) * pstride, pw);
+#pragma unroll
+                for (int y = 0; y < H; ++y) pwp[y] = 0;
+            } else {
+                p16_load<R, PK, NL>(prof, g, cc[x + 1] * pstride, pw);
+                p16_load<R, PK, NL>(prof, g, cc[x] * pstride, pwp);
+            }
+            p16_step<R, PK>(st, pw, pwp, S.top[k0 + x], lane == 0, c);
+            const int jj = j - h;
+            if (mine && jj >= 0 && jj < n) {
+#pragma unroll
+                for (int y = H - 1; y >= 0; --y)
+                    if (y < row && y < nrows && (h ? p16_hi(st.U[y]) : p16_lo(st.U[y])) == want) { row = y; col = jj; }
+            }
         }
     }
     row = __shfl_sync(kFull, row, pos >> 1);
@@ -520,8 +529,8 @@ struct P16Shared {
     P16Snap<R> snap[W][3];
     int poff[kQB];                         // profile offset per column
     int2 ring0[kP16QS];                    // (H - open, F), absolute: the strip's boundary row
-    uint2 ring[W][kP16QS];                 // channel w + 1: after step s of warp w, at slot s, (w, F of the bottom row)
-    int base[W][kP16QS / kP16CH];          // base of warp w per chunk
+    uint2 ring[W][kP16RS];                 // channel w + 1: after step s of warp w, at slot s, (w, F of the bottom row)
+    int base[W][kP16RS / kP16CH];          // base of warp w per chunk
     int4 cand[W];
     long long tk;
     int prod[W + 1];                       // columns available in channel k
@@ -547,8 +556,8 @@ wavefront16_kernel(const FillLaunch L)
     constexpr int H = R / 2;
     constexpr int HC = W * 32 * R;
     constexpr int NL = W * 32;
-    constexpr int CH = kP16CH, QS = kP16QS, QB = kQB, LAG = kP16Lag;
-    static_assert(QS >= 2 * 64 + 2 * CH + 2 * kP16Pos, "ring too small");
+    constexpr int CH = kP16CH, QS = kP16QS, RS = kP16RS, QB = kQB, LAG = kP16Lag;
+    static_assert(QS >= 2 * 64 + 2 * CH && RS >= 2 * CH + 2 * kP16Pos, "ring too small");
     static_assert(QB >= W * (kP16Pos + CH) + kP16Pos + 2 + 128, "the last warp's offsets must not be overwritten");
     constexpr int UNR = kP16Unroll;
     static_assert(CH % UNR == 0 && UNR % 4 == 0, "chunks are whole unrolled groups of four steps");
@@ -558,8 +567,8 @@ wavefront16_kernel(const FillLaunch L)
     P16Shared<R, W> &S = *reinterpret_cast<P16Shared<R, W> *>(p16_smem);
     int8_t *const prof = p16_smem + p16_shared_bytes<R, W>();
     int2 *const ring0 = S.ring0;
-    uint2 (*const ring)[kP16QS] = S.ring;
-    int (*const s_base)[kP16QS / kP16CH] = S.base;
+    uint2 (*const ring)[kP16RS] = S.ring;
+    int (*const s_base)[kP16RS / kP16CH] = S.base;
     int *const s_poff = S.poff, *const prod = S.prod, *const cons = S.cons;
     P16Snap<R> (*const s_snap)[3] = S.snap;
     int4 *const s_cand = S.cand;
@@ -591,25 +600,28 @@ wavefront16_kernel(const FillLaunch L)
         const int n_ext = (n + LAG + CH - 1) / CH * CH + 2;
 
         const int pstride = PK == kP16Pair ? H * NL * 4 : 2 * HC;   // bytes per profile entry
+        // query profile of the strip's rows, S(a_r, c) + open, padding rows and columns at kPadScore: a thread takes a
+        // row (pair profile: the packed row of a lane) and runs over the residues, so that a row's residue is read
+        // once and no index is divided (464 x 503 protein: the fill 69 -> 55 us)
         if constexpr (PK == kP16Pair) {
-            const int ncc = (K + 1) * (K + 1);
             uint32_t *pw32 = reinterpret_cast<uint32_t *>(prof);
-            for (int idx = threadIdx.x; idx < ncc * NL * H; idx += blockDim.x) {
-                const int k = idx % H, g = (idx / H) % NL, cc = idx / (H * NL);
-                const int ct = cc / (K + 1), cb = cc % (K + 1);
-                const int rt = g * R + k, rb = g * R + H + k;
-                const bool okt = rt < SH && rbase + rt < T.rows && ct < K;
-                const bool okb = rb < SH && rbase + rb < T.rows && cb < K;
-                const int vt = okt ? SC.mat[min((int)T.a[rbase + rt], K - 1) * K + ct] + go : kPadScore;
-                const int vb = okb ? SC.mat[min((int)T.a[rbase + rb], K - 1) * K + cb] + go : kPadScore;
-                pw32[cc * NL * H + p16_pair_word<H>(k, g, NL)] = p16_pack(vt, vb);
+            for (int idx = threadIdx.x; idx < SW * 32 * H; idx += blockDim.x) {
+                const int k = idx % H, pg = idx / H;
+                const int rt = rbase + pg * R + k, rb = rt + H;
+                const int8_t *mt = rt < T.rows ? SC.mat + min((int)T.a[rt], K - 1) * K : nullptr;
+                const int8_t *mb = rb < T.rows ? SC.mat + min((int)T.a[rb], K - 1) * K : nullptr;
+                uint32_t *dst = pw32 + p16_pair_word<H>(k, pg, NL);
+                for (int ct = 0; ct <= K; ++ct) {
+                    const int vt = mt && ct < K ? mt[ct] + go : kPadScore;
+                    for (int cb = 0; cb <= K; ++cb)
+                        dst[(ct * (K + 1) + cb) * (NL * H)] = p16_pack(vt, mb && cb < K ? mb[cb] + go : kPadScore);
+                }
             }
         } else {
             int16_t *p16 = reinterpret_cast<int16_t *>(prof);
-            for (int idx = threadIdx.x; idx < (K + 1) * HC; idx += blockDim.x) {
-                const int lr = idx % HC, c = idx / HC;
-                const bool ok = lr < SH && rbase + lr < T.rows && c < K;
-                p16[idx] = (int16_t)(ok ? SC.mat[min((int)T.a[rbase + lr], K - 1) * K + c] + go : kPadScore);
+            for (int lr = threadIdx.x; lr < SH; lr += blockDim.x) {
+                const int8_t *m = rbase + lr < T.rows ? SC.mat + min((int)T.a[rbase + lr], K - 1) * K : nullptr;
+                for (int c = 0; c <= K; ++c) p16[c * HC + lr] = (int16_t)(m && c < K ? m[c] + go : kPadScore);
             }
         }
         // the offset ring starts as padding (the warm-up chunk below reads columns down to -96); its last kP16Pos
@@ -633,7 +645,7 @@ wavefront16_kernel(const FillLaunch L)
             p16_input_warp<QS, QB, PK>(T, L, strip, slot, n, n_ext, go, K, Wa, ring0, s_poff, pstride, prod, &S.res, cons,
                                             s_abort, lane);
         } else if (warp == W + 1) {
-            p16_output_warp<QS>(T, L, strip, slot, n, go, SH, Wa, ring[Wa - 1], s_base[Wa - 1], prod, cons, s_abort,
+            p16_output_warp(T, L, strip, slot, n, go, SH, Wa, ring[Wa - 1], s_base[Wa - 1], prod, cons, s_abort,
                                 lane);
         } else if (warp >= Wa) {
             if (lane == 0) s_cand[warp] = make_int4(0, 0x7fffffff, 0x7fffffff, 0);
@@ -678,7 +690,7 @@ wavefront16_kernel(const FillLaunch L)
             for (int s0 = sbeg; s0 < n + LAG; s0 += CH) {
                 // the chunk's rows above, the profile offsets one step ahead, and room in the ring below
                 const int ring_hi = s0 + CH - LAG, out_hi = min(n, ring_hi);
-                if (!p16_wait3(&prod[warp], min(n, s0 + CH), &S.res, s0 + CH + 2, &cons[warp + 1], ring_hi - QS, s_abort,
+                if (!p16_wait3(&prod[warp], min(n, s0 + CH), &S.res, s0 + CH + 2, &cons[warp + 1], ring_hi - RS, s_abort,
                                spin_limit, err)) {
                     *s_abort = 1;
                     ok = false;
@@ -703,8 +715,8 @@ wavefront16_kernel(const FillLaunch L)
                     if (warp == 0) {
                         tv = ring0[tcol & (QS - 1)];
                     } else {
-                        tv.x = (int)ring[warp - 1][(tcol + LAG) & (QS - 1)].x;
-                        tB = s_base[warp - 1][((tcol + LAG) / CH) & (QS / CH - 1)];
+                        tv.x = (int)ring[warp - 1][(tcol + LAG) & (RS - 1)].x;
+                        tB = s_base[warp - 1][((tcol + LAG) / CH) & (RS / CH - 1)];
                     }
                 }
                 {   // the warp's base follows lane 0's first row
@@ -736,7 +748,7 @@ wavefront16_kernel(const FillLaunch L)
                     for (int k = 0; k < p16_snap_words(R) / 4; ++k)
                         snap.st[k][lane] = make_uint4(q[4 * k], q[4 * k + 1], q[4 * k + 2], q[4 * k + 3]);
                     if (lane0) {
-                        s_base[warp][(s0 / CH) & (QS / CH - 1)] = B;
+                        s_base[warp][(s0 / CH) & (RS / CH - 1)] = B;
                         snap.s0 = s0; snap.B = B;
                     }
                     unsigned t = tcol < 0 ? cst.ngo2 : cst.neg2;
@@ -748,7 +760,7 @@ wavefront16_kernel(const FillLaunch L)
                     __syncwarp();
                 }
                 st.cmx = 0x80008000u;
-                uint2 *rc = rout + (s0 & (QS - 1));
+                uint2 *rc = rout + (s0 & (RS - 1));
 #pragma unroll 1
                 for (int gs = 0; gs < CH; gs += UNR) {                 // (a lane past the task's columns steps over padding)
 #pragma unroll

@@ -453,21 +453,35 @@ def test_bounded_wait_timeout(oracle_mod, monkeypatch):
         c2.close()
 
 
-@pytest.fixture(scope="module", params=[8, 12, 16])
+@pytest.fixture(scope="module", params=[8, 10, 12, 14, 16, 20, 26])
 def packed_ctx(request):
-    """A context on the packed fill with a fixed number of rows a lane."""
+    """A context on the packed fill with a fixed number of rows a lane (shapes above 8 other
+    than 12 and 16 serve small alphabets only; larger ones take the int32 fill there)."""
     from paper_2211_10769_gb300 import binding
-    old = os.environ.get("SWGB_FWD")
-    os.environ["SWGB_FWD"] = "%d,4,0,2,1" % request.param
+    env = {"SWGB_FWD": "%d,4,0,2,1" % request.param, "SWGB_ONE_ROUND": "0"}
+    old = {k: os.environ.get(k) for k in env}
+    os.environ.update(env)
     try:
         c = binding.Context(0)
     finally:
-        if old is None:
-            del os.environ["SWGB_FWD"]
-        else:
-            os.environ["SWGB_FWD"] = old
+        for k, v in old.items():
+            if v is None:
+                del os.environ[k]
+            else:
+                os.environ[k] = v
     yield c
     c.close()
+
+
+@pytest.mark.parametrize("m,n", [(7000, 6543), (3330, 9001), (26 * 128, 26 * 128 + 1)])
+def test_packed_align_shapes(packed_ctx, oracle_mod, m, n):
+    """Paths over tiles whose left columns the packed fill wrote at another number of rows a lane
+    than the traceback fill's: straightened columns, tiles of partial strips, the matrix's edges."""
+    sc = W.dna_scoring()
+    a = W.uniform_dna(m, W.BASE_SEED + 8700 + m)
+    core = W.mutate(a[m // 9:], 4, W.BASE_SEED + 8701 + n)[:n - 50]
+    b = np.concatenate([core, W.uniform_dna(n - len(core), W.BASE_SEED + 8702)])
+    _align_case(packed_ctx, oracle_mod, a, b, sc.matrix, sc.gap_open, sc.gap_extend)
 
 
 def test_packed_end_cell_among_ties(packed_ctx, oracle_mod):
