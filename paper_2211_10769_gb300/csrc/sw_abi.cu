@@ -269,6 +269,7 @@ FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t col
     if (!c->fwd_auto) {
         FillConfig f = c->fwd;
         f.P16 = f.P16 && p16_fits(s, f.R) && f.W == 4;
+        if (!f.P16 && f.R != 4 && f.R != 8 && f.R != 12 && f.R != 16) f.R = 8;   // a shape of the packed fill only
         return f;
     }
     if (c->p16 && rows + cols >= kPackedMinSum) {
