@@ -2,14 +2,12 @@
 // the test of whether a scoring scheme and tile shape keep it exact.
 #include "sw.h"
 #include "sw_ctx.h"
-#include "straighten.cuh"
-#include "wavefront16.cuh"
+#include "fill16_launch.cuh"
 
 #include <algorithm>
 
 using namespace swgb;
 
-#define CU(x) do { if ((x) != cudaSuccess) { cudaGetLastError(); return SW_ECUDA; } } while (0)
 
 namespace {
 
@@ -17,73 +15,15 @@ namespace {
 constexpr double kP16ChainSteps = 105;
 constexpr double p16_step_clocks(int R) { return R <= 8 ? 70 + 3.3 * R : (R <= 16 ? 53 + 5.4 * R : 46 + 6.1 * R); }
 
-// largest pair profile (small alphabets); larger alphabets take the int16 profile
-constexpr size_t kPairProfileMax = 170 * 1024;
-constexpr size_t kSharedMax = 227 * 1024;          // shared memory a block can have
-
-template <int R, int W, int MODE, int PK, bool LEFT>
-int launch16(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int max_blocks) {
-    auto kern = wavefront16_kernel<R, W, MODE, PK, LEFT>;
-    const size_t smem = p16_shared_bytes<R, W>() + p16_profile_bytes(R, W, K, PK);
-    static int attr_set[64] = {0};
-    if (c->device >= 64 || !attr_set[c->device]) {
-        const size_t cap = p16_shared_bytes<R, W>() + (PK == kP16Pair ? kPairProfileMax : p16_profile_bytes(R, W, kMaxAlphabet, PK));
-        CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(cap, kSharedMax)));
-        if (c->device < 64) attr_set[c->device] = 1;
-    }
-    int occ = 0;
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, (W + 2) * 32, smem));
-    if (occ < 1) return SW_ECUDA;
-    if (max_blocks > 0) occ = std::min(occ, max_blocks);
-    const long long grid = std::min<long long>(tickets, (long long)occ * c->nsm);
-    const int kp = kt_begin(c, SW_KT_FILL);
-    kern<<<(unsigned)grid, (W + 2) * 32, smem, c->stream>>>(L);
-    kt_end(c, kp);
-    CU(cudaGetLastError());
-    ++c->launches;
-    return SW_OK;
-}
-
-// Whether a block of W compute warps at R rows a lane takes the pair profile for K residue codes (it has to fit).
-template <int R, int W>
-bool pair_profile_fits(int K) {
-    const size_t p = p16_profile_bytes(R, W, K, kP16Pair);
-    return p <= kPairProfileMax && p16_shared_bytes<R, W>() + p <= kSharedMax;
-}
-
-template <int R, int MODE, bool LEFT = false, int W = 4>
-int launch16_pk(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int B) {
-    if (pair_profile_fits<R, W>(K)) return launch16<R, W, MODE, kP16Pair, LEFT>(c, L, K, tickets, B);
-    if constexpr (R == 8 || R == 12 || R == 16) return launch16<R, W, MODE, kP16Int16, LEFT>(c, L, K, tickets, B);
-    else return SW_EINVAL;                          // (p16_fits keeps other shapes to small alphabets)
-}
-
-// left: the coarse-tile refills (checkpoint mode only), whose tasks enter the
-// fill at a checkpoint column.  W = 2 (score mode only): blocks of two compute
-// warps for batches, whose pairs' last strips are partly empty (a strip of
-// four warps runs its pair's width with one to four of them busy).
+// W = 2 (score mode only): blocks of two compute warps for batches, whose
+// pairs' last strips are partly empty (a strip of four warps runs its pair's
+// width with one to four of them busy).
 template <int R>
 int launch16_mode(sw_ctx *c, int mode, bool left, int W, const FillLaunch &L, int K, long long tickets, int B) {
     if constexpr (R == 8 || R == 12 || R == 16)
         if (W == 2) return mode == kModeScore && !left ? launch16_pk<R, kModeScore, false, 2>(c, L, K, tickets, B) : SW_EINVAL;
     if (W != 4) return SW_EINVAL;
-    if (left) return mode == kModeScoreCk ? launch16_pk<R, kModeScoreCk, true>(c, L, K, tickets, B) : SW_EINVAL;
-    switch (mode) {
-        case kModeScore: return launch16_pk<R, kModeScore>(c, L, K, tickets, B);
-        case kModeScoreCk: return launch16_pk<R, kModeScoreCk>(c, L, K, tickets, B);
-        default: return SW_EINVAL;
-    }
-}
-
-template <int R>
-int launch_straighten_r(sw_ctx *c, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc) {
-    const int wpt = (max_rows + 32 * R - 1) / (32 * R);
-    const long long threads = 32LL * wpt * ntasks;
-    straighten_kernel<R><<<(unsigned)((threads + kStraightThreads - 1) / kStraightThreads), kStraightThreads, 0,
-                           c->stream>>>(tasks, ntasks, wpt, sc);
-    CU(cudaGetLastError());
-    ++c->launches;
-    return SW_OK;
+    return launch16_mode4<R, true>(c, mode, left, L, K, tickets, B);
 }
 
 // shapes with a pair profile only, for pairs of small alphabets
@@ -100,7 +40,7 @@ bool swgb::p16_fits(const DevScoring &s, int R) {
 #undef SWGB_P16_CASE
         default: return false;
     }
-    if (s.alg != kAlgLocal) return false;            // the packed fill keeps the zero floor
+    if (s.alg != kAlgLocal && R != 8 && R != 12 && R != 16) return false;   // the shapes of fill16_variants.cu
     int lo = 127, hi = -128;
     for (int k = 0; k < s.K * s.K; ++k) { lo = std::min(lo, (int)s.mat[k]); hi = std::max(hi, (int)s.mat[k]); }
     return p16_spread(R, s.go, s.ge, hi, lo) <= kP16Span;
@@ -109,6 +49,7 @@ bool swgb::p16_fits(const DevScoring &s, int R) {
 int swgb::launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K,
                         long long tickets) {
     if (tickets <= 0) return SW_OK;
+    if (cfg.alg != kAlgLocal) return launch_fill16_variant(c, cfg, mode, L, K, tickets);
     switch (cfg.R) {
 #define SWGB_P16_CASE(R) case R: return launch16_mode<R>(c, mode, cfg.left != 0, cfg.W, L, K, tickets, cfg.B);
         SWGB_P16_SHAPES(SWGB_P16_CASE)
@@ -117,10 +58,12 @@ int swgb::launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, const FillLa
     }
 }
 
-int swgb::launch_straighten(sw_ctx *c, int R, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc) {
+int swgb::launch_straighten(sw_ctx *c, int R, bool local, const FillTask *tasks, int ntasks, int max_rows,
+                            const DevScoring *sc) {
     if (ntasks <= 0) return SW_OK;
+    if (!local) return launch_straighten_variant(c, R, tasks, ntasks, max_rows, sc);
     switch (R) {
-#define SWGB_P16_CASE(R) case R: return launch_straighten_r<R>(c, tasks, ntasks, max_rows, sc);
+#define SWGB_P16_CASE(R) case R: return launch_straighten_r<R, true>(c, tasks, ntasks, max_rows, sc);
         SWGB_P16_SHAPES(SWGB_P16_CASE)
 #undef SWGB_P16_CASE
         default: return SW_EINVAL;

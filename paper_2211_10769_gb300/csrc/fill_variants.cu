@@ -81,6 +81,8 @@ int swgb::launch_fill_variant(sw_ctx *c, const FillConfig &cfg, int mode, bool f
     if (tickets <= 0) return SW_OK;
     if (cfg.W != 4) return SW_EINVAL;
     switch (cfg.R) {
+        // traceback tiles of 256 rows (two warps) after a small pair's packed fill
+        case 4: return mode == kModeTb ? launch_v_pk<4, kModeTb>(c, fold, L, K, tickets, cfg.B) : SW_EINVAL;
         case 8: return launch_v_mode<8>(c, mode, fold, L, K, tickets, cfg.B);
         case 12: return launch_v_mode<12>(c, mode, fold, L, K, tickets, cfg.B);
         case 16: return launch_v_mode<16>(c, mode, fold, L, K, tickets, cfg.B);

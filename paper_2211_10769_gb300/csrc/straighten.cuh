@@ -21,7 +21,7 @@ namespace swgb {
 constexpr int kStraightThreads = 128;
 
 // One warp per R * 32 rows of every task with left_split == R; tasks [0, ntasks), wpt warps each (the most any needs).
-template <int R>
+template <int R, bool LOCAL>
 __global__ void __launch_bounds__(kStraightThreads)
 straighten_kernel(const FillTask *tasks, int ntasks, int wpt, const DevScoring *scorings)
 {
@@ -80,8 +80,8 @@ straighten_kernel(const FillTask *tasks, int ntasks, int wpt, const DevScoring *
             for (int x = 0; x < H; ++x) {
                 const int ut = U[x], ub = U[H + x];
                 const int et = __viaddmax_s32(E[x], -ge, ut), eb = __viaddmax_s32(E[H + x], -ge, ub);
-                const int xt = __viaddmax_s32_relu(dt, mt[code[x]] + go, et) - go;
-                const int xb = __viaddmax_s32_relu(db, mb[code[H + x]] + go, eb) - go;
+                const int xt = (LOCAL ? __viaddmax_s32_relu(dt, mt[code[x]] + go, et) : __viaddmax_s32(dt, mt[code[x]] + go, et)) - go;
+                const int xb = (LOCAL ? __viaddmax_s32_relu(db, mb[code[H + x]] + go, eb) : __viaddmax_s32(db, mb[code[H + x]] + go, eb)) - go;
                 if (top) { U[x] = __viaddmax_s32(f, -go, xt); E[x] = et; }
                 U[H + x] = __viaddmax_s32(g, -go, xb);
                 E[H + x] = eb;

@@ -253,6 +253,7 @@ FillConfig swgb::pair_fill_config(const sw_ctx *c, int64_t rows) {
 }
 
 constexpr int64_t kPackedMinSum = 2048;
+constexpr int64_t kPackedMinSumVariant = 1024;
 
 // Tile shape of a single-pair fill with scoring s: the packed 16-bit fill
 // (two cells per lane operation) where it is exact, with the rows a lane that
@@ -263,6 +264,14 @@ constexpr int64_t kPackedMinSum = 2048;
 FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s) {
     if (s.alg != kAlgLocal) {
         FillConfig f = variant_fill_config(c, rows);
+        // (the int32 variants run at 8 rows a lane at least: the packed fill from smaller pairs on)
+        const int R = !c->fwd_auto ? (c->fwd.P16 && p16_fits(s, c->fwd.R) ? c->fwd.R : 0)
+                                   : (c->p16 && rows + cols >= kPackedMinSumVariant ? p16_rows_per_lane(c, rows, cols, s) : 0);
+        if (R > 0) {
+            f = FillConfig{R, 4, 0, 2, 1};
+            f.alg = 1;
+            return f;
+        }
         if (!c->fwd_auto && (c->fwd.R == 8 || c->fwd.R == 12 || c->fwd.R == 16)) f.R = c->fwd.R;   // SWGB_FWD
         return f;
     }
@@ -345,7 +354,7 @@ int swgb::run_fill_with(sw_ctx *c, const FillBufs &b, cudaStream_t st, const Fil
     if (straight_R > 0) {
         int max_rows = 0;
         for (const FillTask &t : tasks) max_rows = std::max(max_rows, t.straight ? t.rows : 0);
-        if (max_rows > 0) rc = launch_straighten(c, straight_R, L.tasks, (int)tasks.size(), max_rows, L.scorings);
+        if (max_rows > 0) rc = launch_straighten(c, straight_R, cfg.alg == kAlgLocal, L.tasks, (int)tasks.size(), max_rows, L.scorings);
     }
     if (!rc) rc = launch_fill(c, cfg, mode, fold, L, K, tickets);
     c->stream = home;

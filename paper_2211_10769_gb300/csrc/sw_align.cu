@@ -220,7 +220,7 @@ constexpr int64_t kOneRoundPackedSide = 4096;
 // straightened, the context's shape (8 rows a lane); after an int32 fill the
 // tiles continue its staircase columns lane by lane, so they take its rows a lane.
 FillConfig traceback_config(const sw_ctx *c, const FillConfig &fwd) {
-    FillConfig t = (fwd.alg == kAlgLocal && (fwd.P16 || c->tbc.R == fwd.R)) ? c->tbc : FillConfig{fwd.R, 4};
+    FillConfig t = (fwd.alg == kAlgLocal && (fwd.P16 || c->tbc.R == fwd.R)) ? c->tbc : FillConfig{fwd.P16 ? 8 : fwd.R, 4};
     t.P16 = 0;
     t.alg = fwd.alg;
     return t;
@@ -236,8 +236,10 @@ long long small_pair_tile(const sw_ctx *c, int64_t m, int64_t n, const DevScorin
     // straightened columns (a launch and 63 dependent steps): 1,000 0.237 against 0.253 ms, 2,800 0.436 against
     // 0.442, 8,000 1.185 against 1.134
     FillConfig fwd = pair_fill_config_for(c, m, n, ds);
-    if (c->fwd_auto && fwd.P16)
-        fwd = std::max(m, n) > kOneRoundPackedSide && p16_fits(ds, 8) ? FillConfig{8, 4, 0, 2, 1} : pair_fill_config(c, m);
+    if (c->fwd_auto && fwd.P16) {
+        if (fwd.alg != kAlgLocal) fwd = p16_fits(ds, 8) ? FillConfig{8, 4, 0, 2, 1, 1} : fwd;
+        else fwd = std::max(m, n) > kOneRoundPackedSide && p16_fits(ds, 8) ? FillConfig{8, 4, 0, 2, 1} : pair_fill_config(c, m);
+    }
     // strips of 256 rows where the fill allows it (one compute warp of the packed fill at 8 rows a lane, two of
     // the int32 fill at 4): a small pair's forward chain has as many warps either way, and a 256-row tile
     // recomputes in about half the steps of a 512-row one
@@ -386,7 +388,7 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
     Lt.total = tickets;
     Lt.ntasks = ntiles;
     if (fwd.P16 && nJ > 1)
-        RC(launch_straighten(c, fwd.R, dtasks + 1, ntiles, (int)std::min<int64_t>(BT, m), L.scorings));
+        RC(launch_straighten(c, fwd.R, ds.alg == kAlgLocal, dtasks + 1, ntiles, (int)std::min<int64_t>(BT, m), L.scorings));
     RC(launch_fill(c, tbc, kModeTb, fold, Lt, ds.K, tickets));
     walk_start_kernel<<<1, 32, 0, c->stream>>>(static_cast<const int4 *>(c->result.p), ds.alg == kAlgLocal ? 1 : 0,
                                                static_cast<WalkState *>(c->walk.p));

@@ -45,7 +45,7 @@ struct FillConfig {
     int S = 0;
     int B = 0;
     int P16 = 0;   // packed 16-bit fill (wavefront16.cuh) instead of the int32 one
-    int alg = 0;   // not kAlgLocal: the int32 fill without the zero floor (fill_variants.cu)
+    int alg = 0;   // not kAlgLocal: the fills without the zero floor (fill_variants.cu, fill16_variants.cu)
     int left = 0;  // packed fill whose tasks may start right of its own checkpoint column
 };
 
@@ -111,7 +111,9 @@ FillConfig pair_fill_config(const sw_ctx *c, int64_t rows);
 FillConfig pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s);   // picks P16 where exact
 int p16_rows_per_lane(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &s);
 // the packed checkpoint columns of tasks with FillTask::straight brought to one column (R: the writer's rows a lane)
-int launch_straighten(sw_ctx *c, int R, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc);
+int launch_straighten(sw_ctx *c, int R, bool local, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc);
+int launch_straighten_variant(sw_ctx *c, int R, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc);
+int launch_fill16_variant(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K, long long tickets);
 bool p16_fits(const DevScoring &s, int R);
 int launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K, long long tickets);
 // the global, semi-global and overlap algorithms: 8 or 16 rows a lane, four compute warps

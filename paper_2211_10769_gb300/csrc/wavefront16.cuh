@@ -225,11 +225,14 @@ struct P16Consts { unsigned nge2, ngo2, neg2; };
 
 // One step of one lane: column s - 2 lane (top half) and the one before (bottom half); top = lane 0's row
 // above for this step, (H - open, F of the first row).
-template <int R, int PK>
+// LOCAL = false: no zero floor, and cmx is kept by the caller (the largest U only matters in the last row).
+// EDGE: a half whose bits are set in hold keeps its state (its column lies outside the task).
+template <int R, int PK, bool LOCAL = true, bool EDGE = false>
 __device__ __forceinline__ void p16_step(P16Lane<R> &st, const uint32_t (&pw)[R / 2], const uint32_t (&pwp)[R / 2],
-                                         unsigned top, bool lane0, const P16Consts &c)
+                                         unsigned top, bool lane0, const P16Consts &c, unsigned hold = 0)
 {
     constexpr int H = R / 2;
+    [[maybe_unused]] auto held = [&](unsigned now, unsigned before) { return EDGE ? (now & ~hold) | (before & hold) : now; };
     unsigned r = __shfl_up_sync(kFull, st.w, 1);
     r = lane0 ? top : r;
     // low half: the row above the top half (lane t-1's bottom half one step earlier); high half: this
@@ -237,26 +240,34 @@ __device__ __forceinline__ void p16_step(P16Lane<R> &st, const uint32_t (&pw)[R 
     const unsigned uup = prmt_c<0x5410>(r, st.U[H - 1]);
     unsigned f = prmt_c<0x5432>(r, st.fb);
     unsigned udiag = st.udiag0;
-    st.udiag0 = uup;
+    st.udiag0 = held(uup, udiag);
 #pragma unroll
     for (int k = 0; k < H; ++k) {
         const unsigned sp = p16_score<R, PK>(pw, pwp, k);
         const unsigned uold = st.U[k];
         const unsigned e = __viaddmax_s16x2(st.E[k], c.nge2, uold);
-        const unsigned x = __viaddmax_s16x2_relu(udiag, sp, e);    // max(H(i-1,j-1) + S, E, 0)
+        const unsigned x = LOCAL ? __viaddmax_s16x2_relu(udiag, sp, e)   // max(H(i-1,j-1) + S, E, 0)
+                                 : __viaddmax_s16x2(udiag, sp, e);
         const unsigned xgo = __viaddmax_s16x2(x, c.ngo2, c.neg2);  // x - open
         const unsigned u = __viaddmax_s16x2(f, c.ngo2, xgo);       // H - open
-        st.E[k] = e;
+        st.E[k] = held(e, st.E[k]);
         udiag = uold;
-        st.U[k] = u;
+        st.U[k] = held(u, uold);
         if (k + 1 < H) f = __viaddmax_s16x2(f, c.nge2, xgo);       // F of the next row
-        else st.fb = __viaddmax_s16x2(f, c.nge2, xgo);             // F of the row below the half
+        else st.fb = held(__viaddmax_s16x2(f, c.nge2, xgo), st.fb);   // F of the row below the half
     }
-    st.flast = f;
+    st.flast = held(f, st.flast);
     st.w = prmt_c<0x7632>(st.U[H - 1], st.fb);
+    if constexpr (LOCAL) {
 #pragma unroll
-    for (int k = 0; k + 1 < H; k += 2) st.cmx = __vimax3_s16x2(st.cmx, st.U[k], st.U[k + 1]);
-    if constexpr (H % 2 == 1) st.cmx = __vmaxs2(st.cmx, st.U[H - 1]);
+        for (int k = 0; k + 1 < H; k += 2) st.cmx = __vimax3_s16x2(st.cmx, st.U[k], st.U[k + 1]);
+        if constexpr (H % 2 == 1) st.cmx = __vmaxs2(st.cmx, st.U[H - 1]);
+    }
+}
+
+// The halves of a lane whose columns j (top) and j - 1 (bottom) lie outside [lo, n).
+__device__ __forceinline__ unsigned p16_hold(int j, int lo, int n) {
+    return ((j >= lo && j < n) ? 0u : 0xffffu) | ((j - 1 >= lo && j - 1 < n) ? 0u : 0xffff0000u);
 }
 
 __device__ __forceinline__ int ld_relaxed(const int *p) {
@@ -268,11 +279,11 @@ __device__ __forceinline__ int ld_relaxed(const int *p) {
 // Input warp of a packed fill block, ahead of the first compute warp: every column's profile offset into the
 // offset ring (published in *res; it goes on past the last column with the padding residue) and the strip's top
 // boundary row (H - open, F; absolute) into channel 0 (published in prod[0]).
-template <int QS, int QB, int PK>
+template <int QS, int QB, int PK, bool LOCAL>
 __device__ __forceinline__ void p16_input_warp(const FillTask &T, const FillLaunch &L, int strip, long long slot,
                                                int n, int n_ext, int go, int K, int Wa, int2 *ring0, int *poff,
                                                int pstride, int *prod, int *res, const int *cons, volatile int *s_abort,
-                                               int lane)
+                                               int lane, int alg, int ge)
 {
     constexpr int kBatch = 64;                 // columns of either stream per turn
     const uint8_t *const b = T.b;
@@ -280,6 +291,7 @@ __device__ __forceinline__ void p16_input_warp(const FillTask &T, const FillLaun
     const int2 *const src = strip == 0 ? T.top : T.bnd + (size_t)((strip - 1) % T.nslot) * n;
     const int *const pprev = L.prog + (slot - 1);
     const long long spin_limit = L.spin_limit;
+    const int col0 = T.col0;
     int next = 0, rnext = 0, avail = strip == 0 ? n : 0;
     long long idle = 0;
     bool warm = true;                          // the first turn runs the boundary code with nothing to move (instruction cache)
@@ -301,7 +313,9 @@ __device__ __forceinline__ void p16_input_warp(const FillTask &T, const FillLaun
             target = max(target, next);
             if (target > next || warm) {
                 const int c0 = next + lane, c1 = c0 + 32;
-                int2 v0 = make_int2(0, kNeg), v1 = v0;
+                // the matrix's top border: H(0, j) of the algorithm, F = -infinity
+                int2 v0 = make_int2(LOCAL ? 0 : (int)top_border_h(alg, (long long)col0 + c0 + 1, go, ge), kNeg);
+                int2 v1 = make_int2(LOCAL ? 0 : (int)top_border_h(alg, (long long)col0 + c1 + 1, go, ge), kNeg);
                 if (src && c0 < target) v0 = __ldcg(src + c0);
                 if (src && c1 < target) v1 = __ldcg(src + c1);
                 if (c0 < target) ring0[c0 & (QS - 1)] = make_int2(v0.x - go, v0.y);
@@ -428,10 +442,10 @@ struct P16Snap {
 };
 
 // The first cell in row-major order, among the valid cells of half-lane pos of the chunk in snapshot S,
-// whose H - open equals u: (row of the half, column), or (R, 0).
-template <int R, int PK, int NL>
+// whose H - open equals u: (row of the half, column), or (R, 0).  Valid: rows [row_lo, row_hi) of the half, real columns.
+template <int R, int PK, int NL, bool LOCAL>
 __device__ __noinline__ int2 p16_locate(const P16Snap<R> &S, const int8_t *prof, int g, int pstride, const FillTask &T,
-                                        int n, int K, int go, int ge, int pos, int u, int nrows)
+                                        int n, int K, int go, int ge, int pos, int u, int row_lo, int row_hi)
 {
     constexpr int H = R / 2;
     const int lane = threadIdx.x & 31;
@@ -473,12 +487,12 @@ __device__ __noinline__ int2 p16_locate(const P16Snap<R> &S, const int8_t *prof,
                 p16_load<R, PK, NL>(prof, g, cc[x + 1] * pstride, pw);
                 p16_load<R, PK, NL>(prof, g, cc[x] * pstride, pwp);
             }
-            p16_step<R, PK>(st, pw, pwp, S.top[k0 + x], lane == 0, c);
+            p16_step<R, PK, LOCAL, !LOCAL>(st, pw, pwp, S.top[k0 + x], lane == 0, c, LOCAL ? 0u : p16_hold(j, first, n));
             const int jj = j - h;
             if (mine && jj >= 0 && jj < n) {
 #pragma unroll
                 for (int y = H - 1; y >= 0; --y)
-                    if (y < row && y < nrows && (h ? p16_hi(st.U[y]) : p16_lo(st.U[y])) == want) { row = y; col = jj; }
+                    if (y < row && y >= row_lo && y < row_hi && (h ? p16_hi(st.U[y]) : p16_lo(st.U[y])) == want) { row = y; col = jj; }
             }
         }
     }
@@ -494,7 +508,7 @@ __device__ __noinline__ int2 p16_locate(const P16Snap<R> &S, const int8_t *prof,
 // -1.  The lane takes that state (relative to a base taken from lane 0) and the
 // sweep goes on from step 0; its first steps recompute real columns left of
 // the task from real residues (the offset ring's slots left of column 0).
-template <int R>
+template <int R, bool LOCAL>
 __device__ __forceinline__ void p16_enter_staircase(const FillTask &T, P16Lane<R> &st, int &B, int grow, int lane, int go,
                                                     int ge) {
     constexpr int H = R / 2;
@@ -509,7 +523,8 @@ __device__ __forceinline__ void p16_enter_staircase(const FillTask &T, P16Lane<R
     const bool in = grow < T.rows;
     const int2 at = in ? __ldcg(T.left_aux + grow / H) : make_int2(-go, kNeg);       // top half
     const int2 ab = in ? __ldcg(T.left_aux + grow / H + 1) : make_int2(-go, kNeg);   // bottom half
-    B = max(0, __shfl_sync(kFull, vU[0], 0) - kP16Center);
+    B = __shfl_sync(kFull, vU[0], 0) - kP16Center;
+    if (LOCAL) B = max(B, 0);
     auto rel = [&](int v) { return max(min(v - B, 32767), kNeg16p); };
 #pragma unroll
     for (int k = 0; k < H; ++k) {
@@ -522,6 +537,9 @@ __device__ __forceinline__ void p16_enter_staircase(const FillTask &T, P16Lane<R
     st.w = prmt_c<0x7632>(st.U[H - 1], st.fb);
 }
 
+
+// A compile-time integer as an argument.
+template <int V> struct P16Int { static constexpr int v = V; };
 
 // Shared memory of a block ahead of its query profile.
 template <int R, int W>
@@ -546,7 +564,8 @@ constexpr size_t p16_shared_bytes() { return (sizeof(P16Shared<R, W>) + 15) / 16
 // LEFT: the tasks may start right of a checkpoint column written by this fill
 // (p16_enter_staircase; the coarse-tile refills of a two-level reconstruction).
 // A separate instantiation, so that the others compile exactly without it.
-template <int R, int W, int MODE, int PK, bool LEFT = false>
+// LOCAL = false: the global, semi-global and overlap algorithms (DevScoring::alg).
+template <int R, int W, int MODE, int PK, bool LEFT = false, bool LOCAL = true>
 __global__ void __launch_bounds__((W + 2) * 32, 1)
 wavefront16_kernel(const FillLaunch L)
 {
@@ -642,13 +661,13 @@ wavefront16_kernel(const FillLaunch L)
         __syncthreads();
 
         if (warp == W) {
-            p16_input_warp<QS, QB, PK>(T, L, strip, slot, n, n_ext, go, K, Wa, ring0, s_poff, pstride, prod, &S.res, cons,
-                                            s_abort, lane);
+            p16_input_warp<QS, QB, PK, LOCAL>(T, L, strip, slot, n, n_ext, go, K, Wa, ring0, s_poff, pstride, prod, &S.res, cons,
+                                            s_abort, lane, SC.alg, ge);
         } else if (warp == W + 1) {
             p16_output_warp(T, L, strip, slot, n, go, SH, Wa, ring[Wa - 1], s_base[Wa - 1], prod, cons, s_abort,
                                 lane);
         } else if (warp >= Wa) {
-            if (lane == 0) s_cand[warp] = make_int4(0, 0x7fffffff, 0x7fffffff, 0);
+            if (lane == 0) s_cand[warp] = make_int4(LOCAL ? 0 : kNoScore, 0x7fffffff, 0x7fffffff, 0);
         } else {
             // ================= compute warp =================
             const int g = warp * 32 + lane;
@@ -661,9 +680,32 @@ wavefront16_kernel(const FillLaunch L)
             for (int k = 0; k < H; ++k) { st.U[k] = cst.ngo2; st.E[k] = cst.neg2; }
             st.fb = cst.ngo2; st.flast = cst.neg2; st.udiag0 = cst.ngo2; st.w = cst.ngo2;   // matrix border: H = 0
             if constexpr (LEFT)
-                if (T.left) p16_enter_staircase<R>(T, st, B, grow, lane, go, ge);
+                if (T.left) p16_enter_staircase<R, LOCAL>(T, st, B, grow, lane, go, ge);
+            // the other algorithms: the matrix's left border H(i, 0) as state, held until a half's column 0; the task's
+            // last row (where it is an end row at every column: semi-global, overlap) as a mask over the packed rows
+            [[maybe_unused]] unsigned tmask[LOCAL ? 1 : H];
+            [[maybe_unused]] int rlast = -1;               // the lane's row that is the task's last one
+            [[maybe_unused]] bool track = false;           // this warp holds the last row and it is an end row
+            if constexpr (!LOCAL) {
+                if (!(LEFT && T.left)) {
+                    auto border = [&](long long i) { return (int)left_border_h(SC.alg, i, go, ge) - go; };
+                    const long long i0 = (long long)T.row0 + grow;
+                    B = border((long long)T.row0 + rbase + warp * 32 * R + 1) - kP16Center;
+#pragma unroll
+                    for (int k = 0; k < H; ++k)
+                        st.U[k] = p16_pack(max(border(i0 + k + 1) - B, kNeg16p), max(border(i0 + H + k + 1) - B, kNeg16p));
+                    st.udiag0 = p16_pack(max(border(i0) - B, kNeg16p), max(border(i0 + H) - B, kNeg16p));
+                    st.fb = cst.neg2;
+                    st.w = prmt_c<0x7632>(st.U[H - 1], st.fb);
+                }
+                const int rl = T.rows - 1 - grow;
+                rlast = rl >= 0 && rl < R ? rl : -1;
+#pragma unroll
+                for (int k = 0; k < H; ++k) tmask[k] = rl == k ? 0xffffu : (rl == H + k ? 0xffff0000u : 0u);
+                track = (SC.alg == kAlgSemiGlobal || SC.alg == kAlgOverlap) && __any_sync(kFull, rlast >= 0);
+            }
             // the warp's best: H - open, half-lane (2 lane + half), and where: snapshot, or row and column once located
-            int bu = 1 - go, brow = R, bcol = 0, bcb = 0;
+            int bu = LOCAL ? 1 - go : -(1 << 30), brow = R, bcol = 0, bcb = 0;
             int pa = 0, pb = 0, npend = 0;      // snapshots that hold the best (the second: the same half-lane again)
 
             unsigned bcm = 0x80008000u;
@@ -675,7 +717,8 @@ wavefront16_kernel(const FillLaunch L)
             auto resolve = [&](int pos) {
                 const int nr = T.rows - (rbase + (warp * 32 + (pos >> 1)) * R + (pos & 1) * H);
                 for (int q = 0; q < npend; ++q) {
-                    const int2 c = p16_locate<R, PK, NL>(s_snap[warp][q ? pb : pa], prof, g, pstride, T, n, K, go, ge, pos, bu, nr);
+                    const int2 c = p16_locate<R, PK, NL, LOCAL>(s_snap[warp][q ? pb : pa], prof, g, pstride, T, n, K, go, ge, pos,
+                                                                bu, LOCAL ? 0 : nr - 1, nr);
                     if (c.x < brow) { brow = c.x; bcol = c.y; }
                 }
             };
@@ -721,8 +764,8 @@ wavefront16_kernel(const FillLaunch L)
                 }
                 {   // the warp's base follows lane 0's first row
                     const int ref = p16_lo(__shfl_sync(kFull, st.U[0], 0));
-                    if (ref > kP16Center + kP16Slack || (B > 0 && ref < kP16Center - kP16Slack)) {
-                        const int Bn = max(0, ref + B - kP16Center);
+                    if (ref > kP16Center + kP16Slack || ((!LOCAL || B > 0) && ref < kP16Center - kP16Slack)) {
+                        const int Bn = LOCAL ? max(0, ref + B - kP16Center) : ref + B - kP16Center;
                         const unsigned d2 = p16_pack(B - Bn, B - Bn);
 #pragma unroll
                         for (int k = 0; k < H; ++k) {
@@ -761,35 +804,57 @@ wavefront16_kernel(const FillLaunch L)
                 }
                 st.cmx = 0x80008000u;
                 uint2 *rc = rout + (s0 & (RS - 1));
-#pragma unroll 1
-                for (int gs = 0; gs < CH; gs += UNR) {                 // (a lane past the task's columns steps over padding)
+                // the chunk's steps; NS: steps an unrolled body, EDGE: halves outside the task hold (the other algorithms)
+                auto sweep = [&](auto ns, auto edge) {
+                    constexpr int NS = decltype(ns)::v;
+                    constexpr bool EDGE = decltype(edge)::v != 0;
+                    [[maybe_unused]] const int lo = LEFT && T.left ? -(1 << 30) : 0;
+                    auto step = [&](const uint32_t (&w)[H], const uint32_t (&wp)[H], unsigned top, int s) {
+                        p16_step<R, PK, LOCAL, EDGE>(st, w, wp, top, lane0, cst, EDGE ? p16_hold(s - 2 * lane, lo, n) : 0u);
+                        if (lane == 31) rc[s - s0] = make_uint2(st.w, st.flast);
+                        if constexpr (!LOCAL) {
+                            if (track) {                   // (one warp of the pair)
+                                unsigned v = 0;
 #pragma unroll
-                    for (int k4 = 0; k4 < UNR; k4 += 4) {
-                        const uint4 tops = *reinterpret_cast<const uint4 *>(&snap.top[gs + k4]);
-#pragma unroll
-                        for (int k2 = 0; k2 < 4; k2 += 2) {
-                            const int k = k4 + k2;
-                            // offsets of steps s + 2, s + 3 (slots an even distance apart from lane to lane)
-                            const int2 offn = *reinterpret_cast<const int2 *>(&s_poff[(s0 + gs + k + 2 - 2 * lane) & (QB - 1)]);
-                            uint32_t pwn[H];
-                            p16_load<R, PK, NL>(prof, g, off.y, pwn);
-                            p16_step<R, PK>(st, pw, pwp, k2 == 0 ? tops.x : tops.z, lane0, cst);
-                            if (lane == 31) rc[gs + k] = make_uint2(st.w, st.flast);
-                            p16_load<R, PK, NL>(prof, g, offn.x, PK == kP16Pair ? pw : pwp);
-                            if constexpr (PK == kP16Pair) {
-                                p16_step<R, PK>(st, pwn, pwp, k2 == 0 ? tops.y : tops.w, lane0, cst);
-                            } else {
-                                uint32_t t2[H];
-#pragma unroll
-                                for (int q = 0; q < H; ++q) t2[q] = pwp[q];      // words of step s + 2
-                                p16_step<R, PK>(st, pwn, pw, k2 == 0 ? tops.y : tops.w, lane0, cst);
-#pragma unroll
-                                for (int q = 0; q < H; ++q) { pwp[q] = pwn[q]; pw[q] = t2[q]; }
+                                for (int k = 0; k < H; ++k) v |= st.U[k] & tmask[k];
+                                st.cmx = __vmaxs2(st.cmx, v);
                             }
-                            if (lane == 31) rc[gs + k + 1] = make_uint2(st.w, st.flast);
-                            off = offn;
+                        }
+                    };
+#pragma unroll 1
+                    for (int gs = 0; gs < CH; gs += NS) {
+#pragma unroll
+                        for (int k4 = 0; k4 < NS; k4 += 4) {
+                            const uint4 tops = *reinterpret_cast<const uint4 *>(&snap.top[gs + k4]);
+#pragma unroll
+                            for (int k2 = 0; k2 < 4; k2 += 2) {
+                                const int s = s0 + gs + k4 + k2;
+                                // offsets of steps s + 2, s + 3 (slots an even distance apart from lane to lane)
+                                const int2 offn = *reinterpret_cast<const int2 *>(&s_poff[(s + 2 - 2 * lane) & (QB - 1)]);
+                                uint32_t pwn[H];
+                                p16_load<R, PK, NL>(prof, g, off.y, pwn);
+                                step(pw, pwp, k2 == 0 ? tops.x : tops.z, s);
+                                p16_load<R, PK, NL>(prof, g, offn.x, PK == kP16Pair ? pw : pwp);
+                                if constexpr (PK == kP16Pair) {
+                                    step(pwn, pwp, k2 == 0 ? tops.y : tops.w, s + 1);
+                                } else {
+                                    uint32_t t2[H];
+#pragma unroll
+                                    for (int q = 0; q < H; ++q) t2[q] = pwp[q];      // words of step s + 2
+                                    step(pwn, pw, k2 == 0 ? tops.y : tops.w, s + 1);
+#pragma unroll
+                                    for (int q = 0; q < H; ++q) { pwp[q] = pwn[q]; pw[q] = t2[q]; }
+                                }
+                                off = offn;
+                            }
                         }
                     }
+                };
+                if constexpr (LOCAL) {
+                    sweep(P16Int<UNR>{}, P16Int<0>{});     // (a lane past the task's columns steps over padding)
+                } else {
+                    if ((s0 >= kP16Pos || (LEFT && T.left)) && s0 + CH <= n) sweep(P16Int<UNR>{}, P16Int<0>{});
+                    else sweep(P16Int<4>{}, P16Int<1>{});
                 }
                 if constexpr (MODE == kModeScoreCk) {
                     if (s0 + CH - 1 == next_ck && next_ck < n) {   // the same for every lane
@@ -806,7 +871,17 @@ wavefront16_kernel(const FillLaunch L)
                         next_ck += T.colck_every;
                     }
                 }
-                {   // a best cell in this chunk?
+                if constexpr (!LOCAL) {
+                    if (track) {                           // the last row's best of the chunk; the first column that holds it wins
+                        const unsigned who = __ballot_sync(kFull, rlast >= 0);
+                        const int v = __shfl_sync(kFull, rlast >= H ? p16_hi(st.cmx) : p16_lo(st.cmx), __ffs(who) - 1) + B;
+                        if (v > bu) {
+                            bu = v; held = true; brow = R;
+                            pa = cur; npend = 1;
+                            cur = (cur + 1) % 3;
+                        }
+                    }
+                } else {   // a best cell in this chunk?
                     const int lo = p16_lo(st.cmx), hi = p16_hi(st.cmx);
                     const int thr = min(bu - B, 32767);
                     if (__any_sync(kFull, max(lo, hi) >= thr)) {
@@ -842,13 +917,38 @@ wavefront16_kernel(const FillLaunch L)
                     if (out_hi > 0) *(volatile int *)&prod[warp + 1] = out_hi;
                 }
             }
-            int cs = 0, cj = 0x7fffffff, ci = 0x7fffffff;
-            if (ok && held) {
-                const int bpos = p16_first_pos(bcm, bu - bcb);
-                resolve(bpos);
-                if (brow < H) {
-                    cs = bu + go; cj = bcol + 1;
-                    ci = T.row0 + rbase + (warp * 32 + (bpos >> 1)) * R + (bpos & 1) * H + brow + 1;
+            int cs = LOCAL ? 0 : kNoScore, cj = 0x7fffffff, ci = 0x7fffffff;
+            if constexpr (LOCAL) {
+                if (ok && held) {
+                    const int bpos = p16_first_pos(bcm, bu - bcb);
+                    resolve(bpos);
+                    if (brow < H) {
+                        cs = bu + go; cj = bcol + 1;
+                        ci = T.row0 + rbase + (warp * 32 + (bpos >> 1)) * R + (bpos & 1) * H + brow + 1;
+                    }
+                }
+            } else {
+                if (ok && held) {                          // the best of the last row (semi-global, overlap)
+                    const int l = __ffs(__ballot_sync(kFull, rlast >= 0)) - 1, r = __shfl_sync(kFull, rlast, l);
+                    resolve(2 * l + (r >= H ? 1 : 0));
+                    if (brow < H) { cs = bu + go; cj = bcol + 1; ci = T.row0 + T.rows; }
+                }
+                // the last column: every row for the overlap algorithm, the last row for the global one
+                if (ok && n > 0 && (SC.alg == kAlgOverlap || SC.alg == kAlgGlobal)) {
+#pragma unroll
+                    for (int k = 0; k < R; ++k) {
+                        const int sc = (k < H ? p16_lo(st.U[k % H]) : p16_hi(st.U[k % H])) + B + go;
+                        const int ii = T.row0 + grow + k + 1;
+                        const bool end = SC.alg == kAlgOverlap ? grow + k < T.rows : k == rlast;
+                        if (end && cand_better(sc, n, ii, cs, cj, ci)) { cs = sc; cj = n; ci = ii; }
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const int os = __shfl_xor_sync(kFull, cs, o);
+                    const int oj = __shfl_xor_sync(kFull, cj, o);
+                    const int oi = __shfl_xor_sync(kFull, ci, o);
+                    if (cand_better(os, oj, oi, cs, cj, ci)) { cs = os; cj = oj; ci = oi; }
                 }
             }
             if (lane == 0) s_cand[warp] = make_int4(cs, ci, cj, 0);
@@ -860,7 +960,7 @@ wavefront16_kernel(const FillLaunch L)
                 const int4 o = s_cand[w];
                 if (cand_better(o.x, o.z, o.y, b.x, b.z, b.y)) b = o;
             }
-            b.w = b.x > 0 ? 1 : 0;
+            b.w = LOCAL ? (b.x > 0 ? 1 : 0) : (b.x != kNoScore ? 1 : 0);
             L.cand[slot] = b;
         }
         __syncthreads();

@@ -236,3 +236,43 @@ def test_local_only_calls_reject_other_algorithms(ctx):
                       a.numel(), ctypes.byref(bad), ctypes.byref(hit))
     assert rc == binding.SW_EINVAL
     db.close()
+
+
+@pytest.mark.parametrize("R", [8, 12, 16])
+@pytest.mark.parametrize("alg", ALGS)
+def test_packed_variant_fill(oracle_mod, monkeypatch, alg, R):
+    """The packed fill without the zero floor, forced for every size: columns left and right of the
+    task held by lane halves, the last row in any half-lane, equal maxima in the last row and column,
+    bases far below zero, one and two checkpoint levels."""
+    from paper_2211_10769_gb300 import binding
+    monkeypatch.setenv("SWGB_FWD", "%d,4,0,2,1" % R)
+    monkeypatch.setenv("SWGB_ONE_ROUND", "0")
+    ctx = binding.Context(0)
+    monkeypatch.setenv("SWGB_TWO_LEVEL", "%d,%d" % (3 * 128 * R, 128 * R))
+    two = binding.Context(0)
+    try:
+        g = np.random.default_rng(W.BASE_SEED + 16100 + 10 * alg + R)
+        for t in range(40):
+            K = int(g.integers(1, 6)) if t % 4 else 20
+            m = int(g.choice([1, 3, R // 2, R, R + 1, 60, 32 * R, 32 * R + 1, 700, 128 * R + 5]))
+            n = int(g.choice([1, 2, 31, 32, 33, 63, 64, 65, 96, 97, 500, 1300]))
+            a, b = g.integers(0, K, size=m).astype(np.uint8), g.integers(0, K, size=n).astype(np.uint8)
+            if t % 3 == 0:
+                b = np.resize(b[:int(g.integers(1, 20))], n)
+            S = g.integers(-5, 6, size=(K, K)).astype(np.int8)
+            o = int(g.integers(0, 14))
+            e = int(g.integers(0, o + 1))
+            _score_case(ctx, oracle_mod, a, b, S, o, e, alg)
+            if t % 5 == 0:
+                _align_case(ctx, oracle_mod, a, b, S, o, e, alg)
+        sc = W.dna_scoring()
+        a = W.uniform_dna(6100, W.BASE_SEED + 16200 + R)
+        b = np.concatenate([W.uniform_dna(700, 5), W.mutate(a[300:5800], 4, W.BASE_SEED + 16300)])
+        _align_case(ctx, oracle_mod, a, b, sc.matrix, sc.gap_open, sc.gap_extend, alg)
+        _align_case(two, oracle_mod, a, b, sc.matrix, sc.gap_open, sc.gap_extend, alg)
+        for o, e in ((300, 20), (60, 60), (2000, 1)):        # steep borders; some beyond the packed fill's bound
+            _score_case(ctx, oracle_mod, a[:1500], b[:5000], sc.matrix, o, e, alg)
+            _score_case(ctx, oracle_mod, b[:5000], a[:1500], sc.matrix, o, e, alg)
+    finally:
+        two.close()
+        ctx.close()
