@@ -65,9 +65,10 @@ struct DbView {
     const int64_t *off;        // subject s = res[off[s] .. off[s+1])
     const int32_t *pairs;      // pair p = subjects pairs[2p], pairs[2p+1] (-1 = none)
     const uint16_t *pres;      // pair p's residues interleaved, column j at pres[poff[p] + j]:
-    const int64_t *poff;       // low byte subject A, high byte subject B, 0xff past a subject's end;
+    const int64_t *poff;       // low byte subject A, high byte subject B, `pad` past a subject's end;
                                // n_p = poff[p+1] - poff[p] - 1 columns plus one padding column
     int32_t npairs;
+    int32_t pad;               // the database's largest residue code + 1: the padding code
     int32_t maxlen;            // longest subject (scratch rows hold maxlen + 1 entries)
     // scratch slots: one per block that can be resident at a time (nslots = SMs x blocks per
     // SM); block b < nslots uses slot b, a later block (an oversubscribed grid) takes a slot a
@@ -81,7 +82,7 @@ struct DbView {
 
 // Interleaved residues of every pair (see DbView::pres): one warp per pair.
 static __global__ void pair_residues_kernel(const uint8_t *res, const int64_t *off, const int32_t *pairs,
-                                            const int64_t *poff, int npairs, uint16_t *pres) {
+                                            const int64_t *poff, int npairs, unsigned pad, uint16_t *pres) {
     const int lane = threadIdx.x & 31;
     const int nw = (int)((gridDim.x * blockDim.x) >> 5);
     for (int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); p < npairs; p += nw) {
@@ -90,8 +91,8 @@ static __global__ void pair_residues_kernel(const uint8_t *res, const int64_t *o
         const int64_t b0 = sb >= 0 ? off[sb] : 0, nb = sb >= 0 ? off[sb + 1] - b0 : 0;
         const int64_t base = poff[p], cols = poff[p + 1] - base;   // n_p + 1
         for (int64_t j = lane; j < cols; j += 32) {
-            const unsigned ca = j < na ? res[a0 + j] : 0xffu;
-            const unsigned cb = j < nb ? res[b0 + j] : 0xffu;
+            const unsigned ca = j < na ? res[a0 + j] : pad;
+            const unsigned cb = j < nb ? res[b0 + j] : pad;
             pres[base + j] = (uint16_t)(ca | (cb << 8));
         }
     }
@@ -152,26 +153,34 @@ __device__ __forceinline__ unsigned merge_row(const uint32_t *wa, const uint32_t
     }
 }
 
-// Profile bytes a lane owns per pass: its R rows rounded up to whole 32-bit
-// words, so that every lane's profile load is aligned (R = 5 or 6 gives
-// 160- or 192-row passes, which pad a short query far less than 256).
-constexpr int db_lane_slot(int R) { return ((R + 3) / 4) * 4; }
+// Profile bytes a lane owns per pass: its R rows rounded up to one 4- or
+// 8-byte load, or to whole 16-byte chunks, each chunk [lane] so that a load is conflict-free.
+constexpr int db_lane_slot(int R) { return R <= 4 ? 4 : (R <= 8 ? 8 : ((R + 15) / 16) * 16); }
 
-template <int R>
+// p: the lane's first chunk; lanes of up to 32 rows have a second one 16 G bytes on.
+template <int R, int G>
 __device__ __forceinline__ void load_prof_words(const int8_t *p, uint32_t (&w)[db_lane_slot(R) / 4]) {
     constexpr int LS = db_lane_slot(R);
+    static_assert(LS <= 32, "at most two chunks a lane");
     if constexpr (LS == 4) {
         w[0] = *reinterpret_cast<const uint32_t *>(p);
     } else if constexpr (LS == 8) {
         const uint2 v = *reinterpret_cast<const uint2 *>(p);
         w[0] = v.x; w[1] = v.y;
-    } else if constexpr (LS == 12) {             // 12-byte lane slots: 4-byte aligned only
-        const uint32_t *q = reinterpret_cast<const uint32_t *>(p);
-        w[0] = q[0]; w[1] = q[1]; w[2] = q[2];
     } else {
-        const uint4 v = *reinterpret_cast<const uint4 *>(p);
-        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+#pragma unroll
+        for (int q = 0; q < LS / 16; ++q) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(p + q * 16 * G);
+            w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+        }
     }
+}
+
+// Byte of row r of lane g within a pass of the profile, and a lane's first byte.
+template <int R, int G>
+__device__ __forceinline__ int db_prof_byte(int g, int r) {
+    constexpr int LS = db_lane_slot(R);
+    return LS <= 8 ? g * LS + r : (r / 16) * 16 * G + g * 16 + r % 16;
 }
 
 // grid: 1D; blocks [jobs[j].block0, jobs[j+1].block0) start on job j (the
@@ -180,7 +189,9 @@ __device__ __forceinline__ void load_prof_words(const int8_t *p, uint32_t (&w)[d
 // the most work left (same scoring), so that the launch ends balanced.
 // Dynamic shared memory: the query profile, (K + 1) * mpad bytes,
 // mpad = passes * 32 * db_lane_slot(R) (lane slots of whole words).
-constexpr int kDbCH = 8;      // steps per chunk of the packed fill (steady chunks skip all range tests)
+// Steps per chunk of the packed fill (steady chunks skip all range tests); 4 for long lanes, whose body of 8
+// steps would be some 2,000 instructions (loops beyond about that fall out of the instruction cache)
+constexpr int db_chunk(int R) { return R <= 16 ? 8 : 4; }
 
 // Per-lane state of the packed fill: U = H and E + open of the lane's R query
 // rows for both subjects (16-bit halves), the bottom row's (H, F + open) of the
@@ -200,7 +211,7 @@ struct DbLane {
 // pair (the first and last G - 1 steps).
 template <int R, int G, bool CHECK>
 __device__ __forceinline__ void db_step(DbLane<R> &st, int s, int gl, int n, const uint16_t *pr, uint2 *bnd,
-                                        bool tops, bool last, int K, int mpad,
+                                        bool tops, bool last, unsigned pad2, int mpad,
                                         unsigned nge2, unsigned ngo2, unsigned ge2, unsigned go2)
 {
     const int j = s - gl;
@@ -212,7 +223,7 @@ __device__ __forceinline__ void db_step(DbLane<R> &st, int s, int gl, int n, con
     unsigned cpn;
     uint2 topn = make_uint2(0u, 0u);
     if (CHECK) {
-        cpn = (jn >= 0 && jn <= n) ? pr[jn] : 0xffffu;
+        cpn = (jn >= 0 && jn <= n) ? pr[jn] : pad2;
         if (tops && s + 1 < n) topn = bnd[s + 1];
     } else {
         cpn = pr[jn];                                   // jn <= n: at most the padding column
@@ -220,8 +231,8 @@ __device__ __forceinline__ void db_step(DbLane<R> &st, int s, int gl, int n, con
     }
     if (!CHECK || (j >= 0 && j < n)) {
         uint32_t wa[db_lane_slot(R) / 4], wb[db_lane_slot(R) / 4];
-        load_prof_words<R>(st.prow + min((int)(st.cp & 0xffu), K) * mpad, wa);
-        load_prof_words<R>(st.prow + min((int)(st.cp >> 8), K) * mpad, wb);
+        load_prof_words<R, G>(st.prow + (int)(st.cp & 0xffu) * mpad, wa);
+        load_prof_words<R, G>(st.prow + (int)(st.cp >> 8) * mpad, wb);
         unsigned udiag = st.udiag0;
         st.udiag0 = uup;
         unsigned f = __viaddmax_s16x2(fup, nge2, uup);
@@ -249,11 +260,12 @@ __device__ __forceinline__ void db_step(DbLane<R> &st, int s, int gl, int n, con
 }
 
 template <int R, int W, bool OVERSUB, int G = 32>
-__global__ void __launch_bounds__(W * 32, W >= 16 ? 1 : (R >= 12 ? 3 : 4))
+__global__ void __launch_bounds__(W * 32, W >= 16 ? 1 : (R > 16 ? 2 : (R >= 12 ? 3 : 4)))
 db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
                 const DevScoring *__restrict__ scorings, uint2 *__restrict__ scratch)
 {
     static_assert(G == 32 || G == 16, "one or two wavefronts a warp");
+    constexpr int kDbCH = db_chunk(R);
     constexpr int NG = 32 / G;                    // wavefronts (pairs of subjects) a warp
     extern __shared__ __align__(16) int8_t prof[];
     // OVERSUB: the grid may exceed the blocks that fit at once (the server's steps); blocks
@@ -281,12 +293,16 @@ db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
         constexpr int LS = db_lane_slot(R), PROWS = G * LS;    // profile bytes per lane and per pass
         const int passes = (m + ROWS - 1) / ROWS;
         const int mpad = passes * PROWS;
-        for (int i = threadIdx.x; i < mpad; i += blockDim.x) {
-            const int r = i % LS, row = (i / PROWS) * ROWS + ((i % PROWS) / LS) * R + r;
+        // (only the database's own codes and the padding one have a row: 21 rather than 25 for 20 amino acids)
+        const int pad = D.pad;
+        for (int i = threadIdx.x; i < passes * G * LS; i += blockDim.x) {
+            const int r = i % LS, g = (i / LS) % G, pass = i / (G * LS);
+            const int row = pass * ROWS + g * R + r;
             const bool ok = r < R && row < m;
             const int qc = ok ? min((int)J.q[row], K - 1) : 0;
-            for (int c = 0; c <= K; ++c)
-                prof[c * mpad + i] = (ok && c < K) ? (int8_t)(SC.mat[qc * K + c] + go) : (int8_t)kPadScore;
+            int8_t *dst = prof + pass * PROWS + db_prof_byte<R, G>(g, r);
+            for (int c = 0; c <= pad; ++c)
+                dst[c * mpad] = (ok && c < pad) ? (int8_t)(SC.mat[qc * K + c] + go) : (int8_t)kPadScore;
         }
         __syncthreads();
 
@@ -297,6 +313,7 @@ db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
         const int gl = lane & (G - 1), grp = lane / G;          // the lane's wavefront and its place there
         const int gwarp = slot * W + (threadIdx.x >> 5);
         uint2 *bnd = scratch + ((size_t)gwarp * NG + grp) * (size_t)(D.maxlen + 1);
+        const unsigned pad2 = (unsigned)pad * 0x0101u;
         const unsigned go2 = pack2(go, go), ge2 = pack2(ge, ge);
         const unsigned ngo2 = pack2(-go, -go), nge2 = pack2(-ge, -ge);
 
@@ -331,7 +348,7 @@ db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
             unsigned cmax = 0;                                      // running max of H
             for (int pass = 0; pass < passes; ++pass) {
                 DbLane<R> st;
-                st.prow = prof + pass * PROWS + gl * LS;
+                st.prow = prof + pass * PROWS + db_prof_byte<R, G>(gl, 0);
     #pragma unroll
                 for (int r = 0; r < R; ++r) { st.U[r] = 0; st.E[r] = go2; }    // H = 0; E = 0 never shows
                 st.ub = 0; st.fb = 0; st.udiag0 = 0;                           // F = -open: F(1) = max(-inf, H - open)
@@ -339,7 +356,7 @@ db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
                 const bool last = pass + 1 == passes;
                 const bool tops = pass > 0;
                 // prefetched inputs of this lane's first column and of lane 0's first top cell
-                st.cp = gl == 0 && n > 0 ? pr[0] : 0xffffu;
+                st.cp = gl == 0 && n > 0 ? pr[0] : pad2;
                 st.topv = (tops && n > 0) ? bnd[0] : make_uint2(0u, 0u);
                 for (int s0 = 0; s0 < nmax + G - 1; s0 += kDbCH) {
                     if (s0 >= G - 1 && s0 + kDbCH <= nmin) {
@@ -347,10 +364,10 @@ db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
                         // column at most the padding column n
     #pragma unroll
                         for (int k = 0; k < kDbCH; ++k)
-                            db_step<R, G, false>(st, s0 + k, gl, n, pr, bnd, tops, last, K, mpad, nge2, ngo2, ge2, go2);
+                            db_step<R, G, false>(st, s0 + k, gl, n, pr, bnd, tops, last, pad2, mpad, nge2, ngo2, ge2, go2);
                     } else {
                         for (int k = 0; k < kDbCH && s0 + k < nmax + G - 1; ++k)
-                            db_step<R, G, true>(st, s0 + k, gl, n, pr, bnd, tops, last, K, mpad, nge2, ngo2, ge2, go2);
+                            db_step<R, G, true>(st, s0 + k, gl, n, pr, bnd, tops, last, pad2, mpad, nge2, ngo2, ge2, go2);
                     }
                 }
                 cmax = st.cmax;

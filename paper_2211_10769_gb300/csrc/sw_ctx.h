@@ -151,10 +151,11 @@ int db_score_all(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m, const
 int db_rescore(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m, const DevScoring &ds,
                const std::vector<int32_t> &flagged, int32_t *dscores);
 int db_topk(sw_ctx *c, const int32_t *dscores, int64_t nseq, int k, int2 *dout);
-int db_shape(int K, int m);                // tile shape (index) for a query of m residues
+// (codes: the database's residue codes, DbView::pad)
+int db_shape(int codes, int m);            // tile shape (index) for a query of m residues
 int db_shape_warps(int shape);
 int db_shape_rows(int shape);              // query rows per pass
-int db_resident_blocks_shape(sw_ctx *c, int shape, int K, int m, int *out);
+int db_resident_blocks_shape(sw_ctx *c, int shape, int codes, int m, int *out);
 // Buffers of a database launch: boundary-row scratch, slot pool, scoring table and error word.
 // Default: the context's; launches that may run while other calls use the context (the
 // server's steps on their own streams) bring their own.
@@ -163,14 +164,10 @@ struct DbBufs {
     const DevScoring *scorings;
     int *err;
 };
-int db_launch_shape(sw_ctx *c, int shape, const DbJob *jobs, int njobs, int nblocks, const DbView &D, int K, int m,
+int db_launch_shape(sw_ctx *c, int shape, const DbJob *jobs, int njobs, int nblocks, const DbView &D, int codes, int m,
                     const DbBufs *bufs = nullptr);
 // the scratch bytes db_launch_shape ensures for that launch (subjects up to maxlen residues)
-int db_scratch_shape(sw_ctx *c, int shape, int K, int m, int maxlen, size_t *row_bytes, size_t *slot_bytes);
-int db_resident_blocks(sw_ctx *c, int K, int m, int *out);
-int db_warps_per_block(int K, int m);
-int db_rows_per_pass(int K, int m);      // query rows per pass of the packed kernel for this launch shape
-int db_launch(sw_ctx *c, const DbJob *jobs, int njobs, int nblocks, const DbView &D, int K, int m);
+int db_scratch_shape(sw_ctx *c, int shape, int codes, int m, int maxlen, size_t *row_bytes, size_t *slot_bytes);
 int db_view(const sw_db *db, DbView *v, int64_t *nseq, int32_t *max_code, int *device);
 int db_chunk_maxlen(const sw_db *db, int32_t pair0, int32_t pair1);
 int64_t db_total_residues(const sw_db *db);

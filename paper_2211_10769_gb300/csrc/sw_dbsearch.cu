@@ -3,7 +3,7 @@
 // 32-bit rescoring of saturating subjects, top-k hits.
 #include "sw.h"
 #include "sw_ctx.h"
-#include "dbsearch.cuh"
+#include "db_launch.cuh"
 #include "wavefront.cuh"
 #include "aux_kernels.cuh"
 
@@ -15,8 +15,6 @@
 
 using namespace swgb;
 
-#define CU(x) do { if ((x) != cudaSuccess) { cudaGetLastError(); return SW_ECUDA; } } while (0)
-#define RC(x) do { int rc_ = (x); if (rc_) return rc_; } while (0)
 
 struct sw_db {
     int device = 0;
@@ -40,181 +38,82 @@ static __global__ void max_code_kernel(const uint8_t *s, long long len, int *out
     if ((threadIdx.x & 31) == 0) atomicMax(out, mx);
 }
 
-constexpr long long kMaxProfileSmem = 200 * 1024;
-
-// Profile bytes of a query of m residues for tile shape (R, G) (whole passes
-// of G lane slots of db_lane_slot(R) bytes, per residue code and padding).
-template <int R, int G>
-size_t db_profile_bytes(int K, int m) {
-    constexpr int ROWS = G * R;
-    const long long mpad = (long long)((m + ROWS - 1) / ROWS) * G * db_lane_slot(R);
-    return (size_t)(K + 1) * (size_t)mpad;
-}
-
-// Scratch of one launch: boundary rows, one per wavefront (32 / G of them a
-// warp) of every block that can be resident at once, and the slot pool's words.
-template <int R, int W, int G>
-int db_scratch(sw_ctx *c, int K, int m, int maxlen, int *nslots, size_t *row_bytes, size_t *slot_bytes) {
-    const size_t smem = db_profile_bytes<R, G>(K, m);
-    int occ = 0;
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, db_s16x2_kernel<R, W, false, G>, W * 32, smem));
-    int occ2 = 0;
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, db_s16x2_kernel<R, W, true, G>, W * 32, smem));
-    occ = std::min(occ, occ2);
-    if (occ < 1) return SW_ECUDA;
-    *nslots = occ * c->nsm;
-    *row_bytes = (size_t)*nslots * W * (32 / G) * (size_t)(maxlen + 1) * sizeof(uint2);
-    *slot_bytes = (size_t)((*nslots + 31) / 32) * sizeof(unsigned);
-    return SW_OK;
-}
-
-template <int R, int W, int G>
-int launch_db(sw_ctx *c, const DbJob *jobs, int njobs, int nblocks, const DbView &D0, int K, int m,
-              const DbBufs &B) {
-    const size_t smem = db_profile_bytes<R, G>(K, m);
-    // boundary rows: one per warp of every block that can be resident at once; a grid larger
-    // than that (the server's steps) takes the kernel whose later blocks share the slots
-    DbView D = D0;
-    size_t row_bytes = 0, slot_bytes = 0;
-    RC((db_scratch<R, W, G>(c, K, m, D.maxlen, &D.nslots, &row_bytes, &slot_bytes)));
-    D.slot_words = (D.nslots + 31) / 32;
-    const bool over = nblocks > D.nslots;
-    RC(B.rows->ensure(row_bytes));
-    RC(B.slots->ensure(slot_bytes));
-    D.slot_pool = static_cast<unsigned *>(B.slots->p);
-    D.err = B.err;
-    D.spin_limit = c->spin_limit;
-    if (over) {
-        init_slot_pool_kernel<<<1, 64, 0, c->stream>>>(D.slot_pool, D.slot_words, D.nslots, D.nslots);
-        CU(cudaGetLastError());
-        ++c->launches;
-    }
-    auto kern = over ? db_s16x2_kernel<R, W, true, G> : db_s16x2_kernel<R, W, false, G>;
-    const int kp = kt_begin(c, SW_KT_DB16);
-    kern<<<(unsigned)nblocks, W * 32, smem, c->stream>>>(jobs, njobs, D, B.scorings,
-                                                         static_cast<uint2 *>(B.rows->p));
-    kt_end(c, kp);
-    CU(cudaGetLastError());
-    ++c->launches;
-    return SW_OK;
-}
-
-template <int R, int W, int G>
-int resident_blocks(sw_ctx *c, int K, int m, int *out) {
-    const size_t smem = db_profile_bytes<R, G>(K, m);
-    if ((long long)smem > kMaxProfileSmem) return SW_ERANGE;
-    static int attr_set[64] = {0};
-    if (c->device < 64 && !attr_set[c->device]) {
-        CU(cudaFuncSetAttribute(db_s16x2_kernel<R, W, false, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kMaxProfileSmem));
-        CU(cudaFuncSetAttribute(db_s16x2_kernel<R, W, true, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)kMaxProfileSmem));
-        attr_set[c->device] = 1;
-    }
-    int occ = 0;
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, db_s16x2_kernel<R, W, false, G>, W * 32, smem));
-    if (occ < 1) return SW_ECUDA;
-    *out = occ * c->nsm;
-    return SW_OK;
-}
-
 // Tile shapes of the packed search: rows a lane, warps a block and lanes a
-// wavefront.  A query is padded to whole passes of G R rows, so short queries
-// want few rows a pass: 144 residues take one 144-row pass in two 16-lane
-// wavefronts a warp at R = 9 (in one 32-lane wavefront: 160 rows at R = 5, with
-// a lane's fixed per-step cost shared by 5 rows instead of 9; measured 4,333
-// against 3,476 GCUPS).  Long queries want R = 16, whose per-step overhead is
-// shared by more rows.  Queries whose profile would not leave room for three
-// blocks an SM take blocks of 16 warps (one per SM) at R = 16.  (Lanes of 4, 5,
-// 6 and 12 rows in 32-lane wavefronts were measured too and never won.)
-#define SWGB_DB_SHAPES(X)                                                                              \
-    X(0, 8, 8, 32) X(1, 16, 8, 32) X(2, 4, 8, 16) X(3, 6, 8, 16) X(4, 9, 8, 16) X(5, 12, 8, 16)          \
-    X(6, 16, 16, 32)
-struct DbShape { int R, W, G; };
-#define SWGB_DB_ROW(i, R, W, G) {R, W, G},
-constexpr DbShape kDbShapes[] = {SWGB_DB_SHAPES(SWGB_DB_ROW)};
-#undef SWGB_DB_ROW
-constexpr int kDbWide = 6;                         // index of the one-block-an-SM shape
-constexpr size_t kDbNarrowProfileMax = 96 * 1024;  // profile bytes of a three-blocks-an-SM shape at most
-// cost model of a shape (db_shape), fitted to measured GCUPS of every shape at query lengths 144,
-// 300, 464, 700, 1,000 and 2,005 (it picks the fastest at each): a lane's fixed per-step cost in
-// rows' worth, a pass boundary in rows, and a typical subject length (a wavefront's skew of
-// G - 1 steps costs about (G - 1) / 360 of a pair's sweep)
-constexpr double kDbStepRows = 2.25, kDbPassRows = 16, kDbTypicalCols = 360;
+// wavefront (16: two wavefronts a warp).  A query is padded to whole passes of
+// 16 R rows.  A lane's fixed per-step work (two shuffles, lane 0's row above,
+// the next residues) is shared by its R rows, so a query wants the most rows a
+// lane whose passes it fills: 144 residues take one pass at R = 9, 464 one at
+// R = 29, 1,000 two at R = 32.  32 lanes a wavefront (1,000: one pass of 32 x 32
+// rows, 5,690 against 5,820 GCUPS) pay more for their skew than a second pass
+// costs; four wavefronts of 8 lanes (144: 4,190 against 4,960) lose to their bank
+// conflicts and uneven pairs.  Blocks of 8 warps, two (above 16 rows a lane: 128
+// registers) to four an SM; queries whose profile would not leave room for two
+// blocks take blocks of 16 warps, one an SM, with 32 lanes a wavefront (5,478
+// residues: 5,760 GCUPS at R = 29, against 5,270 in two wavefronts a warp, whose
+// twice as many boundary rows outgrow the L1 cache that the profile leaves).
+constexpr int kDbA = 6, kDbB = 5, kDbC = 6;        // shapes per translation unit
+constexpr int kDbShapeCount = kDbA + kDbB + kDbC;
+constexpr int kDbWide0 = kDbA + kDbB + 2;          // the first of the one-block-an-SM shapes
+constexpr size_t kDbNarrowProfileMax = 100 * 1024; // profile bytes of a two-blocks-an-SM shape at most
+// cost model of a shape (db_shape), from measured GCUPS of every shape: a lane's fixed per-step cost in
+// rows' worth, and a pass boundary in rows
+constexpr double kDbStepRows = 2.0, kDbPassRows = 2;
 
-size_t shape_profile_bytes(int s, int K, int m) {
-    switch (s) {
-#define SWGB_DB_CASE(i, R, W, G) case i: return db_profile_bytes<R, G>(K, m);
-        SWGB_DB_SHAPES(SWGB_DB_CASE)
-#undef SWGB_DB_CASE
-        default: return 0;
-    }
+const DbShape &shape_at(int s) {
+    static const auto all = [] {
+        std::vector<DbShape> v;
+        for (int k = 0; k < kDbA; ++k) v.push_back(db_shape_a(k));
+        for (int k = 0; k < kDbB; ++k) v.push_back(db_shape_b(k));
+        for (int k = 0; k < kDbC; ++k) v.push_back(db_shape_c(k));
+        return v;
+    }();
+    return all[(size_t)s];
 }
 
 }  // namespace
 
-// The shape for a query of m residues: the least padded work, counting the
-// per-step overhead of a lane, a pass boundary and the wavefront's skew, among
-// the shapes whose profile fits.
-int swgb::db_shape(int K, int m) {
-    // tuning override: SWGB_DB_SHAPE=<index into kDbShapes>, where its profile fits
+// The shape for a query of m residues against a database of `codes` residue codes: the least padded work,
+// counting the per-step overhead of a lane and a pass boundary, among the shapes whose profile fits.
+int swgb::db_shape(int codes, int m) {
+    // tuning override: SWGB_DB_SHAPE=<index of a shape>, where its profile fits
     static const int forced = [] { const char *f = std::getenv("SWGB_DB_SHAPE"); return f ? std::atoi(f) : -1; }();
-    if (forced >= 0 && forced < kDbWide && shape_profile_bytes(forced, K, m) <= kDbNarrowProfileMax) return forced;
-    int best = kDbWide;
+    auto fits = [&](int s) {
+        const size_t p = shape_at(s).profile_bytes(codes, m);
+        return s < kDbWide0 ? p <= kDbNarrowProfileMax : (long long)p <= kMaxProfileSmem;
+    };
+    if (forced >= 0 && forced < kDbShapeCount && fits(forced)) return forced;
+    int best = kDbShapeCount - 1;                   // 16 rows a lane: the most compact profile
     double best_cost = 1e300;
-    for (int s = 0; s < kDbWide; ++s) {
-        if (shape_profile_bytes(s, K, m) > kDbNarrowProfileMax) continue;
-        const int R = kDbShapes[s].R, G = kDbShapes[s].G, rows = G * R;
+    bool narrow = false;
+    for (int s = 0; s < kDbShapeCount; ++s) {
+        if (!fits(s) || (narrow && s >= kDbWide0)) continue;
+        if (s < kDbWide0) narrow = true;
+        const DbShape &q = shape_at(s);
+        const int rows = q.G * q.R;
         const long long passes = (m + rows - 1) / rows;
-        const double cost = (double)passes * rows * (R + kDbStepRows) / R * (1.0 + (G - 1) / kDbTypicalCols) +
-                            kDbPassRows * (double)passes;
+        const double cost = (double)passes * (rows * (q.R + kDbStepRows) / q.R + kDbPassRows);
         if (cost < best_cost) { best_cost = cost; best = s; }
     }
     return best;
 }
 
-int swgb::db_resident_blocks_shape(sw_ctx *c, int shape, int K, int m, int *out) {
-    switch (shape) {
-#define SWGB_DB_CASE(i, R, W, G) case i: return resident_blocks<R, W, G>(c, K, m, out);
-        SWGB_DB_SHAPES(SWGB_DB_CASE)
-#undef SWGB_DB_CASE
-        default: return SW_EINVAL;
-    }
+int swgb::db_resident_blocks_shape(sw_ctx *c, int shape, int codes, int m, int *out) {
+    return shape_at(shape).resident(c, codes, m, out);
 }
 
-int swgb::db_resident_blocks(sw_ctx *c, int K, int m, int *out) {
-    return db_resident_blocks_shape(c, db_shape(K, m), K, m, out);
-}
+int swgb::db_shape_warps(int shape) { return shape_at(shape).W; }
+int swgb::db_shape_rows(int shape) { return shape_at(shape).G * shape_at(shape).R; }
 
-int swgb::db_shape_warps(int shape) { return kDbShapes[shape].W; }
-int swgb::db_shape_rows(int shape) { return kDbShapes[shape].G * kDbShapes[shape].R; }
-int swgb::db_warps_per_block(int K, int m) { return db_shape_warps(db_shape(K, m)); }
-int swgb::db_rows_per_pass(int K, int m) { return db_shape_rows(db_shape(K, m)); }
-
-int swgb::db_launch_shape(sw_ctx *c, int shape, const DbJob *jobs, int njobs, int nblocks, const DbView &D, int K,
+int swgb::db_launch_shape(sw_ctx *c, int shape, const DbJob *jobs, int njobs, int nblocks, const DbView &D, int codes,
                           int m, const DbBufs *bufs) {
     DbBufs B{&c->dbscratch, &c->dbslots, static_cast<const DevScoring *>(c->scorings.p), static_cast<int *>(c->err.p)};
     if (bufs) B = *bufs;
-    switch (shape) {
-#define SWGB_DB_CASE(i, R, W, G) case i: return launch_db<R, W, G>(c, jobs, njobs, nblocks, D, K, m, B);
-        SWGB_DB_SHAPES(SWGB_DB_CASE)
-#undef SWGB_DB_CASE
-        default: return SW_EINVAL;
-    }
+    return shape_at(shape).launch(c, jobs, njobs, nblocks, D, codes, m, B);
 }
 
-int swgb::db_scratch_shape(sw_ctx *c, int shape, int K, int m, int maxlen, size_t *row_bytes, size_t *slot_bytes) {
+int swgb::db_scratch_shape(sw_ctx *c, int shape, int codes, int m, int maxlen, size_t *row_bytes, size_t *slot_bytes) {
     int nslots = 0;
-    switch (shape) {
-#define SWGB_DB_CASE(i, R, W, G) case i: return db_scratch<R, W, G>(c, K, m, maxlen, &nslots, row_bytes, slot_bytes);
-        SWGB_DB_SHAPES(SWGB_DB_CASE)
-#undef SWGB_DB_CASE
-        default: return SW_EINVAL;
-    }
-}
-
-int swgb::db_launch(sw_ctx *c, const DbJob *jobs, int njobs, int nblocks, const DbView &D, int K, int m) {
-    return db_launch_shape(c, db_shape(K, m), jobs, njobs, nblocks, D, K, m);
+    return shape_at(shape).scratch(c, codes, m, maxlen, &nslots, row_bytes, slot_bytes);
 }
 
 int swgb::db_view(const sw_db *db, DbView *v, int64_t *nseq, int32_t *max_code, int *device) {
@@ -224,6 +123,7 @@ int swgb::db_view(const sw_db *db, DbView *v, int64_t *nseq, int32_t *max_code, 
     v->pres = static_cast<const uint16_t *>(db->pres.p);
     v->poff = static_cast<const int64_t *>(db->poff.p);
     v->npairs = db->npairs;
+    v->pad = db->max_code + 1;
     v->maxlen = db->maxlen;
     *nseq = db->nseq;
     *max_code = db->max_code;
@@ -295,15 +195,7 @@ extern "C" int sw_db_create(sw_ctx *c, const uint8_t *residues, const int64_t *o
     if (!pairs.empty())
         ok &= cudaMemcpyAsync(db->pairs.p, pairs.data(), pairs.size() * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
     ok &= cudaMemcpyAsync(db->poff.p, poff.data(), poff.size() * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream) == cudaSuccess;
-    if (ok && db->npairs > 0) {
-        pair_residues_kernel<<<(unsigned)std::min<long long>((db->npairs + 7) / 8, 16LL * c->nsm), 256, 0, c->stream>>>(
-            static_cast<const uint8_t *>(db->res.p), static_cast<const int64_t *>(db->doff.p),
-            static_cast<const int32_t *>(db->pairs.p), static_cast<const int64_t *>(db->poff.p), db->npairs,
-            static_cast<uint16_t *>(db->pres.p));
-        ok &= cudaGetLastError() == cudaSuccess;
-        ++c->launches;
-    }
-    // largest residue code, checked against the alphabet at search time
+    // largest residue code: checked against the alphabet at search time; the next one is the pairs' padding
     ok &= c->misc.ensure(sizeof(int)) == SW_OK;
     ok &= cudaMemsetAsync(c->misc.p, 0, sizeof(int), c->stream) == cudaSuccess;
     if (ok && total > 0) {
@@ -315,6 +207,15 @@ extern "C" int sw_db_create(sw_ctx *c, const uint8_t *residues, const int64_t *o
     int mc = 0;
     ok &= cudaMemcpyAsync(&mc, c->misc.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream) == cudaSuccess;
     ok &= cudaStreamSynchronize(c->stream) == cudaSuccess;
+    if (ok && db->npairs > 0) {
+        pair_residues_kernel<<<(unsigned)std::min<long long>((db->npairs + 7) / 8, 16LL * c->nsm), 256, 0, c->stream>>>(
+            static_cast<const uint8_t *>(db->res.p), static_cast<const int64_t *>(db->doff.p),
+            static_cast<const int32_t *>(db->pairs.p), static_cast<const int64_t *>(db->poff.p), db->npairs,
+            (unsigned)(total > 0 ? mc + 1 : 0), static_cast<uint16_t *>(db->pres.p));
+        ok &= cudaGetLastError() == cudaSuccess;
+        ++c->launches;
+    }
+    ok &= cudaStreamSynchronize(c->stream) == cudaSuccess;   // (the offsets' host copies are read until here)
     if (!ok) { cudaGetLastError(); delete db; return SW_ECUDA; }
     db->max_code = total > 0 ? mc : -1;
     *out = db;
@@ -333,7 +234,6 @@ extern "C" int64_t sw_db_size(const sw_db *db) { return db ? db->nseq : -1; }
 // scores, int32 per subject), flagged subjects rescored exactly.
 int swgb::db_score_all(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m, const DevScoring &ds,
                        int32_t *dscores) {
-    const int K = ds.K;
     RC(c->dbovf.ensure((size_t)std::max<int64_t>(1, db->nseq) * sizeof(int32_t)));
     RC(c->dbjob.ensure(sizeof(DbJob) + 64));
     int32_t *novf = reinterpret_cast<int32_t *>(static_cast<char *>(c->dbjob.p) + sizeof(DbJob));
@@ -355,6 +255,7 @@ int swgb::db_score_all(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m,
     D.pres = static_cast<const uint16_t *>(db->pres.p);
     D.poff = static_cast<const int64_t *>(db->poff.p);
     D.npairs = db->npairs;
+    D.pad = db->max_code + 1;
     D.maxlen = db->maxlen;
     int32_t nflag = 0;
     std::vector<int32_t> flagged;
@@ -362,11 +263,12 @@ int swgb::db_score_all(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m,
     int rc = SW_ERANGE;
     if (packed_ok) {
         int nblk = 0;
-        rc = db_resident_blocks(c, K, (int)m, &nblk);
+        const int shape = db_shape(D.pad, (int)m);
+        rc = db_resident_blocks_shape(c, shape, D.pad, (int)m, &nblk);
         if (!rc) {
-            const int W = db_warps_per_block(K, (int)m);
+            const int W = db_shape_warps(shape);
             nblk = std::max(1, std::min(nblk, (db->npairs + W - 1) / W));
-            rc = db_launch(c, static_cast<const DbJob *>(c->dbjob.p), 1, nblk, D, K, (int)m);
+            rc = db_launch_shape(c, shape, static_cast<const DbJob *>(c->dbjob.p), 1, nblk, D, D.pad, (int)m);
         }
     }
     if (rc == SW_ERANGE) {

@@ -199,7 +199,7 @@ int enqueue_step(sw_server *S, const std::vector<Slot *> &act, InFlight *next, i
     // that pads it least (one shape for all would pad a 100-residue query to a 512-row pass
     // next to a long one); one launch per group
     std::map<int, std::vector<Slot *>> groups;
-    for (Slot *s : act) groups[db_shape(S->ds.K, (int)s->m)].push_back(s);
+    for (Slot *s : act) groups[db_shape(S->view.pad, (int)s->m)].push_back(s);
     std::vector<DbJob> jobs;
     struct Launch { int shape, job0, njobs, nblocks, maxm; };
     std::vector<Launch> launches;
@@ -208,7 +208,7 @@ int enqueue_step(sw_server *S, const std::vector<Slot *> &act, InFlight *next, i
         int64_t maxm = 0;
         for (Slot *s : g.second) maxm = std::max(maxm, s->m);
         int resident = 0;
-        RC(db_resident_blocks_shape(c, shape, S->ds.K, (int)maxm, &resident));
+        RC(db_resident_blocks_shape(c, shape, S->view.pad, (int)maxm, &resident));
         const int W = db_shape_warps(shape), rows = db_shape_rows(shape);
         // a request's work is its query padded to whole passes of `rows` rows
         auto padded = [&](int64_t m) { return (double)((m + rows - 1) / rows) * rows; };
@@ -258,7 +258,7 @@ int enqueue_step(sw_server *S, const std::vector<Slot *> &act, InFlight *next, i
     std::vector<size_t> rneed((size_t)ng), sneed((size_t)ng);
     bool grow = false;
     for (int g = 0; g < ng; ++g) {
-        RC(db_scratch_shape(c, launches[g].shape, S->ds.K, launches[g].maxm, v.maxlen, &rneed[g], &sneed[g]));
+        RC(db_scratch_shape(c, launches[g].shape, S->view.pad, launches[g].maxm, v.maxlen, &rneed[g], &sneed[g]));
         grow = grow || rneed[g] > S->grows[g].cap || sneed[g] > S->gslots[g].cap;
     }
     if (grow) *early = complete_inflight(S);
@@ -286,7 +286,7 @@ int enqueue_step(sw_server *S, const std::vector<Slot *> &act, InFlight *next, i
         DbBufs B{&S->grows[g], &S->gslots[g], static_cast<const DevScoring *>(S->dscore.p),
                  static_cast<int *>(S->derr.p)};
         c->stream = gs;
-        rc = db_launch_shape(c, L.shape, djobs + L.job0, L.njobs, L.nblocks, v, S->ds.K, L.maxm, &B);
+        rc = db_launch_shape(c, L.shape, djobs + L.job0, L.njobs, L.nblocks, v, S->view.pad, L.maxm, &B);
         c->stream = home;
         if (rc == SW_OK && cudaEventRecord(S->gdone[par][g], gs) != cudaSuccess) { cudaGetLastError(); rc = SW_ECUDA; }
         if (rc == SW_OK) ++launched;

@@ -50,11 +50,10 @@ def test_small_database_all_scores(ctx, oracle_mod):
 
 
 def test_every_tile_shape(ctx, oracle_mod):
-    """Query lengths that pick each tile shape of the packed search (two
-    16-lane wavefronts a warp at 4, 6, 9 and 12 rows a lane; one 32-lane
-    wavefront at 8 and 16 rows; 16-warp blocks for long queries), with one or
-    several passes, the last pass partly padding, and warps whose second
-    wavefront finds no pair left."""
+    """Query lengths that pick the tile shapes of the packed search (two
+    16-lane wavefronts a warp at 4 to 32 rows a lane; 16-warp blocks for long
+    queries), with one or several passes, the last pass partly padding, and
+    warps whose second wavefront finds no pair left."""
     sc = W.protein_scoring()
     lengths = (1, 31, 80, 100, 128, 144, 160, 161, 190, 250, 300, 350, 384, 464, 700, 1000, 1500, 4100)
     qs = W.protein_queries(lengths, seed_offset=760)
@@ -63,6 +62,24 @@ def test_every_tile_shape(ctx, oracle_mod):
     db = _db(ctx, subjects)
     for q in qs:
         _check_all(ctx, oracle_mod, db, subjects, q, sc)
+
+
+@pytest.mark.parametrize("codes", [20, 24])
+def test_shape_edges(ctx, oracle_mod, codes):
+    """Queries of exactly 16 R rows and one more for every R of the shapes, one to many passes, up to
+    the blocks of 16 warps; a database whose residues use every code of the alphabet (the padding code
+    is then the alphabet size) and one that stops at 20."""
+    sc = W.protein_scoring()
+    g = np.random.default_rng(W.BASE_SEED + 765 + codes)
+    subjects = [g.integers(0, codes, size=int(n)).astype(np.uint8) for n in (1, 15, 16, 17, 40, 333, 334, 90, 700)]
+    subjects[3][0] = codes - 1
+    db = _db(ctx, subjects)
+    for rows in (4, 7, 9, 11, 13, 16, 18, 20, 22, 24, 26, 29, 32):
+        for m in (16 * rows, 16 * rows + 1):
+            q = g.integers(0, 24, size=m).astype(np.uint8)
+            _check_all(ctx, oracle_mod, db, subjects, q, sc, k=5)
+    for m in (4090, 5200, 6100, 7999):
+        _check_all(ctx, oracle_mod, db, subjects, g.integers(0, 24, size=m).astype(np.uint8), sc, k=5)
 
 
 @pytest.mark.parametrize("nseq", [1, 2, 3, 5, 7])
