@@ -46,10 +46,11 @@ bool swgb::p16_fits(const DevScoring &s, int R) {
     return p16_spread(R, s.go, s.ge, hi, lo) <= kP16Span;
 }
 
-int swgb::launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K,
+int swgb::launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const FillLaunch &L, int K,
                         long long tickets) {
     if (tickets <= 0) return SW_OK;
     if (cfg.alg != kAlgLocal) return launch_fill16_variant(c, cfg, mode, L, K, tickets);
+    if (cfg.P16 == 2 && fold && mode == kModeScore) return launch_fill16_batch(c, cfg, L, K, tickets);
     switch (cfg.R) {
 #define SWGB_P16_CASE(R) case R: return launch16_mode<R>(c, mode, cfg.left != 0, cfg.W, L, K, tickets, cfg.B);
         SWGB_P16_SHAPES(SWGB_P16_CASE)

@@ -18,9 +18,9 @@ namespace swgb {
 inline constexpr size_t kPairProfileMax = 170 * 1024;
 inline constexpr size_t kSharedMax = 227 * 1024;          // shared memory a block can have
 
-template <int R, int W, int MODE, int PK, bool LEFT, bool LOCAL>
+template <int R, int W, int MODE, int PK, bool LEFT, bool LOCAL, int MINB = 1>
 int launch16(sw_ctx *c, const FillLaunch &L, int K, long long tickets, int max_blocks) {
-    auto kern = wavefront16_kernel<R, W, MODE, PK, LEFT, LOCAL>;
+    auto kern = wavefront16_kernel<R, W, MODE, PK, LEFT, LOCAL, MINB>;
     const size_t smem = p16_shared_bytes<R, W>() + p16_profile_bytes(R, W, K, PK);
     static int attr_set[64] = {0};
     if (c->device >= 64 || !attr_set[c->device]) {

@@ -312,7 +312,7 @@ bool swgb::fold_open(const DevScoring &s) {
 int swgb::launch_fill(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const FillLaunch &L, int K,
                       long long tickets) {
     if (tickets <= 0) return SW_OK;
-    if (cfg.P16) return launch_fill16(c, cfg, mode, L, K, tickets);
+    if (cfg.P16) return launch_fill16(c, cfg, mode, fold, L, K, tickets);
     if (cfg.alg != kAlgLocal) return launch_fill_variant(c, cfg, mode, fold, L, K, tickets);
     if (cfg.R == 4 && cfg.W == 4) return launch_fill_rw<4, 4>(c, mode, fold, L, K, tickets, cfg.B);
     if (cfg.R == 8 && cfg.W == 4) return launch_fill_rw<8, 4>(c, mode, fold, L, K, tickets, cfg.B);
@@ -454,7 +454,10 @@ int sw_ctx_create(int device, void *cuda_stream, sw_ctx **out) {
         c->fwd_auto = false;
     }
     if (const char *f = std::getenv("SWGB_TB")) std::sscanf(f, "%d,%d", &c->tbc.R, &c->tbc.W);
-    if (const char *f = std::getenv("SWGB_BATCH")) std::sscanf(f, "%d,%d,%d", &c->bat.R, &c->bat.W, &c->bat.P16);
+    if (const char *f = std::getenv("SWGB_BATCH")) {
+        std::sscanf(f, "%d,%d,%d", &c->bat.R, &c->bat.W, &c->bat.P16);
+        c->bat_auto = false;
+    }
     if (const char *f = std::getenv("SWGB_PROF32")) c->prof32 = std::atoi(f) != 0;
     if (const char *f = std::getenv("SWGB_ONE_ROUND")) c->one_round = std::atoi(f) != 0 ? 1 : 0;
     if (const char *f = std::getenv("SWGB_LOOKAHEAD")) c->lookahead = std::atoi(f) != 0;

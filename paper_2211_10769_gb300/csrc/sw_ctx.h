@@ -44,7 +44,7 @@ struct FillConfig {
     int W;
     int S = 0;
     int B = 0;
-    int P16 = 0;   // packed 16-bit fill (wavefront16.cuh) instead of the int32 one
+    int P16 = 0;   // packed 16-bit fill (wavefront16.cuh) instead of the int32 one; 2: with an int8 profile (batches)
     int alg = 0;   // not kAlgLocal: the fills without the zero floor (fill_variants.cu, fill16_variants.cu)
     int left = 0;  // packed fill whose tasks may start right of its own checkpoint column
 };
@@ -74,6 +74,7 @@ struct sw_ctx {
     bool fwd_auto = true;             // choose R per pair (pair_fill_config)
     swgb::FillConfig tbc{8, 4};       // traceback recompute
     swgb::FillConfig bat{8, 4};       // batches of pairs (unless autotuned)
+    bool bat_auto = true;             // no SWGB_BATCH: batches start from the packed fill where it is exact
     bool prof32 = true;               // int32 query profiles where they fit (small alphabets)
     bool p16 = true;                  // packed 16-bit pair fill where it is exact (p16_fits)
     int tb_band = 0;                  // tile rows per traceback band (0 = about one tile per SM)
@@ -115,7 +116,8 @@ int launch_straighten(sw_ctx *c, int R, bool local, const FillTask *tasks, int n
 int launch_straighten_variant(sw_ctx *c, int R, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc);
 int launch_fill16_variant(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K, long long tickets);
 bool p16_fits(const DevScoring &s, int R);
-int launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K, long long tickets);
+int launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const FillLaunch &L, int K, long long tickets);
+int launch_fill16_batch(sw_ctx *c, const FillConfig &cfg, const FillLaunch &L, int K, long long tickets);
 // the global, semi-global and overlap algorithms: 8 or 16 rows a lane, four compute warps
 FillConfig variant_fill_config(const sw_ctx *c, int64_t rows);
 int launch_fill_variant(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const FillLaunch &L, int K,

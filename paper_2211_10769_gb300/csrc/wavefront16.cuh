@@ -38,8 +38,9 @@
 // 45 instructions a step at 12 rows a lane (77 before), 91 clocks in the
 // loop.  200 kbp score fill 18.85 -> 15.2 ms, 1 Mbp (16 rows a lane) 332 ->
 // 276 ms (GB300, 2,070 MHz).  Tried on the same code: four ALU operations a
-// cell pair and two plain subtractions, as in the database search (no gain
-// with one warp a sub-partition); a third step of skew per lane to take the
+// cell pair and two plain subtractions, as in the database search (26 rows a lane
+// 207 -> 229 clocks a step, 12 rows 115.5 -> 117.6: a lone warp has no issue slots
+// for the extra instruction); a third step of skew per lane to take the
 // shuffle off the chain (the longer fill eats the gain); unrolling 8 (16.4
 // ms) and 32 steps (18.4 ms) instead of 16.
 //
@@ -76,7 +77,8 @@
 //
 // Query profile: for small alphabets a pair profile, one packed word per
 // (residue of the top half, residue of the bottom half) and packed row; else
-// an int16 profile whose two words per packed row are merged with one prmt.
+// an int16 profile whose two words per packed row are merged with one prmt;
+// batches, which want several blocks an SM, an int8 one a quarter its size.
 //
 // Modes: score (end-cell candidate per strip) and score with checkpoints
 // (strip bottom rows, and staircase checkpoint columns in the two-positions
@@ -103,7 +105,11 @@ constexpr int kP16Unroll = 16;
 constexpr int kP16IdleNs = 256;
 
 // Profile kinds of the packed fill.
-enum P16Prof { kP16Pair = 0, kP16Int16 = 1 };
+enum P16Prof { kP16Pair = 0, kP16Int16 = 1, kP16Int8 = 2 };
+
+// Profile words a lane loads per step, and the bytes of its slot in an int8 profile row.
+__host__ __device__ constexpr int p16_words(int R, int PK) { return PK == kP16Int8 ? R / 4 : R / 2; }
+__host__ __device__ constexpr int p16_slot8(int R) { return R <= 8 ? 8 : 16; }
 
 // Bound on the spread of all values a warp touches during one chunk (see the header); the packed
 // fill is exact when it is at most kP16Span.
@@ -117,6 +123,7 @@ inline long long p16_spread(int R, int go, int ge, int max_s, int min_s) {
 // Bytes of the packed fill's query profile for K residue codes.
 inline size_t p16_profile_bytes(int R, int W, int K, int pk) {
     const size_t HC = (size_t)W * 32 * R;
+    if (pk == kP16Int8) return (size_t)(K + 1) * W * 32 * p16_slot8(R);
     return pk == kP16Pair ? (size_t)(K + 1) * (K + 1) * (HC / 2) * 4 : (size_t)(K + 1) * HC * 2;
 }
 
@@ -133,6 +140,12 @@ template <unsigned sel>
 __device__ __forceinline__ unsigned prmt_c(unsigned a, unsigned b) {
     unsigned d;
     asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "n"(sel));
+    return d;
+}
+
+__device__ __forceinline__ unsigned prmt_v(unsigned a, unsigned b, unsigned sel) {
+    unsigned d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
     return d;
 }
 
@@ -159,9 +172,20 @@ __device__ __forceinline__ int p16_pair_word(int k, int g, int NL) {
 
 // Profile words of one step (H per lane) for the column whose profile offset is off.
 template <int R, int PK, int NL>
-__device__ __forceinline__ void p16_load(const int8_t *prof, int g, int off, uint32_t (&w)[R / 2]) {
+__device__ __forceinline__ void p16_load(const int8_t *prof, int g, int off, uint32_t (&w)[p16_words(R, PK)]) {
     constexpr int H = R / 2;
-    if constexpr (PK == kP16Pair) {
+    if constexpr (PK == kP16Int8) {
+        static_assert(R == 8 || R == 12 || R == 16, "int8 profile loads");
+        const int8_t *p = prof + off + g * p16_slot8(R);
+        if constexpr (R == 8) {
+            const uint2 v = *reinterpret_cast<const uint2 *>(p);
+            w[0] = v.x; w[1] = v.y;
+        } else {
+            const uint4 v = *reinterpret_cast<const uint4 *>(p);
+            w[0] = v.x; w[1] = v.y; w[2] = v.z;
+            if constexpr (R == 16) w[3] = v.w;
+        }
+    } else if constexpr (PK == kP16Pair) {
         using C = P16Chunks<H>;
         const int8_t *p = prof + off;
 #pragma unroll
@@ -195,9 +219,14 @@ __device__ __forceinline__ void p16_load(const int8_t *prof, int g, int off, uin
 
 // Score pair S + open of packed row k.
 template <int R, int PK>
-__device__ __forceinline__ unsigned p16_score(const uint32_t (&cur)[R / 2], const uint32_t (&prev)[R / 2], int k) {
+__device__ __forceinline__ unsigned p16_score(const uint32_t (&cur)[p16_words(R, PK)],
+                                              const uint32_t (&prev)[p16_words(R, PK)], int k) {
     if constexpr (PK == kP16Pair) {
         return cur[k];
+    } else if constexpr (PK == kP16Int8) {
+        const int kb = R / 2 + k;    // constants after unrolling: one prmt, both bytes sign-extended
+        const unsigned x = k & 3, y = 4 + (kb & 3);
+        return prmt_v(cur[k >> 2], prev[kb >> 2], x | ((8 | x) << 4) | (y << 8) | ((8 | y) << 12));
     } else {
         constexpr int H = R / 2;
         const int kb = H + k;        // bottom half's row k is lane row R/2 + k
@@ -228,7 +257,8 @@ struct P16Consts { unsigned nge2, ngo2, neg2; };
 // LOCAL = false: no zero floor, and cmx is kept by the caller (the largest U only matters in the last row).
 // EDGE: a half whose bits are set in hold keeps its state (its column lies outside the task).
 template <int R, int PK, bool LOCAL = true, bool EDGE = false>
-__device__ __forceinline__ void p16_step(P16Lane<R> &st, const uint32_t (&pw)[R / 2], const uint32_t (&pwp)[R / 2],
+__device__ __forceinline__ void p16_step(P16Lane<R> &st, const uint32_t (&pw)[p16_words(R, PK)],
+                                         const uint32_t (&pwp)[p16_words(R, PK)],
                                          unsigned top, bool lane0, const P16Consts &c, unsigned hold = 0)
 {
     constexpr int H = R / 2;
@@ -420,7 +450,7 @@ __device__ __forceinline__ bool p16_wait3(const int *a, int wa, const int *b, in
         if (va >= wa && vb >= wb && vc >= wc) break;
         if (*abort_flag) return false;
         if (it > limit) { atomicCAS(err, 0, kErrTimeout); return false; }
-        if (it > 64) __nanosleep(20);
+        if (it > 1) __nanosleep(64);
     }
     __threadfence_block();
     return true;
@@ -478,11 +508,11 @@ __device__ __noinline__ int2 p16_locate(const P16Snap<R> &S, const int8_t *prof,
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const int j = S.s0 + k0 + x - 2 * lane;
-            uint32_t pw[H], pwp[H];
+            uint32_t pw[p16_words(R, PK)], pwp[p16_words(R, PK)];
             if constexpr (PK == kP16Pair) {
                 p16_load<R, PK, NL>(prof, g, (cc[x + 1] * (K + 1) + cc[x]) * pstride, pw);
 #pragma unroll
-                for (int y = 0; y < H; ++y) pwp[y] = 0;
+                for (int y = 0; y < p16_words(R, PK); ++y) pwp[y] = 0;
             } else {
                 p16_load<R, PK, NL>(prof, g, cc[x + 1] * pstride, pw);
                 p16_load<R, PK, NL>(prof, g, cc[x] * pstride, pwp);
@@ -565,12 +595,14 @@ constexpr size_t p16_shared_bytes() { return (sizeof(P16Shared<R, W>) + 15) / 16
 // (p16_enter_staircase; the coarse-tile refills of a two-level reconstruction).
 // A separate instantiation, so that the others compile exactly without it.
 // LOCAL = false: the global, semi-global and overlap algorithms (DevScoring::alg).
-template <int R, int W, int MODE, int PK, bool LEFT = false, bool LOCAL = true>
-__global__ void __launch_bounds__((W + 2) * 32, 1)
+// MINB: blocks an SM to compile for.
+template <int R, int W, int MODE, int PK, bool LEFT = false, bool LOCAL = true, int MINB = 1>
+__global__ void __launch_bounds__((W + 2) * 32, MINB)
 wavefront16_kernel(const FillLaunch L)
 {
     static_assert(R % 2 == 0 && R >= 4, "two halves");
-    static_assert(PK == kP16Pair || R == 8 || R == 12 || R == 16, "int16 profile loads");
+    static_assert(PK == kP16Pair || R == 8 || R == 12 || R == 16, "int16 and int8 profile loads");
+    constexpr int NWD = p16_words(R, PK);
     static_assert(MODE == kModeScore || MODE == kModeScoreCk, "score modes only");
     constexpr int H = R / 2;
     constexpr int HC = W * 32 * R;
@@ -618,7 +650,7 @@ wavefront16_kernel(const FillLaunch L)
         const int Wa = min(SW, (T.rows - rbase + 32 * R - 1) / (32 * R));
         const int n_ext = (n + LAG + CH - 1) / CH * CH + 2;
 
-        const int pstride = PK == kP16Pair ? H * NL * 4 : 2 * HC;   // bytes per profile entry
+        const int pstride = PK == kP16Pair ? H * NL * 4 : (PK == kP16Int8 ? NL * p16_slot8(R) : 2 * HC);   // bytes per profile entry
         // query profile of the strip's rows, S(a_r, c) + open, padding rows and columns at kPadScore: a thread takes a
         // row (pair profile: the packed row of a lane) and runs over the residues, so that a row's residue is read
         // once and no index is divided (464 x 503 protein: the fill 69 -> 55 us)
@@ -635,6 +667,12 @@ wavefront16_kernel(const FillLaunch L)
                     for (int cb = 0; cb <= K; ++cb)
                         dst[(ct * (K + 1) + cb) * (NL * H)] = p16_pack(vt, mb && cb < K ? mb[cb] + go : kPadScore);
                 }
+            }
+        } else if constexpr (PK == kP16Int8) {
+            for (int lr = threadIdx.x; lr < SH; lr += blockDim.x) {
+                const int8_t *m = rbase + lr < T.rows ? SC.mat + min((int)T.a[rbase + lr], K - 1) * K : nullptr;
+                int8_t *dst = prof + lr / R * p16_slot8(R) + lr % R;
+                for (int c = 0; c <= K; ++c) dst[c * (NL * p16_slot8(R))] = (int8_t)(m && c < K ? m[c] + go : kPadScore);
             }
         } else {
             int16_t *p16 = reinterpret_cast<int16_t *>(prof);
@@ -724,7 +762,7 @@ wavefront16_kernel(const FillLaunch L)
             };
             const long long spin_limit = L.spin_limit;
             int *const err = L.err;
-            uint32_t pw[H], pwp[H];
+            uint32_t pw[NWD], pwp[NWD];
             int2 off;                           // profile offsets of the next two steps to load
             bool ok = true;
             // the block's first strip runs one chunk left of the task, which keeps the border state: it brings the
@@ -742,7 +780,7 @@ wavefront16_kernel(const FillLaunch L)
                 if (s0 == sbeg) {
                     if constexpr (PK == kP16Pair) {
 #pragma unroll
-                        for (int q = 0; q < H; ++q) pwp[q] = 0;
+                        for (int q = 0; q < NWD; ++q) pwp[q] = 0;
                     } else {
                         p16_load<R, PK, NL>(prof, g, s_poff[(sbeg - 1 - 2 * lane) & (QB - 1)], pwp);
                     }
@@ -809,7 +847,7 @@ wavefront16_kernel(const FillLaunch L)
                     constexpr int NS = decltype(ns)::v;
                     constexpr bool EDGE = decltype(edge)::v != 0;
                     [[maybe_unused]] const int lo = LEFT && T.left ? -(1 << 30) : 0;
-                    auto step = [&](const uint32_t (&w)[H], const uint32_t (&wp)[H], unsigned top, int s) {
+                    auto step = [&](const uint32_t (&w)[NWD], const uint32_t (&wp)[NWD], unsigned top, int s) {
                         p16_step<R, PK, LOCAL, EDGE>(st, w, wp, top, lane0, cst, EDGE ? p16_hold(s - 2 * lane, lo, n) : 0u);
                         if (lane == 31) rc[s - s0] = make_uint2(st.w, st.flast);
                         if constexpr (!LOCAL) {
@@ -831,19 +869,19 @@ wavefront16_kernel(const FillLaunch L)
                                 const int s = s0 + gs + k4 + k2;
                                 // offsets of steps s + 2, s + 3 (slots an even distance apart from lane to lane)
                                 const int2 offn = *reinterpret_cast<const int2 *>(&s_poff[(s + 2 - 2 * lane) & (QB - 1)]);
-                                uint32_t pwn[H];
+                                uint32_t pwn[NWD];
                                 p16_load<R, PK, NL>(prof, g, off.y, pwn);
                                 step(pw, pwp, k2 == 0 ? tops.x : tops.z, s);
                                 p16_load<R, PK, NL>(prof, g, offn.x, PK == kP16Pair ? pw : pwp);
                                 if constexpr (PK == kP16Pair) {
                                     step(pwn, pwp, k2 == 0 ? tops.y : tops.w, s + 1);
                                 } else {
-                                    uint32_t t2[H];
+                                    uint32_t t2[NWD];
 #pragma unroll
-                                    for (int q = 0; q < H; ++q) t2[q] = pwp[q];      // words of step s + 2
+                                    for (int q = 0; q < NWD; ++q) t2[q] = pwp[q];      // words of step s + 2
                                     step(pwn, pw, k2 == 0 ? tops.y : tops.w, s + 1);
 #pragma unroll
-                                    for (int q = 0; q < H; ++q) { pwp[q] = pwn[q]; pw[q] = t2[q]; }
+                                    for (int q = 0; q < NWD; ++q) { pwp[q] = pwn[q]; pw[q] = t2[q]; }
                                 }
                                 off = offn;
                             }

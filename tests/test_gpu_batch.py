@@ -88,6 +88,26 @@ def test_batch_packed_lanes(oracle_mod, monkeypatch, R, Wc):
         c.close()
 
 
+@pytest.mark.parametrize("R,Wc", [(8, 4), (12, 4), (8, 2), (12, 2)])
+def test_batch_int8_profile(oracle_mod, monkeypatch, R, Wc):
+    """The packed fill with the int8 query profile, and a scoring whose S + open leaves int8 (it takes
+    the other profile)."""
+    from paper_2211_10769_gb300 import binding
+    monkeypatch.setenv("SWGB_BATCH", "%d,%d,2" % (R, Wc))
+    c = binding.Context(0)
+    try:
+        sc = _scorings()
+        for scorings in (sc, [(sc[0][0], 130, 2), (sc[1][0], 100, 1)]):
+            pairs = _mixed_pairs(W.BASE_SEED + 12300 + R, 120, hi=4500)
+            plan = binding.Batch(c, pairs, scorings, flags=0)
+            assert all(lb == 16 for _, _, lb, _ in plan.bins())
+            got = plan.run()
+            assert [(h.score, h.a_end, h.b_end) for h in got] == _oracle_hits(oracle_mod, pairs, scorings)
+            plan.close()
+    finally:
+        c.close()
+
+
 def test_batch_device_inputs_and_empty(ctx, oracle_mod):
     import torch
     from paper_2211_10769_gb300 import binding
