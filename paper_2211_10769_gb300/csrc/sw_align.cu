@@ -107,13 +107,15 @@ int finish_alignment(int alg, int score, int64_t ie, int64_t je, const WalkState
     return SW_OK;
 }
 
+// Traceback words of a tile's row group (diagonal words reach R - 1 columns over its edges).
+long long tb_row_words(long long BT, int R) { return BT + R; }
+
 template <typename Word, int R>
 int launch_walk_t(sw_ctx *c, const void *const *table, int I0, int J0, int nI, int nJ, int BT) {
     if ((long long)nI * nJ > kWalkTableMax || BT < kWalkMinBT || BT % R != 0) return SW_EINVAL;
     TileTable<Word> T;
     T.bits = reinterpret_cast<const Word *const *>(table);
-    T.I0 = I0; T.J0 = J0; T.nI = nI; T.nJ = nJ; T.BT = BT; T.R = R;
-    T.win_groups = walk_window_groups(BT, R);
+    T.I0 = I0; T.J0 = J0; T.nI = nI; T.nJ = nJ; T.BT = BT; T.ld = (int32_t)tb_row_words(BT, R);
     const size_t smem = walk_window_bytes<R>(sizeof(Word));
     static int attr_set[64] = {0};                       // per instantiation and device
     if (c->device >= 64 || !attr_set[c->device]) {
@@ -282,7 +284,7 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
     const int J0 = 1 - nI, nJw = nI + nJ - 1;
     if ((long long)nI * nJw > kWalkTableMax) return SW_EINVAL;
     const int ntiles = nI * nJ;
-    const size_t tile_bytes = (size_t)(BT / R) * (size_t)BT * (size_t)tb_word_bytes(R);
+    const size_t tile_bytes = (size_t)(BT / R) * (size_t)tb_row_words(BT, R) * (size_t)tb_word_bytes(R);
     const long long nrowck = std::max<long long>(1, m / BT), ncolck = std::max<long long>(1, n / BT);
 
     FillTask t{};                                   // the forward fill, checkpoints every BT
@@ -337,7 +339,7 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
             u.row0 = (int32_t)r0;
             u.col0 = (int32_t)c0;
             u.tb = static_cast<char *>(c->tb.p) + k * tile_bytes;
-            u.tb_ld = BT;
+            u.tb_ld = tb_row_words(BT, R);
             tickets += u.nstrips;
             tasks.push_back(u);
             table[(size_t)ti * nJw + (size_t)(tj - J0 - ti)] = u.tb;
@@ -552,7 +554,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     RC(c->runs.ensure((size_t)(ie + je + 2) * sizeof(int2)));
     WalkState w{ie, je, 0, 0, 0, -1, 0};
     // the band's traceback bits within the budget (at most three tiles a row)
-    const size_t tile_bytes = (size_t)(BT / tbc.R) * (size_t)BT * (size_t)tb_word_bytes(tbc.R);
+    const size_t tile_bytes = (size_t)(BT / tbc.R) * (size_t)tb_row_words(BT, tbc.R) * (size_t)tb_word_bytes(tbc.R);
     // tile rows per band: two or three tiles a row, about one tile per SM (measured at 200 kbp: a
     // band as deep as the SM count, 228 tiles in one round, took 1.18 ms against 1.00 ms for two
     // rounds of one tile per SM)
@@ -665,7 +667,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
                 u.row0 = (int32_t)r0;
                 u.col0 = (int32_t)c0;
                 u.tb = tbp + k * tile_bytes;
-                u.tb_ld = BT;
+                u.tb_ld = tb_row_words(BT, R);
                 bd.tickets += u.nstrips;
                 bd.tasks.push_back(u);
                 bd.table[(size_t)(ti - I0) * nJ + (tj - (kd + I0) - (ti - I0))] = u.tb;

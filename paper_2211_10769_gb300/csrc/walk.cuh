@@ -10,25 +10,28 @@
 //   state E: emit I, go left; back to H if the E-opened bit is set;
 //   state F: emit D, go up; back to H if the F-opened bit is set.
 //
-// The walk is a chain of dependent lookups, so it reads them from shared
-// memory: a window of the decision words that follows the diagonal through
-// the walk's cell (kWinRows rows above it, kWinCols columns per row group,
-// kWinRight of them right of the diagonal).  Warp 0 walks inside one window
-// while warps 1..8 stage the next one in a second buffer: the same band
-// continued above the first, which is where a walk that follows the
-// diagonal leaves it.  Where the walk left the window elsewhere (a long
-// gap drifts it off the diagonal), the next window is staged at its cell
-// while it waits.
-//
-// One warp walks.  Runs are taken 64 cells at a time: in state H the lanes
-// read the cells of the diagonal ahead and the walk jumps over the leading
-// cells whose source is "diagonal"; in state E (F) they read the cells to
-// the left (above) and the walk jumps to the first one whose opened bit is
-// set.  Only the run-ending cell is handled one at a time.
+// The bits come in words of R nibbles along the diagonal (wavefront.cuh): word
+// q of row group g holds row g R + x's nibble of column q + x.  The walk is one
+// warp's chain of dependent lookups, so what bounds it is the number of
+// lookups and the latency of each:
+//   * it reads words from shared memory: a window of row groups by diagonals
+//     around the walk's (kWinRows rows, kWinDiags diagonals; word q of group g lies
+//     on diagonal q - g R, so the window is a rectangle).  Warp 0 walks while the
+//     other warps stage the same diagonals of the groups above into a second
+//     buffer;
+//   * in state H lane l reads the word of the walk's diagonal l groups up: 32 R
+//     cells at once, in which one vote and one shuffle find the cell that ends the
+//     run and its whole nibble, which settles a gap of one cell.  In states E and F
+//     the lanes read the next 32 cells of the row or column.
+// (Before, the words were columns of a row group: a lane read one or two cells, 64
+// a turn at about 780 clocks, and windows met at most 2 x 2 tiles.  200 kbp:
+// 1.65 ms, 100 kbp global with unrelated ends 2.9 ms, 3 kbp on 256-row tiles 129 us.)
 // The walk stops when it reaches a zero cell or the border (done = 1), or
 // when its next cell lies in a tile that was not recomputed this round
 // (done = 0, the host computes that tile next).
 #pragma once
+#include <type_traits>
+
 #include "sw_device.cuh"
 
 namespace swgb {
@@ -45,52 +48,33 @@ struct WalkState {
 // The tiles recomputed in one round: for each tile row I in [I0, I0 + nI), a
 // window of nJ tile columns that follows the diagonal, [J0 + (I - I0),
 // J0 + (I - I0) + nJ); a null entry means the tile was not computed.  Words of
-// a tile: [local row / R][local column], ld = BT.
+// a tile: [local row / R][ld], word q (local) at index q + R - 1.
 template <typename Word>
 struct TileTable {
     const Word *const *bits;   // nI * nJ entries
     int32_t I0, J0, nI, nJ;
     int32_t BT;                // tile side
-    int32_t R;                 // rows per word
-    int32_t win_groups;        // row groups of a window (walk_window_groups)
+    int32_t ld;                // words per row group
 };
 
-constexpr int kLook = 2;              // groups of 32 cells each lane reads ahead per iteration
 constexpr int kWalkTableMax = 4096;   // tile-table entries cached in shared memory
 constexpr int kWinRows = 768;         // rows of a window (a multiple of every R)
-constexpr int kWinCols = 128;         // columns a window keeps per row group
-constexpr int kWinRight = 64;         // ... of them right of the diagonal through the walk's cell
-constexpr int kStageThreads = 256;    // threads staging a window (warps 1..8)
+constexpr int kWinDiags = 128;        // diagonals of a window, the walk's in the middle
+constexpr int kWinMargin = 16;        // diagonals a staged window must leave either side of the walk's
+constexpr int kStageThreads = 512;    // threads staging a window (warps 1..16)
 constexpr int kWalkThreads = 32 + kStageThreads;   // warp 0 walks
-constexpr int kStage = 16;            // window words a thread loads at once
-constexpr int kWinMargin = 16;        // columns a staged window must leave either side of the walk's cell
+constexpr int kStage = 8;             // window words a thread loads at once
 constexpr int kWalkMinBT = 256;       // tiles at least this side
 
-// Row groups of a window on tiles of side BT: its rows, and its band of
-// columns ((groups - 1) R + kWinCols wide), each within BT, so that a window
-// meets 2 x 2 tiles at most (768 rows on tiles of 1,024 and more).
-__host__ __device__ constexpr int walk_min3(int a, int b, int c) { return a < b ? (a < c ? a : c) : (b < c ? b : c); }
-__host__ __device__ constexpr int walk_window_groups(int BT, int R) {
-    return walk_min3(kWinRows / R, BT / R, (BT - kWinCols) / R + 1);
-}
+__device__ __forceinline__ int leading_zeros(unsigned v) { return __clz((int)v); }
+__device__ __forceinline__ int leading_zeros(unsigned long long v) { return __clzll((long long)v); }
 
 template <int R>
-constexpr size_t walk_window_bytes(size_t word_bytes) { return 2 * (size_t)(kWinRows / R) * kWinCols * word_bytes; }
+constexpr size_t walk_window_bytes(size_t word_bytes) { return 2 * (size_t)(kWinRows / R) * kWinDiags * word_bytes; }
 
-// Where a window lies (all coordinates 0-based).  Row groups g = 0 .. ng-1
-// hold rows r_lo + g*R .. r_lo + g*R + R - 1 (r_lo a multiple of R); group
-// g keeps columns [clo(g), clo(g) + kWinCols) with clo(g) = chi - (ng-1-g)*R,
-// so the kept band slides along the diagonal.  The window meets at most two
-// tile rows (the second from window row lrb on) and two tile columns (the
-// second from column cb on); tile (x, y) starts at row rbase[x], column
-// cbase[y], its words are tp[2x + y] and bit 2x + y of pres says whether it
-// was recomputed.
+// Row groups [g_lo, g_lo + ng), diagonals (column - row, 0-based) [dlo, dlo + kWinDiags).
 struct WalkWindow {
-    int r_lo, ng, chi;
-    int lrb, cb;
-    int rbase[2], cbase[2];
-    int pres;
-    const void *tp[4];
+    int g_lo, ng, dlo;
 };
 
 template <typename Word>
@@ -99,103 +83,60 @@ __device__ __forceinline__ const Word *tile_ptr(const TileTable<Word> &T, const 
     return (ti >= 0 && tj >= 0 && ti < T.nI && tj < T.nJ) ? tiles[ti * T.nJ + tj] : nullptr;
 }
 
-// The window whose last row group is ghi (>= 0) and keeps columns from chi
-// on in that group.
-template <typename Word, int R>
-__device__ WalkWindow make_window_g(const TileTable<Word> &T, const Word *const *tiles, int ghi, int chi) {
-    const int RG = T.win_groups;
-    constexpr int kNone = 0x7fffffff;
-    WalkWindow m;
+// The window whose last row group is ghi.
+template <int R>
+__device__ __forceinline__ WalkWindow make_window(int ghi, int dlo) {
+    constexpr int RG = kWinRows / R;
     const int glo = max(0, ghi - (RG - 1));
-    m.ng = ghi - glo + 1;
-    m.r_lo = glo * R;
-    m.chi = chi;
-    const int BT = T.BT;
-    const int ia = m.r_lo / BT, ib = (ghi * R + R - 1) / BT;
-    m.lrb = ib > ia ? ib * BT - m.r_lo : kNone;
-    const int cmin = max(0, m.chi - (m.ng - 1) * R), cmax = max(0, m.chi + kWinCols - 1);
-    const int ja = cmin / BT, jb = cmax / BT;
-    m.cb = jb > ja ? jb * BT : kNone;
-    m.rbase[0] = ia * BT; m.rbase[1] = ib * BT;
-    m.cbase[0] = ja * BT; m.cbase[1] = jb * BT;
-    m.pres = 0;
-    for (int x = 0; x < 2; ++x)
-        for (int y = 0; y < 2; ++y) {
-            const Word *b = tile_ptr(T, tiles, x ? ib : ia, y ? jb : ja);
-            m.tp[2 * x + y] = b;
-            if (b) m.pres |= 1 << (2 * x + y);
-        }
-    return m;
+    return WalkWindow{glo, ghi - glo + 1, dlo};
 }
 
-// The window whose last row group holds the walk's cell (r0, c0), with that
-// cell kWinRight columns left of the group's last kept column.
-template <typename Word, int R>
-__device__ WalkWindow make_window(const TileTable<Word> &T, const Word *const *tiles, int r0, int c0) {
-    r0 = max(r0, 0);
-    c0 = max(c0, 0);
-    return make_window_g<Word, R>(T, tiles, r0 / R, c0 - (kWinCols - 1 - kWinRight));
-}
-
-// Whether window m holds the cell (r0, c0) at least kWinMargin columns from
-// either side of its band.
+// Whether window m holds the cell (r0, c0) at least kWinMargin diagonals from either side.
 template <int R>
 __device__ __forceinline__ bool window_holds(const WalkWindow &m, int r0, int c0) {
-    const int rr = r0 - m.r_lo;
-    if (m.ng <= 0 || rr < 0 || rr >= m.ng * R) return false;
-    const int k = c0 - m.chi + (m.ng - 1 - rr / R) * R;
-    return k >= kWinMargin && k < kWinCols - kWinMargin;
+    const int g = r0 / R - m.g_lo, d = c0 - r0 - m.dlo;
+    return r0 >= 0 && g >= 0 && g < m.ng && d >= kWinMargin && d < kWinDiags - kWinMargin;
 }
 
-// Stage window m into win: staging thread t (of kStageThreads) takes column
-// k = t % kWinCols of every kStageThreads / kWinCols-th row group, kStage
-// independent loads in flight at a time.
+// Stage window m into win: staging thread t (of kStageThreads) takes diagonal
+// t % kWinDiags of every kStageThreads / kWinDiags-th row group, kStage
+// independent words in flight at a time.  A word that reaches over a tile's right
+// edge is the union of the two tiles' words.  Missing tiles and columns left of
+// the matrix read as 0.
 template <typename Word, int R>
-__device__ __forceinline__ void stage_window(const TileTable<Word> &T, const WalkWindow &m, Word *win, int t) {
-    constexpr int kGroupsPerPass = kStageThreads / kWinCols;
-    static_assert(kStageThreads % kWinCols == 0, "whole row groups per pass");
-    const int k = t % kWinCols;
-    for (int g0 = t / kWinCols; g0 < m.ng; g0 += kStage * kGroupsPerPass) {
-        Word v[kStage];
+__device__ __forceinline__ void stage_window(const TileTable<Word> &T, const Word *const *tiles, const WalkWindow &m,
+                                             Word *win, int t) {
+    constexpr int kStep = kStageThreads / kWinDiags;       // row groups a thread advances
+    static_assert(kStageThreads % kWinDiags == 0, "whole row groups per pass");
+    const int k = t % kWinDiags, BT = T.BT;
+    int g = t / kWinDiags;
+    // the thread's tile and its place in it, advanced with the groups (BT is a multiple of R)
+    const int r = (m.g_lo + g) * R, q = m.dlo + k + r;
+    int I = r / BT, lr = r - I * BT;
+    int J = q >= 0 ? q / BT : -((-q + BT - 1) / BT), lq = q - J * BT;
+    while (g < m.ng) {
+        Word v[kStage], x[kStage];
 #pragma unroll
         for (int u = 0; u < kStage; ++u) {
-            const int g = g0 + u * kGroupsPerPass;
-            const int c = m.chi - (m.ng - 1 - g) * R + k;
-            const int x = g * R >= m.lrb, y = c >= m.cb;
-            const Word *b = static_cast<const Word *>(x ? (y ? m.tp[3] : m.tp[2]) : (y ? m.tp[1] : m.tp[0]));
-            const int rb = x ? m.rbase[1] : m.rbase[0], cbs = y ? m.cbase[1] : m.cbase[0];
-            v[u] = 0;
-            if (g < m.ng && c >= 0 && b)              // a row group never straddles tiles (BT % R == 0)
-                v[u] = __ldcg(b + (size_t)((m.r_lo + g * R - rb) / R) * (size_t)T.BT + (size_t)(c - cbs));
+            v[u] = 0; x[u] = 0;
+            if (g + u * kStep < m.ng) {
+                const size_t row = (size_t)(lr / R) * (size_t)T.ld;
+                const Word *a = tile_ptr(T, tiles, I, J);
+                if (a) v[u] = __ldcg(a + row + lq + R - 1);
+                if (lq > BT - R) {
+                    const Word *b = tile_ptr(T, tiles, I, J + 1);
+                    if (b) x[u] = __ldcg(b + row + lq - BT + R - 1);
+                }
+            }
+            lr += kStep * R; lq += kStep * R;
+            while (lr >= BT) { lr -= BT; ++I; }
+            while (lq >= BT) { lq -= BT; ++J; }
         }
 #pragma unroll
-        for (int u = 0; u < kStage; ++u) {
-            const int g = g0 + u * kGroupsPerPass;
-            if (g < m.ng) win[g * kWinCols + k] = v[u];
-        }
+        for (int u = 0; u < kStage; ++u)
+            if (g + u * kStep < m.ng) win[(g + u * kStep) * kWinDiags + k] = v[u] | x[u];
+        g += kStage * kStep;
     }
-}
-
-// Decision nibble of the cell p steps back along (di, dj) from the walk's
-// cell (r0, c0) = (i - 1, j - 1): -2 at the matrix border, -3 outside the
-// window, -1 in a tile that was not recomputed.  lr0 = r0 - m.r_lo.  Without
-// branches: early returns made the lanes of the walker's warp diverge on its
-// dependency chain (2.01 -> 1.53 ms a 200 kbp alignment without them).
-template <typename Word, int R>
-__device__ __forceinline__ int window_nibble(const WalkWindow &m, const Word *win, int lr0, int c0, int di, int dj, int p) {
-    // every lane loads a word, clamped into the window (rr < ng R always: the walk starts
-    // inside the window and only moves up), and the special cases are selected after
-    const int rr = lr0 - di * p, c = c0 - dj * p;
-    const int rrc = max(rr, 0);
-    const int g = (int)((unsigned)rrc / R);
-    const int k = c - m.chi + (m.ng - 1 - g) * R;
-    const bool border = rr + m.r_lo < 0 || c < 0;
-    const bool outside = rr < 0 || (unsigned)k >= (unsigned)kWinCols;
-    const bool missing = !((m.pres >> (2 * (rrc >= m.lrb) + (c >= m.cb))) & 1);
-    const int kc = min(max(k, 0), kWinCols - 1);
-    const Word w = win[g * kWinCols + kc];
-    const int nib = (int)((unsigned long long)w >> (4 * (rrc - g * R))) & 15;
-    return border ? -2 : (outside ? -3 : (missing ? -1 : nib));
 }
 
 // The walk's start taken from the end cell reduced on the device (res: score,
@@ -216,7 +157,10 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
                                                           long long max_iters)
 {
     static_assert(kWinRows % R == 0, "a window holds whole row groups");
-    constexpr int kWinWords = (kWinRows / R) * kWinCols;
+    constexpr int kWinWords = (kWinRows / R) * kWinDiags;
+    using Wide = typename std::conditional<(R > 8), unsigned long long, unsigned>::type;   // a word, registers whole
+    constexpr int kTop = 8 * (int)sizeof(Wide) - 4;        // shift of a Wide's top nibble
+    constexpr Wide kOnes = (Wide)(0x1111111111111111ull >> (64 - 4 * R));
     extern __shared__ __align__(16) unsigned char walk_smem[];
     Word *s_buf = reinterpret_cast<Word *>(walk_smem);   // two windows
     __shared__ const Word *s_tiles[kWalkTableMax];
@@ -226,46 +170,41 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
     if (blockIdx.x != 0) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ntab = T.nI * T.nJ;
-    if (ntab > kWalkTableMax || T.BT < kWalkMinBT || T.win_groups < 1 || T.win_groups > kWinRows / R ||
-        T.win_groups != walk_window_groups(T.BT, R)) {   // the host keeps bands, tiles and windows within these
+    if (ntab > kWalkTableMax || T.BT < kWalkMinBT || T.BT % R != 0 || T.ld < T.BT + R - 1) {   // the host keeps within these
         if (threadIdx.x == 0) st->done = 2;
         return;
     }
     for (int k = threadIdx.x; k < ntab; k += blockDim.x) s_tiles[k] = T.bits[k];
-    __syncthreads();
     if (threadIdx.x == 0) {
         s_w = *st;
         s_stop = s_w.done != 0;
-        s_mw[0] = make_window<Word, R>(T, s_tiles, s_w.i - 1, s_w.j - 1);
+        const int r0 = max(s_w.i - 1, 0), c0 = max(s_w.j - 1, 0);
+        s_mw[0] = make_window<R>(r0 / R, c0 - r0 - kWinDiags / 2);
     }
     __syncthreads();
-    if (warp > 0 && !s_stop) stage_window<Word, R>(T, s_mw[0], s_buf, threadIdx.x - 32);
+    if (warp > 0 && !s_stop) stage_window<Word, R>(T, s_tiles, s_mw[0], s_buf, threadIdx.x - 32);
     __syncthreads();
-    long long it = 0;                                    // walk iterations (warp 0)
+    long long it = 0;                                    // walk turns (warp 0)
     int cur = 0;
     while (!s_stop) {
         const int nxt = cur ^ 1;
-        if (threadIdx.x == 0) {
-            // the band continued above the current window (none above the first row)
-            const WalkWindow &m = s_mw[cur];
-            WalkWindow p{};
-            if (m.r_lo > 0) p = make_window_g<Word, R>(T, s_tiles, m.r_lo / R - 1, m.chi - m.ng * R);
-            else p.ng = 0;
-            s_mw[nxt] = p;
-        }
-        __syncthreads();
+        const WalkWindow m = s_mw[cur];
+        // the same diagonals above the current window (none above the first row)
+        const WalkWindow up = m.g_lo > 0 ? make_window<R>(m.g_lo - 1, m.dlo) : WalkWindow{0, 0, 0};
         if (warp > 0) {
-            if (s_mw[nxt].ng > 0) stage_window<Word, R>(T, s_mw[nxt], s_buf + nxt * kWinWords, threadIdx.x - 32);
+            if (threadIdx.x == 32) s_mw[nxt] = up;
+            if (up.ng > 0) stage_window<Word, R>(T, s_tiles, up, s_buf + nxt * kWinWords, threadIdx.x - 32);
         } else {
             const Word *s_win = s_buf + cur * kWinWords;
-            const WalkWindow m = s_mw[cur];
             WalkState w = s_w;
+            int nr = 0;                                  // run records written in this window
+            int2 *out = runs + w.nruns;
             // every lane keeps the same (uniform) run state; lane 0 stores the records
             auto emit = [&](int op, int cnt) {
                 if (op == w.cur_op) { w.cur_len += cnt; return; }
                 if (w.cur_len > 0) {
-                    if (lane == 0) runs[w.nruns] = make_int2(w.cur_op, w.cur_len);
-                    ++w.nruns;
+                    if (lane == 0) out[nr] = make_int2(w.cur_op, w.cur_len);
+                    ++nr;
                 }
                 w.cur_op = op;
                 w.cur_len = cnt;
@@ -273,64 +212,77 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
             bool stop = false;                           // back to the host (or finished)
             while (true) {                               // (w.done is 0 here: every exit that sets it breaks)
                 if (++it >= max_iters) { w.done = 2; stop = true; break; }
-                if (w.state == 0 && (w.i == 0 || w.j == 0)) { w.done = 1; stop = true; break; }
-                // the next 32 * kLook cells of the run: the diagonal in state H, the row to
-                // the left in state E, the column above in state F
-                const int di = w.state == 1 ? 0 : 1, dj = w.state == 2 ? 0 : 1;
-                const int mask = w.state == 0 ? 3 : (w.state == 1 ? 4 : 8);
-                const int lr0 = w.i - 1 - m.r_lo, c0 = w.j - 1;
-                int nb[kLook];
-#pragma unroll
-                for (int q = 0; q < kLook; ++q)
-                    nb[q] = window_nibble<Word, R>(m, s_win, lr0, c0, di, dj, q * 32 + lane);
-                // first cell that ends the run: in H a source other than "diagonal", in E / F
-                // the opened bit; the window's edge, a missing tile or the border ends it too.
-                // Both votes at once, one 64-bit scan, one shuffle: no loop, no divergence.
-                static_assert(kLook == 2, "the scan below reads two groups of 32 cells");
-                const bool end0 = nb[0] < 0 || (w.state == 0 ? (nb[0] & 3) != 1 : (nb[0] & mask) != 0);
-                const bool end1 = nb[1] < 0 || (w.state == 0 ? (nb[1] & 3) != 1 : (nb[1] & mask) != 0);
-                const unsigned long long ends = (unsigned long long)__ballot_sync(kFull, end0) |
-                                                ((unsigned long long)__ballot_sync(kFull, end1) << 32);
-                const int pos = ends ? __ffsll((long long)ends) - 1 : 64;
-                const int nbk = __shfl_sync(kFull, pos >= 32 ? nb[1] : nb[0], pos & 31);
-                const int op = w.state;                  // M, I or D runs of states H, E, F
-                if (pos == 64) {                         // the whole look-ahead continues the run
-                    emit(op, pos);
-                    w.i -= di * pos;
-                    w.j -= dj * pos;
-                    continue;
-                }
-                if (nbk == -3) {                         // the window's edge: take what was read
-                    if (pos > 0) emit(op, pos);
-                    w.i -= di * pos;
-                    w.j -= dj * pos;
-                    break;                               // the next window starts here
-                }
+                const int r = w.i - 1, c = w.j - 1;
+                const int g0 = (int)((unsigned)max(r, 0) / R), x0 = r - g0 * R, gl = g0 - m.g_lo, dd = c - r - m.dlo;
                 if (w.state == 0) {
+                    if (w.i == 0 || w.j == 0) { w.done = 1; stop = true; break; }
+                    if (dd < 0 || dd >= kWinDiags) break;   // a gap ran out of the window
+                    // lane l: the walk's diagonal in the l-th group up, from row x0 (lane 0) or the group's last row
+                    const int g = gl - lane, top = lane == 0 ? x0 : R - 1;
+                    const Word wd = s_win[max(g, 0) * kWinDiags + dd];
+                    // a nibble is nonzero here where the H source is not "diagonal"; the top one first
+                    const Wide bad = (((Wide)wd ^ kOnes) & (3 * kOnes)) << (kTop - 4 * top);
+                    const bool in = g >= 0;
+                    const int cnt = bad ? leading_zeros(bad) >> 2 : top + 1;   // leading cells that go on
+                    const bool end = !in || bad != 0;
+                    const unsigned ends = __ballot_sync(kFull, end);
+                    const int before = lane == 0 ? 0 : x0 + 1 + (lane - 1) * R;
+                    const int nib = in ? (int)((Wide)wd >> (4 * max(top - cnt, 0))) & 15 : 16;
+                    const int lim = min(r, c) + 1;       // cells up to the border
+                    if (ends == 0) {                     // all 32 groups go on
+                        const int pos = min(x0 + 1 + 31 * R, lim);
+                        emit(0, pos);
+                        w.i -= pos;
+                        w.j -= pos;
+                        continue;
+                    }
+                    const int val = __shfl_sync(kFull, (before + (in ? cnt : 0)) | (nib << 16), __ffs(ends) - 1);
+                    const int pos = min(val & 0xffff, lim), nbk = val >> 16;
                     if (pos > 0) emit(0, pos);
                     w.i -= pos;
                     w.j -= pos;
-                    if (nbk == -2) { w.done = 1; stop = true; break; }   // reached the border
-                    if (nbk == -1) { stop = true; break; }              // tile not computed: ask the host
+                    if (pos == lim) continue;            // the border
+                    if (nbk == 16) break;                // the window's first row: the next window starts here
                     const int src = nbk & 3;
-                    if (src == 0) { w.done = 1; stop = true; break; }
-                    w.state = (src == 2) ? 1 : 2;
-                } else {
-                    if (nbk == -1) {                     // missing tile: consume what was read
-                        if (pos > 0) emit(op, pos);
-                        w.i -= di * pos;
-                        w.j -= dj * pos;
+                    if (src == 0) {                      // a zero cell, or a tile that was not recomputed
+                        if (tile_ptr(T, s_tiles, (r - pos) / T.BT, (c - pos) / T.BT)) w.done = 1;
                         stop = true;
                         break;
                     }
-                    if (nbk == -2) { w.done = 2; stop = true; break; }  // a gap cannot reach the border
-                    emit(op, pos + 1);                   // the extensions and the opening cell
-                    w.i -= di * (pos + 1);
-                    w.j -= dj * (pos + 1);
-                    w.state = 0;
+                    w.state = src == 2 ? 1 : 2;
+                    if (nbk & (src == 2 ? 4 : 8)) {      // opened here: a gap of one cell
+                        emit(w.state, 1);
+                        if (src == 2) --w.j; else --w.i;
+                        w.state = 0;
+                    }
+                } else {
+                    // lane p: the cell p columns to the left (E) or p rows up (F); a cell of the path in a gap state
+                    // has a nonzero nibble (its H source is not "zero"), so 0 is a tile that was not recomputed
+                    const bool inE = w.state == 1;
+                    const int rp = inE ? r : r - lane, d = inE ? dd - lane : dd + lane;
+                    const int gp = (int)((unsigned)max(rp, 0) / R), gw = gp - m.g_lo;
+                    const bool out_m = rp < 0 || (inE && c - lane < 0);
+                    const bool in = gw >= 0 && d >= 0 && d < kWinDiags;
+                    const Word wd = s_win[max(gw, 0) * kWinDiags + min(max(d, 0), kWinDiags - 1)];
+                    int nib = (int)((Wide)wd >> (4 * max(rp - gp * R, 0))) & 15;
+                    nib = out_m ? 17 : (in ? nib : 16);
+                    const bool end = nib >= 16 || nib == 0 || (nib & (inE ? 4 : 8)) != 0;
+                    const unsigned ends = __ballot_sync(kFull, end);
+                    const int pos = ends ? __ffs(ends) - 1 : 32;
+                    const int nbk = __shfl_sync(kFull, nib, pos & 31);
+                    const bool opened = ends != 0 && nbk != 0 && nbk < 16;
+                    const int step = pos + (opened ? 1 : 0);   // the extensions, and the opening cell
+                    if (ends != 0 && nbk == 17) { w.done = 2; stop = true; break; }   // a gap cannot reach the border
+                    if (step > 0) emit(w.state, step);
+                    if (inE) w.j -= step; else w.i -= step;
+                    if (opened) { w.state = 0; continue; }
+                    if (ends == 0) continue;
+                    if (nbk == 0) stop = true;           // missing tile: ask the host
+                    break;                               // (nbk 16: the window's edge)
                 }
             }
             if (lane == 0) {
+                w.nruns += nr;
                 s_w = w;
                 s_stop = stop;
             }
@@ -339,12 +291,13 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
         if (s_stop) break;
         // the staged window serves if it holds the walk's cell with room to both sides
         if (threadIdx.x == 0) {
-            s_redo = !window_holds<R>(s_mw[nxt], s_w.i - 1, s_w.j - 1);
-            if (s_redo) s_mw[nxt] = make_window<Word, R>(T, s_tiles, s_w.i - 1, s_w.j - 1);
+            const int r0 = max(s_w.i - 1, 0), c0 = max(s_w.j - 1, 0);
+            s_redo = !window_holds<R>(s_mw[nxt], r0, c0);
+            if (s_redo) s_mw[nxt] = make_window<R>(r0 / R, c0 - r0 - kWinDiags / 2);
         }
         __syncthreads();
         if (s_redo) {
-            if (warp > 0) stage_window<Word, R>(T, s_mw[nxt], s_buf + nxt * kWinWords, threadIdx.x - 32);
+            if (warp > 0) stage_window<Word, R>(T, s_tiles, s_mw[nxt], s_buf + nxt * kWinWords, threadIdx.x - 32);
             __syncthreads();
         }
         cur = nxt;

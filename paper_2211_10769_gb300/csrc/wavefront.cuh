@@ -43,8 +43,12 @@
 // column c - l; a task entered from such a column first brings every lane to
 // column c, see FillTask::left).
 // Traceback (TB = true) writes, for every cell, four decision bits
-// {H source: 0 zero, 1 diagonal, 2 E, 3 F; E opened; F opened} packed R
-// nibbles per word, for the walk.
+// {H source: 0 zero, 1 diagonal, 2 E, 3 F; E opened; F opened} for the walk,
+// packed R nibbles per word along the diagonal: word D of a lane's row group
+// holds row x's nibble of column D + x, so that the walk takes R cells of a
+// diagonal run from one word.  A lane finishes word j - (R - 1) at column j and
+// keeps R - 1 partial ones; word D is stored at index D + R - 1, and a word that
+// reaches over the task's left or right edge holds its own columns only.
 #pragma once
 #include "sw_device.cuh"
 
@@ -77,7 +81,7 @@ struct FillTask {
     int32_t row0;          // row index (0-based, in the whole pair) of the task's first row
     int32_t col0;          // column index (0-based, in the whole pair) of the task's first column
     int64_t colck_ld;
-    void *tb;              // traceback words, TB mode: [row group][tb_ld]
+    void *tb;              // traceback words, TB mode: [row group][tb_ld], tb_ld >= ncols + R - 1
     int64_t tb_ld;
     int32_t strip_warps;   // compute warps per strip (rows per strip = strip_warps * 32 * R);
                            // 0 = all W warps of the block
@@ -230,6 +234,7 @@ constexpr int kIOB = 64;      // columns per I/O batch
 template <int R>
 struct LaneState {
     int U[R], E[R];
+    typename TbWord<R>::T pend[R];   // traceback fill: pend[x] holds rows 0 .. x - 1 of word j - x + 1 after column j
     int ub, fb, udiag0;
     int bk, bj;
     int rlast;        // the other algorithms: the lane's row holding the task's last row, or -1
@@ -256,7 +261,8 @@ __device__ __forceinline__ int row_key(int u, int r) { return u * kKeyRows + (R 
 // One column of one lane's R rows (Gotoh recurrence, paper Section 2.1.2),
 // entered with uup / fup = H - open and F of the row above at this column;
 // st.udiag0 holds H - open of the row above at the previous column.  TB
-// collects the four decision bits of every cell into word.
+// adds the four decision bits of every cell to its diagonal's word; word receives
+// the one that this column finishes.
 // LOCAL: the Smith-Waterman zero floor; without it (the global, semi-global and
 // overlap algorithms) H has no floor and no cell has the "zero" source.
 template <int R, int PK, bool TB, bool LOCAL = true>
@@ -282,6 +288,11 @@ __device__ __forceinline__ void column_update(LaneState<R> &st, const uint32_t (
             const unsigned src = (LOCAL && h == 0) ? 0u : (h == diag ? 1u : (h == e ? 2u : 3u));
             const unsigned nib = src | (e == uold ? 4u : 0u) | (f == fopen_ref ? 8u : 0u);
             word |= (typename TbWord<R>::T)nib << (4 * r);
+            if (r + 1 < R) {                               // on to the diagonal that meets the next row at this column
+                const typename TbWord<R>::T next = st.pend[r + 1];
+                st.pend[r + 1] = word;
+                word = next;
+            }
             fopen_ref = u;
         }
         st.E[r] = e;
@@ -574,6 +585,9 @@ wavefront_kernel(const FillLaunch L)
             int next_ck = (MODE == kModeScoreCk && T.colck && T.colck_every > 0) ? T.colck_every - 1 : 0x7fffffff;
             typename TbWord<R>::T *tbw = nullptr;
             if constexpr (MODE == kModeTb)
+#pragma unroll
+                for (int r = 0; r < R; ++r) st.pend[r] = 0;
+            if constexpr (MODE == kModeTb)
                 tbw = reinterpret_cast<typename TbWord<R>::T *>(T.tb) + (size_t)(grow / R) * (size_t)T.tb_ld;
             int2 *rin = ring[warp];
             int2 *rout = ring[warp + 1];
@@ -685,6 +699,10 @@ wavefront_kernel(const FillLaunch L)
                 }
             }
 
+            if constexpr (MODE == kModeTb) {               // the words that reach over the right edge
+#pragma unroll
+                for (int x = 1; x < R; ++x) tbw[n + R - 1 - x] = st.pend[x];
+            }
             if constexpr (MODE != kModeTb) {
                 static_assert(kKeyRows == 16, "key decode assumes 4 row bits");
                 int cs, cj, ci;

@@ -521,3 +521,33 @@ def test_packed_base_moves(packed_ctx, oracle_mod):
     S, o, e = W.protein_scoring().matrix, 10, 1
     a = W.random_protein(4200, W.BASE_SEED + 8610)
     _align_case(packed_ctx, oracle_mod, a, W.mutate(a, 20, W.BASE_SEED + 8611), S, o, e)
+
+
+@pytest.mark.parametrize("tb", ["4,4", "8,4", "12,4", "16,4"])
+def test_walk_windows(oracle_mod, monkeypatch, tb):
+    """The walk's windows, at every traceback tile height: gap runs that end just inside, at and
+    just outside the staged diagonals and the 32 cells of one turn, to both sides of the
+    diagonal, and diagonal runs up to the matrix's first row and column."""
+    from paper_2211_10769_gb300 import binding
+    monkeypatch.setenv("SWGB_TB", tb)
+    c = binding.Context(0)
+    try:
+        S = np.full((4, 4), -4, np.int8)
+        np.fill_diagonal(S, 5)
+        x = W.uniform_dna(4200, W.BASE_SEED + 9870)
+        parts_a, parts_b, at = [], [], 0
+        for k, gap in enumerate([1, 31, 32, 33, 47, 48, 49, 63, 64, 65, 127, 129]):
+            at += 97 + 5 * k                               # a stretch of matches, then letters of one side only
+            parts_a.append(x[at - 97 - 5 * k:at + (gap if k % 2 else 0)])
+            parts_b.append(x[at - 97 - 5 * k:at + (0 if k % 2 else gap)])
+            at += gap
+        a = np.concatenate(parts_a + [x[at:]])
+        b = np.concatenate(parts_b + [x[at:]])
+        for p, q in ((a, b), (b, a), (a[40:], b), (a, b[3:])):
+            for alg in (0, 1, 2, 3):
+                want = oracle_mod.align_alg(p, q, S, 9, 0, alg)
+                got = c.align(p, q, S, 9, 0, alg)
+                assert (got.score, got.a_begin, got.a_end, got.b_begin, got.b_end, got.cigar) == \
+                    (want.score, want.a_begin, want.a_end, want.b_begin, want.b_end, want.cigar)
+    finally:
+        c.close()
