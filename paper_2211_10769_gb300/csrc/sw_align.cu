@@ -27,6 +27,7 @@
 #include "aux_kernels.cuh"
 
 #include <algorithm>
+#include <charconv>
 #include <numeric>
 #include <cstdlib>
 #include <cstring>
@@ -41,7 +42,7 @@ using namespace swgb;
 namespace {
 
 constexpr int kMinBandDepth = 16;         // tile rows per band at least
-constexpr long long kWalkMaxIters = 1LL << 26;
+constexpr int kWalkMaxIters = 1 << 26;
 
 int empty_alignment(sw_alignment *out) {
     char *s = static_cast<char *>(std::malloc(1));
@@ -94,11 +95,14 @@ int finish_alignment(int alg, int score, int64_t ie, int64_t je, const WalkState
     cig.reserve(cig.size() + (size_t)w.nruns * 6);
     static const char opc[3] = {'M', 'I', 'D'};
     char buf[24];
-    for (long long k = w.nruns - 1; k >= 0; --k) {
-        const int2 r = runs[(size_t)k];
-        if (r.x < 0 || r.x > 2) return SW_ECUDA;
-        std::snprintf(buf, sizeof(buf), "%d%c", r.y, opc[r.x]);
-        cig += buf;
+    for (long long k = w.nruns - 1; k >= 0;) {
+        const int op = runs[(size_t)k].x;
+        if (op < 0 || op > 2) return SW_ECUDA;
+        long long cells = 0;                               // one run may come in several records
+        for (; k >= 0 && runs[(size_t)k].x == op; --k) cells += runs[(size_t)k].y;
+        char *e = std::to_chars(buf, buf + sizeof(buf) - 1, cells).ptr;
+        *e++ = opc[op];
+        cig.append(buf, e);
     }
     char *s = static_cast<char *>(std::malloc(cig.size() + 1));
     if (!s) return SW_ENOMEM;
@@ -552,7 +556,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     // ---- 2. walk state
     RC(c->walk.ensure(sizeof(WalkState)));
     RC(c->runs.ensure((size_t)(ie + je + 2) * sizeof(int2)));
-    WalkState w{ie, je, 0, 0, 0, -1, 0};
+    WalkState w{ie, je, 0, 0, 0};
     // the band's traceback bits within the budget (at most three tiles a row)
     const size_t tile_bytes = (size_t)(BT / tbc.R) * (size_t)tb_row_words(BT, tbc.R) * (size_t)tb_word_bytes(tbc.R);
     // tile rows per band: two or three tiles a row, about one tile per SM (measured at 200 kbp: a

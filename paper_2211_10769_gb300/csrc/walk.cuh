@@ -40,9 +40,8 @@ struct WalkState {
     int32_t i, j;          // current cell (1-based rows / columns; 0 = border)
     int32_t state;         // 0 = H, 1 = E, 2 = F
     int32_t done;          // 0 running / needs tiles, 1 finished, 2 inconsistent bits
-    int64_t nruns;         // run records written so far
-    int32_t cur_op;        // op of the open run (0 = M, 1 = I, 2 = D, -1 = none)
-    int32_t cur_len;
+    int64_t nruns;         // run records {op: 0 = M, 1 = I, 2 = D; cells > 0} written so far;
+                           // consecutive records may have the same op
 };
 
 // The tiles recomputed in one round: for each tile row I in [I0, I0 + nI), a
@@ -63,16 +62,40 @@ constexpr int kWinDiags = 128;        // diagonals of a window, the walk's in th
 constexpr int kWinMargin = 16;        // diagonals a staged window must leave either side of the walk's
 constexpr int kStageThreads = 512;    // threads staging a window (warps 1..16)
 constexpr int kWalkThreads = 32 + kStageThreads;   // warp 0 walks
-constexpr int kStage = 8;             // window words a thread loads at once
 constexpr int kWalkMinBT = 256;       // tiles at least this side
 
 __device__ __forceinline__ int leading_zeros(unsigned v) { return __clz((int)v); }
 __device__ __forceinline__ int leading_zeros(unsigned long long v) { return __clzll((long long)v); }
 
 template <int R>
-constexpr size_t walk_window_bytes(size_t word_bytes) { return 2 * (size_t)(kWinRows / R) * kWinDiags * word_bytes; }
+constexpr size_t walk_window_bytes(size_t word_bytes) {   // two windows, each below a group of zero words
+    return 2 * (size_t)(kWinRows / R + 1) * kWinDiags * word_bytes;
+}
 
-// Row groups [g_lo, g_lo + ng), diagonals (column - row, 0-based) [dlo, dlo + kWinDiags).
+// Four consecutive words of a row group, loaded and stored as vectors.
+template <typename Word>
+struct alignas(sizeof(Word) == 2 ? 8 : 16) Quad {
+    unsigned v[sizeof(Word)];
+};
+
+template <typename Word>
+__device__ __forceinline__ Quad<Word> load_quad(const Word *p) {
+    Quad<Word> q;
+    if constexpr (sizeof(Word) == 2) {
+        const uint2 x = __ldcg(reinterpret_cast<const uint2 *>(p));
+        q.v[0] = x.x; q.v[1] = x.y;
+    } else {
+#pragma unroll
+        for (int k = 0; k < (int)sizeof(Word) / 4; ++k) {
+            const uint4 x = __ldcg(reinterpret_cast<const uint4 *>(p) + k);
+            q.v[4 * k] = x.x; q.v[4 * k + 1] = x.y; q.v[4 * k + 2] = x.z; q.v[4 * k + 3] = x.w;
+        }
+    }
+    return q;
+}
+
+// Row groups [g_lo, g_lo + ng), diagonals (column - row, 0-based) [dlo, dlo + kWinDiags), dlo = 1 (mod 4), which
+// puts a quad of diagonals at a multiple of four words of a tile's row group.
 struct WalkWindow {
     int g_lo, ng, dlo;
 };
@@ -83,13 +106,15 @@ __device__ __forceinline__ const Word *tile_ptr(const TileTable<Word> &T, const 
     return (ti >= 0 && tj >= 0 && ti < T.nI && tj < T.nJ) ? tiles[ti * T.nJ + tj] : nullptr;
 }
 
-// The window whose last row group is ghi.
+// The window whose last row group is ghi; the first diagonal around the walk's.
 template <int R>
 __device__ __forceinline__ WalkWindow make_window(int ghi, int dlo) {
     constexpr int RG = kWinRows / R;
     const int glo = max(0, ghi - (RG - 1));
     return WalkWindow{glo, ghi - glo + 1, dlo};
 }
+
+__device__ __forceinline__ int window_diag(int d) { return ((d - kWinDiags / 2 - 1) & ~3) + 1; }
 
 // Whether window m holds the cell (r0, c0) at least kWinMargin diagonals from either side.
 template <int R>
@@ -98,43 +123,47 @@ __device__ __forceinline__ bool window_holds(const WalkWindow &m, int r0, int c0
     return r0 >= 0 && g >= 0 && g < m.ng && d >= kWinMargin && d < kWinDiags - kWinMargin;
 }
 
-// Stage window m into win: staging thread t (of kStageThreads) takes diagonal
-// t % kWinDiags of every kStageThreads / kWinDiags-th row group, kStage
-// independent words in flight at a time.  A word that reaches over a tile's right
-// edge is the union of the two tiles' words.  Missing tiles and columns left of
-// the matrix read as 0.
+// Stage window m into win: a warp takes every (kStageThreads / 32)-th row group,
+// four diagonals a lane, kStage independent quads in flight at a time.  A word that reaches
+// over a tile's right edge is the union of the two tiles' words.  Missing tiles and
+// columns left of the matrix read as 0.
 template <typename Word, int R>
 __device__ __forceinline__ void stage_window(const TileTable<Word> &T, const Word *const *tiles, const WalkWindow &m,
                                              Word *win, int t) {
-    constexpr int kStep = kStageThreads / kWinDiags;       // row groups a thread advances
-    static_assert(kStageThreads % kWinDiags == 0, "whole row groups per pass");
-    const int k = t % kWinDiags, BT = T.BT;
-    int g = t / kWinDiags;
+    constexpr int kStep = kStageThreads / 32;              // row groups a thread advances
+    constexpr int kStage = kWinRows / R / kStep < 6 ? kWinRows / R / kStep : 6;   // quads a thread loads at once
+    static_assert(kWinDiags == 128, "a warp takes a row group");
+    static_assert(R % 4 == 0 && kStep * R <= kWalkMinBT, "quads are aligned; a step leaves at most one tile");
+    const int k = 4 * (t & 31), BT = T.BT;
+    int g = t >> 5;
     // the thread's tile and its place in it, advanced with the groups (BT is a multiple of R)
     const int r = (m.g_lo + g) * R, q = m.dlo + k + r;
     int I = r / BT, lr = r - I * BT;
     int J = q >= 0 ? q / BT : -((-q + BT - 1) / BT), lq = q - J * BT;
     while (g < m.ng) {
-        Word v[kStage], x[kStage];
+        Quad<Word> v[kStage];
 #pragma unroll
         for (int u = 0; u < kStage; ++u) {
-            v[u] = 0; x[u] = 0;
+            Quad<Word> x{};
+            v[u] = Quad<Word>{};
             if (g + u * kStep < m.ng) {
                 const size_t row = (size_t)(lr / R) * (size_t)T.ld;
                 const Word *a = tile_ptr(T, tiles, I, J);
-                if (a) v[u] = __ldcg(a + row + lq + R - 1);
+                if (a) v[u] = load_quad(a + row + lq + R - 1);
                 if (lq > BT - R) {
                     const Word *b = tile_ptr(T, tiles, I, J + 1);
-                    if (b) x[u] = __ldcg(b + row + lq - BT + R - 1);
+                    if (b) x = load_quad(b + row + lq - BT + R - 1);
+#pragma unroll
+                    for (int y = 0; y < (int)sizeof(Word); ++y) v[u].v[y] |= x.v[y];
                 }
             }
             lr += kStep * R; lq += kStep * R;
-            while (lr >= BT) { lr -= BT; ++I; }
-            while (lq >= BT) { lq -= BT; ++J; }
+            if (lr >= BT) { lr -= BT; ++I; }
+            if (lq >= BT) { lq -= BT; ++J; }
         }
 #pragma unroll
         for (int u = 0; u < kStage; ++u)
-            if (g + u * kStep < m.ng) win[(g + u * kStep) * kWinDiags + k] = v[u] | x[u];
+            if (g + u * kStep < m.ng) *reinterpret_cast<Quad<Word> *>(win + (g + u * kStep) * kWinDiags + k) = v[u];
         g += kStage * kStep;
     }
 }
@@ -147,17 +176,17 @@ __device__ __forceinline__ void stage_window(const TileTable<Word> &T, const Wor
 static __global__ void walk_start_kernel(const int4 *res, int local, WalkState *st) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const int4 r = *res;
-    WalkState w{r.y, r.z, 0, 0, 0, -1, 0};
+    WalkState w{r.y, r.z, 0, 0, 0};
     if ((local && r.x <= 0) || r.y <= 0 || r.z <= 0) { w.i = 1; w.j = 1; w.done = 3; }
     *st = w;
 }
 
 template <typename Word, int R>
 __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<Word> T, WalkState *st, int2 *runs,
-                                                          long long max_iters)
+                                                          int max_iters)
 {
     static_assert(kWinRows % R == 0, "a window holds whole row groups");
-    constexpr int kWinWords = (kWinRows / R) * kWinDiags;
+    constexpr int kWinWords = (kWinRows / R + 1) * kWinDiags;   // a group of zero words, then the window's
     using Wide = typename std::conditional<(R > 8), unsigned long long, unsigned>::type;   // a word, registers whole
     constexpr int kTop = 8 * (int)sizeof(Wide) - 4;        // shift of a Wide's top nibble
     constexpr Wide kOnes = (Wide)(0x1111111111111111ull >> (64 - 4 * R));
@@ -179,12 +208,14 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
         s_w = *st;
         s_stop = s_w.done != 0;
         const int r0 = max(s_w.i - 1, 0), c0 = max(s_w.j - 1, 0);
-        s_mw[0] = make_window<R>(r0 / R, c0 - r0 - kWinDiags / 2);
+        s_mw[0] = make_window<R>(r0 / R, window_diag(c0 - r0));
     }
+    if (threadIdx.x < kWinDiags) { s_buf[threadIdx.x] = 0; s_buf[kWinWords + threadIdx.x] = 0; }
+    s_buf += kWinDiags;
     __syncthreads();
     if (warp > 0 && !s_stop) stage_window<Word, R>(T, s_tiles, s_mw[0], s_buf, threadIdx.x - 32);
     __syncthreads();
-    long long it = 0;                                    // walk turns (warp 0)
+    int it = 0;                                          // walk turns (warp 0)
     int cur = 0;
     while (!s_stop) {
         const int nxt = cur ^ 1;
@@ -199,87 +230,82 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
             WalkState w = s_w;
             int nr = 0;                                  // run records written in this window
             int2 *out = runs + w.nruns;
-            // every lane keeps the same (uniform) run state; lane 0 stores the records
             auto emit = [&](int op, int cnt) {
-                if (op == w.cur_op) { w.cur_len += cnt; return; }
-                if (w.cur_len > 0) {
-                    if (lane == 0) out[nr] = make_int2(w.cur_op, w.cur_len);
-                    ++nr;
-                }
-                w.cur_op = op;
-                w.cur_len = cnt;
+                if (lane == 0) out[nr] = make_int2(op, cnt);
+                ++nr;
             };
+            // the cell, relative to the window
+            int rw = w.i - 1 - m.g_lo * R, dd = w.j - w.i - m.dlo, state = w.state;
             bool stop = false;                           // back to the host (or finished)
             while (true) {                               // (w.done is 0 here: every exit that sets it breaks)
                 if (++it >= max_iters) { w.done = 2; stop = true; break; }
-                const int r = w.i - 1, c = w.j - 1;
-                const int g0 = (int)((unsigned)max(r, 0) / R), x0 = r - g0 * R, gl = g0 - m.g_lo, dd = c - r - m.dlo;
-                if (w.state == 0) {
-                    if (w.i == 0 || w.j == 0) { w.done = 1; stop = true; break; }
-                    if (dd < 0 || dd >= kWinDiags) break;   // a gap ran out of the window
-                    // lane l: the walk's diagonal in the l-th group up, from row x0 (lane 0) or the group's last row
-                    const int g = gl - lane, top = lane == 0 ? x0 : R - 1;
-                    const Word wd = s_win[max(g, 0) * kWinDiags + dd];
+                if (rw < 0 || (unsigned)dd >= (unsigned)kWinDiags) break;   // out of the window
+                const int g0 = (int)((unsigned)rw / R), x0 = rw - g0 * R;
+                if (state == 0) {
+                    // lane l: the walk's diagonal in the l-th group up, from row x0 (lane 0) or the group's last
+                    // row; above the window's first group the words are 0, and columns left of the matrix read as 0
+                    const int top = lane == 0 ? x0 : R - 1;
+                    const Word wd = s_win[max(g0 - lane, -1) * kWinDiags + dd];
                     // a nibble is nonzero here where the H source is not "diagonal"; the top one first
                     const Wide bad = (((Wide)wd ^ kOnes) & (3 * kOnes)) << (kTop - 4 * top);
-                    const bool in = g >= 0;
-                    const int cnt = bad ? leading_zeros(bad) >> 2 : top + 1;   // leading cells that go on
-                    const bool end = !in || bad != 0;
-                    const unsigned ends = __ballot_sync(kFull, end);
-                    const int before = lane == 0 ? 0 : x0 + 1 + (lane - 1) * R;
-                    const int nib = in ? (int)((Wide)wd >> (4 * max(top - cnt, 0))) & 15 : 16;
-                    const int lim = min(r, c) + 1;       // cells up to the border
+                    const unsigned ends = __ballot_sync(kFull, bad != 0);
                     if (ends == 0) {                     // all 32 groups go on
-                        const int pos = min(x0 + 1 + 31 * R, lim);
+                        const int pos = x0 + 1 + 31 * R;
                         emit(0, pos);
-                        w.i -= pos;
-                        w.j -= pos;
+                        rw -= pos;
                         continue;
                     }
-                    const int val = __shfl_sync(kFull, (before + (in ? cnt : 0)) | (nib << 16), __ffs(ends) - 1);
-                    const int pos = min(val & 0xffff, lim), nbk = val >> 16;
+                    const int cnt = leading_zeros(bad) >> 2;   // leading cells that go on
+                    const int nib = (int)((Wide)wd >> (4 * max(top - cnt, 0))) & 15;
+                    const int before = max(0, x0 + 1 - R + lane * R);
+                    const int val = __shfl_sync(kFull, (before + cnt) | (nib << 16), __ffs(ends) - 1);
+                    const int pos = val & 0xffff, nbk = val >> 16, src = nbk & 3;
                     if (pos > 0) emit(0, pos);
-                    w.i -= pos;
-                    w.j -= pos;
-                    if (pos == lim) continue;            // the border
-                    if (nbk == 16) break;                // the window's first row: the next window starts here
-                    const int src = nbk & 3;
-                    if (src == 0) {                      // a zero cell, or a tile that was not recomputed
-                        if (tile_ptr(T, s_tiles, (r - pos) / T.BT, (c - pos) / T.BT)) w.done = 1;
+                    rw -= pos;
+                    if (src == 0) {                      // a zero cell, a tile that was not recomputed, or an edge
+                        const int r = rw + m.g_lo * R, c = r + m.dlo + dd;
+                        if (rw < 0 || c < 0) break;
+                        if (tile_ptr(T, s_tiles, r / T.BT, c / T.BT)) w.done = 1;
                         stop = true;
                         break;
                     }
-                    w.state = src == 2 ? 1 : 2;
-                    if (nbk & (src == 2 ? 4 : 8)) {      // opened here: a gap of one cell
-                        emit(w.state, 1);
-                        if (src == 2) --w.j; else --w.i;
-                        w.state = 0;
+                    if (src == 2) {
+                        if (nbk & 4) { emit(1, 1); --dd; }   // opened here: a gap of one cell
+                        else state = 1;
+                    } else {
+                        if (nbk & 8) { emit(2, 1); --rw; ++dd; }
+                        else state = 2;
                     }
                 } else {
                     // lane p: the cell p columns to the left (E) or p rows up (F); a cell of the path in a gap state
                     // has a nonzero nibble (its H source is not "zero"), so 0 is a tile that was not recomputed
-                    const bool inE = w.state == 1;
-                    const int rp = inE ? r : r - lane, d = inE ? dd - lane : dd + lane;
-                    const int gp = (int)((unsigned)max(rp, 0) / R), gw = gp - m.g_lo;
-                    const bool out_m = rp < 0 || (inE && c - lane < 0);
-                    const bool in = gw >= 0 && d >= 0 && d < kWinDiags;
-                    const Word wd = s_win[max(gw, 0) * kWinDiags + min(max(d, 0), kWinDiags - 1)];
-                    int nib = (int)((Wide)wd >> (4 * max(rp - gp * R, 0))) & 15;
-                    nib = out_m ? 17 : (in ? nib : 16);
+                    const bool inE = state == 1;
+                    const int rp = inE ? rw : rw - lane, d = inE ? dd - lane : dd + lane;
+                    const int gp = (int)((unsigned)max(rp, 0) / R);
+                    const bool in = rp >= 0 && d >= 0 && d < kWinDiags;
+                    const Word wd = s_win[gp * kWinDiags + min(max(d, 0), kWinDiags - 1)];
+                    const int nib = in ? (int)((Wide)wd >> (4 * max(rp - gp * R, 0))) & 15 : 16;
                     const bool end = nib >= 16 || nib == 0 || (nib & (inE ? 4 : 8)) != 0;
                     const unsigned ends = __ballot_sync(kFull, end);
                     const int pos = ends ? __ffs(ends) - 1 : 32;
                     const int nbk = __shfl_sync(kFull, nib, pos & 31);
                     const bool opened = ends != 0 && nbk != 0 && nbk < 16;
                     const int step = pos + (opened ? 1 : 0);   // the extensions, and the opening cell
-                    if (ends != 0 && nbk == 17) { w.done = 2; stop = true; break; }   // a gap cannot reach the border
-                    if (step > 0) emit(w.state, step);
-                    if (inE) w.j -= step; else w.i -= step;
-                    if (opened) { w.state = 0; continue; }
+                    if (step > 0) emit(state, step);
+                    if (inE) dd -= step; else { rw -= step; dd += step; }
+                    if (opened) { state = 0; continue; }
                     if (ends == 0) continue;
-                    if (nbk == 0) stop = true;           // missing tile: ask the host
-                    break;                               // (nbk 16: the window's edge)
+                    // the window's edge (nbk 16), a column left of the matrix, or a missing tile: ask the host
+                    if (nbk == 0 && rw + m.g_lo * R + m.dlo + dd >= 0) stop = true;
+                    break;
                 }
+            }
+            w.i = rw + m.g_lo * R + 1;
+            w.j = w.i + m.dlo + dd;
+            w.state = state;
+            if (w.done == 0 && (w.i <= 0 || w.j <= 0)) {   // the border; a gap cannot reach it
+                w.done = state == 0 ? 1 : 2;
+                stop = true;
             }
             if (lane == 0) {
                 w.nruns += nr;
@@ -293,7 +319,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
         if (threadIdx.x == 0) {
             const int r0 = max(s_w.i - 1, 0), c0 = max(s_w.j - 1, 0);
             s_redo = !window_holds<R>(s_mw[nxt], r0, c0);
-            if (s_redo) s_mw[nxt] = make_window<R>(r0 / R, c0 - r0 - kWinDiags / 2);
+            if (s_redo) s_mw[nxt] = make_window<R>(r0 / R, window_diag(c0 - r0));
         }
         __syncthreads();
         if (s_redo) {
@@ -302,15 +328,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
         }
         cur = nxt;
     }
-    if (threadIdx.x == 0) {
-        WalkState w = s_w;
-        if (w.done == 1 && w.cur_len > 0) {
-            runs[w.nruns++] = make_int2(w.cur_op, w.cur_len);
-            w.cur_len = 0;
-            w.cur_op = -1;
-        }
-        *st = w;
-    }
+    if (threadIdx.x == 0) *st = s_w;
 }
 
 }  // namespace swgb

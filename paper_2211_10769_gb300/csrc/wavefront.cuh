@@ -81,7 +81,7 @@ struct FillTask {
     int32_t row0;          // row index (0-based, in the whole pair) of the task's first row
     int32_t col0;          // column index (0-based, in the whole pair) of the task's first column
     int64_t colck_ld;
-    void *tb;              // traceback words, TB mode: [row group][tb_ld], tb_ld >= ncols + R - 1
+    void *tb;              // traceback words, TB mode: [row group][tb_ld], tb_ld >= ncols + R
     int64_t tb_ld;
     int32_t strip_warps;   // compute warps per strip (rows per strip = strip_warps * 32 * R);
                            // 0 = all W warps of the block
@@ -701,7 +701,7 @@ wavefront_kernel(const FillLaunch L)
 
             if constexpr (MODE == kModeTb) {               // the words that reach over the right edge
 #pragma unroll
-                for (int x = 1; x < R; ++x) tbw[n + R - 1 - x] = st.pend[x];
+                for (int x = 0; x < R; ++x) tbw[n + R - 1 - x] = st.pend[x];   // (pend[0] is 0: the row's last word)
             }
             if constexpr (MODE != kModeTb) {
                 static_assert(kKeyRows == 16, "key decode assumes 4 row bits");
