@@ -22,13 +22,16 @@ static __global__ void encode_kernel(const uint8_t *__restrict__ text, long long
     }
 }
 
-// Sets *err = kErrBadCode if any code is >= K.
-static __global__ void validate_codes_kernel(const uint8_t *__restrict__ s, long long len, int K, int *err)
+// Sets *err = kErrBadCode if any code of s (or of t, a second sequence) is >= K.
+static __global__ void validate_codes_kernel(const uint8_t *__restrict__ s, long long len, int K, int *err,
+                                             const uint8_t *__restrict__ t = nullptr, long long len_t = 0)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
     bool bad = false;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < len; k += stride)
         bad |= s[k] >= K;
+    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < len_t; k += stride)
+        bad |= t[k] >= K;
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicCAS(err, 0, kErrBadCode);
 }
 

@@ -115,7 +115,8 @@ int finish_alignment(int alg, int score, int64_t ie, int64_t je, const WalkState
 long long tb_row_words(long long BT, int R) { return BT + R; }
 
 template <typename Word, int R>
-int launch_walk_t(sw_ctx *c, const void *const *table, int I0, int J0, int nI, int nJ, int BT) {
+int launch_walk_t(sw_ctx *c, const void *const *table, int I0, int J0, int nI, int nJ, int BT, const WalkStart &start,
+                  WalkState *st, int2 *runs) {
     if ((long long)nI * nJ > kWalkTableMax || BT < kWalkMinBT || BT % R != 0) return SW_EINVAL;
     TileTable<Word> T;
     T.bits = reinterpret_cast<const Word *const *>(table);
@@ -127,20 +128,20 @@ int launch_walk_t(sw_ctx *c, const void *const *table, int I0, int J0, int nI, i
         if (c->device < 64) attr_set[c->device] = 1;
     }
     const int kp = kt_begin(c, SW_KT_WALK);
-    walk_kernel<Word, R><<<1, kWalkThreads, smem, c->stream>>>(T, static_cast<WalkState *>(c->walk.p),
-                                                               static_cast<int2 *>(c->runs.p), kWalkMaxIters);
+    walk_kernel<Word, R><<<1, kWalkThreads, smem, c->stream>>>(T, start, st, runs, kWalkMaxIters);
     kt_end(c, kp);
     CU(cudaGetLastError());
     ++c->launches;
     return SW_OK;
 }
 
-int launch_walk(sw_ctx *c, const void *const *table, int I0, int J0, int nI, int nJ, int BT, int R) {
+int launch_walk(sw_ctx *c, const void *const *table, int I0, int J0, int nI, int nJ, int BT, int R, const WalkStart &start,
+                WalkState *st, int2 *runs) {
     switch (R) {
-        case 4: return launch_walk_t<uint16_t, 4>(c, table, I0, J0, nI, nJ, BT);
-        case 8: return launch_walk_t<uint32_t, 8>(c, table, I0, J0, nI, nJ, BT);
-        case 12: return launch_walk_t<unsigned long long, 12>(c, table, I0, J0, nI, nJ, BT);
-        case 16: return launch_walk_t<unsigned long long, 16>(c, table, I0, J0, nI, nJ, BT);
+        case 4: return launch_walk_t<uint16_t, 4>(c, table, I0, J0, nI, nJ, BT, start, st, runs);
+        case 8: return launch_walk_t<uint32_t, 8>(c, table, I0, J0, nI, nJ, BT, start, st, runs);
+        case 12: return launch_walk_t<unsigned long long, 12>(c, table, I0, J0, nI, nJ, BT, start, st, runs);
+        case 16: return launch_walk_t<unsigned long long, 16>(c, table, I0, J0, nI, nJ, BT, start, st, runs);
         default: return SW_EINVAL;
     }
 }
@@ -270,10 +271,12 @@ long long small_pair_tile(const sw_ctx *c, int64_t m, int64_t n, const DevScorin
 // the forward fill with checkpoints every BT rows and columns, the end cell
 // reduced on the device, every BT x BT traceback tile of the matrix
 // recomputed from those checkpoints in one launch (independent tasks), the
-// walk started from the end cell there (walk_start_kernel) through a table of
+// walk started from the end cell there (WalkStart) through a table of
 // all tiles, and every result copied back at once.  The banded path needs a
 // host round trip between the end cell and its band; for a pair whose tiles
-// fit one wave on the SMs, recomputing all of them costs no more time.
+// fit one wave on the SMs, recomputing all of them costs no more time.  Such a call
+// is short (0.17 ms at 464 x 503), so it is five or six launches between one copy down and
+// one up: with a copy or memset for each of its parts, seventeen stream operations.
 int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, int64_t n, const DevScoring &ds,
                     bool fold, const FillConfig &fwd, const FillConfig &tbc, int sw, int tsw, long long BT,
                     sw_alignment *out) {
@@ -349,80 +352,72 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
             table[(size_t)ti * nJw + (size_t)(tj - J0 - ti)] = u.tb;
         }
     const long long all = (long long)t.nstrips + tickets;
-    RC(c->tasks.ensure(tasks.size() * sizeof(FillTask)));
-    RC(c->prog.ensure((size_t)all * sizeof(int)));
     RC(c->cand.ensure((size_t)all * sizeof(int4)));
-    RC(c->ticket.ensure(2 * sizeof(unsigned long long)));
-    RC(c->result.ensure(sizeof(int4)));
-    RC(c->walk.ensure(sizeof(WalkState)));
-    RC(c->runs.ensure((size_t)(m + n + 2) * sizeof(int2)));
-    RC(c->misc.ensure(table.size() * sizeof(void *)));
-    // host staging: the tasks and the tile table go down in two copies
-    const size_t task_bytes = tasks.size() * sizeof(FillTask);
-    const size_t tab_off = (task_bytes + 15) / 16 * 16;
-    RC(c->stage.ensure(tab_off + table.size() * sizeof(void *)));
-    std::memcpy(c->stage.p, tasks.data(), task_bytes);
-    std::memcpy(static_cast<char *>(c->stage.p) + tab_off, table.data(), table.size() * sizeof(void *));
-    CU(cudaMemcpyAsync(c->tasks.p, c->stage.p, task_bytes, cudaMemcpyHostToDevice, c->stream));
-    CU(cudaMemcpyAsync(c->misc.p, static_cast<char *>(c->stage.p) + tab_off, table.size() * sizeof(void *),
-                       cudaMemcpyHostToDevice, c->stream));
-    CU(cudaMemsetAsync(c->prog.p, 0, (size_t)all * sizeof(int), c->stream));
-    CU(cudaMemsetAsync(c->ticket.p, 0, 2 * sizeof(unsigned long long), c->stream));
+    // everything the launches read down in one copy (the scoring, the tasks, the tile table, the cleared tickets,
+    // strip progress and error word), everything the host reads back up in one: the error word, the end
+    // cell, the walk's state and the run records
+    size_t at = 0;
+    auto part = [&](size_t bytes) { const size_t o = at; at = (at + bytes + 127) / 128 * 128; return o; };
+    const size_t o_sc = part(sizeof(DevScoring)), o_tasks = part(tasks.size() * sizeof(FillTask)),
+                 o_table = part(table.size() * sizeof(void *)), o_ticket = part(2 * sizeof(unsigned long long)),
+                 o_prog = part((size_t)all * sizeof(int)), o_err = part(sizeof(int));
+    const size_t down_bytes = at;
+    const size_t o_res = part(sizeof(int4)), o_walk = part(sizeof(WalkState)),
+                 o_runs = part((size_t)(m + n + 2) * sizeof(int2));
+    RC(c->round.ensure(at));
+    RC(c->stage.ensure(down_bytes));
+    RC(c->stage3.ensure(at - o_err));
+    char *dev = static_cast<char *>(c->round.p), *down = static_cast<char *>(c->stage.p);
+    std::memcpy(down + o_sc, &ds, sizeof(DevScoring));
+    std::memcpy(down + o_tasks, tasks.data(), tasks.size() * sizeof(FillTask));
+    std::memcpy(down + o_table, table.data(), table.size() * sizeof(void *));
+    std::memset(down + o_ticket, 0, down_bytes - o_ticket);
+    CU(cudaMemcpyAsync(dev, down, down_bytes, cudaMemcpyHostToDevice, c->stream));
 
-    const FillTask *dtasks = static_cast<const FillTask *>(c->tasks.p);
+    const FillTask *dtasks = reinterpret_cast<const FillTask *>(dev + o_tasks);
     FillLaunch L{};
     L.tasks = dtasks;
-    L.scorings = static_cast<const DevScoring *>(c->scorings.p);
-    L.ticket = static_cast<unsigned long long *>(c->ticket.p);
-    L.prog = static_cast<int *>(c->prog.p);
+    L.scorings = reinterpret_cast<const DevScoring *>(dev + o_sc);
+    L.ticket = reinterpret_cast<unsigned long long *>(dev + o_ticket);
+    L.prog = reinterpret_cast<int *>(dev + o_prog);
     L.cand = static_cast<int4 *>(c->cand.p);
-    L.err = static_cast<int *>(c->err.p);
+    L.err = reinterpret_cast<int *>(dev + o_err);
     L.total = t.nstrips;
     L.spin_limit = c->spin_limit;
     L.ntasks = 1;
-    RC(launch_fill(c, fwd, kModeScoreCk, fold, L, ds.K, t.nstrips));
-    reduce_candidates_kernel<<<1, 32, 0, c->stream>>>(dtasks, 1, static_cast<const int4 *>(c->cand.p),
-                                                       static_cast<const DevScoring *>(c->scorings.p),
-                                                       static_cast<int4 *>(c->result.p));
+    validate_codes_kernel<<<(unsigned)std::min<long long>((std::max(m, n) + 255) / 256, 4LL * c->nsm), 256, 0, c->stream>>>(
+        da, m, ds.K, L.err, db, n);
     CU(cudaGetLastError());
     ++c->launches;
+    RC(launch_fill(c, fwd, kModeScoreCk, fold, L, ds.K, t.nstrips));
     FillLaunch Lt = L;                              // the tiles: their own tickets and progress
     Lt.tasks = dtasks + 1;
-    Lt.ticket = static_cast<unsigned long long *>(c->ticket.p) + 1;
-    Lt.prog = static_cast<int *>(c->prog.p) + t.nstrips;
-    Lt.cand = static_cast<int4 *>(c->cand.p) + t.nstrips;
+    Lt.ticket = L.ticket + 1;
+    Lt.prog = L.prog + t.nstrips;
+    Lt.cand = L.cand + t.nstrips;
     Lt.total = tickets;
     Lt.ntasks = ntiles;
     if (fwd.P16 && nJ > 1)
         RC(launch_straighten(c, fwd.R, ds.alg == kAlgLocal, dtasks + 1, ntiles, (int)std::min<int64_t>(BT, m), L.scorings));
     RC(launch_fill(c, tbc, kModeTb, fold, Lt, ds.K, tickets));
-    walk_start_kernel<<<1, 32, 0, c->stream>>>(static_cast<const int4 *>(c->result.p), ds.alg == kAlgLocal ? 1 : 0,
-                                               static_cast<WalkState *>(c->walk.p));
-    CU(cudaGetLastError());
-    ++c->launches;
-    RC(launch_walk(c, static_cast<const void *const *>(c->misc.p), 0, J0, nI, nJw, (int)BT, R));
+    const WalkStart start{dtasks, L.cand, L.scorings, reinterpret_cast<int4 *>(dev + o_res)};
+    RC(launch_walk(c, reinterpret_cast<const void *const *>(dev + o_table), 0, J0, nI, nJw, (int)BT, R, start,
+                   reinterpret_cast<WalkState *>(dev + o_walk), reinterpret_cast<int2 *>(dev + o_runs)));
 
-    // everything back at once: end cell, walk state, error word, run records
-    const size_t runs_off = 128;
-    const size_t runs_bytes = (size_t)(m + n + 2) * sizeof(int2);
-    RC(c->stage3.ensure(runs_off + runs_bytes));
-    char *h = static_cast<char *>(c->stage3.p);
-    CU(cudaMemcpyAsync(h, c->result.p, sizeof(int4), cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaMemcpyAsync(h + 16, c->err.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaMemcpyAsync(h + 32, c->walk.p, sizeof(WalkState), cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaMemcpyAsync(h + runs_off, c->runs.p, runs_bytes, cudaMemcpyDeviceToHost, c->stream));
+    const char *h = static_cast<const char *>(c->stage3.p);
+    CU(cudaMemcpyAsync(c->stage3.p, dev + o_err, at - o_err, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
     int4 res;
     int e;
     WalkState w;
-    std::memcpy(&res, h, sizeof(int4));
-    std::memcpy(&e, h + 16, sizeof(int));
-    std::memcpy(&w, h + 32, sizeof(WalkState));
+    std::memcpy(&e, h, sizeof(int));
+    std::memcpy(&res, h + (o_res - o_err), sizeof(int4));
+    std::memcpy(&w, h + (o_walk - o_err), sizeof(WalkState));
     RC(map_kernel_error(e));
     if (ds.alg == kAlgLocal && res.x <= 0) return empty_alignment(out);
     if (res.y == 0 || res.z == 0) return border_alignment(ds.alg, res.x, res.y, res.z, out);
     if (w.done != 1 || w.nruns < 0 || w.nruns > m + n) return SW_ECUDA;   // every tile is in the table
-    return finish_alignment(ds.alg, res.x, res.y, res.z, w, reinterpret_cast<const int2 *>(h + runs_off), out);
+    return finish_alignment(ds.alg, res.x, res.y, res.z, w, reinterpret_cast<const int2 *>(h + (o_runs - o_err)), out);
 }
 
 }  // namespace
@@ -445,10 +440,6 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     const uint8_t *da, *db;
     RC(stage_seq(c, a, m, c->seq_a, &da));
     RC(stage_seq(c, b, n, c->seq_b, &db));
-    RC(reset_err(c));
-    RC(validate_codes(c, da, m, ds.K));
-    RC(validate_codes(c, db, n, ds.K));
-    RC(upload_scorings(c, {ds}));
     const bool fold = fold_open(ds);
     if (c->one_round != 0 && std::max(m, n) <= kOneRoundSide) {
         // one round: forced (one_round > 0), or by default where every tile fits one wave on the SMs
@@ -459,6 +450,11 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
         if (bt > 0 && (c->one_round > 0 || tiles <= c->nsm))
             return align_one_round(c, da, m, db, n, ds, fold, f1, t1, sw1, tsw1, bt, out);
     }
+
+    RC(reset_err(c));
+    RC(validate_codes(c, da, m, ds.K));
+    RC(validate_codes(c, db, n, ds.K));
+    RC(upload_scorings(c, {ds}));
 
     // ---- tile side: both checkpoint sets within the budget
     // tiles are BT x BT; BT is a multiple of both fills' strip heights, so
@@ -737,7 +733,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
         CU(cudaMemcpyAsync(dtab, c->stage2.p, tbytes, cudaMemcpyHostToDevice, c->stream));
         if (ahead) CU(cudaEventRecord(c->side_go, c->stream));   // the band's tiles are done
         RC(launch_walk(c, static_cast<const void *const *>(dtab), cur.I0, cur.kd + cur.I0, cur.nI, cur.nJ,
-                       (int)BT, R));
+                       (int)BT, R, WalkStart{}, static_cast<WalkState *>(c->walk.p), static_cast<int2 *>(c->runs.p)));
         // the next band up the same diagonal, recomputed on the side stream while the walk runs
         if (ahead && cur.Itop > 0) {
             const long long pi = (long long)cur.Itop * BT, pj = (long long)w.j - ((long long)w.i - pi);

@@ -86,7 +86,7 @@ struct sw_ctx {
     size_t tb_budget = 0;             // bytes of traceback bits per row group
     swgb::DevBuf seq_a, seq_b, tasks, scorings, ticket, prog, cand, result, err, bnd, ckpt, colck, colaux, tb,
         ckpt2, colck2, colaux2,
-        tbbnd, straight, straight_b, runs, walk, misc, dbscratch, dbslots, dbovf, dbjob, dbscores, topk;
+        tbbnd, straight, straight_b, runs, walk, misc, round, dbscratch, dbslots, dbovf, dbjob, dbscores, topk;
     swgb::HostBuf stage, stage2, stage3;
     // sw_align's look-ahead band: a second set of traceback-fill buffers and a stream of their
     // own, so that the next band's tiles are recomputed while the walk goes through the current one

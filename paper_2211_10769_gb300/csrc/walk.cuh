@@ -32,7 +32,7 @@
 #pragma once
 #include <type_traits>
 
-#include "sw_device.cuh"
+#include "wavefront.cuh"
 
 namespace swgb {
 
@@ -168,21 +168,21 @@ __device__ __forceinline__ void stage_window(const TileTable<Word> &T, const Wor
     }
 }
 
-// The walk's start taken from the end cell reduced on the device (res: score,
-// row, column), for an alignment done in one round without a round trip to
-// the host: the end cell in state H, or nothing to walk (done = 3, parked at
-// cell (1, 1), a cell every window can hold) when the local score is 0 or the
-// end cell lies on the border.
-static __global__ void walk_start_kernel(const int4 *res, int local, WalkState *st) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int4 r = *res;
-    WalkState w{r.y, r.z, 0, 0, 0};
-    if ((local && r.x <= 0) || r.y <= 0 || r.z <= 0) { w.i = 1; w.j = 1; w.done = 3; }
-    *st = w;
-}
+// Where a walk starts, for an alignment done in one round without a round trip to the
+// host: at the end cell of the forward fill, reduced from its candidates by the walk's own
+// warp 0 into *result, in state H, or nothing to walk (done = 3, parked at cell (1, 1), a
+// cell every window can hold) when the local score is 0 or the end cell lies on the
+// border.  A null task: the walk goes on from its state.
+struct WalkStart {
+    const FillTask *task;
+    const int4 *cand;
+    const DevScoring *scorings;
+    int4 *result;
+};
 
 template <typename Word, int R>
-__global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<Word> T, WalkState *st, int2 *runs,
+__global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<Word> T, const WalkStart start,
+                                                          WalkState *st, int2 *runs,
                                                           int max_iters)
 {
     static_assert(kWinRows % R == 0, "a window holds whole row groups");
@@ -204,8 +204,18 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
         return;
     }
     for (int k = threadIdx.x; k < ntab; k += blockDim.x) s_tiles[k] = T.bits[k];
+    int4 end;
+    if (start.task && warp == 0)
+        end = reduce_candidates(*start.task, start.cand, start.scorings[start.task->scoring], lane);
     if (threadIdx.x == 0) {
-        s_w = *st;
+        if (start.task) {
+            *start.result = end;
+            s_w = WalkState{end.y, end.z, 0, 0, 0};
+            if ((start.scorings[start.task->scoring].alg == kAlgLocal && end.x <= 0) || end.y <= 0 || end.z <= 0)
+                s_w = WalkState{1, 1, 0, 3, 0};
+        } else {
+            s_w = *st;
+        }
         s_stop = s_w.done != 0;
         const int r0 = max(s_w.i - 1, 0), c0 = max(s_w.j - 1, 0);
         s_mw[0] = make_window<R>(r0 / R, window_diag(c0 - r0));

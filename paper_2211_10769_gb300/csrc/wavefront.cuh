@@ -753,19 +753,9 @@ wavefront_kernel(const FillLaunch L)
     }
 }
 
-// Reduce the per-strip candidates of every task to one end cell:
-// out[k] = (score, a_end, b_end, 0) with a_end/b_end the 1-based cell
-// (= exclusive 0-based ends); local: all zero when the best score is 0;
-// the other algorithms: the end cells on the matrix border are candidates
-// too (a task is a whole pair there).
-static __global__ void reduce_candidates_kernel(const FillTask *tasks, int ntasks, const int4 *cand,
-                                                const DevScoring *scorings, int4 *out)
+// Task T's end cell {score, row, column, 0} from its strips' candidates, by one warp (lane 0 has it).
+__device__ __forceinline__ int4 reduce_candidates(const FillTask &T, const int4 *cand, const DevScoring &SC, int lane)
 {
-    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (k >= ntasks) return;
-    const FillTask &T = tasks[k];
-    const DevScoring &SC = scorings[T.scoring];
     const bool local = SC.alg == kAlgLocal;
     int cs = local ? 0 : kNoScore, cj = 0x7fffffff, ci = 0x7fffffff;
     for (int s = lane; s < T.nstrips; s += 32) {
@@ -779,13 +769,24 @@ static __global__ void reduce_candidates_kernel(const FillTask *tasks, int ntask
         const int oi = __shfl_xor_sync(kFull, ci, off);
         if (cand_better(os, oj, oi, cs, cj, ci)) { cs = os; cj = oj; ci = oi; }
     }
-    if (lane != 0) return;
-    if (local) {
-        out[k] = cs > 0 ? make_int4(cs, ci, cj, 0) : make_int4(0, 0, 0, 0);
-    } else {
-        border_end_candidates(SC.alg, T.rows, T.ncols, SC.go, SC.ge, &cs, &ci, &cj);
-        out[k] = make_int4(cs, ci, cj, 0);
-    }
+    if (local) return cs > 0 ? make_int4(cs, ci, cj, 0) : make_int4(0, 0, 0, 0);
+    border_end_candidates(SC.alg, T.rows, T.ncols, SC.go, SC.ge, &cs, &ci, &cj);
+    return make_int4(cs, ci, cj, 0);
+}
+
+// Reduce the per-strip candidates of every task to one end cell:
+// out[k] = (score, a_end, b_end, 0) with a_end/b_end the 1-based cell
+// (= exclusive 0-based ends); local: all zero when the best score is 0;
+// the other algorithms: the end cells on the matrix border are candidates
+// too (a task is a whole pair there).
+static __global__ void reduce_candidates_kernel(const FillTask *tasks, int ntasks, const int4 *cand,
+                                                const DevScoring *scorings, int4 *out)
+{
+    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (k >= ntasks) return;
+    const int4 r = reduce_candidates(tasks[k], cand, scorings[tasks[k].scoring], lane);
+    if (lane == 0) out[k] = r;
 }
 
 }  // namespace swgb
