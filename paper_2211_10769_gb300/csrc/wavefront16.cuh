@@ -840,6 +840,28 @@ wavefront16_kernel(const FillLaunch L)
                     snap.top[lane] = t;
                     __syncwarp();
                 }
+                if constexpr (MODE == kModeScoreCk) {
+                    // the checkpoint column before this chunk, out of the snapshot by a small loop: unrolled from the
+                    // registers at the chunk's end it slowed every step of the long bodies down (26 rows a lane,
+                    // 505,856 x 500,000: 62.8 against the score fill's 58.5 ms, 62.0 with the store compiled in but
+                    // never reached; this way 59.4).  Bodies of 8 to 16 rows: the same either way
+                    if (s0 - 1 == next_ck && next_ck < n) {   // the same for every lane
+                        const long long kk = (next_ck + 1) / T.colck_every - 1;
+                        int2 *cc = T.colck + kk * T.colck_ld + (T.row0 + grow);
+                        const unsigned *q = reinterpret_cast<const unsigned *>(&snap.st[0][lane]);
+                        auto word = [&](int k) { return q[(k >> 2) * 128 + (k & 3)]; };
+#pragma unroll 1
+                        for (int k = 0; k < H; ++k) {
+                            const unsigned u = word(k), e = word(H + k);
+                            cc[k] = make_int2(p16_lo(u) + B, p16_lo(e) + B);
+                            cc[H + k] = make_int2(p16_hi(u) + B, p16_hi(e) + B);
+                        }
+                        int2 *ca = T.colck_aux + kk * (T.colck_ld / H) + (T.row0 + grow) / H;
+                        ca[0] = make_int2(p16_lo(st.udiag0) + B, p16_lo(st.flast) + B);
+                        ca[1] = make_int2(p16_hi(st.udiag0) + B, p16_hi(st.flast) + B);
+                        next_ck += T.colck_every;
+                    }
+                }
                 st.cmx = 0x80008000u;
                 uint2 *rc = rout + (s0 & (RS - 1));
                 // the chunk's steps; NS: steps an unrolled body, EDGE: halves outside the task hold (the other algorithms)
@@ -893,21 +915,6 @@ wavefront16_kernel(const FillLaunch L)
                 } else {
                     if ((s0 >= kP16Pos || (LEFT && T.left)) && s0 + CH <= n) sweep(P16Int<UNR>{}, P16Int<0>{});
                     else sweep(P16Int<4>{}, P16Int<1>{});
-                }
-                if constexpr (MODE == kModeScoreCk) {
-                    if (s0 + CH - 1 == next_ck && next_ck < n) {   // the same for every lane
-                        const long long kk = (next_ck + 1) / T.colck_every - 1;
-                        int2 *cc = T.colck + kk * T.colck_ld + (T.row0 + grow);
-#pragma unroll
-                        for (int k = 0; k < H; ++k) {
-                            cc[k] = make_int2(p16_lo(st.U[k]) + B, p16_lo(st.E[k]) + B);
-                            cc[H + k] = make_int2(p16_hi(st.U[k]) + B, p16_hi(st.E[k]) + B);
-                        }
-                        int2 *ca = T.colck_aux + kk * (T.colck_ld / H) + (T.row0 + grow) / H;
-                        ca[0] = make_int2(p16_lo(st.udiag0) + B, p16_lo(st.flast) + B);
-                        ca[1] = make_int2(p16_hi(st.udiag0) + B, p16_hi(st.flast) + B);
-                        next_ck += T.colck_every;
-                    }
                 }
                 if constexpr (!LOCAL) {
                     if (track) {                           // the last row's best of the chunk; the first column that holds it wins
