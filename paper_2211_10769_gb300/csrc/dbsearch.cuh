@@ -11,9 +11,9 @@
 // the subjects' columns exactly as in the pairwise fill (bottom H / F to the
 // next lane by shuffle), and longer queries take several passes, the bottom
 // row of one pass feeding the next through a per-warp boundary row in
-// global memory.  Short queries may instead run two independent 16-lane
-// wavefronts per warp (G = 16), each over its own pair of subjects, so that a
-// lane holds more rows of a short query and the skew of a wavefront is 15
+// global memory.  All but the longest queries run two independent 16-lane
+// wavefronts per warp instead (G = 16), each over its own pair of subjects, so
+// that a lane holds more rows of the query and the skew of a wavefront is 15
 // steps rather than 31.  The query profile (int8, S + open, all passes) sits in
 // shared memory; the two residues' score bytes are merged into one packed
 // register with a single prmt.

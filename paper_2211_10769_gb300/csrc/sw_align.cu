@@ -4,13 +4,16 @@
 //
 // 1. Forward fill over the whole matrix (score mode with checkpoints): the
 //    H / F row at every BT-th row and the H / E column at every BT-th
-//    column are kept.  BT is the smallest multiple of both fills' strip
-//    heights (at least 1024) for which both sets of checkpoints fit the
+//    column are kept.  BT is the smallest multiple of the forward fill's
+//    strip height and the traceback fill's (of its row groups after the packed
+//    fill; at least 512 or 1024) for which both sets of checkpoints fit the
 //    checkpoint budget, so memory is O((m + n)^2 / BT) rather than m x n.
 //    The columns are stored in staircase form (each lane of the fill one
 //    column further left than the lane above it, all at one step, so the
-//    sweep needs no per-step test); a tile entered from one first brings its
-//    lanes to the straight column (see FillTask::left).
+//    sweep needs no per-step test).  After the packed fill a launch of its own
+//    straightens the columns of a round's tiles (straighten.cuh), so that the
+//    tiles' rows a lane are free; a tile entered from an int32 fill's staircase
+//    first brings its own lanes to the straight column (see FillTask::left).
 // 2. The end cell (ie, je) comes from the per-strip candidates.
 // 3. With checkpoints on both sides, every BT x BT tile can be recomputed
 //    on its own from its top row and left column.  The walk goes
