@@ -145,6 +145,20 @@ class Hit:
     a_end: int
     b_end: int
 
+    def __init__(self, score: int, a_end: int, b_end: int):
+        # the generated __init__ of a frozen class sets each field by object.__setattr__, twice the time: 0.43
+        # against 0.25 us a hit, which counts where a batch returns thousands
+        d = self.__dict__
+        d["score"] = score
+        d["a_end"] = a_end
+        d["b_end"] = b_end
+
+
+# sw_hit as a numpy record, to read a batch's hits column by column
+_HIT_DTYPE = np.dtype({"names": ["score", "a_end", "b_end"], "formats": [np.int32, np.int64, np.int64],
+                       "offsets": [_Hit.score.offset, _Hit.a_end.offset, _Hit.b_end.offset],
+                       "itemsize": ctypes.sizeof(_Hit)})
+
 
 @dataclass(frozen=True)
 class Alignment:
@@ -317,7 +331,9 @@ class Batch:
 
     def run(self):
         _check(self._lib.sw_batch_run(self.handle, self._out), "sw_batch_run")
-        return [Hit(h.score, h.a_end, h.b_end) for h in self._out[:self.npairs]]
+        # by columns: one ctypes object a pair took 2,000 hits 1.26 ms, this 0.57 (a run's kernels 9 ms)
+        hits = np.frombuffer(self._out, dtype=_HIT_DTYPE)[:self.npairs]
+        return list(map(Hit, hits["score"].tolist(), hits["a_end"].tolist(), hits["b_end"].tolist()))
 
     def close(self):
         if self.handle:
