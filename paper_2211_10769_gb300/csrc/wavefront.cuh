@@ -317,12 +317,28 @@ __device__ __forceinline__ void lane_step(LaneState<R> &st, const uint32_t (&pw)
     int uup = __shfl_up_sync(kFull, st.ub, 1);
     int fup = __shfl_up_sync(kFull, st.fb, 1);
     if (lane == 0) { uup = top.x; fup = top.y; }
-    if (CHECK && (j < 0 || j >= n)) return;
+    const bool in = !CHECK || (unsigned)j < (unsigned)n;
+    if (MODE != kModeTb && !in) return;
     typename TbWord<R>::T word = 0;
-    column_update<R, PK, MODE == kModeTb, LOCAL>(st, pw, uup, fup, go, ge, word);
-    if (lane == 31) ring_out[j & (kQS - 1)] = make_int2(st.ub, st.fb);
+    if constexpr (CHECK && MODE == kModeTb) {
+        // a lane outside the task computes and keeps its state: no branch, so that consecutive steps overlap
+        const LaneState<R> old = st;
+        column_update<R, PK, true, LOCAL>(st, pw, uup, fup, go, ge, word);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            st.U[r] = in ? st.U[r] : old.U[r];
+            st.E[r] = in ? st.E[r] : old.E[r];
+            st.pend[r] = in ? st.pend[r] : old.pend[r];
+        }
+        st.ub = in ? st.ub : old.ub;
+        st.fb = in ? st.fb : old.fb;
+        st.udiag0 = in ? st.udiag0 : old.udiag0;
+    } else {
+        column_update<R, PK, MODE == kModeTb, LOCAL>(st, pw, uup, fup, go, ge, word);
+    }
+    if (in && lane == 31) ring_out[j & (kQS - 1)] = make_int2(st.ub, st.fb);
     if constexpr (MODE == kModeTb) {
-        tbw[j] = word;
+        if (in) tbw[j] = word;
     } else if constexpr (!LOCAL) {
         // semi-global and overlap: the task's last row is an end row at every column
         int ck = st.bk;
@@ -623,8 +639,8 @@ wavefront_kernel(const FillLaunch L)
                 // entered from the matrix border also takes the first chunk this way, computing
                 // the columns left of the task with the padding residue: that keeps a lane at the
                 // border state (H = 0, E and F at -open, which give column 0 the same values)
-                if ((s0 >= 31 || virt_ok) && s0 + CH + 1 <= n) {
-                    // steady state: every lane's column and the prefetched one are in [0, n)
+                // (in traceback mode the prefetched column may be n: lane 0 leaves that one out)
+                if ((s0 >= 31 || virt_ok) && s0 + CH + (MODE == kModeTb ? 0 : 1) <= n) {
 #pragma unroll UNR
                     for (int k = 0; k < CH; ++k) {
                         const int s = s0 + k;
@@ -663,9 +679,25 @@ wavefront_kernel(const FillLaunch L)
                             top = topn;
                         }
                     }
+                } else if constexpr (MODE == kModeTb) {
+                    // the first and last chunk of a traceback tile: whole unrolled groups, lanes outside the task hold
+                    // (a 256-column tile: 2 of 9 chunks; with a branch a step at twice the steady cost, and the chunk that
+                    // ends at column n among them, the tiles of a 2 kbp pair took 61 us; now 48)
+#pragma unroll (R <= 8 ? UNR : 1)
+                    for (int k = 0; k < CH; ++k) {
+                        const int s = s0 + k;
+                        const int jn = s + 1 - lane;
+                        const int cn = ((unsigned)jn < (unsigned)n) ? min((int)bring[jn & (QB - 1)], K) : K;
+                        const int2 topn = rin[(s + 1) & (QS - 1)];   // stale when s + 1 >= n: lane 0 holds
+                        uint32_t pwn[NPW];
+                        load_profile<R, PK, W * 32>(prow + cn * HC * PB, pwn);
+                        lane_step<R, MODE, PK, true, LOCAL>(st, pw, top, s, lane, n, go, ge, rout, tbw);
+#pragma unroll
+                        for (int q = 0; q < NPW; ++q) pw[q] = pwn[q];
+                        top = topn;
+                    }
                 } else {
-                    // traceback tiles and tasks with a left boundary: the first and last 31
-                    // steps with the same prefetch, bounds-checked
+                    // tasks with a left boundary: the first and last 31 steps with the same prefetch, bounds-checked
 #pragma unroll 1
                     for (int k = 0; k < CH; ++k) {
                         const int s = s0 + k;
