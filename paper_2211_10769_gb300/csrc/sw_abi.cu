@@ -394,6 +394,15 @@ int swgb::validate_codes(sw_ctx *c, const uint8_t *d, int64_t len, int K) {
     return SW_OK;
 }
 
+int swgb::validate_pair(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b, int64_t n, int K, int *err) {
+    const int threads = 256;
+    const long long blocks = std::min<long long>((std::max(m, n) + threads - 1) / threads, 4LL * c->nsm);
+    validate_codes_kernel<<<(unsigned)blocks, threads, 0, c->stream>>>(a, m, K, err, b, n);
+    CU(cudaGetLastError());
+    ++c->launches;
+    return SW_OK;
+}
+
 int swgb::read_err(sw_ctx *c, int *e) {
     RC(c->stage3.ensure(64));
     CU(cudaMemcpyAsync(c->stage3.p, c->err.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -551,11 +560,6 @@ int sw_score(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b, int64_t n
     const uint8_t *da, *db;
     RC(stage_seq(c, a, m, c->seq_a, &da));
     RC(stage_seq(c, b, n, c->seq_b, &db));
-    RC(reset_err(c));
-    RC(validate_codes(c, da, m, ds.K));
-    RC(validate_codes(c, db, n, ds.K));
-    RC(upload_scorings(c, {ds}));
-
     const FillConfig fwd = pair_fill_config_for(c, m, n, ds);
     const int sw = pair_strip_warps(c, fwd, m);
     const int SH = sw * 32 * fwd.R;
@@ -570,23 +574,46 @@ int sw_score(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b, int64_t n
     RC(c->bnd.ensure((size_t)t.nslot * (size_t)n * sizeof(int2)));
     t.bnd = static_cast<int2 *>(c->bnd.p);
     t.ckpt_every = 0; t.ckpt = nullptr; t.row0 = 0; t.tb = nullptr; t.tb_ld = 0;
-    RC(run_fill(c, fwd, kModeScore, fold_open(ds), {t}, t.nstrips, ds.K));
+    RC(c->cand.ensure((size_t)t.nstrips * sizeof(int4)));
 
-    RC(c->result.ensure(sizeof(int4)));
-    reduce_candidates_kernel<<<1, 32, 0, c->stream>>>(static_cast<const FillTask *>(c->tasks.p), 1,
-                                                       static_cast<const int4 *>(c->cand.p),
-                                                       static_cast<const DevScoring *>(c->scorings.p),
-                                                       static_cast<int4 *>(c->result.p));
+    // one copy down (the scoring, the task, the cleared ticket, strip progress and error word), one validation, the
+    // fill, the reduction, one copy up (the error word and the end cell): eleven stream operations with a copy or
+    // memset for each (300 x 300: 69 us; this way 60)
+    size_t at = 0;
+    auto part = [&](size_t bytes) { const size_t o = at; at = (at + bytes + 127) / 128 * 128; return o; };
+    const size_t o_sc = part(sizeof(DevScoring)), o_task = part(sizeof(FillTask)), o_ticket = part(sizeof(unsigned long long)),
+                 o_prog = part((size_t)t.nstrips * sizeof(int)), o_err = part(sizeof(int));
+    const size_t down_bytes = at;
+    const size_t o_res = part(sizeof(int4));
+    RC(c->round.ensure(at));
+    RC(c->stage.ensure(down_bytes));
+    RC(c->stage3.ensure(at - o_err));
+    char *dev = static_cast<char *>(c->round.p), *down = static_cast<char *>(c->stage.p);
+    std::memcpy(down + o_sc, &ds, sizeof(DevScoring));
+    std::memcpy(down + o_task, &t, sizeof(FillTask));
+    std::memset(down + o_ticket, 0, down_bytes - o_ticket);
+    CU(cudaMemcpyAsync(dev, down, down_bytes, cudaMemcpyHostToDevice, c->stream));
+    FillLaunch L{};
+    L.tasks = reinterpret_cast<const FillTask *>(dev + o_task);
+    L.scorings = reinterpret_cast<const DevScoring *>(dev + o_sc);
+    L.ticket = reinterpret_cast<unsigned long long *>(dev + o_ticket);
+    L.prog = reinterpret_cast<int *>(dev + o_prog);
+    L.cand = static_cast<int4 *>(c->cand.p);
+    L.err = reinterpret_cast<int *>(dev + o_err);
+    L.total = t.nstrips;
+    L.spin_limit = c->spin_limit;
+    L.ntasks = 1;
+    RC(validate_pair(c, da, m, db, n, ds.K, L.err));
+    RC(launch_fill(c, fwd, kModeScore, fold_open(ds), L, ds.K, t.nstrips));
+    reduce_candidates_kernel<<<1, 32, 0, c->stream>>>(L.tasks, 1, L.cand, L.scorings, reinterpret_cast<int4 *>(dev + o_res));
     CU(cudaGetLastError());
     ++c->launches;
-    CU(cudaMemcpyAsync(c->stage3.p, c->result.p, sizeof(int4), cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaMemcpyAsync(static_cast<char *>(c->stage3.p) + 16, c->err.p, sizeof(int),
-                       cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaMemcpyAsync(c->stage3.p, dev + o_err, at - o_err, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
     int4 res;
     int e;
-    std::memcpy(&res, c->stage3.p, sizeof(int4));
-    std::memcpy(&e, static_cast<char *>(c->stage3.p) + 16, sizeof(int));
+    std::memcpy(&e, c->stage3.p, sizeof(int));
+    std::memcpy(&res, static_cast<char *>(c->stage3.p) + (o_res - o_err), sizeof(int4));
     RC(map_kernel_error(e));
     *out = sw_hit{res.x, 0, (int64_t)res.y, (int64_t)res.z};
     return SW_OK;

@@ -388,10 +388,7 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
     L.total = t.nstrips;
     L.spin_limit = c->spin_limit;
     L.ntasks = 1;
-    validate_codes_kernel<<<(unsigned)std::min<long long>((std::max(m, n) + 255) / 256, 4LL * c->nsm), 256, 0, c->stream>>>(
-        da, m, ds.K, L.err, db, n);
-    CU(cudaGetLastError());
-    ++c->launches;
+    RC(validate_pair(c, da, m, db, n, ds.K, L.err));
     RC(launch_fill(c, fwd, kModeScoreCk, fold, L, ds.K, t.nstrips));
     FillLaunch Lt = L;                              // the tiles: their own tickets and progress
     Lt.tasks = dtasks + 1;
@@ -455,8 +452,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     }
 
     RC(reset_err(c));
-    RC(validate_codes(c, da, m, ds.K));
-    RC(validate_codes(c, db, n, ds.K));
+    RC(validate_pair(c, da, m, db, n, ds.K, static_cast<int *>(c->err.p)));
     RC(upload_scorings(c, {ds}));
 
     // ---- tile side: both checkpoint sets within the budget

@@ -144,6 +144,8 @@ int kt_begin(sw_ctx *c, int kind);         // -1 when not timing; else the pair 
 void kt_end(sw_ctx *c, int pair);
 int reset_err(sw_ctx *c);
 int validate_codes(sw_ctx *c, const uint8_t *d, int64_t len, int K);
+// both sequences of a pair (at least one residue each) in one launch
+int validate_pair(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b, int64_t n, int K, int *err);
 int read_err(sw_ctx *c, int *e);
 // database search pieces shared with the serving loop
 struct DbJob;
