@@ -97,6 +97,12 @@ constexpr int kP16RS = 256;         // steps of the rings between the warps
 constexpr int kP16Pos = 64;         // wavefront positions per warp (two per lane)
 constexpr int kP16CH = 32;          // steps per chunk (hand-off, base change; 16 measured slower)
 constexpr int kP16Lag = kP16Pos - 1;   // lane 31's bottom half trails lane 0's top half
+// Columns left of the last warp's published count whose profile offsets may still be read: lane 31's, one more for
+// the words of the step before, and the chunk left of the task that a block's first strip starts with, when
+// nothing is published yet.
+constexpr int kP16Back = kP16Pos + kP16CH + 2;
+// Columns that may have their profile offset in the ring once the last warp has published `done` columns.
+__host__ __device__ constexpr int p16_offset_room(int done) { return done + kQB - kP16Back; }
 // steps per unrolled body (12 rows a lane at 200 kbp: 8, 16, 32 steps 16.4, 15.2, 18.4 ms; 26 rows: 8 and 16 steps
 // 212 and 205 clocks a step)
 constexpr int kP16Unroll = 16;
@@ -359,7 +365,7 @@ __device__ __forceinline__ void p16_input_warp(const FillTask &T, const FillLaun
         }
         // the offsets run ahead: in idle turns, and whenever they are less than two batches ahead
         if (rnext < n_ext && (!moved || rnext < next + 2 * kBatch)) {
-            const int target = min(n_ext, min(rnext + kBatch, lds_acquire(&prod[Wa]) + QB - (kP16Pos + 2)));
+            const int target = min(n_ext, min(rnext + kBatch, p16_offset_room(lds_acquire(&prod[Wa]))));
             if (target > rnext) {
                 for (int col = rnext + lane; col < target; col += 32) {
                     const int c = col < n ? min((int)__ldg(b + col), K) : K;
@@ -609,7 +615,7 @@ wavefront16_kernel(const FillLaunch L)
     constexpr int NL = W * 32;
     constexpr int CH = kP16CH, QS = kP16QS, RS = kP16RS, QB = kQB, LAG = kP16Lag;
     static_assert(QS >= 2 * 64 + 2 * CH && RS >= 2 * CH + 2 * kP16Pos, "ring too small");
-    static_assert(QB >= W * (kP16Pos + CH) + kP16Pos + 2 + 128, "the last warp's offsets must not be overwritten");
+    static_assert(QB >= W * (kP16Pos + CH) + kP16Back + 128, "the first warp's offsets must fit beside those the last warp still reads");
     constexpr int UNR = kP16Unroll;
     static_assert(CH % UNR == 0 && UNR % 4 == 0, "chunks are whole unrolled groups of four steps");
     static_assert(CH == 32, "one boundary entry a lane");
@@ -683,8 +689,8 @@ wavefront16_kernel(const FillLaunch L)
         }
         // the offset ring starts as padding (the warm-up chunk below reads columns down to -96); its last kP16Pos
         // slots hold the columns left of the task: padding at the matrix border, real residues for a task entered from
-        // a checkpoint column.  The input warp reaches those slots only after the last warp has published a column,
-        // i.e. left them behind
+        // a checkpoint column.  The input warp stays kP16Back slots short of a full ring until the last warp has published
+        // a column, i.e. left all of these behind
         if (first) {
             for (int k = threadIdx.x; k < QB; k += blockDim.x) s_poff[k] = (PK == kP16Pair ? K * (K + 1) + K : K) * pstride;
             __syncthreads();

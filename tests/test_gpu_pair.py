@@ -523,6 +523,23 @@ def test_packed_base_moves(packed_ctx, oracle_mod):
     _align_case(packed_ctx, oracle_mod, a, W.mutate(a, 20, W.BASE_SEED + 8611), S, o, e)
 
 
+@pytest.mark.parametrize("S,o,e", [(5, 8, 1), (1, 3, 0), (9, 0, 0)])
+def test_packed_left_of_the_task(packed_ctx, oracle_mod, S, o, e):
+    """Cheap gaps, rows that match columns 929 .. 957 (the offset slots of the columns left of the task in the
+    chunk that a block's first strip starts with), and paths that start in column 0: a value from left
+    of the task would reach them."""
+    mat = np.full((4, 4), -S, np.int8)
+    np.fill_diagonal(mat, S)
+    g = np.random.default_rng(W.BASE_SEED + 8650 + S)
+    for m in (3000, 26 * 128 * 3):
+        a = g.integers(0, 4, size=m).astype(np.uint8)
+        b = g.integers(0, 4, size=2500).astype(np.uint8)
+        b[929:958] = a[600:629]
+        b[:40] = a[1400:1440]
+        _score_case(packed_ctx, oracle_mod, a, b, mat, o, e)
+        _align_case(packed_ctx, oracle_mod, np.resize(a[600:629], m), b, mat, o, e)
+
+
 @pytest.mark.parametrize("tb", ["4,4", "8,4", "12,4", "16,4"])
 def test_walk_windows(oracle_mod, monkeypatch, tb):
     """The walk's windows, at every traceback tile height: gap runs that end just inside, at and
