@@ -400,7 +400,7 @@ int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, 
     if (fwd.P16 && nJ > 1)
         RC(launch_straighten(c, fwd.R, ds.alg == kAlgLocal, dtasks + 1, ntiles, (int)std::min<int64_t>(BT, m), L.scorings));
     RC(launch_fill(c, tbc, kModeTb, fold, Lt, ds.K, tickets));
-    const WalkStart start{dtasks, L.cand, L.scorings, reinterpret_cast<int4 *>(dev + o_res)};
+    const WalkStart start{dtasks, L.cand, L.scorings, reinterpret_cast<int4 *>(dev + o_res), L.err};
     RC(launch_walk(c, reinterpret_cast<const void *const *>(dev + o_table), 0, J0, nI, nJw, (int)BT, R, start,
                    reinterpret_cast<WalkState *>(dev + o_walk), reinterpret_cast<int2 *>(dev + o_runs)));
 

@@ -172,13 +172,21 @@ __device__ __forceinline__ void stage_window(const TileTable<Word> &T, const Wor
 // host: at the end cell of the forward fill, reduced from its candidates by the walk's own
 // warp 0 into *result, in state H, or nothing to walk (done = 3, parked at cell (1, 1), a
 // cell every window can hold) when the local score is 0 or the end cell lies on the
-// border.  A null task: the walk goes on from its state.
+// border, or when the error word is set: the fill then stopped early, and what stands in place
+// of its candidates and decision words (an earlier call's) may lead anywhere, past the
+// rows + columns run records there is room for.  A null task: the walk goes on from its state.
 struct WalkStart {
     const FillTask *task;
     const int4 *cand;
     const DevScoring *scorings;
     int4 *result;
+    const int *err;
 };
+
+__host__ __device__ __forceinline__ WalkState walk_start(int4 end, bool local, int err) {
+    if (err != 0 || (local && end.x <= 0) || end.y <= 0 || end.z <= 0) return WalkState{1, 1, 0, 3, 0};
+    return WalkState{end.y, end.z, 0, 0, 0};
+}
 
 template <typename Word, int R>
 __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<Word> T, const WalkStart start,
@@ -210,9 +218,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) walk_kernel(const TileTable<W
     if (threadIdx.x == 0) {
         if (start.task) {
             *start.result = end;
-            s_w = WalkState{end.y, end.z, 0, 0, 0};
-            if ((start.scorings[start.task->scoring].alg == kAlgLocal && end.x <= 0) || end.y <= 0 || end.z <= 0)
-                s_w = WalkState{1, 1, 0, 3, 0};
+            s_w = walk_start(end, start.scorings[start.task->scoring].alg == kAlgLocal, *start.err);
         } else {
             s_w = *st;
         }

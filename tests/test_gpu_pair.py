@@ -247,6 +247,25 @@ def test_invalid_arguments(ctx):
     assert ctx.score(a, a, sc.matrix, sc.gap_open, sc.gap_extend).score == 100
 
 
+def test_refused_align_after_a_larger_one(ctx, oracle_mod):
+    """A residue outside the alphabet, in an alignment whose buffers hold a larger one's end cell and
+    decision words: refused, and the next calls are exact."""
+    from paper_2211_10769_gb300 import binding
+    sc = W.dna_scoring()
+    a = W.uniform_dna(7000, W.BASE_SEED + 8900)
+    b = W.mutate(a, 4, W.BASE_SEED + 8901)
+    for n in (300, 700, 2500):
+        _align_case(ctx, oracle_mod, a, b, sc.matrix, sc.gap_open, sc.gap_extend)
+        bad = b[:n].copy()
+        bad[n // 2] = 4
+        for p, q in ((a[:n], bad), (bad, a[:n])):
+            for alg in (0, 1, 2, 3):
+                with pytest.raises(binding.SwError) as ei:
+                    ctx.align(p, q, sc.matrix, sc.gap_open, sc.gap_extend, alg)
+                assert ei.value.status == binding.SW_EINVAL
+        _align_case(ctx, oracle_mod, a[:n], b[:n], sc.matrix, sc.gap_open, sc.gap_extend)
+
+
 def _long_gap_pair(seed, length, cut0, cut1, insert):
     """A and B share A's sequence except that B lacks A[cut0:cut1] (a long
     deletion) or, with insert=True, carries extra random bases there."""
