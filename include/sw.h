@@ -238,10 +238,11 @@ int sw_score_noalloc(void *cuda_stream, const uint8_t *a, int64_t m, const uint8
  *   SW_BATCH_GRAPH     capture each run in a CUDA graph once and replay it;
  *   SW_BATCH_AUTOTUNE  time the candidate tile shapes of every bin on this plan
  *                      and keep the fastest (cached in the context per bin
- *                      size class).  The candidates are int32 lanes of 4 or
- *                      8 rows and, for local bins whose scoring keeps it
- *                      exact, packed 16-bit lanes of 8, 12 or 16 rows; where
- *                      it does not, also int32 lanes of 12 and 16 rows.
+ *                      size class and what the scoring keeps exact).  The
+ *                      candidates are int32 lanes of 4 or 8 rows and, for
+ *                      local bins whose scoring keeps it exact, packed 16-bit
+ *                      lanes of 8, 12 or 16 rows; where it does not, also
+ *                      int32 lanes of 12 and 16 rows.
  *                      Without it a bin takes packed lanes where exact.
  * sw_batch_run writes npairs hits (host memory).  A plan belongs to its
  * context and must be destroyed before it.

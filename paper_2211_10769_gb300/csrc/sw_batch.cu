@@ -307,14 +307,17 @@ int finish_run(sw_batch *B, sw_hit *out) {
     return SW_OK;
 }
 
-// Size class of a bin for the autotune cache: its alphabet, row class, and
-// log2 of its cells and of its pair count.
+// Class of a bin for the autotune cache: its alphabet, which shapes its scoring is exact
+// for (all that is_candidate asks about it), row class, and log2 of its cells and of its
+// pair count.
 long long bin_class(const sw_batch *B, const Bin &bin) {
     double cells = 0;
     for (int32_t p : bin.pairs) cells += (double)B->m[(size_t)p] * (double)B->n[(size_t)p];
     const int lc = cells > 1 ? (int)std::log2(cells) : 0;
     const int lp = bin.pairs.size() > 1 ? (int)std::log2((double)bin.pairs.size()) : 0;
-    return (((long long)B->scorings[(size_t)bin.sidx].K * 2 + bin.rclass) * 64 + lc) * 64 + lp;
+    const DevScoring &s = B->scorings[(size_t)bin.sidx];
+    const int exact = (p16_fits(s, 8) ? 1 : 0) | (p16_fits(s, 12) ? 2 : 0) | (p16_fits(s, 16) ? 4 : 0) | (fold_open(s) ? 8 : 0);
+    return ((((long long)s.K * 16 + exact) * 2 + bin.rclass) * 64 + lc) * 64 + lp;
 }
 
 }  // namespace

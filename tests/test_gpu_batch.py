@@ -108,6 +108,32 @@ def test_batch_int8_profile(oracle_mod, monkeypatch, R, Wc):
         c.close()
 
 
+@pytest.mark.parametrize("flags", [0, 2, 3])
+def test_tuned_shapes_and_another_scoring(oracle_mod, flags):
+    """A context that has tuned a plan meets the same pairs under scorings of the same alphabet that
+    the tuned shapes are not exact for: S + open outside int8, and scores beyond the packed fill."""
+    from paper_2211_10769_gb300 import binding
+    P = W.protein_scoring().matrix
+    big = np.full((24, 24), -60, np.int8)
+    np.fill_diagonal(big, 100)
+    pairs = []
+    for k in range(60):
+        a = W.random_protein(900 + 40 * k, W.BASE_SEED + 12700 + k)
+        pairs.append((a, W.mutate(a, 20, W.BASE_SEED + 12800 + k, p_sub=0.1), 0))
+    c = binding.Context(0)
+    try:
+        tuned = binding.Batch(c, pairs, [(P, 10, 1)], flags=2)
+        assert any(lb == 16 for _, _, lb, _ in tuned.bins())
+        tuned.close()
+        for sc in ((P, 130, 1), (big, 30, 2)):
+            plan = binding.Batch(c, pairs, [sc], flags=flags)
+            got = plan.run()
+            assert [(h.score, h.a_end, h.b_end) for h in got] == _oracle_hits(oracle_mod, pairs, [sc])
+            plan.close()
+    finally:
+        c.close()
+
+
 def test_batch_device_inputs_and_empty(ctx, oracle_mod):
     import torch
     from paper_2211_10769_gb300 import binding
