@@ -427,7 +427,9 @@ extern "C" int sw_batch_create(sw_ctx *c, int64_t npairs, const uint8_t *a_res, 
             if (c->bat_auto && p16_fits(bsc, 12)) bin.cfg = FillConfig{bin.rclass ? 12 : 8, 4, 0, 0, fold_open(bsc) ? 2 : 1};
             if (bin.cfg.P16 && ((bin.cfg.W != 4 && bin.cfg.W != 2) || !p16_fits(B->scorings[(size_t)bin.sidx], bin.cfg.R)))
                 bin.cfg.P16 = 0;
-            if (bin.cfg.P16 == 2 && !fold_open(B->scorings[(size_t)bin.sidx])) bin.cfg.P16 = 1;
+            // the int8 profile (launch_fill16_batch): 8 and 12 rows, S + open within int8
+            if (bin.cfg.P16 == 2 && (!fold_open(B->scorings[(size_t)bin.sidx]) || (bin.cfg.R != 8 && bin.cfg.R != 12)))
+                bin.cfg.P16 = 1;
             if (B->scorings[(size_t)bin.sidx].alg != kAlgLocal) {   // global, semi-global, overlap
                 bin.cfg = FillConfig{bin.rclass ? 16 : 8, 4};
                 bin.cfg.alg = 1;

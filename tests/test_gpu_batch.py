@@ -108,6 +108,24 @@ def test_batch_int8_profile(oracle_mod, monkeypatch, R, Wc):
         c.close()
 
 
+@pytest.mark.parametrize("Wc", [4, 2])
+def test_batch_int8_profile_at_16_rows(oracle_mod, monkeypatch, Wc):
+    """An override that asks for the int8 profile at 16 rows a lane, which has none: the packed fill's other
+    profiles serve it."""
+    from paper_2211_10769_gb300 import binding
+    monkeypatch.setenv("SWGB_BATCH", "16,%d,2" % Wc)
+    c = binding.Context(0)
+    try:
+        sc = _scorings()
+        pairs = _mixed_pairs(W.BASE_SEED + 12400 + Wc, 60, hi=4500)
+        plan = binding.Batch(c, pairs, sc, flags=0)
+        assert all((r, w, lb) == (16, Wc, 16) for r, w, lb, _ in plan.bins())
+        assert [(h.score, h.a_end, h.b_end) for h in plan.run()] == _oracle_hits(oracle_mod, pairs, sc)
+        plan.close()
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("flags", [0, 2, 3])
 def test_tuned_shapes_and_another_scoring(oracle_mod, flags):
     """A context that has tuned a plan meets the same pairs under scorings of the same alphabet that
