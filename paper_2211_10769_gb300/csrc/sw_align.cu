@@ -227,10 +227,12 @@ constexpr int64_t kOneRoundPackedSide = 4096;
 
 // Tile shape of the traceback fill after forward fill fwd: int32 (bits come from
 // the int32 fill); after the packed fill, whose checkpoint columns are
-// straightened, the context's shape (8 rows a lane); after an int32 fill the
-// tiles continue its staircase columns lane by lane, so they take its rows a lane.
+// straightened, the context's shape (8 rows a lane) where it is one that launch_fill has; after
+// an int32 fill the tiles continue its staircase columns lane by lane, so they take its rows a lane.
 FillConfig traceback_config(const sw_ctx *c, const FillConfig &fwd) {
-    FillConfig t = (fwd.alg == kAlgLocal && (fwd.P16 || c->tbc.R == fwd.R)) ? c->tbc : FillConfig{fwd.P16 ? 8 : fwd.R, 4};
+    const int R = c->tbc.R, W = c->tbc.W;
+    const bool built = (W == 4 && (R == 4 || R == 8 || R == 12 || R == 16)) || (W == 8 && R == 8);
+    FillConfig t = (fwd.alg == kAlgLocal && built && (fwd.P16 || R == fwd.R)) ? c->tbc : FillConfig{fwd.P16 ? 8 : fwd.R, 4};
     t.P16 = 0;
     t.alg = fwd.alg;
     return t;

@@ -542,6 +542,23 @@ def test_packed_base_moves(packed_ctx, oracle_mod):
     _align_case(packed_ctx, oracle_mod, a, W.mutate(a, 20, W.BASE_SEED + 8611), S, o, e)
 
 
+@pytest.mark.parametrize("tb", ["16,8", "10,4", "8,8"])
+def test_traceback_overrides_after_a_packed_fill(oracle_mod, monkeypatch, tb):
+    """A traceback shape that is not built gives way to one that is; blocks of eight warps are built at 8
+    rows a lane."""
+    from paper_2211_10769_gb300 import binding
+    monkeypatch.setenv("SWGB_TB", tb)
+    monkeypatch.setenv("SWGB_ONE_ROUND", "0")
+    monkeypatch.setenv("SWGB_FWD", "12,4,0,2,1")
+    c = binding.Context(0)
+    try:
+        sc = W.dna_scoring()
+        a = W.uniform_dna(9100, W.BASE_SEED + 8660)
+        _align_case(c, oracle_mod, a, W.mutate(a, 4, W.BASE_SEED + 8661), sc.matrix, sc.gap_open, sc.gap_extend)
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("S,o,e", [(5, 8, 1), (1, 3, 0), (9, 0, 0)])
 def test_packed_left_of_the_task(packed_ctx, oracle_mod, S, o, e):
     """Cheap gaps, rows that match columns 929 .. 957 (the offset slots of the columns left of the task in the
