@@ -13,6 +13,7 @@ namespace {
 
 // steps by which a warp trails the one above, and clocks of a step (measured, R = 4 .. 26, one strip)
 constexpr double kP16ChainSteps = 105;
+constexpr double kP16TileClocks = 464;
 constexpr double p16_step_clocks(int R) { return R <= 8 ? 70 + 3.3 * R : (R <= 16 ? 53 + 5.4 * R : 46 + 6.1 * R); }
 
 // W = 2 (score mode only): blocks of two compute warps for batches, whose
@@ -45,6 +46,8 @@ bool swgb::p16_fits(const DevScoring &s, int R) {
     for (int k = 0; k < s.K * s.K; ++k) { lo = std::min(lo, (int)s.mat[k]); hi = std::max(hi, (int)s.mat[k]); }
     return p16_spread(R, s.go, s.ge, hi, lo) <= kP16Span;
 }
+
+bool swgb::p16_pair_profile(int K) { return pair_profile_fits<8, 4>(K); }
 
 int swgb::launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const FillLaunch &L, int K,
                         long long tickets) {
@@ -82,7 +85,10 @@ int swgb::launch_straighten(sw_ctx *c, int R, bool local, const FillTask *tasks,
 // fills: 8 kbp R = 4 / 6 / 8: 0.69 / 0.65 / 0.63 ms; 30 kbp R = 6 / 8 / 10:
 // 2.25 / 2.17 / 2.18; 200 kbp R = 12 / 14: 15.3 / 16.0; 1 Mbp R = 14 / 16 / 20:
 // 257 / 270 / 260 ms.
-int swgb::p16_rows_per_lane(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &s) {
+// tiles: an alignment's forward fill.  Its traceback tiles are as high as a strip (128 R rows), and the
+// first round of them runs after the whole fill, kP16TileClocks a row of the side (R = 8 / 12 / 16: 230 / 350 /
+// 458 us at 2,070 MHz).
+int swgb::p16_rows_per_lane(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &s, bool tiles) {
     static constexpr struct { int R; double clk; } kShapes[] = {
 #define SWGB_P16_ROW(R) {R, p16_step_clocks(R)},
         SWGB_P16_SHAPES(SWGB_P16_ROW)
@@ -96,7 +102,7 @@ int swgb::p16_rows_per_lane(const sw_ctx *c, int64_t m, int64_t n, const DevScor
         const double wave = std::max((double)n, c->nsm * kP16ChainSteps * 4);
         const double steps = (double)(last / c->nsm) * wave + (double)(last % c->nsm) * kP16ChainSteps * 4 + (double)n +
                              kP16ChainSteps * std::min<double>(4.0, (double)m / (32.0 * q.R));
-        const double cost = steps * q.clk;
+        const double cost = steps * q.clk + (tiles ? kP16TileClocks * std::min<double>(128.0 * q.R, (double)std::min(m, n)) : 0);
         if (cost < best_cost) { best_cost = cost; best = q.R; }
     }
     return best;

@@ -261,12 +261,13 @@ constexpr int64_t kPackedMinSumVariant = 1024;
 // kPackedMinSum rows plus columns the int32 fill's shorter set-up wins (score:
 // 500 x 500 0.094 against 0.096 ms, 1,000 0.135 against 0.132, 2 kbp 0.221
 // against 0.199, 30 kbp 2.55 against 2.17).
-FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s) {
+FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s,
+                                      bool tiles) {
     if (s.alg != kAlgLocal) {
         FillConfig f = variant_fill_config(c, rows);
         // (the int32 variants run at 8 rows a lane at least: the packed fill from smaller pairs on)
         const int R = !c->fwd_auto ? (c->fwd.P16 && p16_fits(s, c->fwd.R) ? c->fwd.R : 0)
-                                   : (c->p16 && rows + cols >= kPackedMinSumVariant ? p16_rows_per_lane(c, rows, cols, s) : 0);
+                                   : (c->p16 && rows + cols >= kPackedMinSumVariant ? p16_rows_per_lane(c, rows, cols, s, tiles) : 0);
         if (R > 0) {
             f = FillConfig{R, 4, 0, 2, 1};
             f.alg = 1;
@@ -282,7 +283,7 @@ FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t col
         return f;
     }
     if (c->p16 && rows + cols >= kPackedMinSum) {
-        const int R = p16_rows_per_lane(c, rows, cols, s);
+        const int R = p16_rows_per_lane(c, rows, cols, s, tiles);
         if (R > 0) return FillConfig{R, 4, 0, 2, 1};
     }
     return pair_fill_config(c, rows);

@@ -224,6 +224,7 @@ int refill_coarse_tile(sw_ctx *c, const uint8_t *da, const uint8_t *db, int64_t 
 // Sides up to this many cells may take the one-round reconstruction below.
 constexpr int64_t kOneRoundSide = 8192;
 constexpr int64_t kOneRoundPackedSide = 4096;
+constexpr int64_t kTileRows = 20480;
 
 // Tile shape of the traceback fill after forward fill fwd: int32 (bits come from
 // the int32 fill); after the packed fill, whose checkpoint columns are
@@ -236,6 +237,34 @@ FillConfig traceback_config(const sw_ctx *c, const FillConfig &fwd) {
     t.P16 = 0;
     t.alg = fwd.alg;
     return t;
+}
+
+// Forward fill of a pair that is reconstructed in bands (a side above kOneRoundSide).  Local pairs whose sweep is
+// short beside the first round of tiles take the int32 fill, whose tiles of 512 rows at 4 rows a lane take 96 us
+// where those after the packed fill (1,024 rows and more, at 8) take 230 to 458:
+//   * both sides up to kSmallPairSide (int32 tiles of 512 rows), at least 1,000 columns and up to 12,288 rows, or 10,240
+//     with the pair profile, whose sweep is the faster one.  Packed / int32, us: protein 200 x 10,000 800 / 646,
+//     8,300 x 3,000 799 / 644, 10,000 x 10,000 1,127 / 1,055, 12,000 x 1,000 668 / 629; DNA 1,000 x 10,000 829 / 721,
+//     10,000 x 10,000 1,088 / 1,056, beyond the line 12,000 x 12,000 1,226 / 1,295; fewer columns 8,300 x 500
+//     450 / 513;
+//   * more columns and few rows (one or a few strips): up to 3,072 rows (protein 200 x 20,000 1,304 / 1,186, 3,000 x
+//     20,000 1,431 / 1,404, 3,000 x 60,000 3,477 / 3,430), with the pair profile up to 512 rows and 10,240,000 cells (DNA
+//     200 x 20,000 1,240 / 1,186, 300 x 28,000 1,639 / 1,603, beyond the line 500 x 25,000 1,504 / 1,523).
+// Local and overlap pairs of up to kTileRows rows on the packed fill count the tiles in the choice of its rows
+// a lane (protein 16,000 x 3,000 1,113 -> 875, overlap 1,294 -> 977; DNA 20,000 x 1,500 851 -> 842, beyond the line
+// 24,000 x 1,500 903 -> 930).  Elsewhere the choice by the strip chain alone
+// stands: with the tiles counted there too, DNA 200,000 x 50,000 moved to a shape with a second wave, 7.3 -> 11.6 ms,
+// and a tall global pair, whose path runs down a border through every tile row, took more bands (10,000 x 1,500
+// 1,988 -> 2,655).
+FillConfig banded_fill_config(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &ds) {
+    if (c->fwd_auto && ds.alg == kAlgLocal) {
+        const bool pair = p16_pair_profile(ds.K);
+        const bool near = std::max(m, n) <= kSmallPairSide && n >= 1000 && m <= (pair ? 10240 : 12288);
+        const bool wide = n > kSmallPairSide && (pair ? m <= 512 && m * n <= 10240000 : m <= 3072);
+        if (near || wide) return pair_fill_config(c, m);
+    }
+    const bool tiles = m <= kTileRows && (ds.alg == kAlgLocal || ds.alg == kAlgOverlap);
+    return pair_fill_config_for(c, m, n, ds, tiles);
 }
 
 // Tile side of a small pair's reconstruction: a multiple of both fills' strip
@@ -461,7 +490,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     // tiles are BT x BT; BT is a multiple of both fills' strip heights, so
     // checkpoint rows fall on forward-strip bottoms and tiles hold whole
     // traceback strips
-    const FillConfig fwd = pair_fill_config_for(c, m, n, ds);
+    const FillConfig fwd = banded_fill_config(c, m, n, ds);
     const int sw = pair_strip_warps(c, fwd, m);
     const int HC = sw * 32 * fwd.R;
     const FillConfig tbc = traceback_config(c, fwd);

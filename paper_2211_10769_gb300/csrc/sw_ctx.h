@@ -109,13 +109,15 @@ int map_kernel_error(int e);
 int fill_rows_per_strip(const FillConfig &cfg);
 int pair_strip_warps(const sw_ctx *c, const FillConfig &cfg, int64_t rows);
 FillConfig pair_fill_config(const sw_ctx *c, int64_t rows);
-FillConfig pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s);   // picks P16 where exact
-int p16_rows_per_lane(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &s);
+FillConfig pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s,
+                                bool tiles = false);   // picks P16 where exact; tiles: traceback tiles follow (sw_align)
+int p16_rows_per_lane(const sw_ctx *c, int64_t m, int64_t n, const DevScoring &s, bool tiles);
 // the packed checkpoint columns of tasks with FillTask::straight brought to one column (R: the writer's rows a lane)
 int launch_straighten(sw_ctx *c, int R, bool local, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc);
 int launch_straighten_variant(sw_ctx *c, int R, const FillTask *tasks, int ntasks, int max_rows, const DevScoring *sc);
 int launch_fill16_variant(sw_ctx *c, const FillConfig &cfg, int mode, const FillLaunch &L, int K, long long tickets);
 bool p16_fits(const DevScoring &s, int R);
+bool p16_pair_profile(int K);              // the pair profile at 8 rows a lane fits K residue codes (else int16)
 int launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const FillLaunch &L, int K, long long tickets);
 int launch_fill16_batch(sw_ctx *c, const FillConfig &cfg, const FillLaunch &L, int K, long long tickets);
 // the global, semi-global and overlap algorithms: 8 or 16 rows a lane, four compute warps

@@ -542,6 +542,31 @@ def test_packed_base_moves(packed_ctx, oracle_mod):
     _align_case(packed_ctx, oracle_mod, a, W.mutate(a, 20, W.BASE_SEED + 8611), S, o, e)
 
 
+@pytest.mark.parametrize("letters,m,n", [
+    ("protein", 8193, 999), ("protein", 8193, 1000), ("protein", 12288, 1001), ("protein", 12289, 1000),
+    ("dna", 10240, 1000), ("dna", 10241, 1500), ("protein", 200, 8193), ("dna", 1000, 16384), ("protein", 3072, 16385),
+    ("protein", 3073, 16385), ("dna", 512, 20000), ("dna", 512, 20001), ("dna", 513, 16385), ("dna", 20480, 2100),
+    ("dna", 20481, 2100), ("protein", 256, 3000), ("protein", 257, 3000)])
+def test_either_side_of_the_fills_lines(oracle_mod, letters, m, n):
+    """Pairs on both sides of every line between the packed and the int32 forward fill of an alignment in
+    bands, through a context without overrides."""
+    from paper_2211_10769_gb300 import binding
+    dna = letters == "dna"
+    sc = W.dna_scoring() if dna else W.protein_scoring()
+    a = W.uniform_dna(m, W.BASE_SEED + 8670 + n) if dna else W.random_protein(m, W.BASE_SEED + 8670 + n)
+    q = min(m, n)
+    core = W.mutate(a[(m - q) // 2:(m + q) // 2], 4 if dna else 20, W.BASE_SEED + 8671 + m)[:n - 7]
+    rest = n - len(core)
+    flank = W.uniform_dna(rest, 3) if dna else W.random_protein(rest, 3)
+    b = np.concatenate([flank[:rest // 2], core, flank[rest // 2:]])
+    c = binding.Context(0)
+    try:
+        _score_case(c, oracle_mod, a, b, sc.matrix, sc.gap_open, sc.gap_extend)
+        _align_case(c, oracle_mod, a, b, sc.matrix, sc.gap_open, sc.gap_extend)
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("tb", ["16,8", "10,4", "8,8"])
 def test_traceback_overrides_after_a_packed_fill(oracle_mod, monkeypatch, tb):
     """A traceback shape that is not built gives way to one that is; blocks of eight warps are built at 8
