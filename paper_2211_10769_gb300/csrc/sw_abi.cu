@@ -253,6 +253,7 @@ FillConfig swgb::pair_fill_config(const sw_ctx *c, int64_t rows) {
 }
 
 constexpr int64_t kPackedMinSum = 2048;
+constexpr int64_t kPackedMinRows = 257;
 constexpr int64_t kPackedMinSumVariant = 1024;
 
 // Tile shape of a single-pair fill with scoring s: the packed 16-bit fill
@@ -260,7 +261,10 @@ constexpr int64_t kPackedMinSumVariant = 1024;
 // p16_rows_per_lane picks; else the int32 fill of pair_fill_config.  Below
 // kPackedMinSum rows plus columns the int32 fill's shorter set-up wins (score:
 // 500 x 500 0.094 against 0.096 ms, 1,000 0.135 against 0.132, 2 kbp 0.221
-// against 0.199, 30 kbp 2.55 against 2.17).
+// against 0.199, 30 kbp 2.55 against 2.17).  With the int16 profile (larger alphabets) it also keeps the
+// pairs of less than kPackedMinRows rows, one warp of either fill's strip: protein, packed against int32,
+// 64 x 3,000 199 against 182 us, 200 x 3,000 196 against 185, 64 x 100,000 4.99 against 4.85 ms, and beyond the line
+// 500 x 8,000 446 against 448, 1,000 x 8,000 459 against 467.
 FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t cols, const DevScoring &s,
                                       bool tiles) {
     if (s.alg != kAlgLocal) {
@@ -282,7 +286,7 @@ FillConfig swgb::pair_fill_config_for(const sw_ctx *c, int64_t rows, int64_t col
         if (!f.P16 && f.R != 4 && f.R != 8 && f.R != 12 && f.R != 16) f.R = 8;   // a shape of the packed fill only
         return f;
     }
-    if (c->p16 && rows + cols >= kPackedMinSum) {
+    if (c->p16 && rows + cols >= kPackedMinSum && (rows >= kPackedMinRows || p16_pair_profile(s.K))) {
         const int R = p16_rows_per_lane(c, rows, cols, s, tiles);
         if (R > 0) return FillConfig{R, 4, 0, 2, 1};
     }
