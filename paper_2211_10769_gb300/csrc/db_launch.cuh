@@ -92,9 +92,14 @@ int resident_blocks(sw_ctx *c, int codes, int m, int *out) {
     return SW_OK;
 }
 
-// A tile shape and what can be done with it; `codes`: the database's residue codes (DbView::pad).
+// A tile shape, what it measures and what can be done with it; `codes`: the database's residue codes (DbView::pad).
+//   gcups: 10^9 cells a second, padding rows included, all SMs full (60,000 subjects of 360 residues);
+//   clk1, clk: clocks of a step of a warp that has its SM for itself (subjects of 40,000 columns), for
+//   queries of one pass and of several, whose boundary row goes through memory.
+// (GB300, 152 SMs, 2,070 MHz.)
 struct DbShape {
     int R, W, G;
+    double gcups, clk1, clk;
     size_t (*profile_bytes)(int codes, int m);
     int (*scratch)(sw_ctx *c, int codes, int m, int maxlen, int *nslots, size_t *row_bytes, size_t *slot_bytes);
     int (*launch)(sw_ctx *c, const DbJob *jobs, int njobs, int nblocks, const DbView &D, int codes, int m, const DbBufs &B);
@@ -102,12 +107,13 @@ struct DbShape {
 };
 
 template <int R, int W, int G>
-DbShape db_shape_ops() {
-    return DbShape{R, W, G, db_profile_bytes<R, G>, db_scratch<R, W, G>, launch_db<R, W, G>, resident_blocks<R, W, G>};
+DbShape db_shape_ops(double gcups, double clk1, double clk) {
+    return DbShape{R, W, G, gcups, clk1, clk, db_profile_bytes<R, G>, db_scratch<R, W, G>, launch_db<R, W, G>, resident_blocks<R, W, G>};
 }
 
 DbShape db_shape_a(int k);      // the shapes of each translation unit
 DbShape db_shape_b(int k);
 DbShape db_shape_c(int k);
+DbShape db_shape_d(int k);
 
 }  // namespace swgb

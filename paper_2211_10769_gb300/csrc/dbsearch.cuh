@@ -259,8 +259,11 @@ __device__ __forceinline__ void db_step(DbLane<R> &st, int s, int gl, int n, con
     st.topv = topn;
 }
 
+// Blocks of a shape an SM holds: as many as its registers leave room for.
+constexpr int db_blocks_per_sm(int R, int W) { return W >= 16 ? 1 : (R > 16 ? 2 : (R >= 12 ? 3 : 4)); }
+
 template <int R, int W, bool OVERSUB, int G = 32>
-__global__ void __launch_bounds__(W * 32, W >= 16 ? 1 : (R > 16 ? 2 : (R >= 12 ? 3 : 4)))
+__global__ void __launch_bounds__(W * 32, db_blocks_per_sm(R, W))
 db_s16x2_kernel(const DbJob *__restrict__ jobs, int njobs, const DbView D,
                 const DevScoring *__restrict__ scorings, uint2 *__restrict__ scratch)
 {

@@ -94,6 +94,7 @@ struct sw_ctx {
     swgb::HostBuf stage_b;
     cudaStream_t side = nullptr;
     cudaEvent_t side_go = nullptr, side_done = nullptr;
+    int db_forced = -1;               // SWGB_DB_SHAPE: the database search's tile shape, where its profile fits
     bool lookahead = true;
     std::vector<std::pair<long long, swgb::FillConfig>> batch_tune;   // autotuned tile shape per size class
     swgb::KernelTimer timer;
@@ -158,7 +159,13 @@ int db_rescore(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m, const D
                const std::vector<int32_t> &flagged, int32_t *dscores);
 int db_topk(sw_ctx *c, const int32_t *dscores, int64_t nseq, int k, int2 *dout);
 // (codes: the database's residue codes, DbView::pad)
-int db_shape(int codes, int m);            // tile shape (index) for a query of m residues
+// What a launch sweeps: pairs of subjects, their columns (of the longer subject each) and the longest one's.  Queries
+// that run at the same time count in each other's pairs and columns, by their residues.
+struct DbLoad {
+    double pairs, cols;
+    int maxlen;
+};
+int db_shape(const sw_ctx *c, int codes, int m, const DbLoad &ld);   // tile shape (index) for a query of m residues
 int db_shape_warps(int shape);
 int db_shape_rows(int shape);              // query rows per pass
 int db_resident_blocks_shape(sw_ctx *c, int shape, int codes, int m, int *out);
@@ -177,5 +184,6 @@ int db_scratch_shape(sw_ctx *c, int shape, int codes, int m, int maxlen, size_t 
 int db_view(const sw_db *db, DbView *v, int64_t *nseq, int32_t *max_code, int *device);
 int db_chunk_maxlen(const sw_db *db, int32_t pair0, int32_t pair1);
 int64_t db_total_residues(const sw_db *db);
+int64_t db_pair_columns(const sw_db *db);
 
 }  // namespace swgb

@@ -8,6 +8,7 @@
 #include "aux_kernels.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <numeric>
@@ -22,6 +23,7 @@ struct sw_db {
     int32_t npairs = 0;
     int32_t maxlen = 0;
     int32_t max_code = -1;
+    int64_t pcols = 0;                  // columns of all pairs
     std::vector<int64_t> off;           // host copy of the offsets
     std::vector<int32_t> hpairs;        // host copy of the length-sorted pairs
     DevBuf res, doff, pairs, pres, poff;   // pres / poff: interleaved residues of every pair
@@ -40,24 +42,25 @@ static __global__ void max_code_kernel(const uint8_t *s, long long len, int *out
 
 // Tile shapes of the packed search: rows a lane, warps a block and lanes a
 // wavefront (16: two wavefronts a warp).  A query is padded to whole passes of
-// 16 R rows.  A lane's fixed per-step work (two shuffles, lane 0's row above,
-// the next residues) is shared by its R rows, so a query wants the most rows a
-// lane whose passes it fills: 144 residues take one pass at R = 9, 464 one at
+// G R rows.  A lane's fixed per-step work (two shuffles, lane 0's row above,
+// the next residues) is shared by its R rows, so a large database wants the most rows a
+// lane whose passes the query fills: 144 residues take one pass at R = 9, 464 one at
 // R = 29, 1,000 two at R = 32.  32 lanes a wavefront (1,000: one pass of 32 x 32
-// rows, 5,690 against 5,820 GCUPS) pay more for their skew than a second pass
+// rows, 5,690 against 5,820 GCUPS) pay more for their skew there than a second pass
 // costs; four wavefronts of 8 lanes (144: 4,190 against 4,960) lose to their bank
 // conflicts and uneven pairs.  Blocks of 8 warps, two (above 16 rows a lane: 128
-// registers) to four an SM; queries whose profile would not leave room for two
-// blocks take blocks of 16 warps, one an SM, with 32 lanes a wavefront (5,478
+// registers) to four an SM; long queries, whose profile would not leave room for two
+// blocks, take blocks of 16 warps, one an SM, with 32 lanes a wavefront (5,478
 // residues: 5,760 GCUPS at R = 29, against 5,270 in two wavefronts a warp, whose
 // twice as many boundary rows outgrow the L1 cache that the profile leaves).
-constexpr int kDbA = 6, kDbB = 5, kDbC = 6;        // shapes per translation unit
-constexpr int kDbShapeCount = kDbA + kDbB + kDbC;
-constexpr int kDbWide0 = kDbA + kDbB + 2;          // the first of the one-block-an-SM shapes
-constexpr size_t kDbNarrowProfileMax = 100 * 1024; // profile bytes of a two-blocks-an-SM shape at most
-// cost model of a shape (db_shape), from measured GCUPS of every shape: a lane's fixed per-step cost in
-// rows' worth, and a pass boundary in rows
-constexpr double kDbStepRows = 2.0, kDbPassRows = 2;
+// A small database is bound by its longest subject, whose steps follow one another:
+// there 32 lanes a wavefront win, whose steps are shorter (a warp of two wavefronts loads two
+// pairs' profile rows, in conflict) and which need half the passes: 8,000 subjects (the longest of
+// 3,574) x 1,000: 2,632 us at 32 rows in 16 lanes, 1,295 in 32; one subject x 4,000: 772 and 336 us.
+constexpr int kDbA = 6, kDbB = 5, kDbC = 6, kDbD = 8;   // shapes per translation unit
+constexpr int kDbShapeCount = kDbA + kDbB + kDbC + kDbD;
+constexpr int kDbCompact = kDbA + kDbB + kDbC - 1;      // 16 rows a lane in 32 lanes, 16 warps: the last resort
+constexpr size_t kDbNarrowProfileMax = 100 * 1024;      // profile bytes of a two-blocks-an-SM shape at most
 
 const DbShape &shape_at(int s) {
     static const auto all = [] {
@@ -65,34 +68,47 @@ const DbShape &shape_at(int s) {
         for (int k = 0; k < kDbA; ++k) v.push_back(db_shape_a(k));
         for (int k = 0; k < kDbB; ++k) v.push_back(db_shape_b(k));
         for (int k = 0; k < kDbC; ++k) v.push_back(db_shape_c(k));
+        for (int k = 0; k < kDbD; ++k) v.push_back(db_shape_d(k));
         return v;
     }();
     return all[(size_t)s];
 }
 
+// Seconds a shape takes for a query of m residues, by its measured rate and step (DbShape): the work over the chip's
+// rate and the longest pair's chain, in a norm close to their larger one.  Blocks of 16 warps have twice the
+// chains on an SM.  The exponent and the small factors are fitted to every shape's times for 25 query lengths from
+// 30 to 8,000 against eight databases of 1 to 500,000 subjects: the choice is on average 0.1% and at most 6%
+// above the fastest shape (by the work alone 30%, and 2.6 times the time at worst).
+double db_shape_time(const DbShape &q, int m, const DbLoad &ld, int nsm) {
+    const int rows = q.G * q.R, passes = (m + rows - 1) / rows;
+    const double blocks = std::min<double>((double)db_blocks_per_sm(q.R, q.W) * nsm, std::ceil(ld.pairs / q.W));
+    const double used = std::max(1.0, std::min<double>(nsm, blocks));
+    const double work = (double)passes * rows * 2.0 * ld.cols / (q.gcups * 1e9) * (nsm / used) *
+                        (q.G == 16 ? 1.0 : (q.W >= 16 ? 1.02 : 0.98));
+    const double chains = std::min<double>(q.W, ld.pairs * q.G / 32.0);     // at once in a block
+    // (two wavefronts a warp: the longest pair goes on without its neighbour at the end, at a checked step)
+    const double clk = (passes == 1 ? q.clk1 : q.clk) + (q.G == 16 ? 15 : 0);
+    const double chain = (double)passes * (ld.maxlen + q.G) * clk / 2.07e9 * std::max(1.0, 1.25 * chains / 8);
+    return std::sqrt(std::sqrt(work * work * work * work + chain * chain * chain * chain));
+}
+
 }  // namespace
 
-// The shape for a query of m residues against a database of `codes` residue codes: the least padded work,
-// counting the per-step overhead of a lane and a pass boundary, among the shapes whose profile fits.
-int swgb::db_shape(int codes, int m) {
-    // tuning override: SWGB_DB_SHAPE=<index of a shape>, where its profile fits
-    static const int forced = [] { const char *f = std::getenv("SWGB_DB_SHAPE"); return f ? std::atoi(f) : -1; }();
+// The shape for a query of m residues against a database of `codes` residue codes, of which the launch sweeps
+// ld: the fastest by db_shape_time among the shapes whose profile fits.
+int swgb::db_shape(const sw_ctx *c, int codes, int m, const DbLoad &ld) {
     auto fits = [&](int s) {
         const size_t p = shape_at(s).profile_bytes(codes, m);
-        return s < kDbWide0 ? p <= kDbNarrowProfileMax : (long long)p <= kMaxProfileSmem;
+        return shape_at(s).W < 16 ? p <= kDbNarrowProfileMax : (long long)p <= kMaxProfileSmem;
     };
-    if (forced >= 0 && forced < kDbShapeCount && fits(forced)) return forced;
-    int best = kDbShapeCount - 1;                   // 16 rows a lane: the most compact profile
-    double best_cost = 1e300;
-    bool narrow = false;
+    // tuning override: SWGB_DB_SHAPE=<index of a shape>, where its profile fits
+    if (c->db_forced >= 0 && c->db_forced < kDbShapeCount && fits(c->db_forced)) return c->db_forced;
+    int best = kDbCompact;
+    double best_time = 1e300;
     for (int s = 0; s < kDbShapeCount; ++s) {
-        if (!fits(s) || (narrow && s >= kDbWide0)) continue;
-        if (s < kDbWide0) narrow = true;
-        const DbShape &q = shape_at(s);
-        const int rows = q.G * q.R;
-        const long long passes = (m + rows - 1) / rows;
-        const double cost = (double)passes * (rows * (q.R + kDbStepRows) / q.R + kDbPassRows);
-        if (cost < best_cost) { best_cost = cost; best = s; }
+        if (!fits(s)) continue;
+        const double t = db_shape_time(shape_at(s), m, ld, c->nsm);
+        if (t < best_time) { best_time = t; best = s; }
     }
     return best;
 }
@@ -130,6 +146,8 @@ int swgb::db_view(const sw_db *db, DbView *v, int64_t *nseq, int32_t *max_code, 
     *device = db->device;
     return SW_OK;
 }
+
+int64_t swgb::db_pair_columns(const sw_db *db) { return db->pcols; }
 
 int64_t swgb::db_total_residues(const sw_db *db) { return db->off.empty() ? 0 : db->off.back(); }
 
@@ -185,6 +203,7 @@ extern "C" int sw_db_create(sw_ctx *c, const uint8_t *residues, const int64_t *o
         const int64_t nb = sb >= 0 ? offsets[sb + 1] - offsets[sb] : 0;
         poff[(size_t)p + 1] = poff[(size_t)p] + std::max(na, nb) + 1;
     }
+    db->pcols = poff.back() - db->npairs;
     rc = db->pres.ensure(std::max<size_t>(1, (size_t)poff.back()) * sizeof(uint16_t));
     if (!rc) rc = db->poff.ensure(poff.size() * sizeof(int64_t));
     if (rc) { delete db; return rc; }
@@ -263,7 +282,8 @@ int swgb::db_score_all(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m,
     int rc = SW_ERANGE;
     if (packed_ok) {
         int nblk = 0;
-        const int shape = db_shape(D.pad, (int)m);
+        const DbLoad ld{(double)db->npairs, (double)db->pcols, db->maxlen};
+        const int shape = db_shape(c, D.pad, (int)m, ld);
         rc = db_resident_blocks_shape(c, shape, D.pad, (int)m, &nblk);
         if (!rc) {
             const int W = db_shape_warps(shape);

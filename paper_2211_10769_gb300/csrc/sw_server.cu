@@ -199,7 +199,14 @@ int enqueue_step(sw_server *S, const std::vector<Slot *> &act, InFlight *next, i
     // that pads it least (one shape for all would pad a 100-residue query to a 512-row pass
     // next to a long one); one launch per group
     std::map<int, std::vector<Slot *>> groups;
-    for (Slot *s : act) groups[db_shape(S->view.pad, (int)s->m)].push_back(s);
+    const int maxlen = std::max(1, db_chunk_maxlen(S->db, p0, p0 + 1));   // pairs are sorted longest first
+    double residues = 0;
+    for (Slot *s : act) residues += (double)s->m;
+    for (Slot *s : act) {
+        const double all = residues / std::max<double>(1.0, (double)s->m);   // the step's work in this query's
+        const DbLoad ld{chunk_pairs * all, (double)db_pair_columns(S->db) / stride * all, maxlen};
+        groups[db_shape(c, S->view.pad, (int)s->m, ld)].push_back(s);
+    }
     std::vector<DbJob> jobs;
     struct Launch { int shape, job0, njobs, nblocks, maxm; };
     std::vector<Launch> launches;
@@ -237,7 +244,7 @@ int enqueue_step(sw_server *S, const std::vector<Slot *> &act, InFlight *next, i
     }
     const int ng = chunk_pairs > 0 ? (int)launches.size() : 0;
     DbView v = S->view;
-    v.maxlen = std::max(1, db_chunk_maxlen(S->db, p0, p0 + 1));     // pairs are sorted longest first
+    v.maxlen = maxlen;
     while ((int)S->gstreams.size() < ng) {
         cudaStream_t t = nullptr;
         CU(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));

@@ -82,6 +82,30 @@ def test_shape_edges(ctx, oracle_mod, codes):
         _check_all(ctx, oracle_mod, db, subjects, g.integers(0, 24, size=m).astype(np.uint8), sc, k=5)
 
 
+SHAPES = [(r, 16) for r in (4, 7, 9, 11, 13, 16, 18, 20, 22, 24, 26, 29, 32)] + \
+    [(32, 32), (29, 32), (24, 32), (16, 32), (6, 16), (4, 32), (8, 32), (12, 32), (16, 32), (24, 32), (32, 32), (12, 16)]
+
+
+@pytest.mark.parametrize("shape", range(len(SHAPES)))
+def test_forced_shapes(oracle_mod, monkeypatch, shape):
+    """Every tile shape (by its index) at one pass less a row, exactly one, one row more and two and a half passes,
+    over subjects shorter than, equal to and longer than a wavefront, an odd number of them."""
+    from paper_2211_10769_gb300 import binding
+    monkeypatch.setenv("SWGB_DB_SHAPE", str(shape))
+    c = binding.Context(0)
+    try:
+        sc = W.protein_scoring()
+        g = np.random.default_rng(W.BASE_SEED + 790 + shape)
+        subjects = [g.integers(0, 20, size=int(n)).astype(np.uint8) for n in (1, 15, 16, 17, 31, 32, 33, 90, 333, 334, 800)]
+        db = _db(c, subjects)
+        rows = SHAPES[shape][0] * SHAPES[shape][1]
+        for m in (rows - 1, rows, rows + 1, 2 * rows + rows // 2):
+            _check_all(c, oracle_mod, db, subjects, g.integers(0, 24, size=m).astype(np.uint8), sc, k=5)
+        db.close()
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("nseq", [1, 2, 3, 5, 7])
 def test_tiny_databases_short_queries(ctx, oracle_mod, nseq):
     """One to four subject pairs against queries that take the two-wavefront
