@@ -166,6 +166,7 @@ struct DbLoad {
     int maxlen;
 };
 int db_shape(const sw_ctx *c, int codes, int m, const DbLoad &ld);   // tile shape (index) for a query of m residues
+double db_shape_seconds(const sw_ctx *c, int shape, int m, const DbLoad &ld);   // the time it is taken for
 int db_shape_warps(int shape);
 int db_shape_rows(int shape);              // query rows per pass
 int db_resident_blocks_shape(sw_ctx *c, int shape, int codes, int m, int *out);

@@ -113,6 +113,10 @@ int swgb::db_shape(const sw_ctx *c, int codes, int m, const DbLoad &ld) {
     return best;
 }
 
+double swgb::db_shape_seconds(const sw_ctx *c, int shape, int m, const DbLoad &ld) {
+    return db_shape_time(shape_at(shape), m, ld, c->nsm);
+}
+
 int swgb::db_resident_blocks_shape(sw_ctx *c, int shape, int codes, int m, int *out) {
     return shape_at(shape).resident(c, codes, m, out);
 }
@@ -285,6 +289,12 @@ int swgb::db_score_all(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m,
         const DbLoad ld{(double)db->npairs, (double)db->pcols, db->maxlen};
         const int shape = db_shape(c, D.pad, (int)m, ld);
         rc = db_resident_blocks_shape(c, shape, D.pad, (int)m, &nblk);
+        // A long query against few subjects: one int32 task a subject puts all SMs on the query's rows, where the
+        // packed search has a warp for each pair.  270 us and 590 GCUPS as measured (9,000 residues, packed / int32: 1 subject 0.79 /
+        // 0.29 ms, 30 2.64 / 0.38, 1,000 8.5 / 5.5, 8,000 13.8 / 43.2)
+        if (!rc && c->db_forced < 0 &&
+            db_shape_seconds(c, shape, (int)m, ld) > 270e-6 + (double)m * (double)db_total_residues(db) / 590e9)
+            rc = SW_ERANGE;
         if (!rc) {
             const int W = db_shape_warps(shape);
             nblk = std::max(1, std::min(nblk, (db->npairs + W - 1) / W));
@@ -292,7 +302,7 @@ int swgb::db_score_all(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m,
         }
     }
     if (rc == SW_ERANGE) {
-        // the packed kernel cannot take this query / scoring: score every subject in int32
+        // the packed kernel cannot take this query or scoring, or not as fast: score every subject in int32
         flagged.resize((size_t)db->nseq);
         std::iota(flagged.begin(), flagged.end(), 0);
     } else {

@@ -82,6 +82,19 @@ def test_shape_edges(ctx, oracle_mod, codes):
         _check_all(ctx, oracle_mod, db, subjects, g.integers(0, 24, size=m).astype(np.uint8), sc, k=5)
 
 
+def test_long_query_few_subjects(ctx, oracle_mod):
+    """Queries on both sides of the line above which a few subjects are scored in int32 tasks, up to one that the
+    packed profile has no room for with this database's codes."""
+    sc = W.protein_scoring()
+    g = np.random.default_rng(W.BASE_SEED + 795)
+    subjects = [g.integers(0, 20, size=int(n)).astype(np.uint8) for n in (700, 3, 1, 333, 90, 1500)]
+    db = _db(ctx, subjects)
+    for m in (500, 1500, 2500, 4000, 9000, 10000):
+        q = np.concatenate([W.mutate(subjects[5], 20, W.BASE_SEED + 796), W.random_protein(m, W.BASE_SEED + m)])[:m]
+        _check_all(ctx, oracle_mod, db, subjects, q, sc, k=4)
+    db.close()
+
+
 SHAPES = [(r, 16) for r in (4, 7, 9, 11, 13, 16, 18, 20, 22, 24, 26, 29, 32)] + \
     [(32, 32), (29, 32), (24, 32), (16, 32), (6, 16), (4, 32), (8, 32), (12, 32), (16, 32), (24, 32), (32, 32), (12, 16)]
 
