@@ -243,7 +243,9 @@ int sw_score_noalloc(void *cuda_stream, const uint8_t *a, int64_t m, const uint8
  *                      local bins whose scoring keeps it exact, packed 16-bit
  *                      lanes of 8, 12 or 16 rows; where it does not, also
  *                      int32 lanes of 12 and 16 rows.
- *                      Without it a bin takes packed lanes where exact.
+ *                      Without it a bin takes packed lanes where exact, but
+ *                      int32 ones where no pair has more than 800 rows and
+ *                      columns together.
  * sw_batch_run writes npairs hits (host memory).  A plan belongs to its
  * context and must be destroyed before it.
  */

@@ -66,6 +66,7 @@ bool is_candidate(const FillConfig &f, const DevScoring &s) {
 }
 
 constexpr int64_t kShortRows = 1024;      // row classes: queries up to this many rows, and longer
+constexpr int64_t kShortPair = 800;       // rows and columns of the pairs that keep the int32 fill
 
 // ticket counter of bin b starts at the bin's first ticket
 static __global__ void set_counters_kernel(unsigned long long *ctr, const long long *base, int nbins) {
@@ -422,9 +423,19 @@ extern "C" int sw_batch_create(sw_ctx *c, int64_t npairs, const uint8_t *a_res, 
         std::stable_sort(bins.begin(), bins.end(), [&](const Bin &x, const Bin &y) { return bin_cells(x) > bin_cells(y); });
         for (Bin &bin : bins) {
             bin.cfg = c->bat;
-            // without autotuning: the packed fill where it is exact (10,000 uneven pairs: within a few percent of the tuned plan)
+            // without autotuning: the packed fill where it is exact (10,000 uneven pairs: within a few percent of the tuned
+            // plan), but for short pairs the int32 fill, whose set-up is shorter (DNA, int32 / packed, us: 1 pair of 20 to 60 residues
+            // 31 / 41, 32 of 60 to 200 49 / 54, 600 of 100 to 400 216 / 230, beyond the line 4 of 300 to 1,000 107 / 93); and 12 rows a
+            // lane in place of 8 where the longer queries fill the SMs more than twice over (8 / 12 rows: 1 pair of 1,025 to 3,000
+            // 153 / 177, 64 of 1,100 to 9,000 723 / 762, beyond 256 of 1,025 to 3,000 558 / 549)
             const DevScoring &bsc = B->scorings[(size_t)bin.sidx];
-            if (c->bat_auto && p16_fits(bsc, 12)) bin.cfg = FillConfig{bin.rclass ? 12 : 8, 4, 0, 0, fold_open(bsc) ? 2 : 1};
+            int64_t longest = 0, strips = 0;
+            for (int32_t p : bin.pairs) {
+                longest = std::max(longest, B->m[(size_t)p] + B->n[(size_t)p]);
+                strips += (B->m[(size_t)p] + kShortRows - 1) / kShortRows;
+            }
+            if (c->bat_auto && longest > kShortPair && p16_fits(bsc, 12))
+                bin.cfg = FillConfig{bin.rclass && strips > 2 * c->nsm ? 12 : 8, 4, 0, 0, fold_open(bsc) ? 2 : 1};
             if (bin.cfg.P16 && ((bin.cfg.W != 4 && bin.cfg.W != 2) || !p16_fits(B->scorings[(size_t)bin.sidx], bin.cfg.R)))
                 bin.cfg.P16 = 0;
             // the int8 profile (launch_fill16_batch): 8 and 12 rows, S + open within int8

@@ -126,6 +126,22 @@ def test_batch_int8_profile_at_16_rows(oracle_mod, monkeypatch, Wc):
         c.close()
 
 
+@pytest.mark.parametrize("rows,cols,bits", [(400, 400, 32), (400, 401, 16)])
+def test_short_pairs_keep_int32(ctx, oracle_mod, rows, cols, bits):
+    """An untuned bin whose longest pair has 800 rows and columns runs in int32 lanes, one of 801 in packed ones."""
+    from paper_2211_10769_gb300 import binding
+    sc = _scorings()
+    pairs = [(W.random_protein(n, k), W.mutate(W.random_protein(n, k), 20, k, p_sub=0.3), 1) for k, n in enumerate((1, 30, 200, 399))]
+    a = W.uniform_dna(rows, W.BASE_SEED + 12500)
+    pairs += [(a, W.uniform_dna(cols, W.BASE_SEED + 12501), 0), (a[:3], a[1:60], 0)]
+    c = binding.Context(0)                   # (no tuned shapes)
+    plan = binding.Batch(c, pairs, sc, flags=0)
+    assert [lb for _, _, lb, n in plan.bins() if n == 2] == [bits]
+    assert [(h.score, h.a_end, h.b_end) for h in plan.run()] == _oracle_hits(oracle_mod, pairs, sc)
+    plan.close()
+    c.close()
+
+
 @pytest.mark.parametrize("flags", [0, 2, 3])
 def test_tuned_shapes_and_another_scoring(oracle_mod, flags):
     """A context that has tuned a plan meets the same pairs under scorings of the same alphabet that
