@@ -481,13 +481,23 @@ extern "C" int sw_batch_create(sw_ctx *c, int64_t npairs, const uint8_t *a_res, 
                 if (!is_candidate(cand, B->scorings[(size_t)B->bins[k].sidx])) continue;
                 B->bins[k].cfg = cand;
                 rc = build_plan(B);
-                if (!rc) rc = cudaEventRecord(e0, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
-                if (!rc) rc = enqueue_run(B);
-                if (!rc) rc = cudaEventRecord(e1, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
-                if (!rc) rc = cudaStreamSynchronize(B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
-                float ms = 0;
-                if (!rc) rc = cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess ? SW_OK : SW_ECUDA;
+                // a kernel's first run also loads it, and a run of less than a millisecond varies by a quarter: the
+                // best of two and of three (a single run picked 41 us in place of 30 for one pair of 20 to 60 residues)
+                const long long key = (&cand - kCandidates) * 64 + B->scorings[(size_t)B->bins[k].sidx].K;
+                const bool fresh = std::find(c->batch_ran.begin(), c->batch_ran.end(), key) == c->batch_ran.end();
+                float ms = 1e30f;
+                for (int run = 0, runs = fresh ? 2 : 1; !rc && run < runs; ++run) {
+                    rc = cudaEventRecord(e0, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
+                    if (!rc) rc = enqueue_run(B);
+                    if (!rc) rc = cudaEventRecord(e1, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
+                    if (!rc) rc = cudaStreamSynchronize(B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
+                    float t = 0;
+                    if (!rc) rc = cudaEventElapsedTime(&t, e0, e1) == cudaSuccess ? SW_OK : SW_ECUDA;
+                    ms = std::min(ms, t);
+                    if (ms < 1.0f) runs = 3;
+                }
                 if (rc) break;
+                if (fresh) c->batch_ran.push_back(key);
                 if (ms < best) { best = ms; pick = cand; }
             }
             B->bins[k].cfg = pick;
