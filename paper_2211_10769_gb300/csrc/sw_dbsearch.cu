@@ -325,7 +325,9 @@ int swgb::db_rescore(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m, c
                      const std::vector<int32_t> &flagged, int32_t *dscores) {
     const int K = ds.K;
     RC(upload_scorings(c, {ds}));
-    const int HC = fill_rows_per_strip(c->bat);
+    // (SWGB_BATCH may name a packed shape, which need not be exact for this scoring)
+    const FillConfig cfg = c->bat.P16 ? FillConfig{8, 4} : c->bat;
+    const int HC = fill_rows_per_strip(cfg);
     std::vector<FillTask> tasks;
     tasks.reserve(flagged.size());
     long long tickets = 0;
@@ -353,7 +355,7 @@ int swgb::db_rescore(sw_ctx *c, const sw_db *db, const uint8_t *dq, int64_t m, c
         if (n == 0) { u.nstrips = 0; }
         tasks.push_back(u);
     }
-    RC(run_fill(c, c->bat, kModeScore, fold_open(ds), tasks, tickets, K));
+    RC(run_fill(c, cfg, kModeScore, fold_open(ds), tasks, tickets, K));
     const int nt = (int)tasks.size();
     RC(c->result.ensure((size_t)nt * sizeof(int4)));
     reduce_candidates_kernel<<<(nt + 7) / 8, 256, 0, c->stream>>>(static_cast<const FillTask *>(c->tasks.p), nt,

@@ -192,6 +192,26 @@ def test_half_beside_a_saturated_one(ctx, oracle_mod, go, ge):
         assert scores.tolist() == want.tolist()
 
 
+@pytest.mark.parametrize("shape", ["12,4,1", "8,2,2"])
+def test_rescoring_under_a_packed_batch_override(oracle_mod, monkeypatch, shape):
+    """The rescoring of saturated subjects is an int32 fill whatever shape batches are told to take: here
+    the packed one, with scores it is not exact for."""
+    from paper_2211_10769_gb300 import binding
+    monkeypatch.setenv("SWGB_BATCH", shape)
+    c = binding.Context(0)
+    try:
+        S = np.full((24, 24), -60, np.int8)
+        np.fill_diagonal(S, 90)
+        a = W.random_protein(900, W.BASE_SEED + 798)
+        subjects = [a, W.mutate(a, 20, W.BASE_SEED + 799, p_sub=0.05), W.random_protein(300, W.BASE_SEED + 800)]
+        want = oracle_mod.db_scores(a, subjects, S, 30, 2)
+        assert max(want) > 32767
+        hits, scores = _db(c, subjects).search(a, S, 30, 2, k=2, all_scores=True)
+        assert scores.tolist() == want.tolist()
+    finally:
+        c.close()
+
+
 def test_degenerate_databases(ctx, oracle_mod):
     sc = W.protein_scoring()
     q = W.random_protein(200, W.BASE_SEED + 760)
