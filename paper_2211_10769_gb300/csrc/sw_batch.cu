@@ -308,6 +308,24 @@ int finish_run(sw_batch *B, sw_hit *out) {
     return SW_OK;
 }
 
+// Launches the fill of shape f without strips, so that its kernel is loaded.
+int load_fill(sw_batch *B, const FillConfig &f, const DevScoring &sc) {
+    sw_ctx *c = B->c;
+    DevBuf none;                       // the ticket counter and the error word
+    RC(none.ensure(64));
+    CU(cudaMemsetAsync(none.p, 0, 64, B->stream));
+    FillLaunch L{};
+    L.ticket = static_cast<unsigned long long *>(none.p);
+    L.err = static_cast<int *>(none.p) + 4;
+    L.total = 0;
+    const cudaStream_t saved = c->stream;
+    c->stream = B->stream;
+    const int rc = launch_fill(c, f, kModeScore, fold_open(sc), L, sc.K, 1);
+    c->stream = saved;
+    CU(cudaStreamSynchronize(B->stream));
+    return rc;
+}
+
 // Class of a bin for the autotune cache: its alphabet, which shapes its scoring is exact
 // for (all that is_candidate asks about it), row class, and log2 of its cells and of its
 // pair count.
@@ -481,12 +499,12 @@ extern "C" int sw_batch_create(sw_ctx *c, int64_t npairs, const uint8_t *a_res, 
                 if (!is_candidate(cand, B->scorings[(size_t)B->bins[k].sidx])) continue;
                 B->bins[k].cfg = cand;
                 rc = build_plan(B);
-                // a kernel's first run also loads it, and a run of less than a millisecond varies by a quarter: the
-                // best of two and of three (a single run picked 41 us in place of 30 for one pair of 20 to 60 residues)
-                const long long key = (&cand - kCandidates) * 64 + B->scorings[(size_t)B->bins[k].sidx].K;
-                const bool fresh = std::find(c->batch_ran.begin(), c->batch_ran.end(), key) == c->batch_ran.end();
+                // a kernel's first launch also loads it: one without strips before it is timed; and a run of less than a
+                // millisecond varies by a quarter: the best of three (a single, first run picked 41 us in place of 30 for
+                // one pair of 20 to 60 residues)
+                if (!rc) rc = load_fill(B, cand, B->scorings[(size_t)B->bins[k].sidx]);
                 float ms = 1e30f;
-                for (int run = 0, runs = fresh ? 2 : 1; !rc && run < runs; ++run) {
+                for (int run = 0, runs = 1; !rc && run < runs; ++run) {
                     rc = cudaEventRecord(e0, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
                     if (!rc) rc = enqueue_run(B);
                     if (!rc) rc = cudaEventRecord(e1, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
@@ -497,7 +515,6 @@ extern "C" int sw_batch_create(sw_ctx *c, int64_t npairs, const uint8_t *a_res, 
                     if (ms < 1.0f) runs = 3;
                 }
                 if (rc) break;
-                if (fresh) c->batch_ran.push_back(key);
                 if (ms < best) { best = ms; pick = cand; }
             }
             B->bins[k].cfg = pick;

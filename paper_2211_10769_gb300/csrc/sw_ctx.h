@@ -97,7 +97,6 @@ struct sw_ctx {
     int db_forced = -1;               // SWGB_DB_SHAPE: the database search's tile shape, where its profile fits
     bool lookahead = true;
     std::vector<std::pair<long long, swgb::FillConfig>> batch_tune;   // autotuned tile shape per size class
-    std::vector<long long> batch_ran;                                 // candidates the autotuner has run (and so loaded)
     swgb::KernelTimer timer;
 };
 
