@@ -11,10 +11,11 @@
 // the subjects' columns exactly as in the pairwise fill (bottom H / F to the
 // next lane by shuffle), and longer queries take several passes, the bottom
 // row of one pass feeding the next through a per-warp boundary row in
-// global memory.  All but the longest queries run two independent 16-lane
-// wavefronts per warp instead (G = 16), each over its own pair of subjects, so
-// that a lane holds more rows of the query and the skew of a wavefront is 15
-// steps rather than 31.  The query profile (int8, S + open, all passes) sits in
+// global memory.  Against large databases all but the longest queries run two
+// independent 16-lane wavefronts per warp instead (G = 16), each over its own pair
+// of subjects, so that a lane holds more rows of the query and the skew of a wavefront is 15
+// steps rather than 31; a small database is bound by its longest pair's steps, which are fewer
+// and shorter in 32 lanes.  The query profile (int8, S + open, all passes) sits in
 // shared memory; the two residues' score bytes are merged into one packed
 // register with a single prmt.
 //
@@ -187,8 +188,8 @@ __device__ __forceinline__ int db_prof_byte(int g, int r) {
 // host gives each job blocks in proportion to its work); block: W warps.  A
 // block whose job has no pairs left moves on to the job of the launch with
 // the most work left (same scoring), so that the launch ends balanced.
-// Dynamic shared memory: the query profile, (K + 1) * mpad bytes,
-// mpad = passes * 32 * db_lane_slot(R) (lane slots of whole words).
+// Dynamic shared memory: the query profile, (DbView::pad + 1) * mpad bytes,
+// mpad = passes * G * db_lane_slot(R) (lane slots of whole words).
 // Steps per chunk of the packed fill (steady chunks skip all range tests); 4 for long lanes, whose body of 8
 // steps would be some 2,000 instructions (loops beyond about that fall out of the instruction cache)
 constexpr int db_chunk(int R) { return R <= 16 ? 8 : 4; }

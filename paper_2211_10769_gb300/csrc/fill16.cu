@@ -11,7 +11,9 @@ using namespace swgb;
 
 namespace {
 
-// steps by which a warp trails the one above, and clocks of a step (measured, R = 4 .. 26, one strip)
+// Steps by which a warp trails the one above, and clocks of a step over the sweep (one strip, measured with the pair
+// profile of DNA at the shapes below, and at 4 and 6 rows, which are not built).  The int16 profile's steps are some 5%
+// longer at every shape, which leaves the order of the shapes as it is.
 constexpr double kP16ChainSteps = 105;
 constexpr double kP16TileClocks = 464;
 constexpr double p16_step_clocks(int R) { return R <= 8 ? 70 + 3.3 * R : (R <= 16 ? 53 + 5.4 * R : 46 + 6.1 * R); }
@@ -82,9 +84,9 @@ int swgb::launch_straighten(sw_ctx *c, int R, bool local, const FillTask *tasks,
 //   (columns x whole waves before the last strip + its place in the chain + columns) x step(R),
 // with step(R) the measured clocks of a step of one strip (GB300): few rows a
 // lane leave a long chain of short steps, many leave SMs idle.  Measured, score
-// fills: 8 kbp R = 4 / 6 / 8: 0.69 / 0.65 / 0.63 ms; 30 kbp R = 6 / 8 / 10:
-// 2.25 / 2.17 / 2.18; 200 kbp R = 12 / 14: 15.3 / 16.0; 1 Mbp R = 14 / 16 / 20:
-// 257 / 270 / 260 ms.
+// fills: 30 kbp R = 8 / 10: 2.17 / 2.18 ms; 200 kbp R = 12 / 14: 15.3 / 16.0;
+// 1 Mbp R = 14 / 16 / 20 / 26: 257 / 270 / 260 / 214 ms.  (4 and 6 rows a lane were tried
+// and not kept: 8 kbp R = 4 / 6 / 8 0.69 / 0.65 / 0.63 ms, 30 kbp R = 6 2.25.)
 // tiles: an alignment's forward fill.  Its traceback tiles are as high as a strip (128 R rows), and the
 // first round of them runs after the whole fill, kP16TileClocks a row of the side (R = 8 / 12 / 16: 230 / 350 /
 // 458 us at 2,070 MHz).

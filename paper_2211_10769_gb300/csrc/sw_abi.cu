@@ -261,7 +261,10 @@ constexpr int64_t kPackedMinSumVariant = 1024;
 // p16_rows_per_lane picks; else the int32 fill of pair_fill_config.  Below
 // kPackedMinSum rows plus columns the int32 fill's shorter set-up wins (score:
 // 500 x 500 0.094 against 0.096 ms, 1,000 0.135 against 0.132, 2 kbp 0.221
-// against 0.199, 30 kbp 2.55 against 2.17).  With the int16 profile (larger alphabets) it also keeps the
+// against 0.199, 30 kbp 2.55 against 2.17; protein pairs, whose steps are longer: 1,500 x 1,500 0.161
+// against 0.162, 2,000 0.198 against 0.186, 8,000 0.708 against 0.623, 35,000 3.03 against 2.61; the algorithms
+// without the zero floor from kPackedMinSumVariant on: protein NW 512 x 512 0.112 against 0.077, 8,000 1.16
+// against 0.68).  With the int16 profile (larger alphabets) it also keeps the
 // pairs of less than kPackedMinRows rows, one warp of either fill's strip: protein, packed against int32,
 // 64 x 3,000 199 against 182 us, 200 x 3,000 196 against 185, 64 x 100,000 4.99 against 4.85 ms, and beyond the line
 // 500 x 8,000 446 against 448, 1,000 x 8,000 459 against 467.

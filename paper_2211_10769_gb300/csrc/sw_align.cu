@@ -309,7 +309,7 @@ long long small_pair_tile(const sw_ctx *c, int64_t m, int64_t n, const DevScorin
 // all tiles, and every result copied back at once.  The banded path needs a
 // host round trip between the end cell and its band; for a pair whose tiles
 // fit one wave on the SMs, recomputing all of them costs no more time.  Such a call
-// is short (0.17 ms at 464 x 503), so it is five or six launches between one copy down and
+// is short (0.14 ms at 464 x 503), so it is five or six launches between one copy down and
 // one up: with a copy or memset for each of its parts, seventeen stream operations.
 int align_one_round(sw_ctx *c, const uint8_t *da, int64_t m, const uint8_t *db, int64_t n, const DevScoring &ds,
                     bool fold, const FillConfig &fwd, const FillConfig &tbc, int sw, int tsw, long long BT,
@@ -500,7 +500,7 @@ extern "C" int sw_align(sw_ctx *c, const uint8_t *a, int64_t m, const uint8_t *b
     // tiles hold whole traceback strips of an int32 forward fill's rows a lane; after the packed fill whole
     // row groups are enough (the last strip of a tile may be partial)
     const int HT = fwd.P16 ? 32 * tbc.R : fill_rows_per_strip(tbc);
-    const int HC2 = 4 * 32 * fwd.R;                // strip height of a coarse tile's refill (int32, 4 warps)
+    const int HC2 = 4 * 32 * fwd.R;                // strip height of a coarse tile's refill (4 warps)
     const long long BL = std::lcm((long long)HC, (long long)HT);
     const long long BL2 = std::lcm((long long)HC2, (long long)HT);
     auto ck_bytes = [&](long long bt) {

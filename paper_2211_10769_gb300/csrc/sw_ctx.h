@@ -121,7 +121,7 @@ bool p16_fits(const DevScoring &s, int R);
 bool p16_pair_profile(int K);              // the pair profile at 8 rows a lane fits K residue codes (else int16)
 int launch_fill16(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const FillLaunch &L, int K, long long tickets);
 int launch_fill16_batch(sw_ctx *c, const FillConfig &cfg, const FillLaunch &L, int K, long long tickets);
-// the global, semi-global and overlap algorithms: 8 or 16 rows a lane, four compute warps
+// the int32 fill of the global, semi-global and overlap algorithms: 8, 12 or 16 rows a lane, four compute warps
 FillConfig variant_fill_config(const sw_ctx *c, int64_t rows);
 int launch_fill_variant(sw_ctx *c, const FillConfig &cfg, int mode, bool fold, const FillLaunch &L, int K,
                         long long tickets);

@@ -195,9 +195,9 @@ int enqueue_step(sw_server *S, const std::vector<Slot *> &act, InFlight *next, i
     const int np = S->view.npairs;
     const int p0 = S->cur_chunk, p1 = np, stride = S->chunks;
     const int chunk_pairs = p0 < np ? (np - p0 + stride - 1) / stride : 0;
-    // the requests of a step run in groups of one tile shape each, every query with the shape
-    // that pads it least (one shape for all would pad a 100-residue query to a 512-row pass
-    // next to a long one); one launch per group
+    // the requests of a step run in groups of one tile shape each, every query with the shape that is
+    // fastest beside the step's other requests (one shape for all would pad a 100-residue query to a
+    // 512-row pass next to a long one); one launch per group
     std::map<int, std::vector<Slot *>> groups;
     const int maxlen = std::max(1, db_chunk_maxlen(S->db, p0, p0 + 1));   // pairs are sorted longest first
     double residues = 0;

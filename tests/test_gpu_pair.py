@@ -26,8 +26,8 @@ def ctx(request):
     runs on all three."""
     from paper_2211_10769_gb300 import binding, build
     build.build()
-    # packed16: the packed fill forced at 8 rows a lane (by default pairs up to 152 x 512 rows take
-    # the int32 fill, which has more SMs to use there)
+    # packed16: the packed fill forced at 8 rows a lane (by default small pairs take the int32
+    # fill, and the others the rows a lane of a model)
     env = {"SWGB_P16": "0" if request.param == "int32" else "1",
            "SWGB_ONE_ROUND": "1" if request.param == "one_round" else "0"}
     if request.param == "packed16":
