@@ -308,21 +308,17 @@ int finish_run(sw_batch *B, sw_hit *out) {
     return SW_OK;
 }
 
-// Launches the fill of shape f without strips, so that its kernel is loaded.
-int load_fill(sw_batch *B, const FillConfig &f, const DevScoring &sc) {
+// Launches the fill of shape f without strips, so that its kernel is loaded; zeros: a cleared ticket counter and error word.
+int load_fill(sw_batch *B, const FillConfig &f, const DevScoring &sc, const DevBuf &zeros) {
     sw_ctx *c = B->c;
-    DevBuf none;                       // the ticket counter and the error word
-    RC(none.ensure(64));
-    CU(cudaMemsetAsync(none.p, 0, 64, B->stream));
     FillLaunch L{};
-    L.ticket = static_cast<unsigned long long *>(none.p);
-    L.err = static_cast<int *>(none.p) + 4;
+    L.ticket = static_cast<unsigned long long *>(zeros.p);
+    L.err = static_cast<int *>(zeros.p) + 4;
     L.total = 0;
     const cudaStream_t saved = c->stream;
     c->stream = B->stream;
     const int rc = launch_fill(c, f, kModeScore, fold_open(sc), L, sc.K, 1);
     c->stream = saved;
-    CU(cudaStreamSynchronize(B->stream));
     return rc;
 }
 
@@ -490,7 +486,9 @@ extern "C" int sw_batch_create(sw_ctx *c, int64_t npairs, const uint8_t *a_res, 
         cudaEvent_t e0, e1;
         CU(cudaEventCreate(&e0));
         CU(cudaEventCreate(&e1));
-        int rc = SW_OK;
+        DevBuf zeros;
+        int rc = zeros.ensure(64);
+        if (!rc) rc = cudaMemsetAsync(zeros.p, 0, 64, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
         for (size_t k = 0; k < B->bins.size() && rc == SW_OK; ++k) {
             if (tuned[k]) continue;
             float best = 1e30f;
@@ -499,21 +497,16 @@ extern "C" int sw_batch_create(sw_ctx *c, int64_t npairs, const uint8_t *a_res, 
                 if (!is_candidate(cand, B->scorings[(size_t)B->bins[k].sidx])) continue;
                 B->bins[k].cfg = cand;
                 rc = build_plan(B);
-                // a kernel's first launch also loads it: one without strips before it is timed; and a run of less than a
-                // millisecond varies by a quarter: the best of three (a single, first run picked 41 us in place of 30 for
-                // one pair of 20 to 60 residues)
-                if (!rc) rc = load_fill(B, cand, B->scorings[(size_t)B->bins[k].sidx]);
-                float ms = 1e30f;
-                for (int run = 0, runs = 1; !rc && run < runs; ++run) {
-                    rc = cudaEventRecord(e0, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
-                    if (!rc) rc = enqueue_run(B);
-                    if (!rc) rc = cudaEventRecord(e1, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
-                    if (!rc) rc = cudaStreamSynchronize(B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
-                    float t = 0;
-                    if (!rc) rc = cudaEventElapsedTime(&t, e0, e1) == cudaSuccess ? SW_OK : SW_ECUDA;
-                    ms = std::min(ms, t);
-                    if (ms < 1.0f) runs = 3;
-                }
+                // a kernel's first launch also loads it: one without strips before it is timed (a first run picked 41 us in
+                // place of 30 for one pair of 20 to 60 residues; the best of three after it picked the same as one, at
+                // twice the time of the whole plan's making)
+                if (!rc) rc = load_fill(B, cand, B->scorings[(size_t)B->bins[k].sidx], zeros);
+                if (!rc) rc = cudaEventRecord(e0, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
+                if (!rc) rc = enqueue_run(B);
+                if (!rc) rc = cudaEventRecord(e1, B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
+                if (!rc) rc = cudaStreamSynchronize(B->stream) == cudaSuccess ? SW_OK : SW_ECUDA;
+                float ms = 0;
+                if (!rc) rc = cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess ? SW_OK : SW_ECUDA;
                 if (rc) break;
                 if (ms < best) { best = ms; pick = cand; }
             }
