@@ -42,8 +42,8 @@ WORKLOAD = "dna_pair_200kbp_align"
 # DRAM traffic of the forward fill measured by ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum of one full-size launch) per cell, and the kernel
 # sources it was taken on (None: not measured on the current kernel).
-FILL_TRAFFIC = {"mode": "align", "bytes_per_cell": 397.21e6 / (200_000 * 200_000),
-                "source_sha256": "5183a719e52367bf69a0a91a164dc189b2b80607905c3700eb55fd150f3c994f"}
+FILL_TRAFFIC = {"mode": "align", "bytes_per_cell": 396.68e6 / (200_000 * 200_000),
+                "source_sha256": "a81520930a8948710473e86cec0add85ef3e0577e341cb68e2c5847701d5f32e"}
 
 
 def parse():

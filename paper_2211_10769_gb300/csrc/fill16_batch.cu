@@ -1,7 +1,8 @@
 // fill16_batch.cu -- the packed 16-bit pair fill for batches: an int8 query
 // profile, so that three to five blocks fit an SM.  A batch's strips are
 // independent enough to fill several blocks an SM, where the ALU pipe is the
-// bound (79% busy with two blocks of four warps at 8 rows a lane).  1,500 pairs of
+// bound: 79% busy with the pair profile in two blocks of four warps at 8 rows a lane, 89%
+// with three blocks at 12 rows and the int8 profile.  1,500 pairs of
 // 3,072 x 4,000: DNA 3,280 GCUPS with the pair profile at its best shape (8 rows,
 // two blocks), 3,530 with 12 rows, int8 and three blocks; protein 3,050 and 3,350.
 #include "sw.h"
